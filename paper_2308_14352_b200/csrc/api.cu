@@ -8,6 +8,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "act_tile.cuh"
 #include "common.cuh"
 
 using namespace emoe;
@@ -78,8 +79,10 @@ WorkspaceLayout make_layout(const LayerDims& L, int T) {
   w.perm = o;         o += align_up(P * 4);
   w.slot_of_pair = o; o += align_up(P * 4);
   w.plan = o;         o += 2 * align_up(plan_bytes(L.E));  // two plans: one per kernel family of a forward call
-  w.xs = o;           o += align_up(L.act_bf16 ? P * L.d_model * 2 : 0);
-  w.hidden = o;       o += align_up(P * L.d_ff * (L.act_bf16 ? 2 : 4));
+  // activations: rows, or (weight-streaming kernel) tiles with the sums of their segments
+  const bool tiles = ffn_tma_supported(L);
+  w.xs = o;           o += align_up(L.act_bf16 ? P * (tiles ? act_slot_bytes(L.d_model) : static_cast<size_t>(L.d_model) * 2) : 0);
+  w.hidden = o;       o += align_up(P * (tiles ? act_slot_bytes(L.d_ff) : static_cast<size_t>(L.d_ff) * (L.act_bf16 ? 2 : 4)));
   // block scales of the integer activations (int8 tensor-core kernel): one fp32 per 128 inputs
   w.xsc = o;          o += align_up(ffn_i8_supported(L) ? P * (L.d_model / 128) * 4 : 0);
   w.hsc = o;          o += align_up(ffn_i8_supported(L) ? P * (L.d_ff / 128) * 4 : 0);
@@ -420,37 +423,36 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
     if (out_perm) EMOE_CUDA(ctx, cudaMemcpyAsync(out_perm, perm, sizeof(int32_t) * P, cudaMemcpyDeviceToDevice, st));
     return EMOE_OK;
   }
+  // rows of the tcgen05 kernel's activations: as far apart as a slot of the streaming kernel's tiles, so that the two
+  // families can share the buffers
+  const int xs_stride = static_cast<int>(act_slot_bytes(L.d_model) / 2), hid_stride = static_cast<int>(act_slot_bytes(L.d_ff) / 2);
   if (use_hybrid) {
-    // experts with up to HYBRID_STREAM_TOKENS tokens: passes of 8-token tiles through the streaming
+    // experts with up to HYBRID_STREAM_TOKENS tokens: one or two passes of the streaming
     // kernel; the others: 128-token tiles on tcgen05.  Each family has its own plan and writes only
     // its own slots of xs / hidden / o_part.
 #ifndef EMOE_HYBRID_TOKENS
 #define EMOE_HYBRID_TOKENS 32
 #endif
-#ifndef EMOE_HYBRID_TILES
-#define EMOE_HYBRID_TILES 1  // 8-token tiles per pass of the streaming family
-#endif
     constexpr int HYBRID_STREAM_TOKENS = EMOE_HYBRID_TOKENS;
     int* plan_heavy = reinterpret_cast<int*>(reinterpret_cast<char*>(plan) + align_up(plan_bytes(L.E)));
-    __nv_bfloat16* hid = reinterpret_cast<__nv_bfloat16*>(hidden);
     // many tokens in the call: the streaming family's tail matters little, every further split-K plane costs a
     // cleared and a re-read [P][d] fp32 array
     ksplit = ffn_tma_ksplit(L, T) < 2 ? ffn_tma_ksplit(L, T) : 2;
     EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, plan, xs, nullptr, P, 1, 1, HYBRID_STREAM_TOKENS, ctx->check_word, st));
-    EMOE_LAUNCH(ctx, launch_scatter_x16(L, table, x, ids_use, perm, off, plan_heavy, xs, P, HYBRID_STREAM_TOKENS + 1, INT_MAX, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_scatter_x16(L, table, x, ids_use, perm, off, plan_heavy, xs, xs_stride, P, HYBRID_STREAM_TOKENS + 1, INT_MAX, ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
     // the tcgen05 kernel writes plane 0 only: the other split-K planes of its slots must read as zero
     if (ksplit > 1)
       EMOE_CUDA(ctx, cudaMemsetAsync(o_part + static_cast<size_t>(P) * L.d_model, 0,
                                      static_cast<size_t>(ksplit - 1) * P * L.d_model * sizeof(float), st));
     if (ctx->fuse_projections) {
-      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 2, L, table, tmaps, xs, off, plan, hid, o_part, ksplit, P, T, EMOE_HYBRID_TILES, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
     } else {
-      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, table, tmaps, xs, off, plan, hid, o_part, ksplit, P, T, EMOE_HYBRID_TILES, ctx->check_word, st));
-      EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, table, tmaps, xs, off, plan, hid, o_part, ksplit, P, T, EMOE_HYBRID_TILES, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
     }
-    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, hidden, o_part, um_scratch, P, 1, ctx->check_word, st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hidden, o_part, um_scratch, P, 1, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, um_scratch, P, 1, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, um_scratch, P, 1, ctx->check_word, st));
     if (ev[1]) {  // one interval for the whole expert stage
       EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
       ctx->events_one_launch[ctx->events_used / 3 - 1] = 1;
@@ -463,11 +465,11 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
       ksplit = ffn_umma_zsplit(L, T, sms);
       if (ksplit > w.ksplit) ksplit = w.ksplit;  // the workspace holds w.ksplit planes
     }
-    EMOE_LAUNCH(ctx, launch_scatter_x16(L, table, x, ids_use, perm, off, plan, xs, P, 1, INT_MAX, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_scatter_x16(L, table, x, ids_use, perm, off, plan, xs, xs_stride, P, 1, INT_MAX, ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan, xs, hidden, o_part, um_scratch, P, 1, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan, xs, xs_stride, hidden, hid_stride, o_part, um_scratch, P, 1, ctx->check_word, st));
     if (ev[1]) EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan, hidden, hidden, o_part, um_scratch, P, ksplit, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan, hidden, hid_stride, hidden, hid_stride, o_part, um_scratch, P, ksplit, ctx->check_word, st));
   } else if (use_i8) {
     ksplit = ffn_i8_ksplit(L, T);
     if (one_launch_route)
@@ -508,19 +510,18 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
     else
       EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, plan, xs, nullptr, P, 1, 1, INT_MAX, ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
-    __nv_bfloat16* hid = reinterpret_cast<__nv_bfloat16*>(hidden);
     if (ctx->fuse_projections) {
       // one launch: an expert's second projection starts when its hidden vectors are complete
-      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 2, L, table, tmaps, xs, off, plan, hid, o_part, ksplit, P, T, 0, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
       if (ev[1]) {  // one interval only: the end event of the triple stays unused
         EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
         ctx->events_one_launch[ctx->events_used / 3 - 1] = 1;
         ev[2] = nullptr;
       }
     } else {
-      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, table, tmaps, xs, off, plan, hid, o_part, ksplit, P, T, 0, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
       if (ev[1]) EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
-      EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, table, tmaps, xs, off, plan, hid, o_part, ksplit, P, T, 0, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
     }
   } else if (use_mma) {
     ksplit = ffn_mma_ksplit(L, T);

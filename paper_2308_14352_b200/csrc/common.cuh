@@ -106,7 +106,7 @@ int ffn_mma_ksplit(const LayerDims& L, int T);
 int ffn_token_tiles(const LayerDims& L, int T);
 bool ffn_many_tokens(const LayerDims& L, int T);
 // plan (nullable): plan_bytes(E) bytes, the work plan for the persistent TMA kernels, filled by block 0.
-// fmt: 0 = bf16, 1 = fp16 (saturating; same layout: the TMA-staged kernel's input), 2 = two-limb
+// fmt: 0 = bf16, 1 = fp16 tiles (act_tile.cuh, saturating: the TMA-staged kernel's input), 2 = two-limb
 // block-scaled integers (act_q.cuh: the int8 tensor-core kernel's input; xsc receives the block scales).
 // cnt_lo .. cnt_hi: only experts with that many tokens are listed in the plan and have their rows
 // written (1 .. INT_MAX: all activated experts); lets two kernel families share one forward call.
@@ -144,11 +144,9 @@ int ffn_tma_ksplit(const LayerDims& L, int T);
 int encode_weight_tmap(void* out_map, const void* packed, int N, int K, int bits);
 // Phases [phase_begin, phase_end) of the FFN in one launch: (0,1) first projection, (1,2) second,
 // (0,2) both, the second projection of an expert starting as soon as its hidden vectors are complete.
-// token_tiles: 8-token tiles per pass (1, 2 or 4), 0 = by the routing statistics of (L, T).
-cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, const ExpertDev* experts,
-                           const void* tmaps, const __nv_bfloat16* xs, const int32_t* off, int* plan,
-                           __nv_bfloat16* hidden, float* o_part, int ksplit, int n_pairs, int T, int token_tiles,
-                           int* check_word, cudaStream_t st);
+// xs / hidden: activation tiles (act_tile.cuh).
+cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, const void* tmaps, const void* xs, int* plan,
+                           void* hidden, float* o_part, int ksplit, int n_pairs, int* check_word, cudaStream_t st);
 
 // The weight-streaming kernel on 8-bit integer tensor-core operands (tcgen05 kind::i8, accumulators
 // and unpacked codes in tensor memory).  xq / hq: activations as two-limb block-scaled integers
@@ -170,14 +168,15 @@ int encode_tmap_2d(void* out_map, int dtype, const void* base, uint64_t inner, u
                    uint32_t box_inner, uint32_t box_outer, bool swizzle128 = true);
 
 // tcgen05 grouped GEMM for experts with many tokens (fp16 operands, fp32 accumulation in tensor
-// memory).  xs16 / hidden16: activations in expert order, fp16, pair order; o: [n_pairs][d_model].
+// memory).  xs16 / hidden16: activations in expert order, fp16, pair order, rows xs_stride / hid_stride
+// values apart; o: [n_pairs][d_model].
 bool ffn_umma_supported(const LayerDims& L);
 cudaError_t launch_scatter_x16(const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* ids,
-                               const int32_t* perm, const int32_t* off, int* plan, void* xs16, int n_pairs,
+                               const int32_t* perm, const int32_t* off, int* plan, void* xs16, int xs_stride, int n_pairs,
                                int cnt_lo, int cnt_hi, int* check_word, cudaStream_t st);
 size_t ffn_umma_scratch_bytes(const LayerDims& L);  // scratch of the gated first projection (0 for other layers)
-cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, const int* plan, const void* in16,
-                            void* hidden16, float* o, float* scratch, int n_pairs, int zsplit, int* check_word,
+cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, const int* plan, const void* in16, int in_stride,
+                            void* hidden16, int hid_stride, float* o, float* scratch, int n_pairs, int zsplit, int* check_word,
                             cudaStream_t st);
 int ffn_umma_zsplit(const LayerDims& L, int T, int sms);  // 1 or 2 slices of the second projection's inputs per unit
 

@@ -220,7 +220,8 @@ __global__ void __launch_bounds__(128)
   if (e_slot < 0 || e_slot >= E) return;  // a slot the permutation did not write (stale entry behind a dropped pair)
   const int cnt_slot = off[e_slot + 1] - off[e_slot];
   if (cnt_slot < cnt_lo || cnt_slot > cnt_hi) return;  // this expert's rows belong to another kernel family
-  scatter_any(x + static_cast<size_t>(pair / top_k) * d, xs, xsc, slot, d, experts[e_slot].bits, fmt, check_word);
+  scatter_any(x + static_cast<size_t>(pair / top_k) * d, xs, xsc, off[e_slot], cnt_slot, slot - off[e_slot], d, experts[e_slot].bits, fmt,
+              check_word);
 }
 
 // Permutation and scatter in one launch for small batches (at most PS_MAX_PAIRS pairs): one CTA
@@ -237,7 +238,7 @@ __global__ void __launch_bounds__(128)
                            __nv_bfloat16* __restrict__ xs, float* __restrict__ xsc) {
   __shared__ int s_ids[PS_MAX_PAIRS];
   __shared__ int s_off[EMOE_MAX_EXPERTS + 1];
-  __shared__ int s_red[2][4];
+  __shared__ int s_red[3][4];
   pdl_wait();
   pdl_trigger();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -246,24 +247,27 @@ __global__ void __launch_bounds__(128)
   const int p = blockIdx.x;
   const int e = s_ids[p];
   const bool valid = e >= 0 && e < E;
-  // pairs in front of this one in expert order
-  int before = 0, same = 0;
+  // pairs of lower experts, and pairs of this one's expert: in front of it and in all
+  int lower = 0, rank = 0, same = 0;
   for (int q = tid; q < n_pairs; q += blockDim.x) {
     const int eq = s_ids[q];
-    before += (eq >= 0 && eq < e) || (eq == e && q < p);
+    lower += eq >= 0 && eq < e;
+    rank += eq == e && q < p;
     same += eq == e;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    before += __shfl_xor_sync(0xffffffffu, before, o);
-    same += __shfl_xor_sync(0xffffffffu, same, o);
-  }
+  lower = __reduce_add_sync(0xffffffffu, lower);
+  rank = __reduce_add_sync(0xffffffffu, rank);
+  same = __reduce_add_sync(0xffffffffu, same);
   if (lane == 0) {
-    s_red[0][warp] = before;
-    s_red[1][warp] = same;
+    s_red[0][warp] = lower;
+    s_red[1][warp] = rank;
+    s_red[2][warp] = same;
   }
   __syncthreads();
-  const int slot = s_red[0][0] + s_red[0][1] + s_red[0][2] + s_red[0][3];
+  lower = s_red[0][0] + s_red[0][1] + s_red[0][2] + s_red[0][3];
+  rank = s_red[1][0] + s_red[1][1] + s_red[1][2] + s_red[1][3];
+  same = s_red[2][0] + s_red[2][1] + s_red[2][2] + s_red[2][3];
+  const int slot = lower + rank;
   if (p == 0) {
     // counts, offsets, plan (this CTA only); invalid ids are reported and own no slot
     for (int ee = tid; ee <= E; ee += blockDim.x) s_off[ee] = 0;
@@ -289,9 +293,8 @@ __global__ void __launch_bounds__(128)
     perm[slot] = p;
     slot_of_pair[p] = slot;
   }
-  scatter_any(x + static_cast<size_t>(p / top_k) * d, xs, xsc, slot, d, experts[e].bits, fmt, check_word);
+  scatter_any(x + static_cast<size_t>(p / top_k) * d, xs, xsc, lower, same, rank, d, experts[e].bits, fmt, check_word);
 }
-
 
 }  // namespace
 

@@ -1,38 +1,49 @@
-// Grouped expert FFN on packed weights: TMA-staged weight stream + tensor-core multiply-adds,
-// for bf16 activations in the decode regime.  Paper Sections 1/2.1 (each activated expert is an
-// independent FFN) on the Section 3.2 storage (b-bit codes + scale channel, w~ = q * s formed
-// in registers).
+// Grouped expert FFN on packed weights: TMA-staged weight stream + tensor-core multiply-adds, for
+// bf16 activations with up to some tens of tokens per expert (decode, small prefill).  Paper
+// Sections 1/2.1 (each activated expert is an independent FFN) on the Section 3.2 storage (b-bit
+// codes + scale channel, w~ = q * s formed in registers).
 //
-// Same shape of arithmetic as ffn_mma.cu (codes as exact small integers in the A operand of
-// mma.m16n8k16, tokens as the N dimension, fp32 accumulation per 128-input segment, then
-// total += scale * segment), with two differences.  The operands are fp16: the codes are read
-// as offset codes c + q with one logic instruction per pair and the constant is taken out
-// again per segment (ffn_tile.cuh), and the activations (bf16 values) travel as fp16, exact
-// inside the fp16 range and saturated outside.  And the bytes travel differently: the kernel is
-// bound by streaming packed weights from HBM, so the bytes in flight must not depend on registers:
-//   * the kernel is persistent and runs BOTH projections of a layer: a CTA pulls work items
-//     (activated expert, block of output rows[, split-K slice]) from a device-side counter, the
-//     first projection's items before the second's, most expensive bitwidth first, and its
-//     producer warp runs ahead across item boundaries, so the weight stream never drains
-//     between tiles; an item of the second projection waits until the consumers of the first
-//     have counted the expert's hidden vectors complete (release / acquire on a counter in
-//     the expert's plan record);
-//   * the producer keeps a ring of STAGES shared-memory stages full.  One stage holds two
-//     64-row x 128-byte boxes of packed codes, fetched by two TMA tensor copies (128-byte
-//     swizzle, so that the consumers' 128-bit reads are conflict free), the matching slice of
-//     the expert's activations, fetched by one bulk copy per token row, and a small record
-//     that tells the consumers which item and which inputs the stage belongs to;
-//   * the producer's lanes also start small asynchronous copies (cp.async) of the stage's
-//     scales (128 rows x up to 4 segments, 16 bytes per row) that complete on the same
-//     mbarrier, so that no warp ever waits on a global load of a scale;
-//   * four consumer warps wait on the stage's mbarrier, read their 16-row tiles from shared
-//     memory, unpack step by step, issue the MMAs, and hand the stage back through a second
-//     mbarrier.
+// The codes are the A operand of mma.m16n8k16 (rows = output channels), tokens the N dimension,
+// products accumulate in fp32 per 128-input segment, then total += scale * segment.  The work is
+// bound by streaming packed weights from HBM and, at 4 and 2 bits, by the logic pipe (one
+// instruction per pair of codes, at half the issue rate), so both are kept lean:
+//   * the kernel is persistent and runs BOTH projections of a layer.  Every CTA takes every n-th item of
+//     a list: the first projection's (activated expert, block of output rows), then the second's
+//     (.., split-K slice), most expensive bitwidth first.  The stream runs ahead across items, so
+//     it never drains between tiles; an item of the second projection waits until the expert's
+//     hidden vectors are complete (release / acquire on a counter in the expert's plan record);
+//   * a stage holds two 64-row x 128-byte boxes of packed codes (two TMA tensor copies, 128-byte
+//     swizzle: the consumers' reads are conflict free), the rows' scales (cp.async) and the matching
+//     slice of the pass's activation tile (ONE bulk copy: the tile is stored segment-major, see
+//     act_tile.cuh).  Stages are cut from a ring in shared memory, each as large as it needs to
+//     be, because the activation part varies from 0.3 to 17 KB.  Two CTAs with some four stages
+//     each in flight reach the copy rate of the HBM (6.5 to 6.9 TB/s measured with idle consumers;
+//     one feeding thread per SM tops out at 5.2);
+//   * two feeding warps: one for the codes, one for activations and scales, so that a wait for hidden
+//     vectors does not keep the weight stream from running ahead.  They come first in the CTA: the
+//     schedulers favour old warps.  Items are decoded 32 at a time by the lanes of the first; a
+//     feeding thread between eight computing warps needs about twenty cycles per instruction,
+//     and whatever it does per stage shows;
+//   * eight consumer warps take one 16-row tile of the stage each (gated projection: eight rows of
+//     w1 and the same eight of w3, so that the activation is formed in one lane).  Sixteen consumer
+//     warps per SM alone, out of shared memory, run at 12 / 7.3 / 3.5 TB/s of 8 / 4 / 2-bit codes;
+//   * up to 8 tokens per pass: a code field is read in place as the mantissa of a SUBNORMAL fp16
+//     number ((q + 2^(b-1)) * 2^(p-24) for a field at bit p): one logic instruction per pair of
+//     codes, one shift per word.  Fields at different positions go to accumulators of their own,
+//     which are brought together once per segment; the offset's share 2^(b-1) * sum(x) comes with
+//     the activation tile.  The offset is as small as it can be (8 against codes of magnitude
+//     up to 8), so nothing is lost to cancellation.  9 to 16 tokens per pass: exact codes (one
+//     fp16x2 subtraction more per pair, shared by two token tiles).
 // 128 bytes of a row are 128 / 256 / 512 inputs at 8 / 4 / 2 bits, so a stage covers 1 / 2 / 4
 // scale segments.  Every wait is bounded: a wait that runs out sets a bit in the context's
 // check word and the CTA winds down without touching the stage.
+//
+// Measured (expert launch alone, start of comparison: one feeding and four computing warps per CTA, three CTAs,
+// 16 / 8-token tiles by the launch's mean): Mixtral-like layer (d 4096, f 14336), 23 tokens 245 -> 218 us
+// (3.7 TB/s of packed bytes), 4 tokens of 4-bit experts 2.8 -> 3.6 TB/s, 8 bits 4.7 -> 4.9, 2 bits 1.8 -> 2.2.
 #include <cuda.h>
 
+#include "act_tile.cuh"
 #include "common.cuh"
 #include "ffn_tile.cuh"
 #include "pipe.cuh"
@@ -40,36 +51,21 @@
 namespace emoe {
 namespace {
 
-// Consumer warps of a CTA: four, each with two 16-row tiles of a stage's 128 rows; or (SPLIT) eight,
-// one tile each, in CTAs that are fewer per SM but bring more consumer warps to it in all: the
-// consumers are bound by the latency of their own instruction stream, which more warps hide.
-__host__ __device__ constexpr int consumer_warps(bool split) { return split ? 8 : 4; }
-__host__ __device__ constexpr int tma_threads(bool split) { return (consumer_warps(split) + 1) * 32; }  // + the producer warp
-#ifndef EMOE_TMA_SPLIT_NT1
-#define EMOE_TMA_SPLIT_NT1 0  // 1: 8-token tiles take the eight-warp variant (as measured: slower, see consumer_warps)
+constexpr int ST_WARPS = 8;                      // consumer warps of a CTA
+constexpr int ST_THREADS = (ST_WARPS + 2) * 32;  // + the weight warp and the activation warp
+constexpr int ST_PLAN_CACHE = 64;                // plan records a CTA keeps in shared memory
+constexpr int ST_CTAS = 2;                       // per SM
+constexpr int ST_BOX_ROWS = 64;
+constexpr int ST_BOX_BYTES = ST_BOX_ROWS * 128;  // 8 KB
+constexpr int ST_X_OFFSET = 2 * ST_BOX_BYTES + 2 * ST_BOX_ROWS * 16;  // a stage: two boxes, 16 bytes of scales per row, the activation slice
+#ifndef EMOE_ST_RING_KB
+#define EMOE_ST_RING_KB 96
 #endif
-#ifndef EMOE_TMA_SPLIT_STAGES
-#define EMOE_TMA_SPLIT_STAGES 4
-#endif
-#ifndef EMOE_TMA_SPLIT_CTAS
-#define EMOE_TMA_SPLIT_CTAS 2
-#endif
-constexpr int TMA_SCALE_BYTES = 128 * 16;                   // raw scales of a stage: 16 bytes per row
-constexpr int TMA_BOX_ROWS = 64;
-constexpr int TMA_BOX_BYTES = TMA_BOX_ROWS * 128;  // 8 KB
-constexpr int TMA_XROW_MAX = 512 * 2 + 64;         // bytes per token row of a stage (row stride = 64 mod 128)
-#ifndef EMOE_TMA_STAGES_NT1
-#define EMOE_TMA_STAGES_NT1 2
-#endif
-#ifndef EMOE_TMA_UNROLL_SEGS
-#define EMOE_TMA_UNROLL_SEGS 0
-#endif
-#ifndef EMOE_TMA_L2PROMO
-#define EMOE_TMA_L2PROMO CU_TENSOR_MAP_L2_PROMOTION_L2_256B
-#endif
-#ifndef EMOE_TMA_CTAS_NT1
-#define EMOE_TMA_CTAS_NT1 3
-#endif
+constexpr int ST_RING = EMOE_ST_RING_KB * 1024;
+constexpr int ST_SLOTS = 8;                      // stages in flight at most (barriers, records)
+constexpr int ST_HID_BYTES = ACT_PASS_MAX * 256;  // one segment of hidden values on their way out
+constexpr int ST_SMEM = ST_RING + 2 * ST_HID_BYTES + 1024;  // + slack to align the base to 1024
+static_assert(ST_X_OFFSET + 4 * (ACT_PASS_MAX * 256) + 1023 <= ST_RING / 2, "two of the largest stages fit the ring");
 
 // MMA row g of a 16-row tile -> row of the shared-memory box, chosen per bitwidth so that the
 // lanes of one shared-memory transaction fall into different 16-byte columns after the swizzle.
@@ -80,60 +76,19 @@ __device__ __forceinline__ int box_row_of(int g) {
   return ((g & 3) << 1) | (g >> 2);
 }
 
-// the lane's raw codes of one row for segment `sg` of the stage: `row` points at the row's 128
-// bytes inside a swizzled box, `swz` is the row's swizzle term (row index mod 8)
-template <int BITS>
-__device__ __forceinline__ Raw<BITS> lds_raw(const unsigned char* row, int swz, int sg, int t);
-template <>
-__device__ __forceinline__ Raw<8> lds_raw<8>(const unsigned char* row, int swz, int sg, int t) {
-  (void)sg;
-  Raw<8> r;
-  r.v[0] = *reinterpret_cast<const uint4*>(row + (((2 * t) ^ swz) << 4));
-  r.v[1] = *reinterpret_cast<const uint4*>(row + (((2 * t + 1) ^ swz) << 4));
-  return r;
-}
-template <>
-__device__ __forceinline__ Raw<4> lds_raw<4>(const unsigned char* row, int swz, int sg, int t) {
-  Raw<4> r;
-  r.v[0] = *reinterpret_cast<const uint4*>(row + (((4 * sg + t) ^ swz) << 4));
-  return r;
-}
-template <>
-__device__ __forceinline__ Raw<2> lds_raw<2>(const unsigned char* row, int swz, int sg, int t) {
-  Raw<2> r;
-  r.v[0] = *reinterpret_cast<const uint2*>(row + (((2 * sg + (t >> 1)) ^ swz) << 4) + ((t & 1) << 3));
-  return r;
-}
-
-// a stage = two weight boxes + the activation tile, padded so that every stage (and with it
-// every swizzled box) starts on a 1024-byte boundary
-__host__ __device__ constexpr int stage_bytes_for(int nt) {
-  return 2 * TMA_BOX_BYTES + (nt * 8 * TMA_XROW_MAX + TMA_SCALE_BYTES + 1023) / 1024 * 1024;
-}
-__host__ __device__ constexpr int scale_tile_offset(int nt) { return 2 * TMA_BOX_BYTES + nt * 8 * TMA_XROW_MAX; }
-
-// The scales a stage needs from row n (groups of inputs k0 .. k0 + 128*segs) sit in one short
-// byte window of the scale channel; it is copied from the 4-byte boundary at or below its start.
-// group index of input k (groups of G inputs, G a multiple of 128 or the whole row);
-// gshift = log2(G) when G is a power of two, else -1
-__device__ __forceinline__ int group_of(int k, int gshift, int G, int ngroups) {
-  return ngroups == 1 ? 0 : (gshift >= 0 ? (k >> gshift) : k / G);
-}
-
 struct TmaArgs {
   int phase_begin, phase_end;  // projections this launch runs: [0,1), [1,2) or both, [0,2)
   LayerDims L;
-  const ExpertDev* experts;
   const CUtensorMap* tmaps;  // [E][3]
-  const __half* xs;          // input of the first projection (tokens in expert order, fp16)
-  const int32_t* off;
-  int* plan;  // header {activated experts, item counters} + one PlanRec per activated expert
-  __half* hidden;         // output of the first projection, input of the second (bf16 values as fp16)
+  const unsigned char* xs;   // input tiles of the first projection (act_tile.cuh)
+  int* plan;                 // header {activated experts, item counters} + one PlanRec per activated expert
+  unsigned char* hidden;     // output tiles of the first projection, input of the second
   float* o_part;
   int ksplit;         // split-K slices of the second projection
   int row_blocks[2];  // row blocks of an expert per projection
   int ngroups[2];     // scale groups per row, per projection
-  int gshift;         // log2(group size) if it is a power of two, else -1
+  bool scale_pairs[2];  // one fp16 scale per segment, an even number of them per row, per projection
+  unsigned gmul;      // scale group of segment s: (s * gmul) >> 20 (2^20 / segments per group, rounded up; 0: one group per row)
   int n_pairs;
   int* check_word;
   // floor(2^32 / d) + 1 for the divisors of the item index, per projection: n / d = umulhi(n, magic) for the
@@ -143,171 +98,145 @@ struct TmaArgs {
 
 __host__ __device__ inline uint32_t div_magic(uint32_t d) { return d <= 1 ? 0u : static_cast<uint32_t>((1ull << 32) / d) + 1u; }
 __device__ __forceinline__ int fast_div(int n, int d, uint32_t magic) { return d <= 1 ? n : static_cast<int>(__umulhi(static_cast<uint32_t>(n), magic)); }
+// exact for rows of up to 2^17 inputs: s * (segments per group) stays below 2^20
+__device__ __forceinline__ int group_of_seg(const TmaArgs& a, int seg) { return static_cast<int>((static_cast<unsigned>(seg) * a.gmul) >> 20); }
 
-// what differs between the two projections
-struct PhaseDims {
-  int K, N, rows_per_item, row_blocks, ksplit, mat_first;
-  bool swiglu_in;
-  uint32_t mg_units, mg_ksplit, mg_rb;
+// One item of a CTA's list: a block of output rows of an expert (and a slice of the inputs in the second
+// projection), all tokens of the expert in passes of at most ACT_PASS_MAX.
+struct __align__(16) ItemRec {
+  int flags;            // ITEM_*; bits 8.. the width of the codes
+  int nst, seg0, last;  // stages per pass, first segment, segments of the last stage (0: an empty split-K slice)
+  int begin, cnt;       // the expert's slots
+  int rbz, ai;          // row block | slice << 16, plan record
+  const char* scales[2];   // scale channels of the item's matrices (second: w3 of a gated projection)
+  const CUtensorMap* map;  // packed codes; a gated projection's w3 follows
+  int row0, pad;
 };
-__device__ __forceinline__ PhaseDims phase_dims(const TmaArgs& a, int phase) {
-  PhaseDims d;
-  d.K = phase == 0 ? a.L.d_model : a.L.d_ff;
-  d.N = phase == 0 ? a.L.d_ff : a.L.d_model;
-  d.swiglu_in = phase == 0 && a.L.act == EMOE_ACT_SWIGLU;
-  d.rows_per_item = d.swiglu_in ? TMA_BOX_ROWS : 2 * TMA_BOX_ROWS;
-  d.row_blocks = a.row_blocks[phase];
-  d.ksplit = phase == 0 ? 1 : a.ksplit;
-  d.mat_first = phase == 0 ? 0 : (a.L.act == EMOE_ACT_SWIGLU ? 2 : 1);
-  d.mg_units = a.mg_units[phase];
-  d.mg_ksplit = a.mg_ksplit[phase];
-  d.mg_rb = a.mg_rb[phase];
-  return d;
-}
-
-// what a stage holds, written by the producer before it arms the stage's barrier
-struct StageMeta {
-  int e, rb, z, begin, p0, ntok, k0, bits;
-  int flags;  // 1 = first stage of an item pass, 2 = last, 4 = no more work, 8 = stage carries no inputs,
-              // 16 = last stage of a first-projection item whose completion the second projection waits for
-  int phase;
-  int ai;  // index of the expert's plan record
-  int pad;
-};
-constexpr int META_FIRST = 1, META_LAST = 2, META_STOP = 4, META_EMPTY = 8, META_DONE = 16;
+constexpr int ITEM_STOP = 1;
+constexpr int ITEM_SECOND = 2;  // of the second projection
+constexpr int ST_QUEUE = 64;    // records kept: decoded 32 at a time, nobody is more than ST_SLOTS stages behind
+static_assert(ST_QUEUE >= 64, "a half of the queue is rewritten while the other is in use");
 
 // How long the second projection of an expert waits for its hidden vectors (polls of ~0.1 us).
 constexpr unsigned DEP_WAIT_LIMIT = 1u << 20;
 
-template <int BITS, int NT, bool SPLIT>
-__device__ __forceinline__ void consume_stage(const TmaArgs& a, int phase, int rb, int k0, int ntok,
-                                              const unsigned char* st, int warp_full, int lane, uint32_t bar_empty,
-                                              float (&tot)[2][NT][4]) {
-  // SPLIT: warps 2p and 2p+1 share the 32 rows (or the w1 / w3 tiles) that warp p owns otherwise
-  const int warp = SPLIT ? warp_full >> 1 : warp_full;
-  const int mt_own = warp_full & 1;
-  constexpr int KSPAN = 1024 / BITS;  // inputs per stage (128 bytes of a row)
-  constexpr int SEGS = KSPAN / 128;   // scale segments per stage
-  // one token tile: offset codes (fewest instructions per code); more: exact codes (no MMAs for
-  // the constants, which would have to be repeated per token tile)
-  constexpr bool OFFSET_CODES = NT == 1 && BITS != 8;
-  const LayerDims& L = a.L;
-  const int K = phase == 0 ? L.d_model : L.d_ff;
-  const bool swiglu_in = phase == 0 && L.act == EMOE_ACT_SWIGLU;
-  const int g = lane >> 2, t = lane & 3;
-  const int gp = box_row_of<BITS>(g);
-  const int N = phase == 0 ? L.d_ff : L.d_model;
-  const int ngroups = a.ngroups[phase];
-  const int ssz = L.scale_f16 ? 2 : 4;
-  const int nseg = min(SEGS, (K - k0) / 128);
-  const int g0 = group_of(k0, a.gshift, L.group, ngroups);
-  // Everything that does not depend on the segment, once per stage.  The lane's four rows (2
-  // tiles x rows gp, gp+8) sit at fixed distances from the first one, in the boxes (128 bytes
-  // per row) and in the scale tile (16 bytes per row): tile 1 is the other box (gated
-  // projection) or 16 rows further down, rows gp+8 are 8 rows further down.  A row's scale
-  // window starts at the 4-byte boundary at or below its first scale of the stage; the rows of a
-  // lane are an even number of rows apart, so the distance to that boundary is the same for all.
-  const int swz = gp & 7;  // swizzle term of all four rows (they differ by multiples of 8)
-  const int box_first = swiglu_in ? 0 : (warp >> 1);
-  const int r_first = (swiglu_in ? 16 * warp : 32 * (warp & 1)) + gp;
-  const int nrow = (swiglu_in ? rb * TMA_BOX_ROWS + 16 * warp : rb * 2 * TMA_BOX_ROWS + 32 * warp) + gp;
-  const int dmt = swiglu_in ? TMA_BOX_BYTES : 16 * 128;
-  const unsigned char* row_base = st + box_first * TMA_BOX_BYTES + r_first * 128;
-  const unsigned char* sc_base = st + scale_tile_offset(NT) + (box_first * TMA_BOX_ROWS + r_first) * 16 +
-                                 (((min(nrow, N - 1) * ngroups + g0) * ssz) & 3);
-  const unsigned char* xlane = st + 2 * TMA_BOX_BYTES + g * TMA_XROW_MAX + t * 16;
-#if EMOE_TMA_UNROLL_SEGS
+// ---- codes -> A operand registers --------------------------------------------------------------
+// The MMA `m` (0..7) of a segment takes two pairs of codes per row (registers lo, hi), class
+// code_class(m) of field positions; see act_tile.cuh for the order of the inputs.
+template <int BITS>
+__device__ __forceinline__ constexpr int code_class(int m) { return BITS == 2 ? (m & 3) : (m & 1); }
+template <int BITS>
+__device__ __forceinline__ constexpr int field_pos(int m) { return BITS == 8 ? 0 : (BITS == 4 ? 4 * (m & 1) : 2 * (m & 3)); }
+template <int BITS>
+__device__ __forceinline__ constexpr int word_of(int m) { return BITS == 8 ? m : (BITS == 4 ? m >> 1 : m >> 2); }
+template <int BITS>
+__device__ __forceinline__ constexpr uint32_t field_mask() { return BITS == 8 ? 0x00FF00FFu : (BITS == 4 ? 0x000F000Fu : 0x00030003u); }
+template <int BITS>
+__device__ __forceinline__ constexpr uint32_t sign_bits() { return BITS == 8 ? 0x00800080u : (BITS == 4 ? 0x00080008u : 0x00020002u); }
+
+// offset codes as subnormal fp16 numbers: (q + 2^(b-1)) * 2^(pos - 24)
+template <int BITS>
+__device__ __forceinline__ uint32_t code_sub(uint32_t w, int pos) { return and_xor(w, field_mask<BITS>() << pos, sign_bits<BITS>() << pos); }
+// exact codes: the field under the exponent that makes its lowest bit weigh 1, the constant subtracted
+template <int BITS>
+__device__ __forceinline__ uint32_t code_exact(uint32_t w, int pos) {
+  const uint32_t one = (static_cast<uint32_t>(25 - pos) << 10) * 0x00010001u;  // 2^(10-pos): mantissa bit pos weighs 1
+  const uint32_t c = one | (sign_bits<BITS>() << pos);                         // 2^(10-pos) + 2^(b-1)
+  return f16x2_sub(and_xor(w, field_mask<BITS>() << pos, c), c);
+}
+
+// Where a lane finds its operands in a stage: its first row of codes (the 16-byte column of segment 0 under the
+// swizzle: the columns of later segments differ by an XOR), the distance to its second row, the even
+// chunks of the activation tile (the odd ones: XOR 64), the code offset's shares, and its rows' scales.
+struct StageLane {
+  int row, drow, xe, init, sc, dsc;
+  bool halves;  // the offset's share comes in two halves
+};
+
+// One segment (128 inputs) of the warp's 16 rows; SG: its index in the stage.
+template <int BITS, int NT>
+__device__ __forceinline__ void consume_segment(const unsigned char* stage, const StageLane& p, int sg, int xoff, float s0, float s1,
+                                                float (&tot)[NT][4]) {
+  constexpr int NW = BITS;  // 32-bit words of the lane's 32 codes of a row
+  uint32_t w[2][NW];
 #pragma unroll
-#else
-#pragma unroll 1
-#endif
-  for (int sg = 0; sg < SEGS; ++sg) {
-    if (sg < nseg) {
-      // B fragments: piece q of lane t sits at (q*4 + t) * 16 bytes of the segment
-      uint4 bq[NT][4];
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        if (nt * 8 < ntok) {
-          const unsigned char* src = xlane + nt * 8 * TMA_XROW_MAX + sg * 256;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) bq[nt][q] = *reinterpret_cast<const uint4*>(src + q * 64);
-        }
-      }
-      // - sum_k c_k x_k of the segment (see ffn_tile.cuh): the same for every output channel, so
-      // one pair of MMAs per step, with the constants as A operand, serves both 16-row tiles
-      float osum[NT][2];  // per token (2t, 2t+1)
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        float da[4] = {0.0f, 0.0f, 0.0f, 0.0f}, db[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        if (OFFSET_CODES && nt * 8 < ntok) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            mma_f16(da, offset_const<BITS>(0), offset_const<BITS>(0), offset_const<BITS>(1), offset_const<BITS>(1),
-                    bq[nt][q].x, bq[nt][q].y);
-            mma_f16(db, offset_const<BITS>(2), offset_const<BITS>(2), offset_const<BITS>(3), offset_const<BITS>(3),
-                    bq[nt][q].z, bq[nt][q].w);
-          }
-        }
-        osum[nt][0] = -(da[0] + db[0]);
-        osum[nt][1] = -(da[1] + db[1]);
-      }
-      const int sdelta = (group_of(k0 + sg * 128, a.gshift, L.group, ngroups) - g0) * ssz;
-      // one 16-row tile at a time, one k16-pair step at a time: the codes of a step live in 8
-      // registers and go straight into the MMAs.  The k-steps alternate between two partial
-      // accumulators so that consecutive MMAs do not depend on each other; the first starts from
-      // the constant's share.
-#pragma unroll
-      for (int mi = 0; mi < (SPLIT ? 1 : 2); ++mi) {
-        const int mt = SPLIT ? mt_own : mi;  // which tile; its totals live in tot[mi]
-        const Raw<BITS> raw0 = lds_raw<BITS>(row_base + mt * dmt, swz, sg, t);
-        const Raw<BITS> raw1 = lds_raw<BITS>(row_base + mt * dmt + 8 * 128, swz, sg, t);
-        const unsigned char* sc = sc_base + mt * (dmt >> 3) + sdelta;
-        float s0, s1;
-        if (ssz == 2) {
-          s0 = __half2float(*reinterpret_cast<const __half*>(sc));
-          s1 = __half2float(*reinterpret_cast<const __half*>(sc + 8 * 16));
-        } else {
-          s0 = *reinterpret_cast<const float*>(sc);
-          s1 = *reinterpret_cast<const float*>(sc + 8 * 16);
-        }
-        float pa[NT][4], pb[NT][4];
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          pa[nt][0] = pa[nt][2] = osum[nt][0];
-          pa[nt][1] = pa[nt][3] = osum[nt][1];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) pb[nt][i] = 0.0f;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          uint32_t c0[4], c1[4];
-          if (OFFSET_CODES) {
-            unpack_step_off(raw0, q, c0);
-            unpack_step_off(raw1, q, c1);
-          } else {
-            unpack_step_exact(raw0, q, c0);
-            unpack_step_exact(raw1, q, c1);
-          }
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt)
-            if (nt * 8 < ntok) {
-              mma_f16(pa[nt], c0[0], c1[0], c0[1], c1[1], bq[nt][q].x, bq[nt][q].y);
-              mma_f16(pb[nt], c0[2], c1[2], c0[3], c1[3], bq[nt][q].z, bq[nt][q].w);
-            }
-        }
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          tot[mi][nt][0] = fmaf(s0, pa[nt][0] + pb[nt][0], tot[mi][nt][0]);
-          tot[mi][nt][1] = fmaf(s0, pa[nt][1] + pb[nt][1], tot[mi][nt][1]);
-          tot[mi][nt][2] = fmaf(s1, pa[nt][2] + pb[nt][2], tot[mi][nt][2]);
-          tot[mi][nt][3] = fmaf(s1, pa[nt][3] + pb[nt][3], tot[mi][nt][3]);
-        }
+  for (int i = 0; i < 2; ++i) {
+    if constexpr (BITS == 2) {
+      const uint2 v = *reinterpret_cast<const uint2*>(stage + (p.row ^ (sg << 5)) + i * p.drow);
+      w[i][0] = v.x, w[i][1] = v.y;
+    } else {
+      const uint4 v = *reinterpret_cast<const uint4*>(stage + (p.row ^ (BITS == 4 ? sg << 6 : 0)) + i * p.drow);
+      w[i][0] = v.x, w[i][1] = v.y, w[i][2] = v.z, w[i][3] = v.w;
+      if constexpr (BITS == 8) {
+        const uint4 u = *reinterpret_cast<const uint4*>(stage + (p.row ^ 16) + i * p.drow);
+        w[i][4] = u.x, w[i][5] = u.y, w[i][6] = u.z, w[i][7] = u.w;
       }
     }
   }
-  // shared memory of the stage is no longer needed
-  __syncwarp();
-  if (lane == 0) mbar_arrive(bar_empty);
+  if constexpr (NT == 1) {
+    constexpr int NC = BITS == 2 ? 4 : 2;
+    float acc[NC][4];
+    float2 off = *reinterpret_cast<const float2*>(stage + p.init + xoff);
+    if (p.halves) {
+      const float2 o2 = *reinterpret_cast<const float2*>(stage + p.init + xoff + 32);
+      off.x += o2.x;
+      off.y += o2.y;
+    }
+    acc[0][0] = acc[0][2] = off.x;
+    acc[0][1] = acc[0][3] = off.y;
+#pragma unroll
+    for (int c = 1; c < NC; ++c)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[c][i] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint4 b = *reinterpret_cast<const uint4*>(stage + (p.xe ^ ((q & 1) << 6)) + xoff + 128 * (q >> 1));
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int m = 2 * q + j, pos = field_pos<BITS>(m);
+        const uint32_t u0 = w[0][word_of<BITS>(m)], u1 = w[1][word_of<BITS>(m)];
+        mma_f16(acc[code_class<BITS>(m)], code_sub<BITS>(u0, pos), code_sub<BITS>(u1, pos), code_sub<BITS>(u0 >> 8, pos),
+                code_sub<BITS>(u1 >> 8, pos), j ? b.z : b.x, j ? b.w : b.y);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float v;
+      if constexpr (BITS == 8) v = acc[0][i] + acc[1][i];
+      else if constexpr (BITS == 4) v = fmaf(acc[1][i], 0.0625f, acc[0][i]);
+      else v = fmaf(fmaf(acc[3][i], 0.25f, acc[2][i]), 0.0625f, fmaf(acc[1][i], 0.25f, acc[0][i]));
+      tot[0][i] = fmaf(i < 2 ? s0 : s1, v, tot[0][i]);
+    }
+  } else {
+    float acc[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[nt][i] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t c[2][4];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int m = 2 * q + j, pos = field_pos<BITS>(m);
+          const uint32_t u = w[i][word_of<BITS>(m)];
+          c[i][2 * j] = code_exact<BITS>(u, pos);
+          c[i][2 * j + 1] = code_exact<BITS>(u >> 8, pos);
+        }
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        const uint4 b = *reinterpret_cast<const uint4*>(stage + (p.xe ^ ((q & 1) << 6)) + xoff + 128 * (q >> 1) + nt * 2048);
+        mma_f16(acc[nt], c[0][0], c[1][0], c[0][1], c[1][1], b.x, b.y);
+        mma_f16(acc[nt], c[0][2], c[1][2], c[0][3], c[1][3], b.z, b.w);
+      }
+    }
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) tot[nt][i] = fmaf(i < 2 ? s0 : s1, acc[nt][i], tot[nt][i]);
+  }
 }
 
 // This warp's share of an expert's hidden vectors is written: make it visible to the bulk copies
@@ -321,445 +250,522 @@ __device__ __forceinline__ void count_item_done(PlanRec* recs, int ai, int lane)
     asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(&recs[ai].done), "r"(1) : "memory");
 }
 
-// the hidden vector is rounded to bf16 (the layer's activation type), then carried as fp16;
-// the same without the report: a saturated value is recognised afterwards by its bit pattern (+-65504 is
-// not a bf16 number, so a hidden value can only be there by saturation), for the positions that are stored
+// the hidden vector is rounded to bf16 (the layer's activation type), then carried as fp16; a
+// saturated value is recognised by its bit pattern (+-65504 is not a bf16 number, so a hidden value
+// can only be there by saturation)
 __device__ __forceinline__ __half hidden_half(float h) { return f32_to_f16_sat(__bfloat162float(__float2bfloat16_rn(h))); }
 __device__ __forceinline__ bool half_saturated(__half v) { return (__half_as_ushort(v) & 0x7fffu) == 0x7bffu; }
 
-// results of one item pass: lane holds rows (gp, gp+8) x tokens (2t, 2t+1) of every tile.
-// SPLIT: a warp holds one tile (tot[0]); in a gated first projection the warp with the w3 tile
-// hands its totals to the warp with the w1 tile of the same rows through shared memory (xch, one
-// slot per warp pair, guarded by a full / free pair of barriers with bounded waits).
-template <int BITS, int NT, bool SPLIT>
-__device__ __forceinline__ bool store_item(const TmaArgs& a, const StageMeta& m, int warp_full, int lane,
-                                           float (&tot)[2][NT][4], float* xch, uint32_t bar_x, int& n_exchanged,
-                                           volatile int* abort_flag) {
-  const LayerDims& L = a.L;
-  const int N = m.phase == 0 ? L.d_ff : L.d_model;
-  const bool swiglu_in = m.phase == 0 && L.act == EMOE_ACT_SWIGLU;
-  const int warp = SPLIT ? warp_full >> 1 : warp_full;
-  const int mt_own = warp_full & 1;
+// Hidden values of a first-projection item: the lane's results (rows gp, gp+8 x tokens 2t, 2t+1 of
+// every 8-token tile) into the warp-shared tile segment in shared memory, in the order the second
+// projection reads them.
+template <int BITS, int NT>
+__device__ __forceinline__ void hidden_to_smem(bool gated, int rb, int ntok, int warp, int lane, const float (&tot)[NT][4],
+                                               unsigned char* hid, int* check_word) {
   const int g = lane >> 2, t = lane & 3;
   const int gp = box_row_of<BITS>(g);
-  if (SPLIT && swiglu_in) {
-    float* slot = xch + warp * (NT * 4 * 32);
-    const uint32_t full = bar_x + 8 * (2 * warp), free_ = bar_x + 8 * (2 * warp + 1);
-    const uint32_t par = n_exchanged & 1;
-    ++n_exchanged;
-    if (mt_own == 1) {  // the w3 tile: hand over, nothing to store
-      if (!mbar_wait(free_, par ^ 1, a.check_word, abort_flag)) return false;
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) slot[(nt * 4 + i) * 32 + lane] = tot[0][nt][i];
-      __syncwarp();
-      if (lane == 0) mbar_arrive(full);
-      return true;
-    }
-    if (!mbar_wait(full, par, a.check_word, abort_flag)) return false;
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) tot[1][nt][i] = slot[(nt * 4 + i) * 32 + lane];
-    __syncwarp();
-    if (lane == 0) mbar_arrive(free_);
-  }
-  // Values first, for all positions at once (independent instruction streams), then the stores under
-  // their predicates: a position-by-position loop with early exits ran as one long dependent chain.
   bool beyond = false;
-  if (swiglu_in) {
-    __half hv[NT][4];
+  if (gated) {
+    const int n = (rb & 1) * 64 + 8 * warp + gp;  // channel inside its 128-input segment
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
+    for (int nt = 0; nt < NT; ++nt) {
+      if (nt * 8 >= ntok) break;
+      __half hv[2];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float av = tot[0][nt][i], bv = tot[1][nt][i];
-        hv[nt][i] = hidden_half(av / (1.0f + expf(-av)) * bv);
+      for (int i = 0; i < 2; ++i) {
+        const float av = tot[nt][i], bv = tot[nt][i + 2];
+        hv[i] = hidden_half(av / (1.0f + expf(-av)) * bv);
       }
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
+      for (int i = 0; i < 2; ++i) {
+        const int tok = nt * 8 + 2 * t + i;
+        if (tok < ntok) {
+          *reinterpret_cast<__half*>(hid + tok * 256 + act_tile_pos<BITS>(n, tok)) = hv[i];
+          beyond |= half_saturated(hv[i]);
+        }
+      }
+    }
+  } else {
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      if (nt * 8 >= ntok) break;
+      __half hv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) hv[i] = hidden_half(fmaxf(tot[nt][i], 0.0f));
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int tok = nt * 8 + 2 * t + (i & 1);
-        const int n = m.rb * TMA_BOX_ROWS + 16 * warp + gp + 8 * (i >> 1);
-        if (tok < m.ntok && n < N) {
-          a.hidden[static_cast<size_t>(m.begin + m.p0 + tok) * N + act_pos<BITS>(n)] = hv[nt][i];
-          beyond |= half_saturated(hv[nt][i]);
+        if (tok < ntok) {
+          *reinterpret_cast<__half*>(hid + tok * 256 + act_tile_pos<BITS>(16 * warp + gp + 8 * (i >> 1), tok)) = hv[i];
+          beyond |= half_saturated(hv[i]);
         }
       }
-  } else if (m.phase == 0) {
-    __half hv[2][NT][4];
-#pragma unroll
-    for (int mi = 0; mi < (SPLIT ? 1 : 2); ++mi)
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) hv[mi][nt][i] = hidden_half(fmaxf(tot[mi][nt][i], 0.0f));
-#pragma unroll
-    for (int mi = 0; mi < (SPLIT ? 1 : 2); ++mi)
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int mt = SPLIT ? mt_own : mi;
-          const int tok = nt * 8 + 2 * t + (i & 1);
-          const int n = m.rb * 2 * TMA_BOX_ROWS + 32 * warp + 16 * mt + gp + 8 * (i >> 1);
-          if (tok < m.ntok && n < N) {
-            a.hidden[static_cast<size_t>(m.begin + m.p0 + tok) * N + act_pos<BITS>(n)] = hv[mi][nt][i];
-            beyond |= half_saturated(hv[mi][nt][i]);
-          }
-        }
-  } else {
-    float* plane = a.o_part + static_cast<size_t>(m.z) * a.n_pairs * N;
-#pragma unroll
-    for (int mi = 0; mi < (SPLIT ? 1 : 2); ++mi)
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int mt = SPLIT ? mt_own : mi;
-          const int tok = nt * 8 + 2 * t + (i & 1);
-          const int n = m.rb * 2 * TMA_BOX_ROWS + 32 * warp + 16 * mt + gp + 8 * (i >> 1);
-          if (tok < m.ntok && n < N) plane[static_cast<size_t>(m.begin + m.p0 + tok) * N + n] = tot[mi][nt][i];
-        }
+    }
   }
-  if (beyond) atomicOr(a.check_word, CHECK_F16_RANGE);  // saturated above: reported, not silent
+  if (beyond) atomicOr(check_word, CHECK_F16_RANGE);  // saturated above: reported, not silent
+}
+
+// The staged segment to global memory, a warp per token: 8 bytes per lane, and the sum of the
+// token's values for the offset codes of the second projection.
+__device__ __forceinline__ void hidden_to_global(const TmaArgs& a, bool gated, int rb, int slot0, int ntok, int bits, int warp,
+                                                 int lane, const unsigned char* hid) {
+  const int seg = gated ? rb >> 1 : rb, half = gated ? rb & 1 : 0;
+  unsigned char* tile = a.hidden + act_tile_offset(slot0, a.L.d_ff) + static_cast<size_t>(seg) * act_seg_bytes(ntok);
+  const bool mine = !gated || ((lane >> 2) & 1) == half;  // a gated item fills half of the segment: inputs of lanes t = 2*half, 2*half+1
+  for (int tok = warp; tok < ntok; tok += ST_WARPS) {
+    float sum = 0.0f;
+    if (mine) {
+      const uint2 v = *reinterpret_cast<const uint2*>(hid + tok * 256 + lane * 8);
+      *reinterpret_cast<uint2*>(tile + tok * 256 + lane * 8) = v;
+      const float2 p = __half22float2(*reinterpret_cast<const __half2*>(&v.x)), q = __half22float2(*reinterpret_cast<const __half2*>(&v.y));
+      sum = (p.x + p.y) + (q.x + q.y);
+    }
+    if (ntok <= 8) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (lane == 0) {
+        act_tile_offset_share(tile + ntok * 256, tok, half, sum, bits);
+      }
+    }
+  }
+}
+
+template <int BITS, int NT>
+__device__ __forceinline__ void store_output(const TmaArgs& a, int rb, int z, int slot0, int ntok, int warp, int lane,
+                                             const float (&tot)[NT][4]) {
+  const int g = lane >> 2, t = lane & 3;
+  const int N = a.L.d_model;
+  float* dst = a.o_part + (static_cast<size_t>(z) * a.n_pairs + slot0) * N + rb * 128 + 16 * warp + box_row_of<BITS>(g);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    if (nt * 8 >= ntok) break;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int tok = nt * 8 + 2 * t + (i & 1);
+      if (tok < ntok) dst[static_cast<size_t>(tok) * N + 8 * (i >> 1)] = tot[nt][i];
+    }
+  }
+}
+
+// Item k of the CTA's list, decoded by one thread.  Every CTA takes every gridDim.x-th item: the items of the
+// first projection, then those of the second, most expensive bitwidth first, so that the shares are even to
+// about one of the cheapest items; the list is known without asking, 32 items are decoded at a time.
+template <bool SF16>
+__device__ __forceinline__ void decode_item(const TmaArgs& a, const PlanRec* s_plan, const PlanRec* recs, int n_active, int k, ItemRec* out) {
+  const int n_items0 = a.phase_begin == 0 ? n_active * a.row_blocks[0] : 0;
+  const int n_items1 = a.phase_end == 2 ? n_active * a.row_blocks[1] * a.ksplit : 0;
+  const int item = static_cast<int>(blockIdx.x) + k * static_cast<int>(gridDim.x);
+  if (item >= n_items0 + n_items1) {
+    out->flags = ITEM_STOP;
+    return;
+  }
+  const int phase = item < n_items0 ? 0 : 1;
+  const int li = item - (phase == 0 ? 0 : n_items0);
+  const bool gated = phase == 0 && a.L.act == EMOE_ACT_SWIGLU;
+  const int row_blocks = a.row_blocks[phase], ksplit = phase == 0 ? 1 : a.ksplit;
+  const int mat_first = phase == 0 ? 0 : (a.L.act == EMOE_ACT_SWIGLU ? 2 : 1);
+  const int ai = fast_div(li, ksplit * row_blocks, a.mg_units[phase]);
+  const PlanRec& rec = ai < ST_PLAN_CACHE ? s_plan[ai] : recs[ai];
+  const int lz = fast_div(li, ksplit, a.mg_ksplit[phase]);  // (expert, row block) index
+  const int z = li - lz * ksplit;
+  const int rb = lz - fast_div(lz, row_blocks, a.mg_rb[phase]) * row_blocks;
+  const int bits = rec.bits;
+  const int sh = bits == 8 ? 0 : (bits == 4 ? 1 : 2);  // log2 of the 128-input segments per stage
+  const int seg_total = (phase == 0 ? a.L.d_model : a.L.d_ff) >> 7;
+  const int steps_total = (seg_total + (1 << sh) - 1) >> sh;
+  const int spz = fast_div(steps_total + ksplit - 1, ksplit, a.mg_ksplit[phase]);
+  const int step_begin = z * spz;
+  const int nsteps = max(0, min(steps_total, step_begin + spz) - step_begin);
+  const int nst = max(nsteps, 1);  // an empty split-K slice still has to store its zeros
+  out->flags = (phase == 1 ? ITEM_SECOND : 0) | (bits << 8);
+  out->nst = nst;
+  out->seg0 = step_begin << sh;
+  out->last = nsteps > 0 ? min(1 << sh, seg_total - ((step_begin + nst - 1) << sh)) : 0;
+  out->begin = rec.begin;
+  out->cnt = rec.cnt;
+  out->rbz = rb | (z << 16);
+  out->ai = ai;
+  out->scales[0] = static_cast<const char*>(mat_first == 0 ? rec.scales[0] : (mat_first == 1 ? rec.scales[1] : rec.scales[2]));
+  out->scales[1] = gated ? static_cast<const char*>(rec.scales[1]) : out->scales[0];
+  out->map = a.tmaps + static_cast<size_t>(rec.e) * 3 + mat_first;
+  out->row0 = rb * (gated ? ST_BOX_ROWS : 2 * ST_BOX_ROWS);
+}
+
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+template <bool SF16>
+__device__ __forceinline__ float scale_at(const unsigned char* p) {
+  if constexpr (SF16) return __half2float(*reinterpret_cast<const __half*>(p));
+  else return *reinterpret_cast<const float*>(p);
+}
+
+// what the consumer warps share
+struct Pipe {
+  const unsigned char* ring;
+  unsigned char* hid_stage;
+  const int* offset;  // of the stage in a slot
+  const ItemRec* queue;
+  uint32_t bar_full, bar_empty, bar_issued, bar_hid;
+  PlanRec* recs;
+  bool fused;
+  volatile int* abort_flag;
+};
+// where a consumer warp stands
+struct Cursor {
+  int it;          // next stage
+  int n_hidden;    // first-projection items stored so far
+  int pending_ai;  // expert whose finished item is still to be counted (-1: none)
+};
+
+// One pass of an item by a consumer warp, its first stage having arrived: all its stages, then the results.
+template <int BITS, bool SF16, int NT>
+__device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, int k, int p0, int warp, int lane, Cursor& cur) {
+  constexpr int SEGS = 8 / BITS;
+  const ItemRec& rec = pp.queue[k % ST_QUEUE];
+  const int nst = rec.nst, seg0 = rec.seg0, last = rec.last, cnt = rec.cnt, tok0 = rec.begin + p0;
+  const int ntok = min(ACT_PASS_MAX, cnt - p0);
+  const int phase = rec.flags & ITEM_SECOND ? 1 : 0;
+  const bool gated = phase == 0 && a.L.act == EMOE_ACT_SWIGLU;
+  constexpr int ssz = SF16 ? 2 : 4;
+  const int g = lane >> 2, t = lane & 3;
+  const int gp = box_row_of<BITS>(g);
+  StageLane p;
+  // rows of a warp: 16 of one matrix, or eight of w1 (first box) and the same eight of w3 (second).  8 bits:
+  // columns 2t and 2t+1; 4 bits: column t of the segment's four; 2 bits: half of column t/2 of its two
+  p.row = ((gated ? 8 : 16) * warp + gp) * 128 + (((BITS == 8 ? 2 * t : (BITS == 4 ? t : t >> 1)) ^ gp) << 4) + (BITS == 2 ? (t & 1) << 3 : 0);
+  p.drow = gated ? ST_BOX_BYTES : 8 * 128;
+  p.xe = ST_X_OFFSET + g * 256 + t * 16 + ((g & 1) << 6);
+  p.init = ST_X_OFFSET + ntok * 256 + t * 8;
+  p.halves = phase == 1 && a.L.act == EMOE_ACT_SWIGLU;
+  const int xstride = act_seg_bytes(ntok);
+  float tot[NT][4];
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tot[nt][i] = 0.0f;
+  // scales: 16 bytes per row of the stage, from the 4-byte boundary at or below the first one
+  p.sc = 2 * ST_BOX_BYTES + ((gated ? 8 : 16) * warp + gp) * 16;
+  p.dsc = gated ? ST_BOX_ROWS * 16 : 8 * 16;
+  const int row_bytes = a.ngroups[phase] * ssz, row_off = (rec.row0 + (gated ? 8 : 16) * warp + gp) * row_bytes;
+#pragma unroll 1
+  for (int s = 0; s < nst; ++s) {
+    const int slot = cur.it % ST_SLOTS;
+    if (s > 0 && !__all_sync(0xffffffffu, mbar_wait(pp.bar_full + 8 * slot, (cur.it / ST_SLOTS) & 1, a.check_word, pp.abort_flag)))
+      return false;
+    const unsigned char* stage = pp.ring + pp.offset[slot];
+    const int seg = seg0 + s * SEGS, g0 = group_of_seg(a, seg);
+    const unsigned char* sc = stage + p.sc + ((row_off + g0 * ssz) & 3);
+    const int nseg = s == nst - 1 ? last : SEGS;
+    if (nseg == SEGS) {
+#pragma unroll
+      for (int sg = 0; sg < SEGS; ++sg) {
+        const int d = sg == 0 ? 0 : (group_of_seg(a, seg + sg) - g0) * ssz;
+        consume_segment<BITS, NT>(stage, p, sg, sg * xstride, scale_at<SF16>(sc + d), scale_at<SF16>(sc + d + p.dsc), tot);
+      }
+    } else {
+#pragma unroll 1
+      for (int sg = 0; sg < nseg; ++sg) {
+        const int d = (group_of_seg(a, seg + sg) - g0) * ssz;
+        consume_segment<BITS, NT>(stage, p, sg, sg * xstride, scale_at<SF16>(sc + d), scale_at<SF16>(sc + d + p.dsc), tot);
+      }
+    }
+    // shared memory of the stage is no longer needed
+    __syncwarp();
+    if (lane == 0) mbar_arrive(pp.bar_empty + 8 * slot);
+    ++cur.it;
+    if (s == 0 && cur.pending_ai >= 0) {
+      count_item_done(pp.recs, cur.pending_ai, lane);
+      cur.pending_ai = -1;
+    }
+  }
+  const bool last_pass = p0 + ACT_PASS_MAX >= cnt;
+  const int rb = rec.rbz & 0xffff, z = rec.rbz >> 16, ai = rec.ai;
+  if (NT == 1) {  // the subnormal codes weigh 2^-24
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tot[0][i] *= 16777216.0f;
+  }
+  if (phase == 0) {
+    // two staging buffers in turn: a warp can be one item ahead of the slowest, not two
+    unsigned char* hid = pp.hid_stage + (cur.n_hidden & 1) * ST_HID_BYTES;
+    hidden_to_smem<BITS, NT>(gated, rb, ntok, warp, lane, tot, hid, a.check_word);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(pp.bar_hid);
+    if (!__all_sync(0xffffffffu, mbar_wait(pp.bar_hid, cur.n_hidden & 1, a.check_word, pp.abort_flag))) return false;
+    ++cur.n_hidden;
+    hidden_to_global(a, gated, rb, tok0, ntok, BITS, warp, lane, hid);
+    if (pp.fused && last_pass) cur.pending_ai = ai;
+  } else {
+    store_output<BITS, NT>(a, rb, z, tok0, ntok, warp, lane, tot);
+  }
   return true;
 }
 
-// ring depth and CTAs per SM by token-tile count: more, smaller CTAs when registers allow, so
-// that every scheduler has several consumer warps to switch between
-template <int NT, bool SPLIT>
-__host__ __device__ constexpr int stages_for() { return SPLIT ? EMOE_TMA_SPLIT_STAGES : (NT == 1 ? EMOE_TMA_STAGES_NT1 : 3); }
-template <int NT, bool SPLIT>
-__host__ __device__ constexpr int ctas_per_sm_for() { return SPLIT ? EMOE_TMA_SPLIT_CTAS : (NT == 1 ? EMOE_TMA_CTAS_NT1 : (NT == 2 ? 2 : 1)); }
-
-template <int NT, bool SPLIT>
-__host__ __device__ constexpr int smem_bytes_for() {
-  return stages_for<NT, SPLIT>() * stage_bytes_for(NT) + 1024;  // + slack to align the base to 1024
-}
-
-template <int NT, bool SPLIT>
-__global__ void __launch_bounds__(tma_threads(SPLIT), ctas_per_sm_for<NT, SPLIT>()) ffn_tma_kernel(const __grid_constant__ TmaArgs a) {
-  constexpr int TMA_CONSUMER_WARPS = consumer_warps(SPLIT);
-  constexpr int STAGES = stages_for<NT, SPLIT>();
-  constexpr int STAGE_BYTES = stage_bytes_for(NT);
+template <bool SF16>
+__global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __grid_constant__ TmaArgs a) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 8];  // full, empty; SPLIT: (full, free) per warp pair of the w3 -> w1 hand-over
-  __shared__ __align__(16) StageMeta meta[STAGES];
-  __shared__ float xch[SPLIT ? 4 * NT * 4 * 32 : 1];
+  __shared__ __align__(8) uint64_t bars[3 * ST_SLOTS + 1];  // full, empty, issued (weight warp -> activation warp), hidden segment staged
+  __shared__ ItemRec queue[ST_QUEUE];
+  __shared__ __align__(16) PlanRec s_plan[ST_PLAN_CACHE];
+  __shared__ int s_active, s_vstart[ST_SLOTS], s_offset[ST_SLOTS];
   __shared__ int abort_word;
   volatile int* abort_flag = &abort_word;
-  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // an offset from the array, not a rounded address: the compiler then knows that every access is to shared memory
+  unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  unsigned char* hid_stage = ring + ST_RING;
+  // The feeding warps come first: the schedulers favour the oldest warp, and a feeding warp that has to wait for
+  // eight computing ones to stall leaves them without work soon after.
+  const int lane = threadIdx.x & 31, warp_id = threadIdx.x >> 5, warp = warp_id < 2 ? ST_WARPS + warp_id : warp_id - 2;
+  const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + ST_SLOTS), bar_issued = smem_u32(bars + 2 * ST_SLOTS), bar_hid = smem_u32(bars + 3 * ST_SLOTS);
 
   if (threadIdx.x == 0) {
     abort_word = 0;
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(smem_u32(bars + s), 33);  // full: lane 0's arrival (+ bulk-copy bytes) and every lane's scale copies
-      mbar_init(smem_u32(bars + STAGES + s), TMA_CONSUMER_WARPS);  // empty: one arrival per consumer warp
+    for (int s = 0; s < ST_SLOTS; ++s) {
+      mbar_init(bar_full + 8 * s, 34);          // weight warp and activation warp (+ the bytes of their copies), every lane's scale copies
+      mbar_init(bar_issued + 8 * s, 1);
+      mbar_init(bar_empty + 8 * s, ST_WARPS);   // one arrival per consumer warp
     }
-    for (int i = 0; i < 8; ++i) mbar_init(smem_u32(bars + 2 * STAGES + i), 1);
+    mbar_init(bar_hid, ST_WARPS);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // Token rows of a stage that no copy fills keep whatever shared memory held.  That is
-  // harmless: a column of the MMA result depends only on its own column of B, and columns past
-  // the expert's token count are never stored.
   __syncthreads();
-  // Everything above overlaps the tail of the kernel in front.  A launch that starts with the
-  // first projection needs that kernel's results (the plan) at once; a launch of the second
-  // projection alone finds plan, weights and scales older than the kernel in front, so its
-  // producer starts fetching them and waits only before the first copy of a hidden vector (see
-  // `waited` below).
-  if (warp == TMA_CONSUMER_WARPS) {
+  // Everything above overlaps the tail of the kernel in front.
+  if (warp == ST_WARPS) {
     // The tensor maps are older than every kernel of the chain: pull them towards L2 now, so that
     // the first copy of an expert's matrix does not wait for its descriptor to come from HBM.
     const int n_maps = 3 * a.L.E;
     const int i = (static_cast<int>(blockIdx.x) * 32 + lane) % ((n_maps + 31) / 32 * 32);
     if (i < n_maps) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.tmaps + i));
   }
-  if (a.phase_begin == 0) pdl_wait();
+  pdl_wait();
   pdl_trigger();
+  {  // the plan into shared memory: header and records in one round trip
+    const int4* src = reinterpret_cast<const int4*>(reinterpret_cast<const char*>(a.plan) + PLAN_HEADER_BYTES);
+    const int n = min(a.L.E, ST_PLAN_CACHE) * static_cast<int>(sizeof(PlanRec) / 16);
+    for (int i = threadIdx.x; i < n; i += ST_THREADS) reinterpret_cast<int4*>(s_plan)[i] = __ldcg(src + i);
+    if (threadIdx.x == 0) s_active = __ldcg(a.plan);
+    __syncthreads();
+  }
 
-  const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + STAGES);
   const LayerDims& L = a.L;
   PlanRec* recs = reinterpret_cast<PlanRec*>(reinterpret_cast<char*>(a.plan) + PLAN_HEADER_BYTES);
   // both projections in this launch: an item of the second projection waits until the expert's
   // hidden vectors are complete (PlanRec::done, raised by the consumers of the first projection)
   const bool fused = a.phase_begin == 0 && a.phase_end == 2;
 
-  if (warp == TMA_CONSUMER_WARPS) {
-    // ---------------- producer warp ----------------
-    // the record the CTA's first item most likely needs, requested together with the header
-    const int ai_guess = min(static_cast<int>(blockIdx.x) / (a.phase_begin == 0 ? a.row_blocks[0] : a.row_blocks[1] * a.ksplit),
-                             L.E - 1);
-    const PlanRec rec_guess = recs[ai_guess];
-    const int n_active = *reinterpret_cast<volatile const int*>(a.plan);
-    // items: the first projection's (expert, row block), then the second's (expert, row block,
-    // split-K slice), each list expert-major in plan order
-    const int n_items0 = a.phase_begin == 0 ? n_active * a.row_blocks[0] : 0;
-    const int n_items1 = a.phase_end == 2 ? n_active * a.row_blocks[1] * a.ksplit : 0;
-    const int n_items = n_items0 + n_items1;
-    const int ssz = L.scale_f16 ? 2 : 4;
-    int it = 0;
-    bool ok = true;
-    bool waited = a.phase_begin == 0;  // false: copies of activation rows are parked until pdl_wait()
-    int n_parked = 0;
-    int park_stage[STAGES], park_row[STAGES], park_k0[STAGES], park_klen[STAGES], park_ntok[STAGES];
-    // A CTA's first item is its own index; the counter hands out the items after those.
-    int item_cur = blockIdx.x, item_next = 0;
-    while (ok) {
-      const int item = item_cur;
-      if (item >= n_items || *abort_flag) break;
-      const int phase = item < n_items0 ? 0 : 1;
-      const int li = item - (phase == 0 ? 0 : n_items0);
-      const PhaseDims pd = phase_dims(a, phase);
-      const int K = pd.K;
-      const bool swiglu_in = pd.swiglu_in;
-      const int mat_first = pd.mat_first;
-      const int ngroups_k = a.ngroups[phase];
-      const int ai = fast_div(li, pd.ksplit * pd.row_blocks, pd.mg_units);
-      const PlanRec rec = (it == 0 && ai == ai_guess) ? rec_guess : recs[ai];
-      const __half* in = phase == 0 ? a.xs : a.hidden;
-      const int lz = fast_div(li, pd.ksplit, pd.mg_ksplit);  // (expert, row block) index
-      const int z = li - lz * pd.ksplit;
-      const int rb = lz - fast_div(lz, pd.row_blocks, pd.mg_rb) * pd.row_blocks;
-      const int e = rec.e;
-      const int begin = rec.begin;
-      const int cnt = rec.cnt;
-      const CUtensorMap* maps = a.tmaps + static_cast<size_t>(e) * 3;
-      const int bits = rec.bits;
-      const int kshift = bits == 8 ? 7 : (bits == 4 ? 8 : 9);  // log2 of the inputs per stage
-      const int kspan = 1 << kshift;
-      const int steps_total = (K + kspan - 1) >> kshift;
-      const int spz = fast_div(steps_total + pd.ksplit - 1, pd.ksplit, pd.mg_ksplit);
-      const int step_begin = z * spz;
-      const int nsteps = max(0, min(steps_total, step_begin + spz) - step_begin);
-      const int npass = (cnt + NT * 8 - 1) / (NT * 8);
-      const int row0 = rb * pd.rows_per_item;
-      bool need_dep = fused && phase == 1;
-      // scale rows of the item this lane copies (rows l, l+32, l+64, l+96 of a stage, box-major): start
-      // of each row's scale channel as a byte offset from its 4-byte-aligned matrix base
-      const char* srow_base[4];
-      int srow_off[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int row = lane + 32 * r;  // neighbouring lanes take neighbouring rows: their 4-byte copies spread over the banks
-        const int n = min(swiglu_in ? row0 + (row & 63) : row0 + row, pd.N - 1);
-        // constant indices only: a record indexed by a variable would live in local memory
-        const void* sc_first = mat_first == 0 ? rec.scales[0] : (mat_first == 1 ? rec.scales[1] : rec.scales[2]);
-        srow_base[r] = static_cast<const char*>(swiglu_in ? ((row >> 6) ? rec.scales[1] : rec.scales[0]) : sc_first);
-        srow_off[r] = n * ngroups_k * ssz;
+  if (warp == ST_WARPS) {
+    // ---------------- weight warp: items, ring, packed codes ----------------
+    // The ring: stages lie one behind the other, a stage that would run over the end starts at the
+    // beginning again.  head and vstart are positions on an endless tape; a stage may be written
+    // once nothing live lies within a ring's length behind its end.  This thread feeds eight
+    // computing warps: whatever it does per stage is kept to a few instructions.
+    int it = 0, oldest = 0, head = 0, phys = 0;
+    int more = 1;
+    for (int k0 = 0; more; k0 += 32) {
+      decode_item<SF16>(a, s_plan, recs, s_active, k0 + lane, &queue[(k0 + lane) % ST_QUEUE]);
+      __syncwarp();
+      if (lane == 0) {
+        for (int k = k0; k < k0 + 32 && more; ++k) {
+          const ItemRec& rec = queue[k % ST_QUEUE];
+          const int flags = rec.flags;
+          if (flags & ITEM_STOP) {  // tell the others that nothing else comes
+            const int slot = it % ST_SLOTS;
+            if (it < ST_SLOTS || mbar_wait(bar_empty + 8 * slot, ((it / ST_SLOTS) & 1) ^ 1, a.check_word, abort_flag)) {
+              mbar_arrive(bar_full + 8 * slot);
+              mbar_arrive(bar_issued + 8 * slot);
+            }
+            more = 0;
+            break;
+          }
+          const int bits = flags >> 8, nst = rec.nst, last = rec.last, cnt = rec.cnt, row0 = rec.row0;
+          const bool gated = !(flags & ITEM_SECOND) && L.act == EMOE_ACT_SWIGLU;
+          const CUtensorMap* map0 = rec.map;
+          const CUtensorMap* map1 = gated ? map0 + 1 : map0;
+          const int row1 = gated ? row0 : row0 + ST_BOX_ROWS;
+          const int c_first = rec.seg0 * 16 * bits;  // byte column: 128 inputs = 16 * bits bytes
+          for (int p0 = 0; p0 < cnt && more; p0 += ACT_PASS_MAX) {
+            const int xseg = act_seg_bytes(min(ACT_PASS_MAX, cnt - p0));
+            const int need_full = ST_X_OFFSET + (((8 / bits) * xseg + 1023) & ~1023);
+            const int need_last = last > 0 ? ST_X_OFFSET + ((last * xseg + 1023) & ~1023) : 0;
+            for (int s = 0, c0 = c_first; s < nst; ++s, ++it, c0 += 128) {
+              const int need = s == nst - 1 ? need_last : need_full;
+              if (phys + need > ST_RING) {  // does not fit in front of the end of the ring
+                head += ST_RING - phys;
+                phys = 0;
+              }
+              while (oldest < it && (it - oldest >= ST_SLOTS || head + need > s_vstart[oldest % ST_SLOTS] + ST_RING)) {
+                if (!mbar_wait(bar_empty + 8 * (oldest % ST_SLOTS), (oldest / ST_SLOTS) & 1, a.check_word, abort_flag)) {
+                  more = 0;
+                  break;
+                }
+                ++oldest;
+              }
+              if (!more) break;
+              const int slot = it % ST_SLOTS;
+              const uint32_t full = bar_full + 8 * slot;
+              if (need > 0) {
+                const uint32_t st = smem_u32(ring + phys);
+                mbar_expect_tx(full, 2 * ST_BOX_BYTES);
+                tma_load_2d(st, map0, c0, row0, full);
+                tma_load_2d(st + ST_BOX_BYTES, map1, c0, row1, full);
+              } else {
+                mbar_arrive(full);
+              }
+              s_vstart[slot] = head;
+              s_offset[slot] = phys;
+              mbar_arrive(bar_issued + 8 * slot);  // over to the activation warp
+              head += need;
+              phys += need;
+            }
+          }
+        }
       }
-      for (int pass = 0; pass < npass && ok; ++pass) {
-        const int p0 = pass * NT * 8;
-        const int ntok = min(NT * 8, cnt - p0);
-        const int nst = max(nsteps, 1);  // an empty split-K slice still has to store its zeros
+      more = __shfl_sync(0xffffffffu, more, 0);
+    }
+  } else if (warp == ST_WARPS + 1) {
+    // ---------------- activation warp: the activation slice and the scales of every stage ----------------
+    // On its own so that a wait for hidden vectors does not keep the weight stream from running ahead.
+    int ready_ai = -1;  // the expert whose hidden vectors are known to be complete
+    bool ok = true;
+    int it = 0;
+    for (int k = 0; ok; ++k) {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_issued + 8 * (it % ST_SLOTS), (it / ST_SLOTS) & 1, a.check_word, abort_flag))) break;
+      const ItemRec& rec = queue[k % ST_QUEUE];
+      const int flags = rec.flags;
+      if (flags & ITEM_STOP) {
+        mbar_arrive(bar_full + 8 * (it % ST_SLOTS));
+        if (lane == 0) mbar_arrive(bar_full + 8 * (it % ST_SLOTS));
+        break;
+      }
+      const int phase = flags & ITEM_SECOND ? 1 : 0, bits = flags >> 8, nst = rec.nst, last = rec.last, cnt = rec.cnt, seg0 = rec.seg0;
+      const bool gated = phase == 0 && L.act == EMOE_ACT_SWIGLU;
+      constexpr int ssz = SF16 ? 2 : 4;
+      // the lane's rows of the stage: lane, lane + 32, ...
+      const int row_bytes = a.ngroups[phase] * ssz;
+      const char* sc_a = rec.scales[0];
+      const char* sc_b = rec.scales[1];
+      const char* sc_row[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        sc_row[i] = (gated && i >= 2 ? sc_b : sc_a) + static_cast<size_t>(rec.row0 + (gated ? (lane + 32 * i) & 63 : lane + 32 * i)) * row_bytes;
+      const bool pairs = a.scale_pairs[phase];
+      {  // pull the item's scales towards L2, where the copies below find them
+        for (int b = lane * 128; b < (gated ? ST_BOX_ROWS : 2 * ST_BOX_ROWS) * row_bytes && (phase == 0 || a.ksplit == 1); b += 32 * 128) {
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(sc_a + static_cast<size_t>(rec.row0) * row_bytes + b));
+          if (gated) asm volatile("prefetch.global.L2 [%0];" ::"l"(sc_b + static_cast<size_t>(rec.row0) * row_bytes + b));
+        }
+      }
+      if (fused && phase == 1 && rec.ai != ready_ai && last > 0) {
+        // The codes of the stage are on their way; the hidden vectors may still be in the making on other
+        // SMs.  (Every lane acquires the counter itself.)
+        const int expect = a.row_blocks[0] * ST_WARPS;  // every consumer warp counts once per item
+        const int* done = &recs[rec.ai].done;
+        bool ready = false;
+        for (unsigned i = 0; i < DEP_WAIT_LIMIT; ++i) {
+          int v;
+          asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
+          ready = __all_sync(0xffffffffu, v >= expect);
+          if (ready || __any_sync(0xffffffffu, *abort_flag)) break;
+          __nanosleep(100);
+        }
+        if (!ready) {
+          if (lane == 0) {
+            *abort_flag = 1;
+            atomicOr(a.check_word, CHECK_WAIT_TIMEOUT);
+          }
+          break;
+        }
+        asm volatile("fence.proxy.async.global;" ::: "memory");  // generic-proxy stores (global memory) -> bulk-copy reads
+        ready_ai = rec.ai;
+      }
+      const int K = phase == 0 ? L.d_model : L.d_ff;
+      const unsigned char* base = phase == 0 ? a.xs : a.hidden;
+      for (int p0 = 0; p0 < cnt && ok; p0 += ACT_PASS_MAX) {
+        const uint32_t xseg = act_seg_bytes(min(ACT_PASS_MAX, cnt - p0));
+        const unsigned char* src = base + act_tile_offset(rec.begin + p0, K) + static_cast<size_t>(seg0) * xseg;
         for (int s = 0; s < nst; ++s, ++it) {
-          const int stage = it % STAGES;
-          const uint32_t par = (it / STAGES) & 1;
-          if (!mbar_wait(bar_empty + 8 * stage, par ^ 1, a.check_word, abort_flag)) {
+          const int slot = it % ST_SLOTS;
+          if ((s > 0 || p0 > 0) &&
+              !__all_sync(0xffffffffu, mbar_wait(bar_issued + 8 * slot, (it / ST_SLOTS) & 1, a.check_word, abort_flag))) {
             ok = false;
             break;
           }
-          unsigned char* st = smem + stage * STAGE_BYTES;
-          const uint32_t full = bar_full + 8 * stage;
-          const int k0 = (step_begin + s) * kspan;
-          const int klen = nsteps > 0 ? min(kspan, K - k0) : 0;
-          // Lanes 30 and 31 start the two weight boxes at once; lane 0 writes the record and announces
-          // the bytes.  The order among them is free: the stage cannot complete before all 33
-          // arrivals are in, and the byte count may run ahead of its announcement.
-          if (klen > 0 && lane >= 30) {
-            const int c0 = k0 * bits / 8;
-            const int bx = lane - 30;
-            if (swiglu_in) tma_load_2d(smem_u32(st + bx * TMA_BOX_BYTES), maps + bx, c0, row0, full);
-            else tma_load_2d(smem_u32(st + bx * TMA_BOX_BYTES), maps + mat_first, c0, row0 + bx * TMA_BOX_ROWS, full);
-          }
-          if (lane == 0) {
-            const int flags = (s == 0 ? META_FIRST : 0) | (s == nst - 1 ? META_LAST : 0) | (klen == 0 ? META_EMPTY : 0) |
-                              (fused && phase == 0 && s == nst - 1 && pass == npass - 1 ? META_DONE : 0);
-            // the record as three 16-byte stores (field order of StageMeta)
-            uint4* mq = reinterpret_cast<uint4*>(&meta[stage]);
-            mq[0] = make_uint4(e, rb, z, begin);
-            mq[1] = make_uint4(p0, ntok, k0, bits);
-            mq[2] = make_uint4(flags, phase, ai, 0);
-            if (klen > 0) mbar_expect_tx(full, 2 * TMA_BOX_BYTES + ntok * klen * 2);
-            else mbar_arrive(full);
-          }
-          __syncwarp();
-          if (klen > 0) {
-            // scales: lane l copies the windows of rows l, l+32, l+64, l+96 of the stage (box-major)
-            const int nseg = klen / 128;
-            const int g0 = group_of(k0, a.gshift, L.group, ngroups_k),
-                      g1 = group_of(k0 + (nseg - 1) * 128, a.gshift, L.group, ngroups_k);
-            const uint32_t sdst = smem_u32(st + scale_tile_offset(NT));
+          const uint32_t full = bar_full + 8 * slot;
+          const int nseg = s == nst - 1 ? last : 8 / bits;
+          if (nseg > 0) {
+            const uint32_t st = smem_u32(ring + s_offset[slot]);
+            if (lane == 0) {
+              mbar_expect_tx(full, nseg * xseg);
+              bulk_load(st + ST_X_OFFSET, src, nseg * xseg, full);
+            }
+            src += nseg * xseg;
+            const int seg = seg0 + s * (8 / bits);
+            const uint32_t dst = st + 2 * ST_BOX_BYTES + lane * 16;
+            if (pairs) {  // one scale per segment, rows of whole 4-byte words: one word, or two at 2 bits
+              const int b0 = (seg * 2) & ~3;
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              const int b0 = (srow_off[r] + g0 * ssz) & ~3;
-              const int b1 = srow_off[r] + (g1 + 1) * ssz;
+              for (int i = 0; i < 4; ++i) cp_async4(dst + 512 * i, sc_row[i] + b0);
+              if (nseg > 2) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) cp_async4(dst + 512 * i + 4, sc_row[i] + b0 + 4);
+              }
+            } else {  // the words that hold the stage's scales, from the 4-byte boundary at or below the first
+              const int g0 = group_of_seg(a, seg) * ssz, g1 = (group_of_seg(a, seg + nseg - 1) + 1) * ssz;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const char* from = reinterpret_cast<const char*>(reinterpret_cast<uintptr_t>(sc_row[i] + g0) & ~static_cast<uintptr_t>(3));
 #pragma unroll 1
-              for (int w = 0; b0 + 4 * w < b1; ++w)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sdst + (lane + 32 * r) * 16 + 4 * w),
-                             "l"(srow_base[r] + b0 + 4 * w)
-                             : "memory");
+                for (int w = 0; from + w < sc_row[i] + g1; w += 4) cp_async4(dst + 512 * i + w, from + w);
+              }
             }
             asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(full) : "memory");
-            if (need_dep) {
-              // The codes and scales of the stage are on their way; the hidden vectors may still be
-              // in the making on other SMs.  Every lane acquires the counter itself, so that its
-              // own copies below are ordered behind the writers' stores.
-              need_dep = false;
-              // every consumer warp that stores hidden values counts once per item (SPLIT, gated layer: the
-              // warps with the w1 tiles only)
-              const int expect = a.row_blocks[0] * ((SPLIT && L.act == EMOE_ACT_SWIGLU) ? 4 : TMA_CONSUMER_WARPS);
-              const int* done = &recs[ai].done;
-              bool ready = false;
-              for (unsigned i = 0; i < DEP_WAIT_LIMIT; ++i) {
-                int v;
-                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(done) : "memory");
-                ready = __all_sync(0xffffffffu, v >= expect);
-                if (ready || *abort_flag) break;
-                __nanosleep(100);
-              }
-              if (!ready) {
-                if (lane == 0) {
-                  *abort_flag = 1;
-                  atomicOr(a.check_word, CHECK_WAIT_TIMEOUT);
-                }
-                ok = false;
-                break;
-              }
-              asm volatile("fence.proxy.async.global;" ::: "memory");  // generic-proxy stores (global memory) -> bulk-copy reads
-            }
-            if (waited) {
-              for (int r = lane; r < ntok; r += 32)
-                bulk_load(smem_u32(st + 2 * TMA_BOX_BYTES + r * TMA_XROW_MAX),
-                          in + static_cast<size_t>(begin + p0 + r) * K + k0, klen * 2, full);
-            } else {
-              park_stage[n_parked] = stage;
-              park_row[n_parked] = begin + p0;
-              park_k0[n_parked] = k0;
-              park_klen[n_parked] = klen;
-              park_ntok[n_parked] = ntok;
-              ++n_parked;
-            }
           } else {
-            mbar_arrive(full);  // with lane 0's arrival above: 33 in all
-          }
-          if (!waited && n_parked == STAGES) {  // the ring is full: nothing more can be fetched early
-            pdl_wait();
-            waited = true;
-            for (int i = 0; i < n_parked; ++i)
-              for (int r = lane; r < park_ntok[i]; r += 32)
-                bulk_load(smem_u32(smem + park_stage[i] * STAGE_BYTES + 2 * TMA_BOX_BYTES + r * TMA_XROW_MAX),
-                          a.hidden + static_cast<size_t>(park_row[i] + r) * K + park_k0[i], park_klen[i] * 2,
-                          bar_full + 8 * park_stage[i]);
-            n_parked = 0;
+            mbar_arrive(full);
+            if (lane == 0) mbar_arrive(full);
           }
         }
-      }
-      // the ring still holds several stages of work for the consumers: fetching the next item
-      // only now costs them nothing and no CTA sits on items it is not yet working on
-      if (lane == 0) item_next = gridDim.x + atomicAdd(a.plan + 1 + a.phase_begin, 1);
-      item_cur = __shfl_sync(0xffffffffu, item_next, 0);
-      if (item_cur < n_items) {
-        // pull the next item's scale rows towards L2 while its codes are still far away
-        const int phn = item_cur < n_items0 ? 0 : 1;
-        const int lin = item_cur - (phn == 0 ? 0 : n_items0);
-        const PhaseDims pn = phase_dims(a, phn);
-        const PlanRec rn = recs[fast_div(lin, pn.ksplit * pn.row_blocks, pn.mg_units)];
-        const int lzn = fast_div(lin, pn.ksplit, pn.mg_ksplit);
-        const int rbn = lzn - fast_div(lzn, pn.row_blocks, pn.mg_rb) * pn.row_blocks;
-        const int ngroups = a.ngroups[phn];
-        const int rows = min(pn.rows_per_item, pn.N - rbn * pn.rows_per_item);
-        const int lines = (rows * ngroups * ssz + 127) / 128;
-        const size_t offs = static_cast<size_t>(rbn) * pn.rows_per_item * ngroups * ssz;
-        const int nm = pn.swiglu_in ? 2 : 1;
-        for (int i = lane; i < nm * lines; i += 32) {
-          const int second = i >= lines ? 1 : 0;  // nm is 1 or 2: no division needed
-          const char* base = static_cast<const char*>(pn.swiglu_in ? (second ? rn.scales[1] : rn.scales[0]) : (pn.mat_first == 0 ? rn.scales[0] : (pn.mat_first == 1 ? rn.scales[1] : rn.scales[2]))) + offs;
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(base + static_cast<size_t>(i - second * lines) * 128));
-        }
-      }
-    }
-    if (!waited) {  // fewer stages than the ring holds: release the parked copies now
-      pdl_wait();
-      waited = true;
-      for (int i = 0; i < n_parked; ++i)
-        for (int r = lane; r < park_ntok[i]; r += 32)
-          bulk_load(smem_u32(smem + park_stage[i] * STAGE_BYTES + 2 * TMA_BOX_BYTES + r * TMA_XROW_MAX),
-                    a.hidden + static_cast<size_t>(park_row[i] + r) * L.d_ff + park_k0[i], park_klen[i] * 2,
-                    bar_full + 8 * park_stage[i]);
-      n_parked = 0;
-    }
-    if (ok && !*abort_flag) {  // tell the consumers that nothing else comes
-      const int stage = it % STAGES;
-      const uint32_t par = (it / STAGES) & 1;
-      if (mbar_wait(bar_empty + 8 * stage, par ^ 1, a.check_word, abort_flag)) {
-        if (lane == 0) {
-          meta[stage].flags = META_STOP;
-          mbar_arrive(bar_full + 8 * stage);  // lane 0 arrives twice: once for itself, once in place of a copy
-        }
-        __syncwarp();
-        mbar_arrive(bar_full + 8 * stage);
       }
     }
   } else {
     // ---------------- consumer warps ----------------
-    float tot[2][NT][4];
-    int n_exchanged = 0;
-    const uint32_t bar_x = smem_u32(bars + 2 * STAGES);
+    const Pipe pp = {ring, hid_stage, s_offset, queue, bar_full, bar_empty, bar_issued, bar_hid, recs, fused, abort_flag};
     // A finished first-projection item is counted one stage late: by then its stores have long
     // been acknowledged and the fence in front of the count costs nothing.  It is never held back
     // across a wait, because the stage waited for may be the one that waits for this count.
-    int pending_ai = -1;
-    for (int it = 0;; ++it) {
-      const int stage = it % STAGES;
-      const uint32_t par = (it / STAGES) & 1;
-      if (pending_ai >= 0 && !__shfl_sync(0xffffffffu, mbar_try_wait(bar_full + 8 * stage, par) ? 1 : 0, 0)) {
-        count_item_done(recs, pending_ai, lane);
-        pending_ai = -1;
+    Cursor cur = {0, 0, -1};
+    bool ok = true;
+    for (int k = 0, p0 = 0; ok;) {
+      const int slot = cur.it % ST_SLOTS;
+      const uint32_t par = (cur.it / ST_SLOTS) & 1;
+      if (cur.pending_ai >= 0 && !__all_sync(0xffffffffu, mbar_try_wait(bar_full + 8 * slot, par))) {
+        count_item_done(recs, cur.pending_ai, lane);
+        cur.pending_ai = -1;
       }
-      if (!mbar_wait(bar_full + 8 * stage, par, a.check_word, abort_flag)) break;
-      const StageMeta m = meta[stage];
-      if (m.flags & META_STOP) break;
-      if (m.flags & META_FIRST) {
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) tot[mt][nt][i] = 0.0f;
-      }
-      const unsigned char* st = smem + stage * STAGE_BYTES;
-      if (!(m.flags & META_EMPTY)) {
-        switch (m.bits) {
-          case 2: consume_stage<2, NT, SPLIT>(a, m.phase, m.rb, m.k0, m.ntok, st, warp, lane, bar_empty + 8 * stage, tot); break;
-          case 4: consume_stage<4, NT, SPLIT>(a, m.phase, m.rb, m.k0, m.ntok, st, warp, lane, bar_empty + 8 * stage, tot); break;
-          default: consume_stage<8, NT, SPLIT>(a, m.phase, m.rb, m.k0, m.ntok, st, warp, lane, bar_empty + 8 * stage, tot); break;
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_full + 8 * slot, par, a.check_word, abort_flag))) break;
+      const ItemRec& rec = queue[k % ST_QUEUE];
+      const int flags = rec.flags, cnt = rec.cnt;
+      if (flags & ITEM_STOP) break;
+      if (cnt - p0 <= 8) {
+        switch (flags >> 8) {
+          case 2: ok = consume_pass<2, SF16, 1>(a, pp, k, p0, warp, lane, cur); break;
+          case 4: ok = consume_pass<4, SF16, 1>(a, pp, k, p0, warp, lane, cur); break;
+          default: ok = consume_pass<8, SF16, 1>(a, pp, k, p0, warp, lane, cur); break;
         }
       } else {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_empty + 8 * stage);
-      }
-      if (m.flags & META_LAST) {
-        bool ok;
-        switch (m.bits) {
-          case 2: ok = store_item<2, NT, SPLIT>(a, m, warp, lane, tot, xch, bar_x, n_exchanged, abort_flag); break;
-          case 4: ok = store_item<4, NT, SPLIT>(a, m, warp, lane, tot, xch, bar_x, n_exchanged, abort_flag); break;
-          default: ok = store_item<8, NT, SPLIT>(a, m, warp, lane, tot, xch, bar_x, n_exchanged, abort_flag); break;
+        switch (flags >> 8) {
+          case 2: ok = consume_pass<2, SF16, 2>(a, pp, k, p0, warp, lane, cur); break;
+          case 4: ok = consume_pass<4, SF16, 2>(a, pp, k, p0, warp, lane, cur); break;
+          default: ok = consume_pass<8, SF16, 2>(a, pp, k, p0, warp, lane, cur); break;
         }
-        if (!ok) break;
       }
-      if (pending_ai >= 0) {
-        count_item_done(recs, pending_ai, lane);
-        pending_ai = -1;
+      p0 += ACT_PASS_MAX;
+      if (p0 >= cnt) {
+        p0 = 0;
+        ++k;
       }
-      // the warps that stored hidden values count the item (SPLIT, gated layer: not the w3 warps)
-      if ((m.flags & META_LAST) && (m.flags & META_DONE) && !(SPLIT && a.L.act == EMOE_ACT_SWIGLU && (warp & 1))) pending_ai = m.ai;
     }
-    if (pending_ai >= 0) count_item_done(recs, pending_ai, lane);
+    if (cur.pending_ai >= 0) count_item_done(recs, cur.pending_ai, lane);
   }
   if (*abort_flag) {
     // a wait ran out: give copies that may still be in flight time to land before the CTA's
@@ -769,27 +775,25 @@ __global__ void __launch_bounds__(tma_threads(SPLIT), ctas_per_sm_for<NT, SPLIT>
   }
 }
 
-template <int NT, bool SPLIT>
-cudaError_t launch_nt(const TmaArgs& a, int max_items, cudaStream_t st) {
-  constexpr int SMEM = smem_bytes_for<NT, SPLIT>();
-  constexpr int TMA_THREADS = tma_threads(SPLIT);
+template <bool SF16>
+cudaError_t launch_sf(const TmaArgs& a, long long items, cudaStream_t st) {
   static int ctas_per_device[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!ctas_per_device[dev]) {
-    e = cudaFuncSetAttribute(ffn_tma_kernel<NT, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    e = cudaFuncSetAttribute(ffn_tma_kernel<SF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM);
     if (e != cudaSuccess) return e;
     int per_sm = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ffn_tma_kernel<NT, SPLIT>, TMA_THREADS, SMEM);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ffn_tma_kernel<SF16>, ST_THREADS, ST_SMEM);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     ctas_per_device[dev] = (per_sm > 0 ? per_sm : 1) * sms;
   }
-  const int grid = max_items < ctas_per_device[dev] ? max_items : ctas_per_device[dev];
-  return launch_chain(ffn_tma_kernel<NT, SPLIT>, dim3(grid), dim3(TMA_THREADS), SMEM, st, a);
+  const int grid = items < ctas_per_device[dev] ? static_cast<int>(items) : ctas_per_device[dev];
+  return launch_chain(ffn_tma_kernel<SF16>, dim3(grid), dim3(ST_THREADS), ST_SMEM, st, a);
 }
 
 }  // namespace
@@ -797,24 +801,22 @@ cudaError_t launch_nt(const TmaArgs& a, int max_items, cudaStream_t st) {
 bool ffn_tma_supported(const LayerDims& L) {
   // tensor maps use 128-byte x 64-row boxes: every packed row must hold at least 128 bytes at
   // the narrowest width (2 bits)
-  return ffn_mma_supported(L) && L.d_model >= 512 && L.d_ff >= 512;
+  return ffn_mma_supported(L) && L.d_model >= 512 && L.d_ff >= 512 && L.d_model <= (1 << 17) && L.d_ff <= (1 << 17);
 }
 
 int ffn_tma_ksplit(const LayerDims& L, int T) {
-  const int row_blocks = (L.d_model + 2 * TMA_BOX_ROWS - 1) / (2 * TMA_BOX_ROWS);
+  const int row_blocks = (L.d_model + 2 * ST_BOX_ROWS - 1) / (2 * ST_BOX_ROWS);
   const long long pairs = static_cast<long long>(T) * L.top_k;
   const long long active = pairs < L.E ? pairs : L.E;
   const long long ctas = row_blocks * active;
   const int steps_min = (L.d_ff + 511) / 512;  // stages at the widest span (2 bits)
-  // enough slices that the second projection's items outnumber the resident CTAs (3 per SM)
-  // about four times: short items at the end of the launch keep its tail short (as measured: the
-  // same on the Switch-base-like layer at 64 tokens as twice as many CTAs' worth, 3 % faster on
-  // the Mixtral-like layer at 4 tokens; fewer slices were slower on both)
+  // enough slices that the second projection's items outnumber the resident CTAs (2 per SM)
+  // several times: short items at the end of the launch keep its tail short
   long long z = (12 * 148 + ctas - 1) / ctas;
   // A handful of tokens leaves most SMs without an item: the slices are then cut as fine as the
   // 8-bit stages allow (narrower experts get empty slices, which only store zeros), so that the
   // second projection of the one or two activated experts is a short step on many SMs instead
-  // of a chain of stages on a few (single token, Switch-base-like layer: 8 % off the launch).
+  // of a chain of stages on a few.
   const int steps_max = (L.d_ff + 127) / 128;
   const int cap = ctas * 4 <= 148 ? steps_max : steps_min;
   if (z > cap) z = cap;
@@ -823,31 +825,26 @@ int ffn_tma_ksplit(const LayerDims& L, int T) {
   return static_cast<int>(z);
 }
 
-cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, const ExpertDev* experts,
-                           const void* tmaps, const __nv_bfloat16* xs, const int32_t* off, int* plan,
-                           __nv_bfloat16* hidden, float* o_part, int ksplit, int n_pairs, int T, int token_tiles,
-                           int* check_word, cudaStream_t st) {
+cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, const void* tmaps, const void* xs, int* plan,
+                           void* hidden, float* o_part, int ksplit, int n_pairs, int* check_word, cudaStream_t st) {
   if (phase_begin < 0 || phase_end > 2 || phase_begin >= phase_end) return cudaErrorInvalidValue;
-  const int rows_first = L.act == EMOE_ACT_SWIGLU ? TMA_BOX_ROWS : 2 * TMA_BOX_ROWS;
+  const int rows_first = L.act == EMOE_ACT_SWIGLU ? ST_BOX_ROWS : 2 * ST_BOX_ROWS;
   TmaArgs a;
   a.phase_begin = phase_begin;
   a.phase_end = phase_end;
   a.L = L;
-  a.experts = experts;
   a.tmaps = static_cast<const CUtensorMap*>(tmaps);
-  a.xs = reinterpret_cast<const __half*>(xs);
-  a.off = off;
+  a.xs = static_cast<const unsigned char*>(xs);
   a.plan = plan;
-  a.hidden = reinterpret_cast<__half*>(hidden);
+  a.hidden = static_cast<unsigned char*>(hidden);
   a.o_part = o_part;
   a.ksplit = ksplit;
-  a.row_blocks[0] = (L.d_ff + rows_first - 1) / rows_first;
-  a.row_blocks[1] = (L.d_model + 2 * TMA_BOX_ROWS - 1) / (2 * TMA_BOX_ROWS);
+  a.row_blocks[0] = L.d_ff / rows_first;
+  a.row_blocks[1] = L.d_model / (2 * ST_BOX_ROWS);
   a.ngroups[0] = L.group > 0 ? L.d_model / L.group : 1;
   a.ngroups[1] = L.group > 0 ? L.d_ff / L.group : 1;
-  a.gshift = -1;
-  for (int b = 7; b < 31; ++b)
-    if (L.group == (1 << b)) a.gshift = b;
+  a.gmul = L.group > 0 ? ((1u << 20) + static_cast<unsigned>(L.group / 128) - 1) / static_cast<unsigned>(L.group / 128) : 0u;
+  for (int p = 0; p < 2; ++p) a.scale_pairs[p] = L.scale_f16 && L.group == 128 && a.ngroups[p] % 2 == 0;
   a.n_pairs = n_pairs;
   a.check_word = check_word;
   for (int p = 0; p < 2; ++p) {
@@ -861,11 +858,7 @@ cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, c
   if (phase_begin == 0) per_expert += a.row_blocks[0];
   if (phase_end == 2) per_expert += static_cast<long long>(a.row_blocks[1]) * ksplit;
   const long long items = active_max * per_expert;
-  const int max_items = items > (1 << 30) ? (1 << 30) : static_cast<int>(items);
-  const int nt = token_tiles > 0 ? token_tiles : ffn_token_tiles(L, T);
-  if (nt == 1) return launch_nt<1, EMOE_TMA_SPLIT_NT1 != 0>(a, max_items, st);
-  if (nt == 2) return launch_nt<2, false>(a, max_items, st);
-  return launch_nt<4, false>(a, max_items, st);
+  return L.scale_f16 ? launch_sf<true>(a, items, st) : launch_sf<false>(a, items, st);
 }
 
 // Host-side tensor-map encoder (driver entry point looked up once; no link against libcuda).
@@ -890,7 +883,7 @@ int encode_tmap_2d(void* out_map, int dtype, const void* base, uint64_t inner, u
   const cuuint32_t estr[2] = {1, 1};
   const CUresult r = fn(static_cast<CUtensorMap*>(out_map), dtype == 1 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8,
                         2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, EMOE_TMA_L2PROMO,
+                        swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : -3;
 }
@@ -906,8 +899,8 @@ int encode_scale_tmap(void* out_map, const void* scales, int N, int row_bytes) {
 // One tensor map per packed matrix: a [N][row_bytes] byte image, 64-row x 128-byte boxes, 128-byte swizzle.
 int encode_weight_tmap(void* out_map, const void* packed, int N, int K, int bits) {
   const uint64_t row_bytes = static_cast<uint64_t>(K) * bits / 8;
-  if (row_bytes < 128 || N < TMA_BOX_ROWS) return -2;
-  return encode_tmap_2d(out_map, 0, packed, row_bytes, static_cast<uint64_t>(N), row_bytes, 128, TMA_BOX_ROWS);
+  if (row_bytes < 128 || N < ST_BOX_ROWS) return -2;
+  return encode_tmap_2d(out_map, 0, packed, row_bytes, static_cast<uint64_t>(N), row_bytes, 128, ST_BOX_ROWS);
 }
 
 }  // namespace emoe

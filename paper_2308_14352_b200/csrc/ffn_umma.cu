@@ -157,7 +157,8 @@ struct UmmaArgs {
   LayerDims L;
   const CUtensorMap* wmaps;  // [E][3] packed-weight tensor maps (boxes of 64 rows x 128 bytes)
   const int* plan;           // header + PlanRec per activated expert
-  __half* hidden16;          // first projection's output (fp16, pair order)
+  __half* hidden16;          // first projection's output (fp16, pair order), rows hid_stride values apart
+  int hid_stride;
   float* o;                  // second projection's output [n_pairs][d_model]
   int zsplit;                // second projection: slices of the inputs per unit (1 or 2), slice z into plane z of o
   size_t plane_stride;       // floats between the planes of o
@@ -478,7 +479,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
             for (int c = 0; c < 32; ++c)
               if (c < live) dst[static_cast<size_t>(c) * N] = __uint_as_float(va[c]);
           } else {
-            __half* dst = a.hidden16 + (slot0 + cc) * N + hpos;
+            __half* dst = a.hidden16 + (slot0 + cc) * a.hid_stride + hpos;
             bool beyond = false;
             if (gated) {
               float av[32];
@@ -488,15 +489,15 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
               for (int c = 0; c < 32; ++c) {
                 // the hidden vector is a bf16 tensor
                 const float h = __bfloat162float(__float2bfloat16_rn(av[c] / (1.0f + expf(-av[c])) * __uint_as_float(va[c])));
-                beyond |= beyond_f16(h);
-                if (c < live) dst[static_cast<size_t>(c) * N] = __float2half_rn(fminf(fmaxf(h, -65504.0f), 65504.0f));
+                beyond |= c < live && beyond_f16(h);  // columns past the last token read whatever lies behind it
+                if (c < live) dst[static_cast<size_t>(c) * a.hid_stride] = __float2half_rn(fminf(fmaxf(h, -65504.0f), 65504.0f));
               }
             } else {
 #pragma unroll
               for (int c = 0; c < 32; ++c) {
                 const float h = __bfloat162float(__float2bfloat16_rn(fmaxf(__uint_as_float(va[c]), 0.0f)));
-                beyond |= beyond_f16(h);
-                if (c < live) dst[static_cast<size_t>(c) * N] = __float2half_rn(fminf(h, 65504.0f));
+                beyond |= c < live && beyond_f16(h);  // columns past the last token read whatever lies behind it
+                if (c < live) dst[static_cast<size_t>(c) * a.hid_stride] = __float2half_rn(fminf(h, 65504.0f));
               }
             }
             if (beyond) atomicOr(a.check_word, CHECK_F16_RANGE);  // saturated above: reported, not silent
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(128)
     scatter_x16_kernel(const ExpertDev* __restrict__ experts, const __nv_bfloat16* __restrict__ x,
                        const int32_t* __restrict__ ids, const int32_t* __restrict__ perm, const int32_t* __restrict__ off,
                        int E, int* __restrict__ plan, int top_k, int d, int n_pairs, int cnt_lo, int cnt_hi,
-                       __half* __restrict__ xs, int* __restrict__ check_word) {
+                       __half* __restrict__ xs, int xs_stride, int* __restrict__ check_word) {
   pdl_wait();
   pdl_trigger();
   if (plan && blockIdx.x == 0 && threadIdx.x < 32) {
@@ -568,7 +569,7 @@ __global__ void __launch_bounds__(128)
   if (cnt_slot < cnt_lo || cnt_slot > cnt_hi) return;  // this expert's rows belong to another kernel family
   const int bits = experts[e_slot].bits;
   const __nv_bfloat16* src = x + static_cast<size_t>(pair / top_k) * d;
-  __half* dst = xs + static_cast<size_t>(slot) * d;
+  __half* dst = xs + static_cast<size_t>(slot) * xs_stride;
   bool beyond = false;
   for (int k = threadIdx.x; k < d; k += blockDim.x) {
     const float xv = __bfloat162float(src[k]);
@@ -586,10 +587,10 @@ bool ffn_umma_supported(const LayerDims& L) {
 }
 
 cudaError_t launch_scatter_x16(const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* ids,
-                               const int32_t* perm, const int32_t* off, int* plan, void* xs16, int n_pairs,
+                               const int32_t* perm, const int32_t* off, int* plan, void* xs16, int xs_stride, int n_pairs,
                                int cnt_lo, int cnt_hi, int* check_word, cudaStream_t st) {
   return launch_chain(scatter_x16_kernel, dim3(n_pairs), dim3(128), 0, st, experts, reinterpret_cast<const __nv_bfloat16*>(x), ids,
-                      perm, off, L.E, plan, L.top_k, L.d_model, n_pairs, cnt_lo, cnt_hi, reinterpret_cast<__half*>(xs16), check_word);
+                      perm, off, L.E, plan, L.top_k, L.d_model, n_pairs, cnt_lo, cnt_hi, reinterpret_cast<__half*>(xs16), xs_stride, check_word);
 }
 
 size_t ffn_umma_scratch_bytes(const LayerDims& L) {
@@ -610,15 +611,15 @@ int ffn_umma_zsplit(const LayerDims& L, int T, int sms) {
   return (halves_ok && halves > whole + 0.03) ? 2 : 1;
 }
 
-cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, const int* plan, const void* in16,
-                            void* hidden16, float* o, float* scratch, int n_pairs, int zsplit, int* check_word,
+cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, const int* plan, const void* in16, int in_stride,
+                            void* hidden16, int hid_stride, float* o, float* scratch, int n_pairs, int zsplit, int* check_word,
                             cudaStream_t st) {
   if (phase == 0 && L.act == EMOE_ACT_SWIGLU && !scratch) return cudaErrorInvalidValue;
   const int N = phase == 0 ? L.d_ff : L.d_model;
   const int K = phase == 0 ? L.d_model : L.d_ff;
   CUtensorMap tmap_b;
   if (encode_tmap_2d(&tmap_b, /*fp16*/ 1, in16, static_cast<uint64_t>(K), static_cast<uint64_t>(n_pairs),
-                     static_cast<uint64_t>(K) * 2, UM_BK, UM_TOK) != 0)
+                     static_cast<uint64_t>(in_stride) * 2, UM_BK, UM_TOK) != 0)
     return cudaErrorInvalidValue;
   static int sms_of_device[64] = {};
   int dev = 0;
@@ -642,6 +643,7 @@ cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, co
   a.wmaps = static_cast<const CUtensorMap*>(wmaps);
   a.plan = plan;
   a.hidden16 = reinterpret_cast<__half*>(hidden16);
+  a.hid_stride = hid_stride;
   a.o = o;
   a.scratch = scratch;
   a.zsplit = zsplit < 1 ? 1 : zsplit;

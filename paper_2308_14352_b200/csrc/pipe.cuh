@@ -6,7 +6,7 @@
 
 namespace emoe {
 
-constexpr unsigned PIPE_WAIT_LIMIT = 1u << 22;  // polls before a wait gives up (~0.2 s)
+constexpr unsigned PIPE_WAIT_LIMIT = 1u << 22;  // polls before a polling wait gives up (~0.2 s)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
@@ -40,16 +40,26 @@ __device__ __forceinline__ bool mbar_try_wait_parked(uint32_t bar, uint32_t pari
       : "memory");
   return ok != 0;
 }
-// Bounded wait.  Returns false (after flagging the check word) if the phase never completed.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* check_word, volatile int* abort_flag) {
-  for (unsigned i = 0; i < PIPE_WAIT_LIMIT; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
+constexpr unsigned long long PIPE_WAIT_NS = 500000000ull;  // a wait gives up after half a second
+constexpr uint32_t PIPE_PARK_NS = 20000;                   // how long a waiting thread may be parked at a time
+
+// The rest of a wait whose first test failed.  Parked, not polled: the warps that feed a pipeline wait for most
+// of its time, and their polling was a third of the instructions the SM executed.
+static __device__ __noinline__ bool mbar_wait_parked(uint32_t bar, uint32_t parity, int* check_word, volatile int* abort_flag) {
+  unsigned long long t0, t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  do {
+    if (mbar_try_wait_parked(bar, parity, PIPE_PARK_NS)) return true;
     if (*abort_flag) return false;
-    if (i > 64) __nanosleep(40);
-  }
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  } while (t - t0 < PIPE_WAIT_NS);
   *abort_flag = 1;
   atomicOr(check_word, CHECK_WAIT_TIMEOUT);
   return false;
+}
+// Bounded wait.  Returns false (after flagging the check word) if the phase never completed.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* check_word, volatile int* abort_flag) {
+  return mbar_try_wait(bar, parity) || mbar_wait_parked(bar, parity, check_word, abort_flag);
 }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int c0, int c1, uint32_t bar) {
   asm volatile(

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(ROUTER_THREADS)
   extern __shared__ float smem[];
   __shared__ int s_ids[RPS_MAX_PAIRS];
   __shared__ int s_off[EMOE_MAX_EXPERTS + 1];
-  __shared__ int s_red[2][ROUTER_THREADS / 32];
+  __shared__ int s_red[3][ROUTER_THREADS / 32];
   __shared__ int s_ok;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t = blockIdx.x;
@@ -127,24 +127,36 @@ __global__ void __launch_bounds__(ROUTER_THREADS)
   for (int j = 0; j < top_k; ++j) {
     const int p = t * top_k + j;
     const int e = s_ids[p];
-    int before = 0;
+    int lower = 0, rank = 0, same = 0;
     for (int q = tid; q < n_pairs; q += ROUTER_THREADS) {
       const int eq = s_ids[q];
-      before += eq < e || (eq == e && q < p);
+      lower += eq < e;
+      rank += eq == e && q < p;
+      same += eq == e;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    lower = __reduce_add_sync(0xffffffffu, lower);
+    rank = __reduce_add_sync(0xffffffffu, rank);
+    same = __reduce_add_sync(0xffffffffu, same);
     __syncthreads();  // s_red of the previous pair has been read
-    if (lane == 0) s_red[0][warp] = before;
+    if (lane == 0) {
+      s_red[0][warp] = lower;
+      s_red[1][warp] = rank;
+      s_red[2][warp] = same;
+    }
     __syncthreads();
-    int slot = 0;
+    lower = rank = same = 0;
 #pragma unroll
-    for (int w = 0; w < ROUTER_THREADS / 32; ++w) slot += s_red[0][w];
+    for (int w = 0; w < ROUTER_THREADS / 32; ++w) {
+      lower += s_red[0][w];
+      rank += s_red[1][w];
+      same += s_red[2][w];
+    }
+    const int slot = lower + rank;
     if (tid == 0) {
       perm[slot] = p;
       slot_of_pair[p] = slot;
     }
-    scatter_any(x + static_cast<size_t>(t) * d, xs_out, xsc, slot, d, experts[e].bits, fmt, check_word);
+    scatter_any(x + static_cast<size_t>(t) * d, xs_out, xsc, lower, same, rank, d, experts[e].bits, fmt, check_word);
   }
 }
 
