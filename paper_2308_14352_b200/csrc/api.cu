@@ -69,6 +69,7 @@ WorkspaceLayout make_layout(const LayerDims& L, int T) {
   const size_t P = static_cast<size_t>(T) * L.top_k;
   w.ksplit = 1;
   if (ffn_mma_supported(L)) w.ksplit = ffn_mma_ksplit(L, T);
+  else w.ksplit = ffn_gemv_ksplit(L);
   if (ffn_tma_supported(L) && ffn_tma_ksplit(L, T) > w.ksplit) w.ksplit = ffn_tma_ksplit(L, T);
   if (ffn_i8_supported(L) && ffn_i8_ksplit(L, T) > w.ksplit) w.ksplit = ffn_i8_ksplit(L, T);
   size_t o = 0;
@@ -532,10 +533,11 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
     EMOE_LAUNCH(ctx, launch_ffn_mma(1, L, table, reinterpret_cast<const __nv_bfloat16*>(hidden), off,
                                   reinterpret_cast<__nv_bfloat16*>(hidden), o_part, ksplit, P, T, st));
   } else {
+    ksplit = ffn_gemv_ksplit(L) < w.ksplit ? ffn_gemv_ksplit(L) : w.ksplit;
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
-    EMOE_LAUNCH(ctx, launch_ffn_gemv(0, L, table, x, perm, off, hidden, o_part, P, st));
+    EMOE_LAUNCH(ctx, launch_ffn_gemv(0, L, table, x, perm, off, hidden, o_part, ksplit, P, st));
     if (ev[1]) EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
-    EMOE_LAUNCH(ctx, launch_ffn_gemv(1, L, table, x, perm, off, hidden, o_part, P, st));
+    EMOE_LAUNCH(ctx, launch_ffn_gemv(1, L, table, x, perm, off, hidden, o_part, ksplit, P, st));
   }
   if (ev[2]) EMOE_CUDA(ctx, cudaEventRecord(ev[2], st));
   EMOE_LAUNCH(ctx, launch_combine(o_part, ksplit, static_cast<size_t>(P), gates_use, slot_of_pair, T, L.top_k, L.d_model,

@@ -60,7 +60,7 @@ bool dims_from_desc(const emoe_layer_desc* d, LayerDims* L) {
 StaticLayout layout_for(const LayerDims& L, int T) {
   StaticLayout w{};
   const size_t P = static_cast<size_t>(T) * L.top_k;
-  w.ksplit = ffn_mma_supported(L) ? ffn_mma_ksplit(L, T) : 1;
+  w.ksplit = ffn_mma_supported(L) ? ffn_mma_ksplit(L, T) : ffn_gemv_ksplit(L);
   size_t o = 0;
   w.check = o;        o += align_up(sizeof(int));
   w.table = o;        o += align_up(sizeof(ExpertDev) * L.E);
@@ -170,9 +170,9 @@ extern "C" int emoe_moe_forward_routed_static(int device, const emoe_layer_desc*
                             reinterpret_cast<__nv_bfloat16*>(hidden), o_part, w.ksplit, P, T, st));
     EMOE_TRY(launch_combine(o_part, w.ksplit, static_cast<size_t>(P), gates, slot_of_pair, T, L.top_k, L.d_model, y, st));
   } else {
-    EMOE_TRY(launch_ffn_gemv(0, L, table, x, perm, off, hidden, o_part, P, st));
-    EMOE_TRY(launch_ffn_gemv(1, L, table, x, perm, off, hidden, o_part, P, st));
-    EMOE_TRY(launch_combine(o_part, 1, static_cast<size_t>(P), gates, slot_of_pair, T, L.top_k, L.d_model, y, st));
+    EMOE_TRY(launch_ffn_gemv(0, L, table, x, perm, off, hidden, o_part, w.ksplit, P, st));
+    EMOE_TRY(launch_ffn_gemv(1, L, table, x, perm, off, hidden, o_part, w.ksplit, P, st));
+    EMOE_TRY(launch_combine(o_part, w.ksplit, static_cast<size_t>(P), gates, slot_of_pair, T, L.top_k, L.d_model, y, st));
   }
 #undef EMOE_TRY
   return EMOE_OK;

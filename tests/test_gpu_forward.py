@@ -61,6 +61,22 @@ def test_forward_cuda_core_path(act, adt, group, sdt, d, f, E, k, gate, bits, T)
     _run_case(shape, bits, T, seed=21, path=1)
 
 
+GEMV_EDGE_CASES = [
+    # rows shorter than a lane group's words, slices of unequal length, one to many tokens per expert, several passes
+    ("relu", "f32", 0, "f32", 64, 32, 2, 1, "softmax", [4, 8], 1),
+    ("swiglu", "f32", 64, "f16", 64, 1088, 2, 2, "softmax_renorm", [2, 4], 3),        # 1088 = one slice of 576 and one of 512
+    ("relu", "f32", 0, "f32", 1024, 2112, 3, 1, "softmax", [8, 4, 2], 33),
+    ("swiglu", "bf16", 64, "f16", 1088, 1024, 2, 1, "softmax", [4, 8], 21),
+    ("relu", "f32", 0, "f16", 32, 17408, 2, 1, "softmax", [4, 8], 2),                 # more slices than partial-sum planes
+]
+
+
+@pytest.mark.parametrize("act,adt,group,sdt,d,f,E,k,gate,bits,T", GEMV_EDGE_CASES)
+def test_forward_cuda_core_path_at_the_edges_of_its_slices(act, adt, group, sdt, d, f, E, k, gate, bits, T):
+    shape = inputs.LayerShape(d, f, E, k, act, gate, group, sdt, adt)
+    _run_case(shape, bits, T, seed=23, path=1)
+
+
 MMA_CASES = [
     ("relu", 128, "f16", 256, 512, 4, 1, "softmax", [2, 4, 8, 4], 10),
     ("relu", 128, "f16", 768, 3072, 8, 1, "softmax", [8, 4, 2, 4, 8, 2, 4, 8], 64),
