@@ -408,6 +408,21 @@ int emoe_cache_acquire(emoe_ctx* ctx, const int64_t* ids, int n, int current_lay
  * load into one of these slots waits (on the device) until that point of the stream. */
 int emoe_cache_release(emoe_ctx* ctx, const int64_t* ids, int n, void* compute_stream);
 
+/* One layer of a stack whose experts live in the cache, as one call (Section 3.3's pipeline: route,
+ * preload what the next layer will probably need, get this layer's experts, compute):
+ *   emoe_router_topk -> ids, gates (device) and pinned_ids;  synchronise compute_stream (the picks
+ *   decide which experts are needed);  emoe_rank_experts(prior, picks) and emoe_prefetch_experts
+ *   for the n_prefetch first ids (prior NULL or n_prefetch 0: no prefetch);  emoe_cache_acquire for the
+ *   activated experts;  emoe_moe_forward_routed -> y;  emoe_cache_release.
+ * Expert e of this layer is registered as first_id + e, of the next layer as next_first_id + e.
+ * prior: host array as for emoe_rank_experts; ids / gates / y: device buffers as for
+ * emoe_moe_forward; pinned_ids: [T][top_k] in pinned host memory, valid when the call returns.
+ * Decisions, counters and results are those of the single calls. */
+int emoe_cached_layer(emoe_ctx* ctx, const emoe_layer_desc* desc, int layer, const void* x, int T, const float* router_W,
+                      const float* router_bias, int bias_token_stride, int64_t first_id, const float* prior, int n_prefetch,
+                      int64_t next_first_id, int32_t* ids, float* gates, float* y, int32_t* pinned_ids, void* compute_stream,
+                      void* copy_stream);
+
 /* Slot that holds the expert, -1 if none. */
 int emoe_cache_slot_of(emoe_ctx* ctx, int64_t id);
 int emoe_cache_get_stats(emoe_ctx* ctx, emoe_cache_stats* out);

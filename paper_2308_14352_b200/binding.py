@@ -40,7 +40,7 @@ EXPORTS = (
     "emoe_set_fused_projections", "emoe_set_fused_routing", "emoe_set_fused_layer", "emoe_kernels_last_forward", "emoe_set_wait_limit",
     "emoe_debug_expect_extra_completions",
     "emoe_cache_create", "emoe_register_expert", "emoe_prefetch_experts", "emoe_cache_acquire", "emoe_cache_release",
-    "emoe_cache_slot_of", "emoe_cache_get_stats", "emoe_cache_set_timing", "emoe_last_expert_counts", "emoe_policy_create", "emoe_policy_destroy", "emoe_policy_register",
+    "emoe_cached_layer", "emoe_cache_slot_of", "emoe_cache_get_stats", "emoe_cache_set_timing", "emoe_last_expert_counts", "emoe_policy_create", "emoe_policy_destroy", "emoe_policy_register",
     "emoe_policy_prefetch", "emoe_policy_acquire", "emoe_policy_release", "emoe_policy_get_stats", "emoe_rank_experts",
     "emoe_build_profile2", "emoe_rank_experts2",
 )
@@ -122,6 +122,8 @@ def lib() -> ctypes.CDLL:
         L.emoe_prefetch_experts.argtypes = [vp, ctypes.POINTER(i64), i32, i32, vp]
         L.emoe_cache_acquire.argtypes = [vp, ctypes.POINTER(i64), i32, i32, vp, vp, ctypes.POINTER(emoe_expert)]
         L.emoe_cache_release.argtypes = [vp, ctypes.POINTER(i64), i32, vp]
+        L.emoe_cached_layer.argtypes = [vp, ctypes.POINTER(emoe_layer_desc), i32, vp, i32, vp, vp, i32, i64, vp, i32, i64, vp, vp,
+                                        vp, vp, vp, vp]
         L.emoe_cache_slot_of.argtypes = [vp, i64]
         L.emoe_cache_get_stats.argtypes = [vp, ctypes.POINTER(emoe_cache_stats)]
         L.emoe_cache_set_timing.argtypes = [vp, i32]
@@ -342,6 +344,14 @@ def emoe_cache_acquire(ctx, ids, current_layer: int, compute_stream: int, copy_s
 
 def emoe_cache_release(ctx, ids, compute_stream: int) -> None:
     _check(lib().emoe_cache_release(ctx, _i64_array(ids), len(ids), compute_stream), "emoe_cache_release")
+
+
+def emoe_cached_layer(ctx, desc: emoe_layer_desc, layer: int, x_ptr, T, router_W_ptr, bias_ptr, bias_token_stride, first_id: int,
+                      prior_ptr, n_prefetch: int, next_first_id: int, ids_ptr, gates_ptr, y_ptr, pinned_ids_ptr,
+                      compute_stream: int, copy_stream: int) -> None:
+    _check(lib().emoe_cached_layer(ctx, desc, layer, x_ptr, T, router_W_ptr, bias_ptr, bias_token_stride, first_id, prior_ptr,
+                                   n_prefetch, next_first_id, ids_ptr, gates_ptr, y_ptr, pinned_ids_ptr, compute_stream,
+                                   copy_stream), "emoe_cached_layer")
 
 
 def emoe_cache_slot_of(ctx, expert_id: int) -> int:

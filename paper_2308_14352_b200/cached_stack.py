@@ -4,7 +4,7 @@ library's HBM expert cache: the predict-then-prefetch pipeline of the paper's Se
 (memory, streams, the order of the library calls); the arithmetic runs in the library's kernels
 and the cache decisions in its host code.
 
-Per layer and token batch:
+Per layer and token batch, one call (emoe_cached_layer):
   ids, gates = emoe_router_topk(x, Wr, bias)           # bias ties the routing to the prior
   emoe_prefetch_experts(ranked experts of the next layer)   # copy stream, overlaps this layer
   emoe_cache_acquire(activated experts)                # compute stream waits on the device
@@ -12,7 +12,6 @@ Per layer and token batch:
 """
 from __future__ import annotations
 
-import ctypes
 from typing import List, Optional, Sequence
 
 import numpy as np
@@ -62,11 +61,12 @@ class CachedStack:
                     s = torch.empty(N * (K // G), dtype=sdt, device=self.dev)
                     B.emoe_pack_expert(self.ctx, W.data_ptr(), N, K, self.bits[e], shape.group, _SDT[shape.scale_dtype],
                                        p.data_ptr(), s.data_ptr(), 0)
-                    pm.append(p.cpu().pin_memory())
-                    sm.append(s.cpu().pin_memory())
-                    del W, p, s
-                row.append((pm, sm))
+                    pm.append(p)
+                    sm.append(s)
+                    del W
                 nb = self._nbytes(pm, sm)
+                pm, sm = self._pin(pm, sm, nb)
+                row.append((pm, sm))
                 self.expert_bytes += sum(nb)
                 slot_bytes = max(slot_bytes, sum((b + 255) // 256 * 256 for b in nb))
             self.host.append(row)
@@ -83,6 +83,7 @@ class CachedStack:
         rng = np.random.default_rng(seed)
         self.Wr = [torch.from_numpy((rng.standard_normal((shape.d_model, E)) * 0.02).astype(np.float32)).to(self.dev)
                    for _ in range(n_layers)]
+        self._Wr_ptrs = [w.data_ptr() for w in self.Wr]
         prior = rng.random((E, E)) ** 4          # peaked rows: a few likely successors per expert
         self.prior = (prior / prior.sum(axis=1, keepdims=True)).astype(np.float32)
         self._exposed_ns_seen = 0
@@ -90,6 +91,12 @@ class CachedStack:
         self.gates = torch.empty(max_tokens, shape.top_k, dtype=torch.float32, device=self.dev)
         self.bias = torch.zeros(max_tokens, E, dtype=torch.float32, device=self.dev)
         self.y = torch.empty(max_tokens, shape.d_model, dtype=torch.float32, device=self.dev)
+        # picks of a layer and the router bias on their way to and from the device
+        self._pin_ids = torch.empty(max_tokens, shape.top_k, dtype=torch.int32, pin_memory=True)
+        self._pin_bias = torch.empty(max_tokens, E, dtype=torch.float32, pin_memory=True)
+        # one previous pick per token: the bias is a row of a fixed table
+        self._bias_rows = (beta * np.log(self.prior[:, None].mean(axis=1) + 1e-9)).astype(np.float32)
+        self._bias_rows_dev = torch.from_numpy(self._bias_rows).to(self.dev)
         torch.cuda.synchronize(self.dev)
 
     def draw_matrix(self, l: int, e: int, m: int) -> torch.Tensor:
@@ -97,6 +104,23 @@ class CachedStack:
         N, K = self.shape.matrix_shape(m)
         self._gen.manual_seed((self.seed << 32) ^ (l << 16) ^ (e << 4) ^ m)
         return torch.randn(N, K, generator=self._gen, device=self.dev, dtype=torch.float32) * 0.02
+
+    @staticmethod
+    def _pin(pm, sm, nb):
+        """Copies of the matrices and scales in one pinned block, at the 256-byte boundaries they will have in a cache slot
+        (the library then loads an expert with one copy)."""
+        at, total = [], 0
+        for b in nb:
+            at.append(total)
+            total += (b + 255) // 256 * 256
+        block = torch.empty(total, dtype=torch.uint8, pin_memory=True)
+
+        def put(t, o):
+            v = block[o:o + t.numel() * t.element_size()].view(t.dtype)
+            v.copy_(t)
+            return v
+
+        return [put(t, at[m]) for m, t in enumerate(pm)], [put(t, at[3 + m]) for m, t in enumerate(sm)]
 
     @staticmethod
     def _nbytes(pm, sm):
@@ -132,51 +156,42 @@ class CachedStack:
         Returns the picks of every layer (host arrays).  With measure=True the library brackets
         every acquire by two events on the compute stream (emoe_cache_set_timing): their distance is
         the time the compute stream stood still for a load (the exposed copy time).  If `outputs` is a list, every
-        layer appends (gates, y) of the batch to it (device copies)."""
+        layer appends (gates, y) of the batch to it (device tensors of their own)."""
         sh, E = self.shape, self.shape.n_experts
         T = xs[0].shape[0]
         cs, cps = self.compute.cuda_stream, self.copy.cuda_stream
         picks = []
         prev = None
+        B.emoe_cache_set_timing(self.ctx, measure)
+        host_ids, host_bias = self._pin_ids.numpy()[:T], self._pin_bias.numpy()
+        n_prefetch = (E if T > 1 else self.n_prefetch) if prefetch else 0
+        ids_ptr, pin_ids_ptr, prior_ptr = self.ids.data_ptr(), self._pin_ids.data_ptr(), self.prior.ctypes.data
+        gates_ptr, y_ptr, gates_step, y_step = self.gates.data_ptr(), self.y.data_ptr(), 0, 0
         with torch.cuda.stream(self.compute):
+            if outputs is not None:  # straight into the tensors that are handed out
+                gates = torch.empty((self.n_layers, T, sh.top_k), dtype=torch.float32, device=self.dev)
+                y = torch.empty((self.n_layers, T, sh.d_model), dtype=torch.float32, device=self.dev)
+                outputs.extend(zip(gates.unbind(), y.unbind()))
+                gates_ptr, y_ptr, gates_step, y_step = gates.data_ptr(), y.data_ptr(), T * sh.top_k * 4, T * sh.d_model * 4
             for l in range(self.n_layers):
                 bias_ptr, stride = None, 0
                 if prev is not None:
                     # routing follows the prior: bias[t] = beta * log(mean of the prior rows of t's previous picks)
-                    b = self.beta * np.log(self.prior[prev].mean(axis=1) + 1e-9)
-                    self.bias[:T].copy_(torch.from_numpy(b.astype(np.float32)), non_blocking=True)
-                    bias_ptr, stride = self.bias.data_ptr(), E
-                B.emoe_router_topk(self.ctx, xs[l].data_ptr(), B.DTYPE_BF16, T, sh.d_model, self.Wr[l].data_ptr(), bias_ptr,
-                                   stride, E, sh.top_k, B.GATE_SOFTMAX_RENORM if sh.gate_mode == "softmax_renorm" else B.GATE_SOFTMAX,
-                                   self.ids.data_ptr(), self.gates.data_ptr(), None, cs)
-                ids = self.ids[:T].cpu().numpy()      # the picks decide which experts are needed: read back
-                picks.append(ids)
-                active = sorted(set(ids.reshape(-1).tolist()))
-                if prefetch and l + 1 < self.n_layers:
-                    order = B.emoe_rank_experts(self.prior, np.array(active, dtype=np.int32))
-                    n = E if T > 1 else self.n_prefetch
-                    B.emoe_prefetch_experts(self.ctx, [self.expert_id(l + 1, int(e)) for e in order[:n]], l, cps)
-                eids = [self.expert_id(l, e) for e in active]
-                B.emoe_cache_set_timing(self.ctx, measure)
-                acq = B.emoe_cache_acquire(self.ctx, eids, l, cs, cps)
-                by_e = {e: acq[i] for i, e in enumerate(active)}
-                first = acq[0]
-                table = (B.emoe_expert * E)()
-                for e in range(E):
-                    # entries of experts nobody picked are never read; they borrow an acquired expert
-                    # whole (pointers AND width, so that whatever is derived from an entry stays
-                    # inside that expert's slot)
-                    src = by_e.get(e, first)
-                    table[e].bits = self.bits[e] if e in by_e else self.bits[active[0]]
-                    for m in range(3):
-                        table[e].packed[m] = src.packed[m]
-                        table[e].scales[m] = src.scales[m]
-                B.emoe_moe_forward_routed(self.ctx, self.desc, xs[l].data_ptr(), T, self.ids.data_ptr(), self.gates.data_ptr(),
-                                          table, self.y.data_ptr(), None, cs)
-                B.emoe_cache_release(self.ctx, eids, cs)
-                if outputs is not None:
-                    outputs.append((self.gates[:T].clone(), self.y[:T].clone()))
-                prev = ids
+                    if T == 1 and sh.top_k == 1:
+                        bias_ptr, stride = self._bias_rows_dev.data_ptr() + int(prev[0, 0]) * E * 4, E
+                    else:
+                        if sh.top_k == 1:
+                            host_bias[:T] = self._bias_rows[prev[:, 0]]
+                        else:
+                            host_bias[:T] = self.beta * np.log(self.prior[prev].mean(axis=1) + 1e-9)
+                        self.bias[:T].copy_(self._pin_bias[:T], non_blocking=True)
+                        bias_ptr, stride = self.bias.data_ptr(), E
+                more = l + 1 < self.n_layers
+                B.emoe_cached_layer(self.ctx, self.desc, l, xs[l].data_ptr(), T, self._Wr_ptrs[l], bias_ptr, stride,
+                                    self.expert_id(l, 0), prior_ptr if more else None, n_prefetch, self.expert_id(l + 1, 0),
+                                    ids_ptr, gates_ptr + l * gates_step, y_ptr + l * y_step, pin_ids_ptr, cs, cps)
+                prev = host_ids.copy()
+                picks.append(prev)
         return picks
 
     def exposed_ms(self) -> float:

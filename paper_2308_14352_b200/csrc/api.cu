@@ -29,7 +29,8 @@ constexpr size_t TABLE_BLOCK_BYTES = TABLE_SMAPS_OFFSET + TMAP_BYTES * 3 * EMOE_
 
 struct TableEntry {
   std::vector<emoe_expert> host;
-  int d_model = 0, d_ff = 0, act = 0;
+  int d_model = 0, d_ff = 0, act = 0, group = 0, scale_f16 = 0;
+  bool maps_built = false;  // the tensor maps were asked for (has_tmaps: and exist)
   bool has_tmaps = false;
   bool scales16 = false;  // every scale channel is 16-byte aligned (bulk copies of scales are possible)
 };
@@ -189,52 +190,16 @@ int cached_tmap(emoe_ctx* ctx, int kind, void* out, const void* ptr, int a, int 
   return it->second.rc;
 }
 
-// Device copy of a host expert table (entries + tensor maps); uploaded on `st` the first time
-// its content is seen.  *tmaps is null when the shape has no TMA path.
-int get_table(emoe_ctx* ctx, const LayerDims& L, const emoe_expert* host, cudaStream_t st, const ExpertDev** out,
-              const void** tmaps, const void** smaps) {
-  const int E = L.E;
-  for (size_t i = 0; i < ctx->tables.size(); ++i) {
-    const TableEntry& te = ctx->tables[i];
-    if (static_cast<int>(te.host.size()) != E || te.d_model != L.d_model || te.d_ff != L.d_ff || te.act != L.act) continue;
-    bool same = true;
-    for (int e = 0; e < E && same; ++e) {
-      same = te.host[e].bits == host[e].bits;
-      for (int m = 0; m < 3 && same; ++m)
-        same = te.host[e].packed[m] == host[e].packed[m] && te.host[e].scales[m] == host[e].scales[m];
-    }
-    if (same) {
-      ctx->table_used[i] = ++ctx->table_clock;
-      *out = reinterpret_cast<const ExpertDev*>(ctx->tables_dev + i * TABLE_BLOCK_BYTES);
-      *tmaps = te.has_tmaps ? ctx->tables_dev + i * TABLE_BLOCK_BYTES + TABLE_MAPS_OFFSET : nullptr;
-      *smaps = te.has_tmaps && te.scales16 ? ctx->tables_dev + i * TABLE_BLOCK_BYTES + TABLE_SMAPS_OFFSET : nullptr;
-      return EMOE_OK;
-    }
-  }
-  // A new table: the next unused block, or (tables that change from call to call, e.g. pointers
-  // into an expert cache) the block that was used longest ago, once its upload has left the
-  // pinned mirror.  Kernels that read the old device copy were enqueued earlier on the stream.
-  size_t slot = ctx->tables.size();
-  const bool recycle = slot >= MAX_TABLES;
-  if (recycle) {
-    slot = 0;
-    for (size_t i = 1; i < ctx->tables.size(); ++i)
-      if (ctx->table_used[i] < ctx->table_used[slot]) slot = i;
-    EMOE_CUDA(ctx, cudaEventSynchronize(ctx->table_events[slot]));
-  }
+// The tensor maps of a table (weights and, where their rows allow one, scale channels), built in the pinned mirror and
+// uploaded on `st`.
+int upload_maps(emoe_ctx* ctx, const LayerDims& L, size_t slot, cudaStream_t st) {
+  TableEntry& te = ctx->tables[slot];
   char* pin_block = ctx->tables_pin + slot * TABLE_BLOCK_BYTES;
-  ExpertDev* pin = reinterpret_cast<ExpertDev*>(pin_block);
-  const int nmat = L.act == EMOE_ACT_RELU ? 2 : 3;
-  bool maps_ok = ffn_tma_supported(L);
-  bool scales16 = true;
-  const int ssz = L.scale_f16 ? 2 : 4;
-  for (int e = 0; e < E; ++e) {
-    pin[e].bits = host[e].bits;
-    pin[e].pad = 0;
-    for (int m = 0; m < 3; ++m) {
-      pin[e].packed[m] = static_cast<const uint8_t*>(host[e].packed[m]);
-      pin[e].scales[m] = host[e].scales[m];
-    }
+  char* dev = ctx->tables_dev + slot * TABLE_BLOCK_BYTES;
+  const emoe_expert* host = te.host.data();
+  const int E = L.E, nmat = L.act == EMOE_ACT_RELU ? 2 : 3, ssz = L.scale_f16 ? 2 : 4;
+  bool maps_ok = ffn_tma_supported(L), scales16 = true;
+  for (int e = 0; e < E && maps_ok; ++e)
     for (int m = 0; m < nmat && maps_ok; ++m) {
       const bool first = m < nmat - 1;
       const int N = first ? L.d_ff : L.d_model, K = first ? L.d_model : L.d_ff;
@@ -246,37 +211,90 @@ int get_table(emoe_ctx* ctx, const LayerDims& L, const emoe_expert* host, cudaSt
       if (!aligned(host[e].scales[m], 16)) scales16 = false;
       else if (cached_tmap(ctx, 1, smap, host[e].scales[m], N, row_bytes, 0) != 0) std::memset(smap, 0, TMAP_BYTES);
     }
-  }
-  char* dev = ctx->tables_dev + slot * TABLE_BLOCK_BYTES;
-  if (maps_ok) {  // entries + weight maps in one copy, the scale maps (behind the unused weight maps) in another
-    EMOE_CUDA(ctx, cudaMemcpyAsync(dev, pin_block, TABLE_MAPS_OFFSET + TMAP_BYTES * 3 * E, cudaMemcpyHostToDevice, st));
-    if (scales16)
-      EMOE_CUDA(ctx, cudaMemcpyAsync(dev + TABLE_SMAPS_OFFSET, pin_block + TABLE_SMAPS_OFFSET, TMAP_BYTES * 3 * E,
-                                     cudaMemcpyHostToDevice, st));
-  } else {
-    EMOE_CUDA(ctx, cudaMemcpyAsync(dev, pin_block, sizeof(ExpertDev) * E, cudaMemcpyHostToDevice, st));
-  }
-  TableEntry te;
-  te.host.assign(host, host + E);
-  te.d_model = L.d_model;
-  te.d_ff = L.d_ff;
-  te.act = L.act;
+  te.maps_built = true;
   te.has_tmaps = maps_ok;
   te.scales16 = scales16;
-  if (recycle) {
-    ctx->tables[slot] = std::move(te);
-  } else {
-    ctx->tables.push_back(std::move(te));
-    cudaEvent_t ev;
-    EMOE_CUDA(ctx, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-    ctx->table_events.push_back(ev);
-    ctx->table_used.push_back(0);
-  }
+  if (!maps_ok) return EMOE_OK;
+  EMOE_CUDA(ctx, cudaMemcpyAsync(dev + TABLE_MAPS_OFFSET, pin_block + TABLE_MAPS_OFFSET, TMAP_BYTES * 3 * E, cudaMemcpyHostToDevice, st));
+  if (scales16)
+    EMOE_CUDA(ctx, cudaMemcpyAsync(dev + TABLE_SMAPS_OFFSET, pin_block + TABLE_SMAPS_OFFSET, TMAP_BYTES * 3 * E, cudaMemcpyHostToDevice, st));
   EMOE_CUDA(ctx, cudaEventRecord(ctx->table_events[slot], st));
+  return EMOE_OK;
+}
+
+// Device copy of a host expert table (entries + tensor maps); uploaded on `st` the first time its content is
+// seen, the maps the first time a call needs them (want_maps: the one-launch layer does not, and
+// with an expert cache the table changes from call to call).  *tmaps is null when the shape has no
+// TMA path.
+int get_table(emoe_ctx* ctx, const LayerDims& L, const emoe_expert* host, bool want_maps, cudaStream_t st, const ExpertDev** out,
+              const void** tmaps, const void** smaps) {
+  const int E = L.E;
+  size_t slot = ctx->tables.size();
+  for (size_t i = 0; i < ctx->tables.size(); ++i) {
+    const TableEntry& te = ctx->tables[i];
+    if (static_cast<int>(te.host.size()) != E || te.d_model != L.d_model || te.d_ff != L.d_ff || te.act != L.act || te.group != L.group ||
+        te.scale_f16 != L.scale_f16)
+      continue;
+    bool same = true;
+    for (int e = 0; e < E && same; ++e) {
+      same = te.host[e].bits == host[e].bits;
+      for (int m = 0; m < 3 && same; ++m)
+        same = te.host[e].packed[m] == host[e].packed[m] && te.host[e].scales[m] == host[e].scales[m];
+    }
+    if (same) {
+      slot = i;
+      break;
+    }
+  }
+  if (slot == ctx->tables.size()) {
+    // A new table: the next unused block, or (tables that change from call to call, e.g. pointers
+    // into an expert cache) the block that was used longest ago, once its upload has left the
+    // pinned mirror.  Kernels that read the old device copy were enqueued earlier on the stream.
+    const bool recycle = slot >= MAX_TABLES;
+    if (recycle) {
+      slot = 0;
+      for (size_t i = 1; i < ctx->tables.size(); ++i)
+        if (ctx->table_used[i] < ctx->table_used[slot]) slot = i;
+      EMOE_CUDA(ctx, cudaEventSynchronize(ctx->table_events[slot]));
+    }
+    char* pin_block = ctx->tables_pin + slot * TABLE_BLOCK_BYTES;
+    ExpertDev* pin = reinterpret_cast<ExpertDev*>(pin_block);
+    for (int e = 0; e < E; ++e) {
+      pin[e].bits = host[e].bits;
+      pin[e].pad = 0;
+      for (int m = 0; m < 3; ++m) {
+        pin[e].packed[m] = static_cast<const uint8_t*>(host[e].packed[m]);
+        pin[e].scales[m] = host[e].scales[m];
+      }
+    }
+    EMOE_CUDA(ctx, cudaMemcpyAsync(ctx->tables_dev + slot * TABLE_BLOCK_BYTES, pin_block, sizeof(ExpertDev) * E, cudaMemcpyHostToDevice, st));
+    if (!recycle) {
+      cudaEvent_t ev;
+      EMOE_CUDA(ctx, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+      ctx->table_events.push_back(ev);
+      ctx->table_used.push_back(0);
+      ctx->tables.emplace_back();
+    }
+    TableEntry& te = ctx->tables[slot];
+    te.host.assign(host, host + E);
+    te.d_model = L.d_model;
+    te.d_ff = L.d_ff;
+    te.act = L.act;
+    te.group = L.group;
+    te.scale_f16 = L.scale_f16;
+    te.maps_built = te.has_tmaps = te.scales16 = false;
+    EMOE_CUDA(ctx, cudaEventRecord(ctx->table_events[slot], st));
+  }
+  if (want_maps && !ctx->tables[slot].maps_built) {
+    const int rc = upload_maps(ctx, L, slot, st);
+    if (rc != EMOE_OK) return rc;
+  }
   ctx->table_used[slot] = ++ctx->table_clock;
+  const TableEntry& te = ctx->tables[slot];
+  char* dev = ctx->tables_dev + slot * TABLE_BLOCK_BYTES;
   *out = reinterpret_cast<const ExpertDev*>(dev);
-  *tmaps = maps_ok ? dev + TABLE_MAPS_OFFSET : nullptr;
-  *smaps = maps_ok && scales16 ? dev + TABLE_SMAPS_OFFSET : nullptr;
+  *tmaps = te.has_tmaps ? dev + TABLE_MAPS_OFFSET : nullptr;
+  *smaps = te.has_tmaps && te.scales16 ? dev + TABLE_SMAPS_OFFSET : nullptr;
   return EMOE_OK;
 }
 
@@ -320,11 +338,23 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
     ~PdlScope() { g_pdl_enabled = false; }
   } pdl_scope(ctx->pdl && !ctx->timing);
 
+  // a handful of tokens on a small layer: router, both projections and the gate-weighted sum in one launch
+  bool one_launch_layer = false;
+  // as measured on a Switch-base-sized layer: 1.8 x faster than the chain of launches for one pair, 1.5 x for two to four, 1.25 x
+  // for eight, slower for sixteen (the projections then take several passes of dependent loads per warp)
+  const bool layer_wanted = ctx->fuse_layer == 1 || (ctx->fuse_layer == 2 && T * L.top_k <= 8);
+  if (layer_wanted && ctx->ffn_path == 0 && decode_layer_supported(L, T)) {
+    if (ctx->resident_layer_ctas < 0) {
+      ctx->resident_layer_ctas = decode_layer_resident_ctas(ctx->device);
+      EMOE_CUDA(ctx, cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device));
+    }
+    one_launch_layer = ctx->sms >= T && ctx->resident_layer_ctas >= ctx->sms;  // at least one CTA per SM, one per token
+  }
   ctx->kernels_last = 0;
   const ExpertDev* table = nullptr;
   const void* tmaps = nullptr;
   const void* smaps = nullptr;
-  rc = get_table(ctx, L, host_experts, st, &table, &tmaps, &smaps);
+  rc = get_table(ctx, L, host_experts, !one_launch_layer, st, &table, &tmaps, &smaps);
   if (rc != EMOE_OK) return rc;
 
   char* ws = ctx->workspace;
@@ -376,18 +406,6 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   if (ctx->resident_route_ctas < 0) ctx->resident_route_ctas = route_permute_scatter_resident_ctas(ctx->device);
   const bool one_launch_route =
       ctx->fuse_routing && one_launch_permute && !routed && route_permute_scatter_supported(L, T, ctx->resident_route_ctas);
-  // a handful of tokens on a small layer: router, both projections and the gate-weighted sum in one launch
-  bool one_launch_layer = false;
-  // as measured on a Switch-base-sized layer: 1.8 x faster than the chain of launches for one pair, 1.5 x for two to four, 1.25 x
-  // for eight, slower for sixteen (the projections then take several passes of dependent loads per warp)
-  const bool layer_wanted = ctx->fuse_layer == 1 || (ctx->fuse_layer == 2 && P <= 8);
-  if (layer_wanted && ctx->ffn_path == 0 && decode_layer_supported(L, T)) {
-    if (ctx->resident_layer_ctas < 0) {
-      ctx->resident_layer_ctas = decode_layer_resident_ctas(ctx->device);
-      EMOE_CUDA(ctx, cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device));
-    }
-    one_launch_layer = ctx->sms >= T && ctx->resident_layer_ctas >= ctx->sms;  // at least one CTA per SM, one per token
-  }
   if (!routed && !one_launch_route && !one_launch_layer)
     EMOE_LAUNCH(ctx, launch_router_topk(x, L.act_bf16, T, L.d_model, router_W, router_bias, bias_token_stride, L.E,
                                       L.top_k, L.gate_mode == EMOE_GATE_SOFTMAX_RENORM, ids, gates, nullptr, st));
@@ -553,6 +571,7 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
 namespace emoe {
 ExpertCache*& ctx_cache(emoe_ctx* ctx) { return ctx->cache; }
 int ctx_device(const emoe_ctx* ctx) { return ctx->device; }
+bool ctx_dependent_launch(const emoe_ctx* ctx) { return ctx->pdl && !ctx->timing; }
 int ctx_cuda_fail(emoe_ctx* ctx, cudaError_t e) { return cuda_fail(ctx, e); }
 }  // namespace emoe
 

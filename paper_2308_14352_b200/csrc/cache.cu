@@ -26,6 +26,7 @@ struct CacheExpert {
   const void* host[6];  // packed[0..2], scales[0..2] in pinned host memory (null = matrix not present)
   size_t bytes[6];
   size_t offset[6];  // placement inside a slot
+  int run_end[6];    // matrices m .. run_end[m]-1 lie in host memory as in the slot, in one allocation
   int slot;
   int64_t freq;        // activations so far (acquire calls)
   bool by_prefetch;    // brought in by a prefetch and not used since
@@ -228,13 +229,45 @@ int fill_expert(CacheExpert* e, int64_t id, int layer, int bits, const void* con
   return EMOE_OK;
 }
 
+// Which neighbouring matrices can be copied together: same distance in host memory as in the slot, and one host
+// allocation (the bytes between them are then readable, and the copy stays inside one pinned range).
+void find_runs(CacheExpert* e) {
+  typedef int (*AttrFn)(void*, int, unsigned long long);
+  static const AttrFn attr = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    return cudaGetDriverEntryPoint("cuPointerGetAttribute", &p, cudaEnableDefault, &q) == cudaSuccess ? reinterpret_cast<AttrFn>(p) : nullptr;
+  }();
+  constexpr int RANGE_START = 11;  // CU_POINTER_ATTRIBUTE_RANGE_START_ADDR
+  void* start[6] = {};
+  for (int m = 0; m < 6; ++m)
+    if (e->bytes[m] && (!attr || attr(&start[m], RANGE_START, reinterpret_cast<unsigned long long>(e->host[m])) != 0)) start[m] = nullptr;
+  for (int m = 0; m < 6; ++m) {
+    int end = m + 1;
+    for (int k = m + 1; e->bytes[m] && start[m] && k < 6; ++k) {
+      if (!e->bytes[k]) continue;
+      if (start[k] != start[m] || static_cast<const char*>(e->host[k]) - static_cast<const char*>(e->host[m]) !=
+                                      static_cast<ptrdiff_t>(e->offset[k]) - static_cast<ptrdiff_t>(e->offset[m]))
+        break;
+      end = k + 1;
+    }
+    e->run_end[m] = end;
+  }
+}
+
 // enqueue the copies of an expert into its slot on the copy stream, behind the slot's last reader
 cudaError_t load_into_slot(ExpertCache* c, const CacheExpert& e, int s, cudaStream_t copy) {
   cudaError_t err = cudaSuccess;
   if (c->idle_valid[static_cast<size_t>(s)]) err = cudaStreamWaitEvent(copy, c->idle[static_cast<size_t>(s)], 0);
   char* dst = c->base + static_cast<size_t>(s) * c->slot_bytes;
-  for (int m = 0; m < 6 && err == cudaSuccess; ++m)
-    if (e.bytes[m]) err = cudaMemcpyAsync(dst + e.offset[m], e.host[m], e.bytes[m], cudaMemcpyHostToDevice, copy);
+  // matrices that lie in one host allocation as they will lie in the slot travel as one copy: every further one costs
+  // the link some two microseconds
+  for (int m = 0; m < 6 && err == cudaSuccess; m = e.run_end[m]) {
+    if (!e.bytes[m]) continue;
+    int last = e.run_end[m] - 1;
+    while (!e.bytes[last]) --last;
+    err = cudaMemcpyAsync(dst + e.offset[m], e.host[m], e.offset[last] + e.bytes[last] - e.offset[m], cudaMemcpyHostToDevice, copy);
+  }
   if (err == cudaSuccess) err = cudaEventRecord(c->ready[static_cast<size_t>(s)], copy);
   return err;
 }
@@ -254,6 +287,7 @@ void expert_pointers(const ExpertCache* c, const CacheExpert& e, emoe_expert* ou
 // ---- accessors into the context (api.cu) ----------------------------------------------------
 ExpertCache*& ctx_cache(emoe_ctx* ctx);
 int ctx_device(const emoe_ctx* ctx);
+bool ctx_dependent_launch(const emoe_ctx* ctx);
 int ctx_cuda_fail(emoe_ctx* ctx, cudaError_t e);
 
 }  // namespace emoe
@@ -298,6 +332,7 @@ int emoe_register_expert(emoe_ctx* ctx, int64_t id, int layer, int bits, const v
   if (e.offset[5] + e.bytes[5] > c->slot_bytes) return EMOE_ERR_INVALID_ARG;  // does not fit a slot
   for (int m = 0; m < 3; ++m)
     if (e.bytes[m] && (reinterpret_cast<uintptr_t>(e.host[m]) & 15)) return EMOE_ERR_ALIGNMENT;
+  find_runs(&e);
   return c->policy.add(e) < 0 ? EMOE_ERR_INVALID_ARG : EMOE_OK;
 }
 
@@ -390,6 +425,69 @@ int emoe_cache_release(emoe_ctx* ctx, const int64_t* ids, int n, void* compute_s
     c->idle_valid[static_cast<size_t>(s)] = 1;
   }
   return rc;
+}
+
+int emoe_cached_layer(emoe_ctx* ctx, const emoe_layer_desc* desc, int layer, const void* x, int T, const float* router_W,
+                      const float* router_bias, int bias_token_stride, int64_t first_id, const float* prior, int n_prefetch,
+                      int64_t next_first_id, int32_t* ids, float* gates, float* y, int32_t* pinned_ids, void* compute_stream,
+                      void* copy_stream) {
+  if (!ctx || !ctx_cache(ctx) || !desc || !ids || !gates || !y || !pinned_ids || T <= 0) return EMOE_ERR_INVALID_ARG;
+  const int E = desc->n_experts, k = desc->top_k;
+  if (E < 1 || E > EMOE_MAX_EXPERTS || k < 1 || k > EMOE_MAX_TOP_K || k > E || n_prefetch < 0) return EMOE_ERR_INVALID_ARG;
+  if (!x || !router_W || desc->d_model <= 0) return EMOE_ERR_INVALID_ARG;
+  if (desc->act_dtype != EMOE_DTYPE_F32 && desc->act_dtype != EMOE_DTYPE_BF16) return EMOE_ERR_UNSUPPORTED;
+  if (desc->gate_mode != EMOE_GATE_SOFTMAX && desc->gate_mode != EMOE_GATE_SOFTMAX_RENORM) return EMOE_ERR_UNSUPPORTED;
+  if (router_bias && bias_token_stride != 0 && bias_token_stride != E) return EMOE_ERR_INVALID_ARG;
+  cudaStream_t st = static_cast<cudaStream_t>(compute_stream);
+  cudaError_t err = cudaSetDevice(ctx_cache(ctx)->device);
+  // The router kernel forms its product while the layer in front drains, and writes the picks to host memory as well:
+  // they are there some microseconds before a synchronisation would say so.
+  volatile int32_t* seen_ids = pinned_ids;
+  for (int p = 0; p < T * k; ++p) seen_ids[p] = -1;
+  g_pdl_enabled = ctx_dependent_launch(ctx);
+  if (err == cudaSuccess)
+    err = launch_router_topk(x, desc->act_dtype == EMOE_DTYPE_BF16, T, desc->d_model, router_W, router_bias, bias_token_stride, E, k,
+                             desc->gate_mode == EMOE_GATE_SOFTMAX_RENORM, ids, gates, nullptr, st, pinned_ids);
+  g_pdl_enabled = false;
+  if (err != cudaSuccess) return ctx_cuda_fail(ctx, err);
+  // the picks decide which experts are needed
+  for (int p = 0, polls = 0; p < T * k;) {
+    if (seen_ids[p] >= 0) {
+      ++p;
+    } else if (++polls % 4096 == 0) {  // nothing for some microseconds: done, or failed?
+      err = cudaStreamQuery(st);
+      if (err == cudaSuccess) break;
+      if (err != cudaErrorNotReady) return ctx_cuda_fail(ctx, err);
+    }
+  }
+  bool seen[EMOE_MAX_EXPERTS] = {};
+  for (int p = 0; p < T * k; ++p) {
+    if (pinned_ids[p] < 0 || pinned_ids[p] >= E) return EMOE_ERR_DEVICE_CHECK;
+    seen[pinned_ids[p]] = true;
+  }
+  int32_t active[EMOE_MAX_EXPERTS];
+  int64_t expert_ids[EMOE_MAX_EXPERTS];
+  int n = 0;
+  for (int e = 0; e < E; ++e)
+    if (seen[e]) active[n++] = e;
+  if (prior && n_prefetch > 0) {
+    int32_t order[EMOE_MAX_EXPERTS];
+    int rc = emoe_rank_experts(prior, E, active, n, order);
+    const int m = n_prefetch < E ? n_prefetch : E;
+    for (int i = 0; i < m; ++i) expert_ids[i] = next_first_id + order[i];
+    if (rc == EMOE_OK) rc = emoe_prefetch_experts(ctx, expert_ids, m, layer, copy_stream);
+    if (rc != EMOE_OK) return rc;
+  }
+  for (int i = 0; i < n; ++i) expert_ids[i] = first_id + active[i];
+  emoe_expert got[EMOE_MAX_EXPERTS], table[EMOE_MAX_EXPERTS];
+  int rc = emoe_cache_acquire(ctx, expert_ids, n, layer, compute_stream, copy_stream, got);
+  if (rc != EMOE_OK) return rc;
+  // entries of experts nobody picked are never read; they borrow an acquired expert whole (pointers AND
+  // width, so that whatever is derived from an entry stays inside that expert's slot)
+  for (int e = 0, i = 0; e < E; ++e) table[e] = seen[e] ? got[i++] : got[0];
+  rc = emoe_moe_forward_routed(ctx, desc, x, T, ids, gates, table, y, nullptr, compute_stream);
+  const int rc2 = emoe_cache_release(ctx, expert_ids, n, compute_stream);
+  return rc != EMOE_OK ? rc : rc2;
 }
 
 int emoe_cache_slot_of(emoe_ctx* ctx, int64_t id) {

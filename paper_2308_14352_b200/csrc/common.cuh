@@ -85,7 +85,7 @@ cudaError_t launch_requant(const uint8_t* in_packed, const void* in_scales, int 
 
 cudaError_t launch_router_topk(const void* x, int x_bf16, int T, int d, const float* Wr, const float* bias,
                                int bias_stride, int E, int top_k, int renorm, int32_t* ids, float* gates,
-                               float* logits, cudaStream_t st);
+                               float* logits, cudaStream_t st, int32_t* ids_copy = nullptr);  // ids_copy: the picks once more (pinned host memory)
 
 cudaError_t launch_permute(const int32_t* ids, int n_pairs, int E, int32_t* counts, int32_t* off, int32_t* perm,
                            int32_t* slot_of_pair, int* check_word, cudaStream_t st);

@@ -23,7 +23,7 @@ template <int TT>
 __global__ void __launch_bounds__(ROUTER_THREADS)
     router_topk_kernel(const void* __restrict__ x, int x_bf16, int T, int d, const float* __restrict__ Wr,
                        const float* __restrict__ bias, int bias_stride, int E, int EP, int ep_shift, int top_k,
-                       int renorm, int32_t* __restrict__ ids, float* __restrict__ gates,
+                       int renorm, int32_t* __restrict__ ids, int32_t* __restrict__ ids_copy, float* __restrict__ gates,
                        float* __restrict__ logits) {
   extern __shared__ float smem[];
   pdl_trigger();
@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(ROUTER_THREADS)
     router_pick(zs + tt * EP, E, top_k, renorm, lane, my_id, my_gate);
     if (lane < top_k) {
       ids[static_cast<size_t>(t) * top_k + lane] = my_id;
+      if (ids_copy) ids_copy[static_cast<size_t>(t) * top_k + lane] = my_id;
       gates[static_cast<size_t>(t) * top_k + lane] = my_gate;
     }
   }
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(1024)
 
 cudaError_t launch_router_topk(const void* x, int x_bf16, int T, int d, const float* Wr, const float* bias,
                                int bias_stride, int E, int top_k, int renorm, int32_t* ids, float* gates,
-                               float* logits, cudaStream_t st) {
+                               float* logits, cudaStream_t st, int32_t* ids_copy) {
   int EP = 1, sh = 0;
   while (EP < E) {
     EP <<= 1;
@@ -261,12 +262,12 @@ cudaError_t launch_router_topk(const void* x, int x_bf16, int T, int d, const fl
     constexpr int TT = 8;
     const size_t smem = sizeof(float) * (TT * ROUTER_DC + ROUTER_THREADS * TT + TT * EP);  // <= 48 KB
     return launch_chain(router_topk_kernel<TT>, dim3((T + TT - 1) / TT), dim3(ROUTER_THREADS), smem, st, x, x_bf16, T, d, Wr, bias,
-                        bias_stride, E, EP, sh, top_k, renorm, ids, gates, logits);
+                        bias_stride, E, EP, sh, top_k, renorm, ids, ids_copy, gates, logits);
   } else {
     constexpr int TT = 1;
     const size_t smem = sizeof(float) * (TT * ROUTER_DC + ROUTER_THREADS * TT + TT * EP);
     return launch_chain(router_topk_kernel<TT>, dim3(T), dim3(ROUTER_THREADS), smem, st, x, x_bf16, T, d, Wr, bias, bias_stride, E,
-                        EP, sh, top_k, renorm, ids, gates, logits);
+                        EP, sh, top_k, renorm, ids, ids_copy, gates, logits);
   }
   return cudaGetLastError();
 }
