@@ -19,18 +19,24 @@
 namespace emoe {
 namespace {
 
-template <int TT>
-__global__ void __launch_bounds__(ROUTER_THREADS)
+template <int TT, int BC>  // BC: inputs per chunk of the register-tiled product, 0 = one expert per thread
+__global__ void __launch_bounds__(BC > 0 ? ROUTER_BATCH_THREADS : ROUTER_THREADS)
     router_topk_kernel(const void* __restrict__ x, int x_bf16, int T, int d, const float* __restrict__ Wr,
                        const float* __restrict__ bias, int bias_stride, int E, int EP, int ep_shift, int top_k,
                        int renorm, int32_t* __restrict__ ids, int32_t* __restrict__ ids_copy, float* __restrict__ gates,
                        float* __restrict__ logits) {
   extern __shared__ float smem[];
   pdl_trigger();
-  router_logits<TT>(smem, x, x_bf16, T, d, Wr, bias, bias_stride, E, EP, ep_shift, logits);
-  const float* zs = smem + TT * router_dc(TT) + ROUTER_THREADS * TT;
+  const float* zs;
+  if constexpr (BC > 0) {
+    router_logits_batch<TT, BC>(smem, x, x_bf16, T, d, Wr, bias, bias_stride, E, EP, ep_shift, logits);
+    zs = smem + router_batch_floats_w(TT, EP) + TT * BC;
+  } else {
+    router_logits<TT>(smem, x, x_bf16, T, d, Wr, bias, bias_stride, E, EP, ep_shift, logits);
+    zs = smem + TT * router_dc(TT) + ROUTER_THREADS * TT;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int tt = warp; tt < TT; tt += ROUTER_THREADS / 32) {  // a warp per token, in turns when the CTA owns more tokens than warps
+  for (int tt = warp; tt < TT; tt += static_cast<int>(blockDim.x) / 32) {  // a warp per token, in turns when the CTA owns more tokens than warps
     const int t = blockIdx.x * TT + tt;
     if (t >= T) return;
     int my_id;
@@ -255,21 +261,34 @@ cudaError_t launch_router_topk(const void* x, int x_bf16, int T, int d, const fl
     EP <<= 1;
     ++sh;
   }
-  // 8 tokens per CTA once there are enough tokens to fill the GPU that way, else 1 (32 tokens per CTA, which
-  // would cut the re-reads of the router matrix from L2, was measured three times slower at 2048 tokens: 64 CTAs,
-  // each bound by its shared-memory reads)
-  if (T >= 8 * 64) {
-    constexpr int TT = 8;
-    const size_t smem = sizeof(float) * (TT * ROUTER_DC + ROUTER_THREADS * TT + TT * EP);  // <= 48 KB
-    return launch_chain(router_topk_kernel<TT>, dim3((T + TT - 1) / TT), dim3(ROUTER_THREADS), smem, st, x, x_bf16, T, d, Wr, bias,
-                        bias_stride, E, EP, sh, top_k, renorm, ids, ids_copy, gates, logits);
-  } else {
-    constexpr int TT = 1;
-    const size_t smem = sizeof(float) * (TT * ROUTER_DC + ROUTER_THREADS * TT + TT * EP);
-    return launch_chain(router_topk_kernel<TT>, dim3(T), dim3(ROUTER_THREADS), smem, st, x, x_bf16, T, d, Wr, bias, bias_stride, E,
-                        EP, sh, top_k, renorm, ids, ids_copy, gates, logits);
+  // One token per CTA while that fills the GPU no more than once; then eight, sixteen from where they give most SMs a
+  // CTA (every CTA reads the whole router matrix from L2).  Experts in groups of four, rows in
+  // 16-byte pieces: the register-tiled product.
+  const bool tiled = E >= 4 && E % 4 == 0 && d % 8 == 0 && reinterpret_cast<uintptr_t>(Wr) % 16 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
+  const auto launch = [&](auto kernel, int tt, size_t smem, int threads = ROUTER_BATCH_THREADS) -> cudaError_t {
+    if (smem > 48 * 1024) {
+      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+      if (e != cudaSuccess) return e;
+    }
+    return launch_chain(kernel, dim3((T + tt - 1) / tt), dim3(threads), smem, st, x, x_bf16, T, d, Wr, bias, bias_stride, E, EP, sh,
+                        top_k, renorm, ids, ids_copy, gates, logits);
+  };
+  if (tiled && T >= 96 * 16) {
+    const size_t smem = router_batch_smem(16, EP);
+    if (router_batch_chunk(EP) == 512) return launch(router_topk_kernel<16, 512>, 16, smem);
+    if (router_batch_chunk(EP) == 256) return launch(router_topk_kernel<16, 256>, 16, smem);
+    if (router_batch_chunk(EP) == 128) return launch(router_topk_kernel<16, 128>, 16, smem);
+    return launch(router_topk_kernel<16, 64>, 16, smem);
   }
-  return cudaGetLastError();
+  if (tiled && T >= 148) {
+    const size_t smem = router_batch_smem(8, EP);
+    if (router_batch_chunk(EP) == 512) return launch(router_topk_kernel<8, 512>, 8, smem);
+    if (router_batch_chunk(EP) == 256) return launch(router_topk_kernel<8, 256>, 8, smem);
+    if (router_batch_chunk(EP) == 128) return launch(router_topk_kernel<8, 128>, 8, smem);
+    return launch(router_topk_kernel<8, 64>, 8, smem);
+  }
+  if (T >= 8 * 64) return launch(router_topk_kernel<8, 0>, 8, sizeof(float) * (8 * ROUTER_DC + ROUTER_THREADS * 8 + 8 * EP), ROUTER_THREADS);  // <= 48 KB
+  return launch(router_topk_kernel<1, 0>, 1, sizeof(float) * (ROUTER_DC + ROUTER_THREADS + EP), ROUTER_THREADS);
 }
 
 bool route_permute_scatter_supported(const LayerDims& L, int T, int resident_ctas) {

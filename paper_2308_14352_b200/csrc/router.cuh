@@ -88,6 +88,145 @@ __device__ __forceinline__ void router_logits(float* smem, const void* __restric
   __syncthreads();
 }
 
+// Logits of the CTA's TT tokens into zs[TT][EP] as a register-tiled product, for batches: a thread holds TT/2 tokens x
+// four experts and an interleaved part of the inputs, so that an activation is read once per four
+// experts and a router weight once per TT/2 tokens; with one expert per thread (router_logits) every
+// product needed a shared-memory read of its own.  Chunks of BC inputs: the weights arrive by
+// cp.async two chunks ahead, the activations one chunk ahead in registers (they become fp32,
+// [input][token], on their way into shared memory).  E a multiple of four.
+constexpr int ROUTER_BATCH_THREADS = 512;  // sixteen warps: the loop waits for shared memory with fewer
+__host__ __device__ constexpr int router_batch_chunk(int EP) { return EP <= 16 ? 512 : (EP == 32 ? 256 : (EP <= 128 ? 128 : 64)); }
+__host__ __device__ constexpr int router_batch_stages(int EP) { return EP > 64 ? 2 : 3; }
+// weights' stages (the partial sums follow in the same memory), activations, logits
+__host__ __device__ constexpr int router_batch_floats_w(int tt, int EP) {
+  return router_batch_stages(EP) * router_batch_chunk(EP) * EP > 2 * ROUTER_BATCH_THREADS * tt ? router_batch_stages(EP) * router_batch_chunk(EP) * EP
+                                                                                         : 2 * ROUTER_BATCH_THREADS * tt;
+}
+__host__ __device__ constexpr int router_batch_smem(int tt, int EP) {
+  return (router_batch_floats_w(tt, EP) + tt * router_batch_chunk(EP) + tt * EP) * 4;
+}
+
+template <int TT, int BC>
+__device__ __forceinline__ void router_logits_batch(float* smem, const void* __restrict__ x, int x_bf16, int T, int d,
+                                                    const float* __restrict__ Wr, const float* __restrict__ bias, int bias_stride, int E,
+                                                    int EP, int ep_shift, float* __restrict__ logits) {
+  constexpr int TG = 2, TPT = TT / TG;  // token groups, tokens per thread
+  const int stages = router_batch_stages(EP);
+  float* ws = smem;                                   // [stages][BC][E]
+  float* xs = smem + router_batch_floats_w(TT, EP);   // [BC][TT]
+  float* zs = xs + TT * BC;                           // [TT][EP]
+  float* red = smem;                                  // [S][TT][EP]
+  const int tid = threadIdx.x, t0 = blockIdx.x * TT;
+  const int eg_shift = ep_shift - 2;                  // groups of four experts
+  const int eg = tid & ((1 << eg_shift) - 1), tg = (tid >> eg_shift) & (TG - 1), ks = tid >> (eg_shift + 1);
+  const int S = ROUTER_BATCH_THREADS >> (eg_shift + 1);
+  const int nchunks = (d + BC - 1) / BC;
+  unsigned long long acc[TPT / 2][4];  // pairs of tokens: two fp32 products and sums per instruction
+#pragma unroll
+  for (int t = 0; t < TPT / 2; ++t)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[t][i] = 0ull;
+  auto fetch_w = [&](int c) {  // rows c*BC .. of Wr are one contiguous block; one commit group per chunk, empty past the end
+    if (c < nchunks) {
+      const int n16 = min(BC, d - c * BC) * E / 4;
+      const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(ws + (c % stages) * BC * EP));
+      const float* src = Wr + static_cast<size_t>(c) * BC * E;
+      for (int i = tid; i < n16; i += ROUTER_BATCH_THREADS)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(src + 4 * i) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // activations: a thread moves eight inputs of one token at a time; neighbouring threads take neighbouring tokens
+  constexpr int NST = TT * BC / 8 / ROUTER_BATCH_THREADS > 0 ? TT * BC / 8 / ROUTER_BATCH_THREADS : 1;
+  uint4 pre[NST][2];
+  auto fetch_x = [&](int c) {
+#pragma unroll
+    for (int i = 0; i < NST; ++i) {
+      const int u = tid + i * ROUTER_BATCH_THREADS, tok = t0 + u % TT, k = c * BC + u / TT * 8;
+      const bool in = u < TT * BC / 8 && tok < T && k < d;
+      pre[i][0] = pre[i][1] = make_uint4(0u, 0u, 0u, 0u);
+      if (in) {
+        const size_t at = static_cast<size_t>(tok) * d + k;
+        if (x_bf16) {
+          pre[i][0] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(x) + at));
+        } else {
+          pre[i][0] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(x) + at));
+          pre[i][1] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(x) + at) + 1);
+        }
+      }
+    }
+  };
+  for (int c = 0; c + 1 < stages; ++c) fetch_w(c);
+  fetch_x(0);
+  for (int c = 0; c < nchunks; ++c) {
+    const int dc = min(BC, d - c * BC);
+    if (stages == 3) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // the chunk's weights are here, and the chunk in front is used up
+    fetch_w(c + stages - 1);
+#pragma unroll
+    for (int i = 0; i < NST; ++i) {
+      const int u = tid + i * ROUTER_BATCH_THREADS, tok = u % TT, k = u / TT * 8;
+      if (u >= TT * BC / 8) break;
+      const uint32_t w[8] = {pre[i][0].x, pre[i][0].y, pre[i][0].z, pre[i][0].w, pre[i][1].x, pre[i][1].y, pre[i][1].z, pre[i][1].w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        xs[(k + j) * TT + tok] = __uint_as_float(!x_bf16 ? w[j] : ((j & 1) ? w[j >> 1] & 0xffff0000u : w[j >> 1] << 16));
+    }
+    __syncthreads();
+    if (c + 1 < nchunks) fetch_x(c + 1);
+    if (4 * eg < E) {
+      const float* wp = ws + (c % stages) * BC * EP + 4 * eg;
+      const float* xp = xs + tg * TPT;
+#pragma unroll 4
+      for (int i = ks; i < dc; i += S) {
+        const float4 w = *reinterpret_cast<const float4*>(wp + i * E);
+        unsigned long long xv[TPT / 2], wv[4];
+#pragma unroll
+        for (int t = 0; t < TPT / 2; t += 2) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(xp + i * TT + 2 * t);
+          xv[t] = v.x;
+          xv[t + 1] = v.y;
+        }
+        asm("mov.b64 %0, {%1, %1};" : "=l"(wv[0]) : "f"(w.x));
+        asm("mov.b64 %0, {%1, %1};" : "=l"(wv[1]) : "f"(w.y));
+        asm("mov.b64 %0, {%1, %1};" : "=l"(wv[2]) : "f"(w.z));
+        asm("mov.b64 %0, {%1, %1};" : "=l"(wv[3]) : "f"(w.w));
+#pragma unroll
+        for (int t = 0; t < TPT / 2; ++t)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[t][j]) : "l"(xv[t]), "l"(wv[j]));
+      }
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // partial sums [part][token][expert], added in order
+#pragma unroll
+  for (int t = 0; t < TPT / 2; ++t) {
+    float lo[4], hi[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) asm("mov.b64 {%0, %1}, %2;" : "=f"(lo[j]), "=f"(hi[j]) : "l"(acc[t][j]));
+    float* to = red + (ks * TT + tg * TPT + 2 * t) * EP + 4 * eg;
+    *reinterpret_cast<float4*>(to) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+    *reinterpret_cast<float4*>(to + EP) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+  }
+  __syncthreads();
+  pdl_wait();
+  for (int idx = tid; idx < TT * EP; idx += ROUTER_BATCH_THREADS) {
+    const int tt = idx >> ep_shift, ee = idx & (EP - 1);
+    const int t = t0 + tt;
+    float z = 0.0f;
+    for (int s = 0; s < S; ++s) z += red[(s * TT + tt) * EP + ee];
+    if (ee < E && t < T) {
+      if (bias) z += bias[static_cast<size_t>(t) * bias_stride + ee];
+      if (logits) logits[static_cast<size_t>(t) * E + ee] = z;
+    }
+    zs[idx] = z;
+  }
+  __syncthreads();
+}
+
 // Softmax and Top-K of one token by one warp from its row of logits zrow[EP] (shared memory):
 // K rounds of arg-max, ties to the lower expert index.  Lane r < top_k returns the r-th pick.
 __device__ __forceinline__ void router_pick(const float* zrow, int E, int top_k, int renorm, int lane, int& out_id,

@@ -58,7 +58,24 @@ CASES = [
 ]
 
 
-@pytest.mark.parametrize("T,d,E,k,renorm,bf16,bias_kind", CASES)
+EDGE_CASES = [
+    # tokens around the lines between one, 8 and 16 tokens per CTA
+    (147, 256, 8, 1, False, True, None),
+    (148, 256, 8, 1, False, True, None),
+    (1535, 136, 12, 2, True, True, "vec"),
+    (1537, 136, 12, 2, True, True, "vec"),
+    # inputs: one chunk and a remainder of it; experts: the fewest and the most
+    (150, 8, 4, 4, True, False, None),
+    (161, 520, 4, 1, False, False, None),
+    (149, 72, 256, 2, True, True, "tok"),
+    (1545, 264, 256, 1, False, True, None),
+    # rows or columns that the tiled kernel does not take
+    (513, 1028, 32, 1, False, True, None),
+    (160, 512, 30, 1, False, True, None),
+]
+
+
+@pytest.mark.parametrize("T,d,E,k,renorm,bf16,bias_kind", CASES + EDGE_CASES)
 def test_router_topk(ctx, T, d, E, k, renorm, bf16, bias_kind):
     seed = T * 7 + E
     x = inputs.activations(seed, 0, T, d, "bf16" if bf16 else "f32")
