@@ -19,6 +19,9 @@ thread_local bool g_pdl_enabled = false;
 
 namespace {
 
+// calls on both kernel families: experts with up to this many tokens (two passes) take the weight-streaming kernel
+// (16 and 64 instead were up to 13 % and 15 % slower over means of 16 to 64 tokens, even and skewed)
+constexpr int HYBRID_STREAM_TOKENS = 32;
 constexpr int MAX_TABLES = 128;  // distinct expert tables a context can keep on the device
 constexpr size_t TMAP_BYTES = 128;  // sizeof(CUtensorMap)
 // one table block: the expert entries followed by one tensor map per (expert, matrix)
@@ -38,7 +41,7 @@ struct TableEntry {
 inline size_t align_up(size_t v, size_t a = 256) { return (v + a - 1) / a * a; }
 
 struct WorkspaceLayout {
-  size_t ids, gates, counts, off, perm, slot_of_pair, plan, xs, hidden, xsc, hsc, o_part, um_scratch, um_scratch_bytes, total;
+  size_t ids, gates, counts, off, perm, slot_of_pair, plan, xs, hidden, xsc, hsc, o_part, total;
   int ksplit;
 };
 
@@ -89,11 +92,6 @@ WorkspaceLayout make_layout(const LayerDims& L, int T) {
   w.xsc = o;          o += align_up(ffn_i8_supported(L) ? P * (L.d_model / 128) * 4 : 0);
   w.hsc = o;          o += align_up(ffn_i8_supported(L) ? P * (L.d_ff / 128) * 4 : 0);
   w.o_part = o;       o += align_up(static_cast<size_t>(w.ksplit) * P * L.d_model * 4);
-  // scratch of the tcgen05 kernel's gated first projection: only calls with at least one full token tile of
-  // pairs can take that kernel's many-token shapes
-  w.um_scratch = o;
-  w.um_scratch_bytes = (ffn_umma_supported(L) && P >= 128) ? ffn_umma_scratch_bytes(L) : 0;
-  o += align_up(w.um_scratch_bytes);
   w.total = o;
   return w;
 }
@@ -371,7 +369,6 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   float* xsc = reinterpret_cast<float*>(ws + w.xsc);
   float* hsc = reinterpret_cast<float*>(ws + w.hsc);
   float* o_part = reinterpret_cast<float*>(ws + w.o_part);
-  float* um_scratch = w.um_scratch_bytes ? reinterpret_cast<float*>(ws + w.um_scratch) : nullptr;
 
   ctx->last_counts = counts;
   ctx->last_counts_n = L.E;
@@ -379,15 +376,15 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   const float* gates_use = routed ? gates_in : gates;
   const bool can_tma = ffn_tma_supported(L) && tmaps != nullptr;
   const bool can_i8 = ffn_i8_supported(L) && tmaps != nullptr;
-  // (a gated layer needs the kernel's scratch block, which calls below one token tile of pairs do not carry)
-  const bool can_umma = ffn_umma_supported(L) && tmaps != nullptr && (L.act != EMOE_ACT_SWIGLU || um_scratch != nullptr);
+  const bool can_umma = ffn_umma_supported(L) && tmaps != nullptr;
   // many tokens per expert: the tcgen05 grouped GEMM; otherwise the weight-streaming kernels
   const bool many_tokens = ffn_many_tokens(L, T);
   // skewed loads: experts with few tokens stream through the TMA kernel, the others take the
   // tcgen05 grouped GEMM, in the same forward call
-  // ... unless the experts hold hundreds of tokens each on average: then next to nobody is left for the streaming
-  // family, whose launch, cleared split-K plane and second plan would only cost
-  const bool dense_tokens = static_cast<double>(T) * L.top_k / L.E >= 256.0;
+  // ... unless the experts hold 24 tokens each on average: from there on the tcgen05 kernel alone, whose time hardly
+  // depends on the tokens up to 128 an expert, beats both (768 x 3072, 32 experts, us per layer: 777 tokens 100 against
+  // 116 on both families and 97 streaming, 1024 103/127/115, 2048 117/121/207; at 512 93/90/79)
+  const bool dense_tokens = ffn_dense_tokens(L, T);
   const bool use_hybrid = can_umma && can_tma && (ctx->ffn_path == 5 || (ctx->ffn_path == 0 && many_tokens && !dense_tokens));
   const bool use_umma = !use_hybrid && can_umma && (ctx->ffn_path == 4 || (ctx->ffn_path == 0 && many_tokens));
   // the weight-streaming kernels: the fp16 mma.sync one by default (the faster of the two as measured), the
@@ -401,11 +398,11 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   if (ctx->ffn_path == 5 && !use_hybrid) return EMOE_ERR_UNSUPPORTED;
   if (ctx->ffn_path == 6 && !use_i8) return EMOE_ERR_UNSUPPORTED;
   // small batches on the streaming kernels: permutation, scatter and plan in one launch
-  const bool one_launch_permute = (use_tma || use_i8) && ctx->fuse_projections && permute_scatter_supported(L, P);
+  const bool one_launch_permute = (use_tma || use_i8 || use_hybrid || use_umma) && ctx->fuse_projections && permute_scatter_supported(L, P);
   // ... and, when the router runs here too, router and Top-K in that same launch
   if (ctx->resident_route_ctas < 0) ctx->resident_route_ctas = route_permute_scatter_resident_ctas(ctx->device);
   const bool one_launch_route =
-      ctx->fuse_routing && one_launch_permute && !routed && route_permute_scatter_supported(L, T, ctx->resident_route_ctas);
+      ctx->fuse_routing && one_launch_permute && (use_tma || use_i8) && !routed && route_permute_scatter_supported(L, T, ctx->resident_route_ctas);
   if (!routed && !one_launch_route && !one_launch_layer)
     EMOE_LAUNCH(ctx, launch_router_topk(x, L.act_bf16, T, L.d_model, router_W, router_bias, bias_token_stride, L.E,
                                       L.top_k, L.gate_mode == EMOE_GATE_SOFTMAX_RENORM, ids, gates, nullptr, st));
@@ -445,50 +442,44 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   // rows of the tcgen05 kernel's activations: as far apart as a slot of the streaming kernel's tiles, so that the two
   // families can share the buffers
   const int xs_stride = static_cast<int>(act_slot_bytes(L.d_model) / 2), hid_stride = static_cast<int>(act_slot_bytes(L.d_ff) / 2);
+  int* plan_heavy = reinterpret_cast<int*>(reinterpret_cast<char*>(plan) + align_up(plan_bytes(L.E)));
+  const int heavy_above = use_umma ? 0 : HYBRID_STREAM_TOKENS;  // experts with more tokens than this are the tcgen05 kernel's
+  const int zmax = w.ksplit < 4 ? w.ksplit : 4;  // planes of partial sums its second projection may use
   if (use_hybrid) {
-    // experts with up to HYBRID_STREAM_TOKENS tokens: one or two passes of the streaming
-    // kernel; the others: 128-token tiles on tcgen05.  Each family has its own plan and writes only
-    // its own slots of xs / hidden / o_part.
-#ifndef EMOE_HYBRID_TOKENS
-#define EMOE_HYBRID_TOKENS 32
-#endif
-    constexpr int HYBRID_STREAM_TOKENS = EMOE_HYBRID_TOKENS;
-    int* plan_heavy = reinterpret_cast<int*>(reinterpret_cast<char*>(plan) + align_up(plan_bytes(L.E)));
-    // many tokens in the call: the streaming family's tail matters little, every further split-K plane costs a
-    // cleared and a re-read [P][d] fp32 array
+    // Each family has its own plan and writes only its own slots of xs / hidden / o_part.
+    // many tokens in the call: the streaming family's tail matters little, every further split-K plane costs a re-read
+    // [P][d] fp32 array
     ksplit = ffn_tma_ksplit(L, T) < 2 ? ffn_tma_ksplit(L, T) : 2;
-    EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, plan, xs, nullptr, P, 1, 1, HYBRID_STREAM_TOKENS, ctx->check_word, st));
-    EMOE_LAUNCH(ctx, launch_scatter_x16(L, table, x, ids_use, perm, off, plan_heavy, xs, xs_stride, P, HYBRID_STREAM_TOKENS + 1, INT_MAX, ctx->check_word, st));
+    if (one_launch_permute)
+      EMOE_LAUNCH(ctx, launch_permute_scatter(L, table, x, ids_use, counts, off, perm, slot_of_pair, plan, plan_heavy, xs, nullptr, P, 1,
+                                              heavy_above, ctx->check_word, st));
+    else
+      EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, plan, plan_heavy, xs, nullptr, P, 1, heavy_above, ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
-    // the tcgen05 kernel writes plane 0 only: the other split-K planes of its slots must read as zero
-    if (ksplit > 1)
-      EMOE_CUDA(ctx, cudaMemsetAsync(o_part + static_cast<size_t>(P) * L.d_model, 0,
-                                     static_cast<size_t>(ksplit - 1) * P * L.d_model * sizeof(float), st));
     if (ctx->fuse_projections) {
       EMOE_LAUNCH(ctx, launch_ffn_tma(0, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
     } else {
       EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
       EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
     }
-    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, um_scratch, P, 1, ctx->check_word, st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, um_scratch, P, 1, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, ctx->check_word, st));
     if (ev[1]) {  // one interval for the whole expert stage
       EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
       ctx->events_one_launch[ctx->events_used / 3 - 1] = 1;
       ev[2] = nullptr;
     }
   } else if (use_umma) {
-    {  // the second projection's units may be halves of the inputs, summed by the combine step like any split-K
-      int sms = 0;
-      EMOE_CUDA(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
-      ksplit = ffn_umma_zsplit(L, T, sms);
-      if (ksplit > w.ksplit) ksplit = w.ksplit;  // the workspace holds w.ksplit planes
-    }
-    EMOE_LAUNCH(ctx, launch_scatter_x16(L, table, x, ids_use, perm, off, plan, xs, xs_stride, P, 1, INT_MAX, ctx->check_word, st));
+    if (one_launch_permute)
+      EMOE_LAUNCH(ctx, launch_permute_scatter(L, table, x, ids_use, counts, off, perm, slot_of_pair, nullptr, plan_heavy, xs, nullptr, P,
+                                              SCATTER_ROWS16, heavy_above, ctx->check_word, st));
+    else
+      EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, nullptr, plan_heavy, xs, nullptr, P, SCATTER_ROWS16, heavy_above,
+                                        ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan, xs, xs_stride, hidden, hid_stride, o_part, um_scratch, P, 1, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, ctx->check_word, st));
     if (ev[1]) EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan, hidden, hid_stride, hidden, hid_stride, o_part, um_scratch, P, ksplit, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, ctx->check_word, st));
   } else if (use_i8) {
     ksplit = ffn_i8_ksplit(L, T);
     if (one_launch_route)
@@ -496,10 +487,10 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
                                                     off, perm, slot_of_pair, plan, xs, xsc, 2, route_sync, route_wait,
                                                     ctx->dep_extra, ctx->check_word, st));
     else if (one_launch_permute)
-      EMOE_LAUNCH(ctx, launch_permute_scatter(L, table, x, ids_use, counts, off, perm, slot_of_pair, plan, xs, xsc, P, 2,
+      EMOE_LAUNCH(ctx, launch_permute_scatter(L, table, x, ids_use, counts, off, perm, slot_of_pair, plan, nullptr, xs, xsc, P, 2, INT_MAX,
                                               ctx->check_word, st));
     else
-      EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, plan, xs, xsc, P, 2, 1, INT_MAX, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, plan, nullptr, xs, xsc, P, 2, INT_MAX, ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
     if (ctx->fuse_projections) {
       // one launch: an expert's second projection starts when its hidden vectors are complete
@@ -524,10 +515,10 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
                                                     off, perm, slot_of_pair, plan, xs, nullptr, 1, route_sync, route_wait,
                                                     ctx->dep_extra, ctx->check_word, st));
     else if (one_launch_permute)
-      EMOE_LAUNCH(ctx, launch_permute_scatter(L, table, x, ids_use, counts, off, perm, slot_of_pair, plan, xs, nullptr, P, 1,
+      EMOE_LAUNCH(ctx, launch_permute_scatter(L, table, x, ids_use, counts, off, perm, slot_of_pair, plan, nullptr, xs, nullptr, P, 1, INT_MAX,
                                               ctx->check_word, st));
     else
-      EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, plan, xs, nullptr, P, 1, 1, INT_MAX, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, plan, nullptr, xs, nullptr, P, 1, INT_MAX, ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
     if (ctx->fuse_projections) {
       // one launch: an expert's second projection starts when its hidden vectors are complete
@@ -544,7 +535,7 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
     }
   } else if (use_mma) {
     ksplit = ffn_mma_ksplit(L, T);
-    EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, nullptr, xs, nullptr, P, 0, 1, INT_MAX, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, nullptr, nullptr, xs, nullptr, P, 0, INT_MAX, ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
     EMOE_LAUNCH(ctx, launch_ffn_mma(0, L, table, xs, off, reinterpret_cast<__nv_bfloat16*>(hidden), o_part, 1, P, T, st));
     if (ev[1]) EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
@@ -558,8 +549,8 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
     EMOE_LAUNCH(ctx, launch_ffn_gemv(1, L, table, x, perm, off, hidden, o_part, ksplit, P, st));
   }
   if (ev[2]) EMOE_CUDA(ctx, cudaEventRecord(ev[2], st));
-  EMOE_LAUNCH(ctx, launch_combine(o_part, ksplit, static_cast<size_t>(P), gates_use, slot_of_pair, T, L.top_k, L.d_model,
-                                y, st));
+  EMOE_LAUNCH(ctx, launch_combine(o_part, ksplit, static_cast<size_t>(P), gates_use, slot_of_pair, T, L.top_k, L.d_model, y, ids_use, counts,
+                                  heavy_above, use_hybrid || use_umma ? plan_heavy : nullptr, st));
   if (out_ids) EMOE_CUDA(ctx, cudaMemcpyAsync(out_ids, ids_use, sizeof(int32_t) * P, cudaMemcpyDeviceToDevice, st));
   if (out_gates) EMOE_CUDA(ctx, cudaMemcpyAsync(out_gates, gates_use, sizeof(float) * P, cudaMemcpyDeviceToDevice, st));
   if (out_perm) EMOE_CUDA(ctx, cudaMemcpyAsync(out_perm, perm, sizeof(int32_t) * P, cudaMemcpyDeviceToDevice, st));

@@ -106,15 +106,17 @@ bool ffn_mma_supported(const LayerDims& L);
 int ffn_mma_ksplit(const LayerDims& L, int T);
 int ffn_token_tiles(const LayerDims& L, int T);
 bool ffn_many_tokens(const LayerDims& L, int T);
+bool ffn_dense_tokens(const LayerDims& L, int T);
 // plan (nullable): plan_bytes(E) bytes, the work plan for the persistent TMA kernels, filled by block 0.
 // fmt: 0 = bf16, 1 = fp16 tiles (act_tile.cuh, saturating: the TMA-staged kernel's input), 2 = two-limb
 // block-scaled integers (act_q.cuh: the int8 tensor-core kernel's input; xsc receives the block scales).
-// cnt_lo .. cnt_hi: only experts with that many tokens are listed in the plan and have their rows
-// written (1 .. INT_MAX: all activated experts); lets two kernel families share one forward call.
+// Experts with more than heavy_above tokens (INT_MAX: none) are listed in plan_heavy instead and have their rows
+// written as SCATTER_ROWS16: lets two kernel families share one forward call.
+constexpr int SCATTER_ROWS16 = 3;  // fp16 rows of the tcgen05 kernel
 cudaError_t launch_scatter_x(const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* ids,
-                             const int32_t* perm, const int32_t* off, int* plan, __nv_bfloat16* xs, float* xsc, int n_pairs,
-                             int fmt, int cnt_lo, int cnt_hi, int* check_word, cudaStream_t st);
-// Permutation + scatter + plan in one launch (one CTA per pair) for batches of at most 1024 pairs.
+                             const int32_t* perm, const int32_t* off, int* plan, int* plan_heavy, __nv_bfloat16* xs, float* xsc,
+                             int n_pairs, int fmt, int heavy_above, int* check_word, cudaStream_t st);
+// Permutation + scatter + plans in one launch for batches of at most 4096 pairs.
 bool permute_scatter_supported(const LayerDims& L, int n_pairs);
 bool decode_layer_supported(const LayerDims& L, int T);
 int decode_layer_resident_ctas(int device);
@@ -132,8 +134,9 @@ cudaError_t launch_route_permute_scatter(const LayerDims& L, const ExpertDev* ex
                                          float* xsc, int fmt, unsigned* sync, unsigned wait_limit, int extra_arrivals,
                                          int* check_word, cudaStream_t st);
 cudaError_t launch_permute_scatter(const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* ids,
-                                   int32_t* counts, int32_t* off, int32_t* perm, int32_t* slot_of_pair, int* plan,
-                                   __nv_bfloat16* xs, float* xsc, int n_pairs, int fmt, int* check_word, cudaStream_t st);
+                                   int32_t* counts, int32_t* off, int32_t* perm, int32_t* slot_of_pair, int* plan, int* plan_heavy,
+                                   __nv_bfloat16* xs, float* xsc, int n_pairs, int fmt, int heavy_above, int* check_word,
+                                   cudaStream_t st);
 cudaError_t launch_ffn_mma(int phase, const LayerDims& L, const ExpertDev* experts, const __nv_bfloat16* in,
                            const int32_t* off, __nv_bfloat16* hidden, float* o_part, int ksplit, int n_pairs,
                            int T, cudaStream_t st);
@@ -172,18 +175,17 @@ int encode_tmap_2d(void* out_map, int dtype, const void* base, uint64_t inner, u
 // memory).  xs16 / hidden16: activations in expert order, fp16, pair order, rows xs_stride / hid_stride
 // values apart; o: [n_pairs][d_model].
 bool ffn_umma_supported(const LayerDims& L);
-cudaError_t launch_scatter_x16(const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* ids,
-                               const int32_t* perm, const int32_t* off, int* plan, void* xs16, int xs_stride, int n_pairs,
-                               int cnt_lo, int cnt_hi, int* check_word, cudaStream_t st);
-size_t ffn_umma_scratch_bytes(const LayerDims& L);  // scratch of the gated first projection (0 for other layers)
-cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, const int* plan, const void* in16, int in_stride,
-                            void* hidden16, int hid_stride, float* o, float* scratch, int n_pairs, int zsplit, int* check_word,
+// zmax: most planes of partial sums the second projection may leave; how many it does is decided on the device and left in
+// the fourth word of the plan's header.
+cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, int* plan, const void* in16, int in_stride,
+                            void* hidden16, int hid_stride, float* o, int n_pairs, int zmax, int* check_word,
                             cudaStream_t st);
-int ffn_umma_zsplit(const LayerDims& L, int T, int sms);  // 1 or 2 slices of the second projection's inputs per unit
 
 // y[t] = sum_j gates[t][j] * sum_z o_part[z][slot_of_pair[t*k+j]]
-// o_part holds ksplit partial results, each [n_pairs_stride][d].
+// o_part holds ksplit partial results, each [n_pairs_stride][d]; experts with more than heavy_above tokens (ids, counts)
+// have as many as the fourth word of plan_heavy says (plan_heavy null: no such experts).
 cudaError_t launch_combine(const float* o_part, int ksplit, size_t n_pairs_stride, const float* gates,
-                           const int32_t* slot_of_pair, int T, int top_k, int d, float* y, cudaStream_t st);
+                           const int32_t* slot_of_pair, int T, int top_k, int d, float* y, const int32_t* ids, const int32_t* counts,
+                           int heavy_above, const int* plan_heavy, cudaStream_t st);
 
 }  // namespace emoe

@@ -204,39 +204,43 @@ __global__ void __launch_bounds__(MMA_THREADS)
   }
 }
 
-// x rows -> expert-sorted order, in the activation layout of the owning expert's bitwidth
+// x rows -> expert-sorted order, in the activation layout of the owning expert's bitwidth and kernel family: experts
+// with more than `heavy_above` tokens are the tcgen05 kernel's (rows, plan_heavy), the others take `fmt`
+// and `plan`.
 __global__ void __launch_bounds__(128)
     scatter_x_kernel(const ExpertDev* __restrict__ experts, const __nv_bfloat16* __restrict__ x,
                      const int32_t* __restrict__ ids, const int32_t* __restrict__ perm, const int32_t* __restrict__ off,
-                     int E, int* __restrict__ plan, int top_k, int d, int n_pairs, int fmt, int cnt_lo, int cnt_hi,
+                     int E, int* __restrict__ plan, int* __restrict__ plan_heavy, int top_k, int d, int n_pairs, int fmt, int heavy_above,
                      __nv_bfloat16* __restrict__ xs, float* __restrict__ xsc, int* __restrict__ check_word) {
   pdl_wait();
   pdl_trigger();
-  if (plan && blockIdx.x == 0 && threadIdx.x < 32) build_plan(plan, experts, off, E, cnt_lo, cnt_hi, threadIdx.x);
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    if (plan) build_plan(plan, experts, off, E, 1, heavy_above, threadIdx.x);
+    if (plan_heavy) build_plan(plan_heavy, experts, off, E, heavy_above + 1, 0x7fffffff, threadIdx.x);
+  }
   const int slot = blockIdx.x;
   const int pair = perm[slot];
   if (pair < 0 || pair >= n_pairs) return;
   const int e_slot = ids[pair];
   if (e_slot < 0 || e_slot >= E) return;  // a slot the permutation did not write (stale entry behind a dropped pair)
   const int cnt_slot = off[e_slot + 1] - off[e_slot];
-  if (cnt_slot < cnt_lo || cnt_slot > cnt_hi) return;  // this expert's rows belong to another kernel family
-  scatter_any(x + static_cast<size_t>(pair / top_k) * d, xs, xsc, off[e_slot], cnt_slot, slot - off[e_slot], d, experts[e_slot].bits, fmt,
-              check_word);
+  scatter_any(x + static_cast<size_t>(pair / top_k) * d, xs, xsc, off[e_slot], cnt_slot, slot - off[e_slot], d, experts[e_slot].bits,
+              cnt_slot > heavy_above ? SCATTER_ROWS16 : fmt, check_word);
 }
 
-// Permutation and scatter in one launch for small batches (at most PS_MAX_PAIRS pairs): one CTA
-// per pair.  Every CTA reads all expert ids and works out its own pair's slot (pairs with a lower
-// expert id come first, then pairs of the same expert with a lower index: the stable counting
-// sort of the definition), writes perm / slot_of_pair for it and copies its row; CTA 0 also
-// writes counts, offsets and the work plan.  No CTA waits for another.
-constexpr int PS_MAX_PAIRS = 1024;
+// Permutation and scatter in one launch (at most PS_MAX_PAIRS pairs).  A CTA owns one pair, or up to
+// four neighbouring ones of large batches: it reads all expert ids and works out each of its pairs'
+// slots (pairs with a lower expert id come first, then pairs of the same expert with a lower index:
+// the stable counting sort of the definition), writes perm / slot_of_pair and copies the rows;
+// CTA 0 also writes counts, offsets and the work plans.  No CTA waits for another.
+constexpr int PS_MAX_PAIRS = 4096;
 __global__ void __launch_bounds__(128)
     permute_scatter_kernel(const ExpertDev* __restrict__ experts, const __nv_bfloat16* __restrict__ x,
-                           const int32_t* __restrict__ ids, int E, int top_k, int d, int n_pairs, int fmt,
+                           const int32_t* __restrict__ ids, int E, int top_k, int d, int n_pairs, int per_cta, int fmt, int heavy_above,
                            int32_t* __restrict__ counts, int32_t* __restrict__ off, int32_t* __restrict__ perm,
-                           int32_t* __restrict__ slot_of_pair, int* __restrict__ plan, int* __restrict__ check_word,
-                           __nv_bfloat16* __restrict__ xs, float* __restrict__ xsc) {
-  __shared__ int s_ids[PS_MAX_PAIRS];
+                           int32_t* __restrict__ slot_of_pair, int* __restrict__ plan, int* __restrict__ plan_heavy,
+                           int* __restrict__ check_word, __nv_bfloat16* __restrict__ xs, float* __restrict__ xsc) {
+  extern __shared__ int s_ids[];  // [n_pairs]
   __shared__ int s_off[EMOE_MAX_EXPERTS + 1];
   __shared__ int s_red[3][4];
   pdl_wait();
@@ -244,32 +248,8 @@ __global__ void __launch_bounds__(128)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int q = tid; q < n_pairs; q += blockDim.x) s_ids[q] = ids[q];
   __syncthreads();
-  const int p = blockIdx.x;
-  const int e = s_ids[p];
-  const bool valid = e >= 0 && e < E;
-  // pairs of lower experts, and pairs of this one's expert: in front of it and in all
-  int lower = 0, rank = 0, same = 0;
-  for (int q = tid; q < n_pairs; q += blockDim.x) {
-    const int eq = s_ids[q];
-    lower += eq >= 0 && eq < e;
-    rank += eq == e && q < p;
-    same += eq == e;
-  }
-  lower = __reduce_add_sync(0xffffffffu, lower);
-  rank = __reduce_add_sync(0xffffffffu, rank);
-  same = __reduce_add_sync(0xffffffffu, same);
-  if (lane == 0) {
-    s_red[0][warp] = lower;
-    s_red[1][warp] = rank;
-    s_red[2][warp] = same;
-  }
-  __syncthreads();
-  lower = s_red[0][0] + s_red[0][1] + s_red[0][2] + s_red[0][3];
-  rank = s_red[1][0] + s_red[1][1] + s_red[1][2] + s_red[1][3];
-  same = s_red[2][0] + s_red[2][1] + s_red[2][2] + s_red[2][3];
-  const int slot = lower + rank;
-  if (p == 0) {
-    // counts, offsets, plan (this CTA only); invalid ids are reported and own no slot
+  if (blockIdx.x == 0) {
+    // counts, offsets, plans (this CTA only); invalid ids are reported and own no slot
     for (int ee = tid; ee <= E; ee += blockDim.x) s_off[ee] = 0;
     __syncthreads();
     bool bad = false;
@@ -283,17 +263,45 @@ __global__ void __launch_bounds__(128)
     if (warp == 0) counts_to_offsets(s_off, counts, E, lane);
     __syncthreads();
     for (int ee = tid; ee <= E; ee += blockDim.x) off[ee] = s_off[ee];
-    if (warp == 0) build_plan(plan, experts, s_off, E, 1, 0x7fffffff, lane);
+    if (warp == 0 && plan) build_plan(plan, experts, s_off, E, 1, heavy_above, lane);
+    if (warp == 1 && plan_heavy) build_plan(plan_heavy, experts, s_off, E, heavy_above + 1, 0x7fffffff, lane);
   }
-  if (!valid) {
-    if (tid == 0) slot_of_pair[p] = -1;
-    return;
+  const int p_end = min(n_pairs, (static_cast<int>(blockIdx.x) + 1) * per_cta);
+  for (int p = blockIdx.x * per_cta; p < p_end; ++p) {
+    const int e = s_ids[p];
+    if (e < 0 || e >= E) {
+      if (tid == 0) slot_of_pair[p] = -1;
+      continue;
+    }
+    // pairs of lower experts, and pairs of this one's expert: in front of it and in all
+    int lower = 0, rank = 0, same = 0;
+    for (int q = tid; q < n_pairs; q += blockDim.x) {
+      const int eq = s_ids[q];
+      lower += eq >= 0 && eq < e;
+      rank += eq == e && q < p;
+      same += eq == e;
+    }
+    lower = __reduce_add_sync(0xffffffffu, lower);
+    rank = __reduce_add_sync(0xffffffffu, rank);
+    same = __reduce_add_sync(0xffffffffu, same);
+    if (lane == 0) {
+      s_red[0][warp] = lower;
+      s_red[1][warp] = rank;
+      s_red[2][warp] = same;
+    }
+    __syncthreads();
+    lower = s_red[0][0] + s_red[0][1] + s_red[0][2] + s_red[0][3];
+    rank = s_red[1][0] + s_red[1][1] + s_red[1][2] + s_red[1][3];
+    same = s_red[2][0] + s_red[2][1] + s_red[2][2] + s_red[2][3];
+    const int slot = lower + rank;
+    if (tid == 0) {
+      perm[slot] = p;
+      slot_of_pair[p] = slot;
+    }
+    scatter_any(x + static_cast<size_t>(p / top_k) * d, xs, xsc, lower, same, rank, d, experts[e].bits,
+                same > heavy_above ? SCATTER_ROWS16 : fmt, check_word);
+    if (p + 1 < p_end) __syncthreads();  // s_red has been read
   }
-  if (tid == 0) {
-    perm[slot] = p;
-    slot_of_pair[p] = slot;
-  }
-  scatter_any(x + static_cast<size_t>(p / top_k) * d, xs, xsc, lower, same, rank, d, experts[e].bits, fmt, check_word);
 }
 
 }  // namespace
@@ -311,6 +319,7 @@ int ffn_token_tiles(const LayerDims& L, int T) {
 // Enough tokens per expert (mean of 16 under uniform routing) that the experts with many tokens
 // are a dense contraction: those go to the tcgen05 grouped GEMM.
 bool ffn_many_tokens(const LayerDims& L, int T) { return static_cast<double>(T) * L.top_k / L.E >= 16.0; }
+bool ffn_dense_tokens(const LayerDims& L, int T) { return static_cast<double>(T) * L.top_k / L.E >= 24.0; }
 
 bool ffn_mma_supported(const LayerDims& L) {
   if (!L.act_bf16) return false;
@@ -332,20 +341,22 @@ int ffn_mma_ksplit(const LayerDims& L, int T) {
 }
 
 cudaError_t launch_scatter_x(const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* ids,
-                             const int32_t* perm, const int32_t* off, int* plan, __nv_bfloat16* xs, float* xsc, int n_pairs,
-                             int fmt, int cnt_lo, int cnt_hi, int* check_word, cudaStream_t st) {
+                             const int32_t* perm, const int32_t* off, int* plan, int* plan_heavy, __nv_bfloat16* xs, float* xsc,
+                             int n_pairs, int fmt, int heavy_above, int* check_word, cudaStream_t st) {
   return launch_chain(scatter_x_kernel, dim3(n_pairs), dim3(128), 0, st, experts, reinterpret_cast<const __nv_bfloat16*>(x), ids,
-                      perm, off, L.E, plan, L.top_k, L.d_model, n_pairs, fmt, cnt_lo, cnt_hi, xs, xsc, check_word);
+                      perm, off, L.E, plan, plan_heavy, L.top_k, L.d_model, n_pairs, fmt, heavy_above, xs, xsc, check_word);
 }
 
 bool permute_scatter_supported(const LayerDims& L, int n_pairs) { return n_pairs <= PS_MAX_PAIRS && L.E <= EMOE_MAX_EXPERTS; }
 
 cudaError_t launch_permute_scatter(const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* ids,
-                                   int32_t* counts, int32_t* off, int32_t* perm, int32_t* slot_of_pair, int* plan,
-                                   __nv_bfloat16* xs, float* xsc, int n_pairs, int fmt, int* check_word, cudaStream_t st) {
-  return launch_chain(permute_scatter_kernel, dim3(n_pairs), dim3(128), 0, st, experts, reinterpret_cast<const __nv_bfloat16*>(x),
-                      ids, L.E, L.top_k, L.d_model, n_pairs, fmt, counts, off, perm, slot_of_pair, plan, check_word,
-                      xs, xsc);
+                                   int32_t* counts, int32_t* off, int32_t* perm, int32_t* slot_of_pair, int* plan, int* plan_heavy,
+                                   __nv_bfloat16* xs, float* xsc, int n_pairs, int fmt, int heavy_above, int* check_word,
+                                   cudaStream_t st) {
+  const int per_cta = (n_pairs + 1023) / 1024;  // every CTA reads all ids: not more of them than that pays for
+  return launch_chain(permute_scatter_kernel, dim3((n_pairs + per_cta - 1) / per_cta), dim3(128), sizeof(int) * n_pairs, st, experts,
+                      reinterpret_cast<const __nv_bfloat16*>(x), ids, L.E, L.top_k, L.d_model, n_pairs, per_cta, fmt, heavy_above, counts,
+                      off, perm, slot_of_pair, plan, plan_heavy, check_word, xs, xsc);
 }
 
 cudaError_t launch_ffn_mma(int phase, const LayerDims& L, const ExpertDev* experts, const __nv_bfloat16* in,

@@ -461,6 +461,38 @@ def test_forward_tcgen05_path(act, group, sdt, d, f, E, k, gate, bits, T):
     _run_case(shape, bits, T, seed=27, path=4)
 
 
+UMMA_EDGE_CASES = [
+    # inputs that leave the last packed box partly filled (4 and 2 bits), per projection
+    ("relu", 128, "f16", 640, 768, 3, 1, "softmax", [4, 2, 8], 50),
+    ("swiglu", 128, "f16", 768, 640, 3, 2, "softmax_renorm", [2, 4, 8], 33),
+    # tokens of a group at the limits: MMA width (16), one group (320, beyond 256 in two MMAs), two groups
+    ("relu", 128, "f16", 512, 512, 1, 1, "softmax", [4], 16),
+    ("relu", 128, "f16", 512, 512, 1, 1, "softmax", [4], 17),
+    ("swiglu", 128, "f16", 512, 512, 1, 1, "softmax", [2], 257),
+    ("swiglu", 128, "f16", 512, 512, 1, 1, "softmax", [8], 320),
+    ("relu", 128, "f16", 512, 512, 1, 1, "softmax", [4], 321),
+    ("relu", 128, "f32", 512, 2048, 1, 1, "softmax", [2], 129),       # second projection in slices of its inputs
+]
+
+
+@pytest.mark.parametrize("act,group,sdt,d,f,E,k,gate,bits,T", UMMA_EDGE_CASES)
+def test_forward_tcgen05_path_at_the_edges_of_its_groups(act, group, sdt, d, f, E, k, gate, bits, T):
+    shape = inputs.LayerShape(d, f, E, k, act, gate, group, sdt, "bf16")
+    _run_case(shape, bits, T, seed=33, path=4)
+
+
+PERMUTE_EDGE_CASES = [
+    # pairs of a call around the limits of the one-launch permutation (1024 pairs: one per CTA; 4096: four)
+    (3, 1024, 1), (3, 1025, 1), (3, 2047, 2), (3, 2048, 2), (3, 2049, 2), (4, 1366, 3), (5, 1367, 3),
+]
+
+
+@pytest.mark.parametrize("path,T,k", PERMUTE_EDGE_CASES)
+def test_forward_with_many_pairs(path, T, k):
+    shape = inputs.LayerShape(512, 512, 5, k, "relu", "softmax", 128, "f16", "bf16")
+    _run_case(shape, [4, 2, 8, 4, 2], T, seed=34, path=path)
+
+
 HYBRID_CASES = [
     # loads shaped by a router bias so that some experts hold more than 32 tokens and others fewer
     ("relu", 128, "f16", 512, 1024, 8, 1, "softmax", [8, 4, 2, 4, 2, 8, 4, 2], 220, 1.1),
