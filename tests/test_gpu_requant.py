@@ -58,6 +58,45 @@ def test_requantize_bit_exact(ctx, bits_in, bits_out, group, sdt, N, K):
         assert np.array_equal(p_gpu, packed)
 
 
+@pytest.mark.parametrize("bits_out", [4, 2])
+@pytest.mark.parametrize("full_range", [False, True])
+@pytest.mark.parametrize("sdt", ["f16", "f32"])
+def test_requantize_8bit_codes_of_every_magnitude(ctx, bits_out, full_range, sdt):
+    """Groups whose largest code is 0, 1, ... 128 with all codes below it, under scales of many roundings: products that
+    are ties or lie next to one (even maxima), and a number of rows that leaves a warp's last groups empty."""
+    rng = np.random.default_rng(bits_out + 10 * full_range)
+    N, K = 129 * 3, 640
+    codes = np.empty((N, K), dtype=np.int64)
+    for n in range(N):
+        m = n % 129
+        q = np.concatenate([np.arange(-m, m + 1), -np.arange(-m, m + 1)])
+        codes[n] = np.clip(np.resize(q if n < 129 else rng.permutation(q), K), -128, 127)
+        codes[n, ::128] = -m          # every group has the maximum
+    packed = (codes & 0xFF).astype(np.uint8)
+    scales = np.exp(rng.uniform(np.log(1e-6), np.log(10.0), (N, K // 128))).astype(np.float32)
+    if sdt == "f16":
+        scales = scales.astype(np.float16).astype(np.float32)
+    p_ref, s_ref = oracle.requantize(packed, scales, K, 8, bits_out, 128, sdt, full_range)
+    p_gpu, s_gpu = _gpu_requant(ctx, packed, scales, K, 8, bits_out, 128, sdt, full_range)
+    view = SDT[sdt][2]
+    assert np.array_equal(s_gpu.view(view), oracle.scales_storage(s_ref, sdt).view(view))
+    assert np.array_equal(p_gpu, p_ref)
+
+
+@pytest.mark.parametrize("K,group", [(272, 0), (528, 0), (1040, 0), (2064, 0), (4112, 0), (9216, 0),   # one to eight warps per unit
+                                     (96, 48), (1024, 256), (1024, 512), (192, 64)])
+@pytest.mark.parametrize("bits_in,bits_out", [(8, 4), (8, 2), (4, 2), (2, 4)])
+def test_requantize_at_the_edges_of_its_splits(ctx, K, group, bits_in, bits_out):
+    rng = np.random.default_rng(K + group + bits_in)
+    W = (rng.standard_normal((11, K)) * 0.02).astype(np.float32)
+    W[3] = 0.0
+    packed, scales = oracle.pack_expert(W, bits_in, group, "f16")
+    p_ref, s_ref = oracle.requantize(packed, scales, K, bits_in, bits_out, group, "f16")
+    p_gpu, s_gpu = _gpu_requant(ctx, packed, scales, K, bits_in, bits_out, group, "f16")
+    assert np.array_equal(s_gpu.view(np.uint16), oracle.scales_storage(s_ref, "f16").view(np.uint16))
+    assert np.array_equal(p_gpu, p_ref)
+
+
 def test_requantize_equals_pack_of_the_decompressed_matrix(ctx):
     """The definition, end to end on the GPU: requantise == quantise(decompress(stored))."""
     rng = np.random.default_rng(77)
