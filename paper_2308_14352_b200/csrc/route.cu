@@ -19,8 +19,8 @@
 namespace emoe {
 namespace {
 
-template <int TT, int BC>  // BC: inputs per chunk of the register-tiled product, 0 = one expert per thread
-__global__ void __launch_bounds__(BC > 0 ? ROUTER_BATCH_THREADS : ROUTER_THREADS)
+template <int TT, int BC>  // BC: inputs per chunk of the register-tiled product, 0 = one expert per thread, -1 = one token, all loads at once
+__global__ void __launch_bounds__(BC > 0 ? ROUTER_BATCH_THREADS : (BC < 0 ? ROUTER_ONE_THREADS : ROUTER_THREADS))
     router_topk_kernel(const void* __restrict__ x, int x_bf16, int T, int d, const float* __restrict__ Wr,
                        const float* __restrict__ bias, int bias_stride, int E, int EP, int ep_shift, int top_k,
                        int renorm, int32_t* __restrict__ ids, int32_t* __restrict__ ids_copy, float* __restrict__ gates,
@@ -31,6 +31,9 @@ __global__ void __launch_bounds__(BC > 0 ? ROUTER_BATCH_THREADS : ROUTER_THREADS
   if constexpr (BC > 0) {
     router_logits_batch<TT, BC>(smem, x, x_bf16, T, d, Wr, bias, bias_stride, E, EP, ep_shift, logits);
     zs = smem + router_batch_floats_w(TT, EP) + TT * BC;
+  } else if constexpr (BC < 0) {
+    router_logits_one<ROUTER_ONE_THREADS, ROUTER_ONE_FLY>(smem, x, x_bf16, d, Wr, bias, bias_stride, E, ep_shift, logits);
+    zs = smem;
   } else {
     router_logits<TT>(smem, x, x_bf16, T, d, Wr, bias, bias_stride, E, EP, ep_shift, logits);
     zs = smem + TT * router_dc(TT) + ROUTER_THREADS * TT;
@@ -78,13 +81,15 @@ __global__ void __launch_bounds__(ROUTER_THREADS)
   // The next kernel of the chain is scheduled once every CTA of this grid has executed this, i.e.
   // once the whole grid is resident: it cannot take the room of a CTA the wait below needs.
   pdl_trigger();
-  router_logits<1>(smem, x, 1, T, d, Wr, bias, bias_stride, E, EP, ep_shift, nullptr);  // waits on the kernels in front
+  const bool one = router_one_supported(E, Wr);  // as the router kernel does it, to the same bits
+  if (one) router_logits_one<ROUTER_THREADS, 4>(smem, x, 1, d, Wr, bias, bias_stride, E, ep_shift, nullptr);  // (both wait on the kernels in front)
+  else router_logits<1>(smem, x, 1, T, d, Wr, bias, bias_stride, E, EP, ep_shift, nullptr);
   // should this CTA's wait run out, the expert kernel behind must find an empty plan, not an old one
   if (t == 0 && tid == 0) plan[0] = 0;
   if (warp == 0) {
     int my_id;
     float my_gate;
-    router_pick(smem + ROUTER_DC + ROUTER_THREADS, E, top_k, renorm, lane, my_id, my_gate);
+    router_pick(one ? smem : smem + ROUTER_DC + ROUTER_THREADS, E, top_k, renorm, lane, my_id, my_gate);
     if (lane < top_k) {
       ids[static_cast<size_t>(t) * top_k + lane] = my_id;
       gates[static_cast<size_t>(t) * top_k + lane] = my_gate;
@@ -287,6 +292,8 @@ cudaError_t launch_router_topk(const void* x, int x_bf16, int T, int d, const fl
     if (router_batch_chunk(EP) == 128) return launch(router_topk_kernel<8, 128>, 8, smem);
     return launch(router_topk_kernel<8, 64>, 8, smem);
   }
+  if (T < 148 && router_one_supported(E, Wr))
+    return launch(router_topk_kernel<1, -1>, 1, router_one_smem(E), ROUTER_ONE_THREADS);
   if (T >= 8 * 64) return launch(router_topk_kernel<8, 0>, 8, sizeof(float) * (8 * ROUTER_DC + ROUTER_THREADS * 8 + 8 * EP), ROUTER_THREADS);  // <= 48 KB
   return launch(router_topk_kernel<1, 0>, 1, sizeof(float) * (ROUTER_DC + ROUTER_THREADS + EP), ROUTER_THREADS);
 }
@@ -297,7 +304,7 @@ bool route_permute_scatter_supported(const LayerDims& L, int T, int resident_cta
 
 int route_permute_scatter_resident_ctas(int device) {
   int per_sm = 0, sms = 0;
-  const size_t smem = sizeof(float) * (ROUTER_DC + ROUTER_THREADS + EMOE_MAX_EXPERTS);
+  const size_t smem = sizeof(float) * (ROUTER_ONE_THREADS * 4 + 2 * EMOE_MAX_EXPERTS);  // the most that any number of experts takes
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, route_permute_scatter_kernel, ROUTER_THREADS, smem) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
   return per_sm * sms;
@@ -313,7 +320,7 @@ cudaError_t launch_route_permute_scatter(const LayerDims& L, const ExpertDev* ex
     EP <<= 1;
     ++sh;
   }
-  const size_t smem = sizeof(float) * (ROUTER_DC + ROUTER_THREADS + EP);
+  const size_t old_smem = sizeof(float) * (ROUTER_DC + ROUTER_THREADS + EP), one_smem = router_one_smem(L.E), smem = old_smem > one_smem ? old_smem : one_smem;
   return launch_chain(route_permute_scatter_kernel, dim3(T), dim3(ROUTER_THREADS), smem, st,
                       reinterpret_cast<const __nv_bfloat16*>(x), T, L.d_model, Wr, bias, bias_stride, L.E, EP, sh, L.top_k,
                       static_cast<int>(L.gate_mode == EMOE_GATE_SOFTMAX_RENORM), ids, gates, experts, fmt, counts, off, perm,

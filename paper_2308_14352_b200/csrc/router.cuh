@@ -88,6 +88,70 @@ __device__ __forceinline__ void router_logits(float* smem, const void* __restric
   __syncthreads();
 }
 
+// Logits of one token into zs[EP]: bound by the round trips to memory, so everything a thread reads is requested at
+// once, with nothing staged in front: ROUTER_ONE_FLY pieces of four experts' weights per thread and the activation that
+// belongs to each (up to 32 K products per round trip).  E a power of two, at least four: a thread keeps to four
+// experts.  4 tokens x 4096 x 8 experts, back to back: 12.3 us with chunks staged in shared memory, 8.2 so.
+constexpr int ROUTER_ONE_THREADS = 512, ROUTER_ONE_FLY = 16;
+__host__ __device__ constexpr int router_one_rows(int E) { return ROUTER_ONE_THREADS * 4 / (E > 128 ? E : 128); }  // partial sums per expert
+__host__ __device__ constexpr int router_one_smem(int E) { return (router_one_rows(E) + 1) * E * 4; }
+// Can also run on fewer threads (NT), which then take the work of several in turn: the sums are the same to the bit.
+__host__ __device__ __forceinline__ bool router_one_supported(int E, const void* Wr) {
+  return E >= 4 && (E & (E - 1)) == 0 && reinterpret_cast<uintptr_t>(Wr) % 16 == 0;
+}
+template <int NT, int FLY>
+__device__ __forceinline__ void router_logits_one(float* smem, const void* __restrict__ x, int x_bf16, int d, const float* __restrict__ Wr,
+                                                  const float* __restrict__ bias, int bias_stride, int E, int ep_shift,
+                                                  float* __restrict__ logits) {
+  float* zs = smem;        // [E]
+  float* red = smem + E;   // [rows][E]
+  const int tid = threadIdx.x, t = blockIdx.x, sh = ep_shift - 2, quads = 1 << sh;
+  const int n = d << sh;   // pieces
+  for (int vt = tid; vt < ROUTER_ONE_THREADS; vt += NT) {
+    float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int base = vt; base < n; base += FLY * ROUTER_ONE_THREADS) {
+      float4 w[FLY];
+      float v[FLY];
+#pragma unroll
+      for (int u = 0; u < FLY; ++u) {
+        const int i = base + u * ROUTER_ONE_THREADS;
+        w[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        v[u] = 0.0f;
+        if (i < n) {
+          w[u] = __ldg(reinterpret_cast<const float4*>(Wr) + i);
+          const size_t src = static_cast<size_t>(t) * d + (i >> sh);
+          v[u] = x_bf16 ? __bfloat162float(__ldg(reinterpret_cast<const __nv_bfloat16*>(x) + src)) : __ldg(reinterpret_cast<const float*>(x) + src);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < FLY; ++u) {
+        acc.x = fmaf(v[u], w[u].x, acc.x);
+        acc.y = fmaf(v[u], w[u].y, acc.y);
+        acc.z = fmaf(v[u], w[u].z, acc.z);
+        acc.w = fmaf(v[u], w[u].w, acc.w);
+      }
+    }
+    for (int o = 16; o >= quads; o >>= 1) {  // lanes with the same experts
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+      acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
+      acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+    }
+    if ((vt & 31) < quads)
+      *reinterpret_cast<float4*>(red + static_cast<size_t>(vt / max(32, quads)) * E + 4 * (vt & (quads - 1))) = acc;
+  }
+  __syncthreads();
+  pdl_wait();
+  for (int e = tid; e < E; e += NT) {
+    float z = 0.0f;
+    for (int row = 0; row < router_one_rows(E); ++row) z += red[row * E + e];
+    if (bias) z += bias[static_cast<size_t>(t) * bias_stride + e];
+    if (logits) logits[static_cast<size_t>(t) * E + e] = z;
+    zs[e] = z;
+  }
+  __syncthreads();
+}
+
 // Logits of the CTA's TT tokens into zs[TT][EP] as a register-tiled product, for batches: a thread holds TT/2 tokens x
 // four experts and an interleaved part of the inputs, so that an activation is read once per four
 // experts and a router weight once per TT/2 tokens; with one expert per thread (router_logits) every

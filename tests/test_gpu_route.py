@@ -64,6 +64,11 @@ EDGE_CASES = [
     (148, 256, 8, 1, False, True, None),
     (1535, 136, 12, 2, True, True, "vec"),
     (1537, 136, 12, 2, True, True, "vec"),
+    # one token per CTA, all loads at once: a few pieces, more than one round of them, the fewest and the most experts
+    (3, 4, 4, 2, True, True, None),
+    (5, 8200, 4, 1, False, False, "vec"),
+    (2, 1030, 64, 2, True, True, "tok"),
+    (6, 300, 256, 2, True, False, None),
     # inputs: one chunk and a remainder of it; experts: the fewest and the most
     (150, 8, 4, 4, True, False, None),
     (161, 520, 4, 1, False, False, None),
