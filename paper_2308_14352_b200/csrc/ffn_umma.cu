@@ -21,12 +21,17 @@
 //             packed bytes, dequantise to fp16 (code -> exact fp16 integer by mantissa insertion, then one
 //             multiply by the group scale: |error| <= 2^-12 relative, the only approximation of
 //             this path), and store the 64 values as 32 columns of the row's tensor-memory
-//             lane; later the epilogue: tensor memory -> registers -> activation -> global memory (gated:
-//             the threads of a w1 row and of its w3 row exchange halves through shared memory);
+//             lane; later the epilogue: tensor memory -> registers -> activation -> shared memory -> global
+//             memory, where a thread writes 16 bytes of one token (gated: a w1 row and its w3 row lie 16 lanes apart in
+//             one warp and swap halves by shuffles);
 //   warp 1    one thread issues tcgen05.mma (M128, N = the group's tokens rounded up to 16, in two halves
 //             beyond 256, K16, fp16 x fp16 -> fp32) per 16 inputs and commits each stage back.
 // A step costs two cycles per token in the tensor pipe and some 450 in the dequantisation, so groups of
 // about 256 tokens and more are tensor-bound; an expert's tokens are split evenly (choose_cut, TileWalk).
+// Measured (4096 x 14336 gated, 8 experts, 2048 tokens, 4 bits, both launches): 2040 us with one issuing lane in a branch
+// and groups of whole 128-token tiles, 1053 us now: 1.37 PFLOP/s, 0.86 of the measured dense rate.  Few tokens
+// (768 x 3072, 32 experts, 16 each) cost nearly as much as 64 each, 93 and 117 us per layer: an MMA with A in
+// tensor memory takes 120 cycles however narrow it is.
 // Activations travel as fp16 (exact for bf16 values inside the fp16 range, saturated outside);
 // the hidden vector is rounded to bf16 first, as the definition asks, then stored as fp16.
 // The reduction index is enumerated in the order the unpack emits code pairs; the activation
@@ -51,8 +56,8 @@ constexpr int UM_GROUP_TOK = 320;          // tokens that share one dequantised 
 constexpr int UM_BOX_TOK = 64;             // tokens per box of the activations' tensor map
 constexpr int UM_BOX_BYTES = UM_BOX_TOK * 128;
 constexpr int UM_B_STAGE_BYTES = UM_GROUP_TOK * 128;
-constexpr int UM_XCH_BYTES = 32 * 64 * 4;  // exchange of a set: 16 + 16 columns x 64 rows
-constexpr int UM_SMEM_BYTES = UM_RAW_STAGES * UM_TILE_BYTES + UM_STAGES * UM_B_STAGE_BYTES + 2 * UM_XCH_BYTES + 1024;  // 224 KB + alignment slack
+constexpr int UM_OUT_BYTES = 32 * 128 * 2;  // hidden values of a set on their way out: 32 tokens x 128 channels (gated: two turns of 64)
+constexpr int UM_SMEM_BYTES = UM_RAW_STAGES * UM_TILE_BYTES + UM_STAGES * UM_B_STAGE_BYTES + 2 * UM_OUT_BYTES + 1024;  // 224 KB + alignment slack
 constexpr int UM_A_COLS = UM_BK / 2;       // one A stage: 64 fp16 inputs = 32 columns, behind the accumulators
 constexpr int UM_CAPS = 4;                 // limits of a group that are considered: 128, 192, 256, 320 tokens
 __device__ __forceinline__ constexpr int um_cap(int c) { return 128 + 64 * c; }
@@ -282,11 +287,10 @@ struct UmBars {
 // number of steps).  srow: the row's scales from the unit's first step on, spg steps per scale.
 template <int BITS>
 __device__ __forceinline__ bool dequant_unit(const UmmaArgs& a, const UmBars& b, const unsigned char* raw_ring, uint32_t a_col, const void* sp,
-                                             size_t srow, int ngroups, int spg, int kb0, int kb_len, int part, int r, int lane, RingPos& pos,
+                                             size_t srow, int ngroups, int spg, int kb0, int kb_len, int part, int box, int rin, int lane, RingPos& pos,
                                              volatile int* abort_flag) {
   constexpr int KBS = (1024 / BITS) / UM_BK;  // steps per box
   const bool sf16 = a.L.scale_f16 != 0;
-  const int box = r >> 6, rin = r & 63;
   // scales of this set's step, its next one and the one after: a load has two steps to come back from L2; the group
   // index of the step two ahead is kept by counting
   const int first = kb0 + part;
@@ -342,7 +346,6 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
   // an offset from the array, not a rounded address: the compiler then knows that every access is to shared memory
   unsigned char* raw_ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* b_ring = raw_ring + UM_RAW_STAGES * UM_TILE_BYTES;
-  unsigned char* xch = b_ring + UM_STAGES * UM_B_STAGE_BYTES;
   const int lane = threadIdx.x & 31, warp = uniform_warp();
 
   UmBars b;
@@ -490,14 +493,18 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
     const int G = L.group > 0 ? L.group : K;
     const int ngroups = K / G, spg = G / UM_BK;  // G is a multiple of 128, or the whole row
     const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(32 * quarter) << 16);
-    const bool second = gated && quarter >= 2;   // a row of w3
-    float* xbuf = reinterpret_cast<float*>(xch + part * UM_XCH_BYTES);  // [16 columns of w1 | 16 of w3][64 rows]
+    // gated: the upper 16 lanes of a warp hold the w3 rows that belong to the w1 rows of the lower 16
+    const bool second = gated && lane >= 16;
+    const int rin = gated ? 16 * quarter + (lane & 15) : r & 63, box = gated ? lane >> 4 : r >> 6;  // row in which packed box
+    unsigned char* out_stage = b_ring + UM_STAGES * UM_B_STAGE_BYTES + part * UM_OUT_BYTES;
+    const int set_tid = 32 * quarter + lane;
+    int turn = 0;  // gated: the half of the buffer
     RingPos pos = {0, 0};
     int unit_it = 0;
     while (walk.next(tok_first, ntok, rb, z)) {
       const PlanRec& rec = walk.rec;
       const int bits = rec.bits;
-      const int nrow = gated ? rb * 64 + (r & 63) : rb * UM_ROWS + r;  // output channel
+      const int nrow = gated ? rb * 64 + rin : rb * UM_ROWS + r;  // output channel
       const size_t srow = static_cast<size_t>(min(nrow, N - 1)) * ngroups;
       // constant indices only: a record indexed by a variable would live in local memory
       const void* sp = second ? rec.scales[1] : (mat_first == 0 ? rec.scales[0] : (mat_first == 1 ? rec.scales[1] : rec.scales[2]));
@@ -505,16 +512,17 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
       const uint32_t a_col = lane_base + UM_GROUP_TOK;
       bool ok;
       switch (bits) {
-        case 2: ok = dequant_unit<2>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, r, lane, pos, abort_flag); break;
-        case 4: ok = dequant_unit<4>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, r, lane, pos, abort_flag); break;
-        default: ok = dequant_unit<8>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, r, lane, pos, abort_flag); break;
+        case 2: ok = dequant_unit<2>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
+        case 4: ok = dequant_unit<4>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
+        default: ok = dequant_unit<8>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
       }
       if (!ok) break;
       // ---- epilogue: this warp's 32 rows x every other 32 token columns ----
       if (!mbar_wait_warp(b.acc_full, unit_it & 1, a.check_word, abort_flag)) break;
       tc_fence_after();
       const size_t slot0 = static_cast<size_t>(rec.begin) + static_cast<size_t>(tok_first);
-      const int hpos = a.phase == 0 ? pair_pos_rt(bits, min(nrow, N - 1)) : 0;
+      const int u_row0 = rb * (gated ? 64 : UM_ROWS);  // first channel of the unit
+      const int hpos = a.phase == 0 ? pair_pos_rt(bits, nrow) : 0;  // (moves a channel inside its 16)
 #pragma unroll 1
       for (int cc = 32 * part; cc < ntok; cc += 64) {
         uint32_t va[32];
@@ -524,48 +532,58 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
         const int live = min(32, ntok - cc);  // token columns of this chunk that exist
         // one compact unrolled loop per case (the conditions are uniform)
         if (gated) {
-          // the threads of a w1 row and of its w3 row swap halves: the first computes columns 0..15, the second 16..31
-          const int row = r & 63;
-          float* mine = xbuf + (second ? 16 * 64 : 0) + row;
-#pragma unroll
-          for (int c = 0; c < 16; ++c) mine[c * 64] = __uint_as_float(second ? va[c] : va[16 + c]);
-          asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");
-          const float* theirs = xbuf + (second ? 0 : 16 * 64) + row;
+          // the lanes of a w1 row and of its w3 row swap halves: the first computes columns 0..15, the second 16..31
           const int c0 = second ? 16 : 0;
-          __half* dst = a.hidden16 + (slot0 + cc + c0) * a.hid_stride + hpos;
+          unsigned char* stage = out_stage + turn * (UM_OUT_BYTES / 2);  // [32 tokens][64 channels], 64-byte halves swapped from token 16 on
+          unsigned char* mine = stage + c0 * 128 + (((hpos - u_row0) * 2) ^ (second ? 64 : 0));
           bool beyond = false;
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
-            const float own = __uint_as_float(second ? va[16 + c] : va[c]), other = theirs[c * 64];
-            const float av = second ? other : own, bv = second ? own : other;
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, second ? va[c] : va[16 + c], 16);
+            const float av = __uint_as_float(second ? other : va[c]), bv = __uint_as_float(second ? va[16 + c] : other);
             // the hidden vector is a bf16 tensor
             const float h = __bfloat162float(__float2bfloat16_rn(silu_branchless(av) * bv));
-            if (c0 + c < live) {  // columns past the last token read whatever lies behind it
-              beyond |= beyond_f16(h);
-              dst[static_cast<size_t>(c) * a.hid_stride] = __float2half_rn(fminf(fmaxf(h, -65504.0f), 65504.0f));
-            }
+            beyond |= c0 + c < live && beyond_f16(h);  // columns past the last token read whatever lies behind it
+            *reinterpret_cast<__half*>(mine + c * 128) = __float2half_rn(fminf(fmaxf(h, -65504.0f), 65504.0f));
           }
           if (beyond) atomicOr(a.check_word, CHECK_F16_RANGE);  // saturated above: reported, not silent
-          asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");  // the buffer has been read
-        } else if (nrow < N) {
-          if (a.phase != 0) {
-            float* dst = a.o + z * a.plane_stride + (slot0 + cc) * N + nrow;
+          asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");
 #pragma unroll
-            for (int c = 0; c < 32; ++c)
-              if (c < live) dst[static_cast<size_t>(c) * N] = __uint_as_float(va[c]);
-          } else {
-            __half* dst = a.hidden16 + (slot0 + cc) * a.hid_stride + hpos;
-            bool beyond = false;
+          for (int i = 0; i < 2; ++i) {
+            const int tok = (set_tid >> 3) + 16 * i, piece = set_tid & 7;
+            if (tok < live)
+              *reinterpret_cast<uint4*>(a.hidden16 + (slot0 + cc + tok) * a.hid_stride + u_row0 + 8 * piece) =
+                  *reinterpret_cast<const uint4*>(stage + tok * 128 + ((piece * 16) ^ (i ? 64 : 0)));
+          }
+          turn ^= 1;  // whoever writes this half again has passed the next barrier, and with it everybody's reads
+        } else if (a.phase != 0) {
+          float* dst = a.o + z * a.plane_stride + (slot0 + cc) * N + nrow;
+          if (nrow < N) {
 #pragma unroll
             for (int c = 0; c < 32; ++c) {
-              const float h = __bfloat162float(__float2bfloat16_rn(fmaxf(__uint_as_float(va[c]), 0.0f)));
-              if (c < live) {
-                beyond |= beyond_f16(h);
-                dst[static_cast<size_t>(c) * a.hid_stride] = __float2half_rn(fminf(h, 65504.0f));
-              }
+              if (c < live) *dst = __uint_as_float(va[c]);
+              dst += N;
             }
-            if (beyond) atomicOr(a.check_word, CHECK_F16_RANGE);
           }
+        } else {
+          unsigned char* mine = out_stage + (hpos - u_row0) * 2;  // [32 tokens][128 channels]
+          bool beyond = false;
+#pragma unroll
+          for (int c = 0; c < 32; ++c) {
+            const float h = __bfloat162float(__float2bfloat16_rn(fmaxf(__uint_as_float(va[c]), 0.0f)));
+            beyond |= c < live && nrow < N && beyond_f16(h);
+            *reinterpret_cast<__half*>(mine + c * 256) = __float2half_rn(fminf(h, 65504.0f));
+          }
+          if (beyond) atomicOr(a.check_word, CHECK_F16_RANGE);
+          asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int tok = (set_tid >> 4) + 8 * i, ch = 8 * (set_tid & 15);
+            if (tok < live && u_row0 + ch < N)
+              *reinterpret_cast<uint4*>(a.hidden16 + (slot0 + cc + tok) * a.hid_stride + u_row0 + ch) =
+                  *reinterpret_cast<const uint4*>(out_stage + tok * 256 + ch * 2);
+          }
+          asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");  // the buffer has been read
         }
       }
       tc_fence_before();
