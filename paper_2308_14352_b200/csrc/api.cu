@@ -462,8 +462,8 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
       EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
       EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
     }
-    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, ctx->check_word, st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, false, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, false, ctx->check_word, st));
     if (ev[1]) {  // one interval for the whole expert stage
       EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
       ctx->events_one_launch[ctx->events_used / 3 - 1] = 1;
@@ -477,9 +477,9 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
       EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, nullptr, plan_heavy, xs, nullptr, P, SCATTER_ROWS16, heavy_above,
                                         ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, true, ctx->check_word, st));
     if (ev[1]) EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, true, ctx->check_word, st));
   } else if (use_i8) {
     ksplit = ffn_i8_ksplit(L, T);
     if (one_launch_route)

@@ -178,7 +178,7 @@ bool ffn_umma_supported(const LayerDims& L);
 // zmax: most planes of partial sums the second projection may leave; how many it does is decided on the device and left in
 // the fourth word of the plan's header.
 cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, int* plan, const void* in16, int in_stride,
-                            void* hidden16, int hid_stride, float* o, int n_pairs, int zmax, int* check_word,
+                            void* hidden16, int hid_stride, float* o, int n_pairs, int zmax, bool all_experts, int* check_word,
                             cudaStream_t st);
 
 // y[t] = sum_j gates[t][j] * sum_z o_part[z][slot_of_pair[t*k+j]]

@@ -24,13 +24,15 @@
 //             lane; later the epilogue: tensor memory -> registers -> activation -> shared memory -> global
 //             memory, where a thread writes 16 bytes of one token (gated: a w1 row and its w3 row lie 16 lanes apart in
 //             one warp and swap halves by shuffles);
+//   warps 11-14 (calls with few tokens per expert) the epilogue of groups up to 160 tokens, two of which have
+//             accumulators at a time, while the others go on with the next unit;
 //   warp 1    one thread issues tcgen05.mma (M128, N = the group's tokens rounded up to 16, in two halves
 //             beyond 256, K16, fp16 x fp16 -> fp32) per 16 inputs and commits each stage back.
 // A step costs two cycles per token in the tensor pipe and some 450 in the dequantisation, so groups of
 // about 256 tokens and more are tensor-bound; an expert's tokens are split evenly (choose_cut, TileWalk).
 // Measured (4096 x 14336 gated, 8 experts, 2048 tokens, 4 bits, both launches): 2040 us with one issuing lane in a branch
-// and groups of whole 128-token tiles, 1053 us now: 1.37 PFLOP/s, 0.86 of the measured dense rate.  Few tokens
-// (768 x 3072, 32 experts, 16 each) cost nearly as much as 64 each, 93 and 117 us per layer: an MMA with A in
+// and groups of whole 128-token tiles, 1053 us now: 1.37 PFLOP/s, 0.85 of the measured dense rate.  Few tokens
+// (768 x 3072, 32 experts, 16 each) cost nearly as much as 64 each, 92 and 108 us per layer: an MMA with A in
 // tensor memory takes 120 cycles however narrow it is.
 // Activations travel as fp16 (exact for bf16 values inside the fp16 range, saturated outside);
 // the hidden vector is rounded to bf16 first, as the definition asks, then stored as fp16.
@@ -59,11 +61,13 @@ constexpr int UM_B_STAGE_BYTES = UM_GROUP_TOK * 128;
 constexpr int UM_OUT_BYTES = 32 * 128 * 2;  // hidden values of a set on their way out: 32 tokens x 128 channels (gated: two turns of 64)
 constexpr int UM_SMEM_BYTES = UM_RAW_STAGES * UM_TILE_BYTES + UM_STAGES * UM_B_STAGE_BYTES + 2 * UM_OUT_BYTES + 1024;  // 224 KB + alignment slack
 constexpr int UM_A_COLS = UM_BK / 2;       // one A stage: 64 fp16 inputs = 32 columns, behind the accumulators
-constexpr int UM_CAPS = 4;                 // limits of a group that are considered: 128, 192, 256, 320 tokens
-__device__ __forceinline__ constexpr int um_cap(int c) { return 128 + 64 * c; }
+constexpr int UM_TWO_TOK = UM_GROUP_TOK / 2;  // groups up to this size: accumulators of two units in turn
+constexpr int UM_CAPS = 4;                 // limits of a group that are considered
+__host__ __device__ __forceinline__ constexpr int um_cap(int c) { return c == 0 ? 96 : (c == 1 ? 160 : (c == 2 ? 256 : 320)); }
 constexpr int UM_UNPACK_WARPS = 8;         // two sets of four
 constexpr int UM_RAW_WARP = 2 + UM_UNPACK_WARPS;
-constexpr int UM_THREADS = (3 + UM_UNPACK_WARPS) * 32;
+constexpr int UM_STORE_WARPS = 4;           // epilogue of small groups
+constexpr int um_threads(bool store_warps) { return (3 + UM_UNPACK_WARPS + (store_warps ? UM_STORE_WARPS : 0)) * 32; }
 constexpr int UM_TMEM_COLS = 512;
 
 // a / (1 + exp(-a)) without a branch, so that the 16 columns of a thread overlap (the operator's slow path
@@ -242,9 +246,10 @@ struct TileWalk {
 
 // How a launch is cut (one warp): most tokens of a group, slices of the second projection's inputs.  Larger groups share
 // the dequantisation, smaller ones and slices fill the last round of CTAs.  The estimate, in cycles: a
-// step of 64 inputs takes two per token or the 450 of the dequantisation, a unit 1500 + 12 per token
-// to start and store; a further plane of sums costs the combine step its bandwidth (3400 B per cycle).
-__device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, int row_blocks, int kb_total, int lane) {
+// step of 64 inputs takes two per token or the 500 an MMA with A in tensor memory takes at least; storing a unit 30
+// per token with eight warps, behind its last MMA, or 60 with the four that do nothing else, beside the next unit; a further
+// plane of sums costs the combine step its bandwidth (3400 B per cycle).
+__device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, int row_blocks, int kb_total, int lane, bool store_warps) {
   const int n_active = *reinterpret_cast<const volatile int*>(a.plan);
   const PlanRec* recs = reinterpret_cast<const PlanRec*>(reinterpret_cast<const char*>(a.plan) + PLAN_HEADER_BYTES);
   int groups[UM_CAPS] = {}, tokens = 0;
@@ -264,7 +269,8 @@ __device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, int row_blocks, in
     for (int z = 1; z <= a.zmax; z *= 2) {
       if (z > 1 && (kb_total % z != 0 || kb_total / z % 8 != 0)) break;  // a slice starts on a packed box at every width
       const int rounds = (g * row_blocks * z + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
-      const float unit = static_cast<float>(kb_total / z) * fmaxf(450.0f, 2.0f * tok) + 1500.0f + 12.0f * tok;
+      const float steps = static_cast<float>(kb_total / z) * fmaxf(500.0f, 2.0f * tok);
+      const float unit = store_warps && um_cap(c) <= UM_TWO_TOK ? fmaxf(steps + 500.0f, 60.0f * tok) : steps + 3000.0f + 30.0f * tok;
       const float cost = static_cast<float>(rounds) * unit + static_cast<float>(z - 1) * static_cast<float>(tokens) * static_cast<float>(a.L.d_model) * (8.0f / 3400.0f);
       if (cost < best_cost) {
         best_cost = cost;
@@ -278,6 +284,15 @@ __device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, int row_blocks, in
 // where a dequantisation warp stands in the rings
 struct RingPos {
   int raw_it, ab_it;
+};
+// The accumulators of a CTA's n-th unit: where the groups are small enough, two units in turn have columns of their own.
+struct AccSlot {
+  int index, parity, col;
+  __device__ __forceinline__ AccSlot(int n, bool two) {
+    index = two ? n & 1 : 0;
+    parity = two ? (n >> 1) & 1 : n & 1;
+    col = index * UM_TWO_TOK;
+  }
 };
 struct UmBars {
   uint32_t raw_full, raw_empty, ab_full, ab_empty, acc_full, acc_empty;
@@ -335,10 +350,15 @@ __device__ __forceinline__ bool dequant_unit(const UmmaArgs& a, const UmBars& b,
   return true;
 }
 
-__global__ void __launch_bounds__(UM_THREADS, 1)
+// STORE: with the warps that store small groups.  Calls whose experts hold 192 tokens and more on average, and calls that
+// leave only their fullest experts to this kernel, go without: their groups seldom fit two sets of
+// accumulators, and fewer warps may keep more registers (1 to 2 % of the time).  Where they fit, 777 tokens on 32
+// experts of 768 x 3072 take 3 %, 2048 on 128 of 1024 x 4096 6 % less with them.
+template <bool STORE>
+__global__ void __launch_bounds__(um_threads(STORE), 1)
     ffn_umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap tmap_b) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * UM_RAW_STAGES + 2 * UM_STAGES + 2];
+  __shared__ __align__(8) uint64_t bars[2 * UM_RAW_STAGES + 2 * UM_STAGES + 4];
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_word;
   __shared__ int2 cut_slot;
@@ -354,7 +374,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
   b.ab_full = b.raw_empty + 8 * UM_RAW_STAGES;
   b.ab_empty = b.ab_full + 8 * UM_STAGES;
   b.acc_full = b.ab_empty + 8 * UM_STAGES;
-  b.acc_empty = b.acc_full + 8;
+  b.acc_empty = b.acc_full + 16;
 
   if (threadIdx.x == 0) {
     abort_word = 0;
@@ -366,8 +386,6 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
       mbar_init(b.ab_full + 8 * s, 1 + UM_UNPACK_WARPS / 2);  // the activations' producer (+ bytes) and the set that fills A
       mbar_init(b.ab_empty + 8 * s, 1);
     }
-    mbar_init(b.acc_full, 1);
-    mbar_init(b.acc_empty, UM_UNPACK_WARPS);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), UM_TMEM_COLS);  // accumulators + four A stages
@@ -388,14 +406,20 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
 
   TileWalk walk;
   if (warp == 0) {
-    const int2 c = choose_cut(a, row_blocks, kb_total, lane);
+    const int2 c = choose_cut(a, row_blocks, kb_total, lane, STORE);
     if (lane == 0) {
       cut_slot = c;
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(b.acc_full + 8 * i, 1);
+        mbar_init(b.acc_empty + 8 * i, STORE && c.x <= UM_TWO_TOK ? UM_STORE_WARPS : UM_UNPACK_WARPS);
+      }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       if (a.phase == 1 && blockIdx.x == 0) a.plan[3] = c.y;  // for the combine step
     }
   }
   __syncthreads();
   const int2 cut = cut_slot;
+  const bool two = STORE && cut.x <= UM_TWO_TOK;
   const int kb_len = kb_total / cut.y;  // steps of a unit
   walk.init(a.plan, row_blocks, cut);
   int tok_first, ntok, rb, z;
@@ -432,6 +456,18 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
       const int row0 = rb * (gated ? 64 : 128), row1 = gated ? row0 : row0 + 64;
       const int kbs = (1024 / rec.bits) / UM_BK;  // steps per box (128 bytes of a row)
       const int kb_end = (z + 1) * kb_len;
+      if (z == 0) {  // this warp is up to a unit ahead: pull the unit's scales towards L2
+        const int row_bytes = K / (L.group > 0 ? L.group : K) * (L.scale_f16 ? 2 : 4);
+        const int bytes = min(gated ? 64 : 128, N - row0) * row_bytes;
+        const char* sc0 = static_cast<const char*>(mat_first == 0 ? rec.scales[0] : (mat_first == 1 ? rec.scales[1] : rec.scales[2])) +
+                          static_cast<size_t>(row0) * row_bytes;
+        const char* sc1 = static_cast<const char*>(gated ? rec.scales[1] : nullptr) + static_cast<size_t>(row0) * row_bytes;
+        for (int i = lane * 128; i < bytes; i += 32 * 128) {
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(sc0 + i));
+          if (gated) asm volatile("prefetch.global.L2 [%0];" ::"l"(sc1 + i));
+        }
+        __syncwarp();
+      }
       int c0 = z * kb_len / kbs * 128;
       for (int kb = z * kb_len; kb < kb_end; kb += kbs, ++it, c0 += 128) {
         const int s = it % UM_RAW_STAGES;
@@ -459,7 +495,9 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
       const int n1 = cols <= 256 ? cols : ((cols / 2 + 15) & ~15), n2 = cols - n1;
       const uint32_t id1 = idesc | ((n1 >> 3) << 17), id2 = idesc | ((n2 >> 3) << 17);
       const uint32_t on1 = n1 > 0 ? on : 0u, on2 = n2 > 0 ? on : 0u;
-      if (!mbar_wait_warp(b.acc_empty, ((unit_it & 1) ^ 1), a.check_word, abort_flag)) break;
+      const AccSlot acc(unit_it, two);
+      const uint32_t d_t = tmem_base + acc.col;
+      if (!mbar_wait_warp(b.acc_empty + 8 * acc.index, acc.parity ^ 1, a.check_word, abort_flag)) break;
       tc_fence_after();
       for (int kb = 0; kb < kb_len; ++kb, ++ab_it) {
         const int s = ab_it % UM_STAGES;
@@ -473,22 +511,25 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
         const uint64_t db1 = umma_desc(bs);
 #pragma unroll
         for (int k4 = 0; k4 < UM_BK / 16; ++k4)  // 16 inputs: 8 columns of A, 32 bytes (2 descriptor units) of B
-          umma_f16_ts_if(on1, tmem_base, a_t + 8 * k4, db1 + 2 * k4, id1, (kb > 0 || k4 > 0) ? 1u : 0u);
+          umma_f16_ts_if(on1, d_t, a_t + 8 * k4, db1 + 2 * k4, id1, (kb > 0 || k4 > 0) ? 1u : 0u);
         if (n2 > 0) {
           const uint64_t db2 = umma_desc(bs + n1 * 128);
 #pragma unroll
           for (int k4 = 0; k4 < UM_BK / 16; ++k4)
-            umma_f16_ts_if(on2, tmem_base + n1, a_t + 8 * k4, db2 + 2 * k4, id2, (kb > 0 || k4 > 0) ? 1u : 0u);
+            umma_f16_ts_if(on2, d_t + n1, a_t + 8 * k4, db2 + 2 * k4, id2, (kb > 0 || k4 > 0) ? 1u : 0u);
         }
         umma_commit_if(on, b.ab_empty + 8 * s);  // the stage may be refilled once these MMAs have read it
       }
-      if (ok) umma_commit_if(on, b.acc_full);
+      if (ok) umma_commit_if(on, b.acc_full + 8 * acc.index);
       ++unit_it;
     }
   } else {
-    // ---------------- dequantise (a thread per weight row), then epilogue ----------------
+    // ---------------- dequantise (a thread per weight row) and epilogue ----------------
+    // Groups too large for two sets of accumulators: the dequantising warps store a unit before they go on, eight warps
+    // being faster at it and nothing to overlap it with.  Otherwise the last four warps do, and the others go on.
     const int quarter = warp & 3;          // TMEM lanes this warp may access: 32 * quarter ...
-    const int part = (warp - 2) >> 2;      // the set: even or odd steps, and 32-token chunks of the epilogue
+    const int part = STORE && warp > UM_RAW_WARP ? 2 : (warp - 2) >> 2;  // the set: even or odd steps, or the storing warps
+    const int first_chunk = two ? 0 : 32 * part, chunk_step = two ? 32 : 64;
     const int r = 32 * quarter + lane;     // row of the tile = row of the operand = TMEM lane
     const int G = L.group > 0 ? L.group : K;
     const int ngroups = K / G, spg = G / UM_BK;  // G is a multiple of 128, or the whole row
@@ -496,7 +537,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
     // gated: the upper 16 lanes of a warp hold the w3 rows that belong to the w1 rows of the lower 16
     const bool second = gated && lane >= 16;
     const int rin = gated ? 16 * quarter + (lane & 15) : r & 63, box = gated ? lane >> 4 : r >> 6;  // row in which packed box
-    unsigned char* out_stage = b_ring + UM_STAGES * UM_B_STAGE_BYTES + part * UM_OUT_BYTES;
+    unsigned char* out_stage = b_ring + UM_STAGES * UM_B_STAGE_BYTES + (part & 1) * UM_OUT_BYTES;
     const int set_tid = 32 * quarter + lane;
     int turn = 0;  // gated: the half of the buffer
     RingPos pos = {0, 0};
@@ -510,24 +551,31 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
       const void* sp = second ? rec.scales[1] : (mat_first == 0 ? rec.scales[0] : (mat_first == 1 ? rec.scales[1] : rec.scales[2]));
       const int kb0 = z * kb_len;
       const uint32_t a_col = lane_base + UM_GROUP_TOK;
-      bool ok;
-      switch (bits) {
-        case 2: ok = dequant_unit<2>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
-        case 4: ok = dequant_unit<4>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
-        default: ok = dequant_unit<8>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
+      bool ok = true;
+      if (part < 2) {
+        switch (bits) {
+          case 2: ok = dequant_unit<2>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
+          case 4: ok = dequant_unit<4>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
+          default: ok = dequant_unit<8>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
+        }
       }
       if (!ok) break;
-      // ---- epilogue: this warp's 32 rows x every other 32 token columns ----
-      if (!mbar_wait_warp(b.acc_full, unit_it & 1, a.check_word, abort_flag)) break;
+      if (two != (part == 2)) {
+        ++unit_it;
+        continue;
+      }
+      // ---- epilogue: this warp's 32 rows x (every other) 32 token columns ----
+      const AccSlot acc(unit_it, two);
+      if (!mbar_wait_warp(b.acc_full + 8 * acc.index, acc.parity, a.check_word, abort_flag)) break;
       tc_fence_after();
       const size_t slot0 = static_cast<size_t>(rec.begin) + static_cast<size_t>(tok_first);
       const int u_row0 = rb * (gated ? 64 : UM_ROWS);  // first channel of the unit
       const int hpos = a.phase == 0 ? pair_pos_rt(bits, nrow) : 0;  // (moves a channel inside its 16)
 #pragma unroll 1
-      for (int cc = 32 * part; cc < ntok; cc += 64) {
+      for (int cc = first_chunk; cc < ntok; cc += chunk_step) {
         uint32_t va[32];
         __syncwarp();
-        tmem_ld32(lane_base + cc, va);
+        tmem_ld32(lane_base + acc.col + cc, va);
         tmem_ld_wait();
         const int live = min(32, ntok - cc);  // token columns of this chunk that exist
         // one compact unrolled loop per case (the conditions are uniform)
@@ -588,7 +636,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(b.acc_empty);
+      if (lane == 0) mbar_arrive(b.acc_empty + 8 * acc.index);
       ++unit_it;
     }
   }
@@ -612,7 +660,7 @@ bool ffn_umma_supported(const LayerDims& L) {
 }
 
 cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, int* plan, const void* in16, int in_stride,
-                            void* hidden16, int hid_stride, float* o, int n_pairs, int zmax, int* check_word,
+                            void* hidden16, int hid_stride, float* o, int n_pairs, int zmax, bool all_experts, int* check_word,
                             cudaStream_t st) {
   const int N = phase == 0 ? L.d_ff : L.d_model;
   const int K = phase == 0 ? L.d_model : L.d_ff;
@@ -626,7 +674,9 @@ cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, in
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!sms_of_device[dev]) {
-    e = cudaFuncSetAttribute(ffn_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, UM_SMEM_BYTES);
+    e = cudaFuncSetAttribute(ffn_umma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, UM_SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(ffn_umma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, UM_SMEM_BYTES);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms_of_device[dev], cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
@@ -634,7 +684,7 @@ cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, in
   const bool gated = phase == 0 && L.act == EMOE_ACT_SWIGLU;
   const long long row_blocks = gated ? N / (UM_ROWS / 2) : (N + UM_ROWS - 1) / UM_ROWS;
   // upper bound of the tile count: every pair alone in a token tile
-  long long tiles = row_blocks * (static_cast<long long>(n_pairs < L.E ? n_pairs : L.E) + n_pairs / 128) * (phase == 1 && zmax > 1 ? zmax : 1);
+  long long tiles = row_blocks * (static_cast<long long>(n_pairs < L.E ? n_pairs : L.E) + n_pairs / um_cap(0)) * (phase == 1 && zmax > 1 ? zmax : 1);
   const int grid = static_cast<int>(tiles < sms_of_device[dev] ? tiles : sms_of_device[dev]);
   UmmaArgs a;
   a.phase = phase;
@@ -648,7 +698,8 @@ cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, in
   a.n_pairs = n_pairs;
   a.plane_stride = static_cast<size_t>(n_pairs) * L.d_model;
   a.check_word = check_word;
-  return launch_chain(ffn_umma_kernel, dim3(grid), dim3(UM_THREADS), UM_SMEM_BYTES, st, a, tmap_b);
+  if (all_experts && n_pairs < 192LL * L.E) return launch_chain(ffn_umma_kernel<true>, dim3(grid), dim3(um_threads(true)), UM_SMEM_BYTES, st, a, tmap_b);
+  return launch_chain(ffn_umma_kernel<false>, dim3(grid), dim3(um_threads(false)), UM_SMEM_BYTES, st, a, tmap_b);
 }
 
 }  // namespace emoe

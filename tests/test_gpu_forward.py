@@ -472,6 +472,10 @@ UMMA_EDGE_CASES = [
     ("swiglu", 128, "f16", 512, 512, 1, 1, "softmax", [8], 320),
     ("relu", 128, "f16", 512, 512, 1, 1, "softmax", [4], 321),
     ("relu", 128, "f32", 512, 2048, 1, 1, "softmax", [2], 129),       # second projection in slices of its inputs
+    # several units per CTA: accumulators in turn, stored by warps of their own (small groups) or not (large ones)
+    ("relu", 128, "f16", 512, 8192, 4, 1, "softmax", [4, 2, 8, 4], 150),
+    ("swiglu", 128, "f16", 512, 6144, 3, 2, "softmax_renorm", [8, 4, 2], 200),
+    ("swiglu", 128, "f16", 512, 6144, 2, 2, "softmax_renorm", [4, 2], 210),
 ]
 
 
