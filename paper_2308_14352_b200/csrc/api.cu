@@ -20,7 +20,6 @@ thread_local bool g_pdl_enabled = false;
 namespace {
 
 // calls on both kernel families: experts with up to this many tokens (two passes) take the weight-streaming kernel
-// (16 and 64 instead were up to 13 % and 15 % slower over means of 16 to 64 tokens, even and skewed)
 constexpr int HYBRID_STREAM_TOKENS = 32;
 constexpr int MAX_TABLES = 128;  // distinct expert tables a context can keep on the device
 constexpr size_t TMAP_BYTES = 128;  // sizeof(CUtensorMap)
@@ -377,16 +376,24 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   const bool can_tma = ffn_tma_supported(L) && tmaps != nullptr;
   const bool can_i8 = ffn_i8_supported(L) && tmaps != nullptr;
   const bool can_umma = ffn_umma_supported(L) && tmaps != nullptr;
-  // many tokens per expert: the tcgen05 grouped GEMM; otherwise the weight-streaming kernels
-  const bool many_tokens = ffn_many_tokens(L, T);
-  // skewed loads: experts with few tokens stream through the TMA kernel, the others take the
-  // tcgen05 grouped GEMM, in the same forward call
-  // ... unless the experts hold 24 tokens each on average: from there on the tcgen05 kernel alone, whose time hardly
-  // depends on the tokens up to 128 an expert, beats both (768 x 3072, 32 experts, us per layer: 777 tokens 100 against
-  // 116 on both families and 97 streaming, 1024 103/127/115, 2048 117/121/207; at 512 93/90/79)
-  const bool dense_tokens = ffn_dense_tokens(L, T);
-  const bool use_hybrid = can_umma && can_tma && (ctx->ffn_path == 5 || (ctx->ffn_path == 0 && many_tokens && !dense_tokens));
-  const bool use_umma = !use_hybrid && can_umma && (ctx->ffn_path == 4 || (ctx->ffn_path == 0 && many_tokens));
+  // The tcgen05 grouped GEMM comes in two forms (ffn_umma.cu): one rounds code x scale to fp16 and shares the dequantised
+  // weights among up to 320 tokens; the other keeps the codes exact and takes 64 tokens at a time.
+  // Rounded: from 16 tokens per expert on average, on rows of whole packed boxes at every width, for the experts with
+  // more than HYBRID_STREAM_TOKENS tokens, the others stream; from 256 for all (next to nobody would be left to stream).
+  const double mean_tokens = static_cast<double>(P) / L.E;
+  const bool rounded = mean_tokens >= 16.0 && L.d_model % 512 == 0 && L.d_ff % 512 == 0;
+  // Exact: elsewhere, from 192 (token, expert) pairs.  An uneven load can then fill an expert well beyond the 16 tokens that
+  // the streaming kernel takes per pass over the weights; an even one pays some 5 us for two launches that find
+  // nobody.  From 32 tokens per expert on average for all of them; below, for experts beyond 32 tokens, 48 where even
+  // loads reach 32 as well.  us per layer, streaming alone / both, even and skewed (Zipf exponent 1.1) loads:
+  // 768 x 3072, 32 experts, 256 tokens 53/58 and 88/78, 512 tokens 77/81 and 138/103; 1024 x 4096, 128 experts, 1024 tokens 220/226
+  // and 477/179; 1280 x 4480, 64 experts, 800 tokens 209/218 and 373/197; 2048 tokens on the first, all 192/144 and 510/165.
+  const bool exact_pairs = !rounded && P >= 192;
+  const bool one_family = mean_tokens >= (rounded ? 256.0 : 32.0);
+  const bool auto_umma = ctx->ffn_path == 0 && (rounded || exact_pairs);
+  const bool exact_umma = ctx->ffn_path == 0 && !rounded;
+  const bool use_hybrid = can_umma && can_tma && (ctx->ffn_path == 5 || (auto_umma && !one_family));
+  const bool use_umma = !use_hybrid && can_umma && (ctx->ffn_path == 4 || (auto_umma && one_family));
   // the weight-streaming kernels: the fp16 mma.sync one by default (the faster of the two as measured), the
   // one on int8 tcgen05 operands on request
   const bool use_i8 = !use_hybrid && !use_umma && can_i8 && ctx->ffn_path == 6;
@@ -443,13 +450,11 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   // families can share the buffers
   const int xs_stride = static_cast<int>(act_slot_bytes(L.d_model) / 2), hid_stride = static_cast<int>(act_slot_bytes(L.d_ff) / 2);
   int* plan_heavy = reinterpret_cast<int*>(reinterpret_cast<char*>(plan) + align_up(plan_bytes(L.E)));
-  const int heavy_above = use_umma ? 0 : HYBRID_STREAM_TOKENS;  // experts with more tokens than this are the tcgen05 kernel's
+  const int heavy_above = use_umma ? 0 : HYBRID_STREAM_TOKENS + (exact_umma && mean_tokens >= 16.0 ? 16 : 0);  // experts with more tokens than this are the tcgen05 kernel's
   const int zmax = w.ksplit < 4 ? w.ksplit : 4;  // planes of partial sums its second projection may use
   if (use_hybrid) {
     // Each family has its own plan and writes only its own slots of xs / hidden / o_part.
-    // many tokens in the call: the streaming family's tail matters little, every further split-K plane costs a re-read
-    // [P][d] fp32 array
-    ksplit = ffn_tma_ksplit(L, T) < 2 ? ffn_tma_ksplit(L, T) : 2;
+    ksplit = ffn_tma_ksplit(L, T);
     if (one_launch_permute)
       EMOE_LAUNCH(ctx, launch_permute_scatter(L, table, x, ids_use, counts, off, perm, slot_of_pair, plan, plan_heavy, xs, nullptr, P, 1,
                                               heavy_above, ctx->check_word, st));
@@ -462,8 +467,8 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
       EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
       EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
     }
-    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, false, ctx->check_word, st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, false, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, exact_umma, exact_umma, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, exact_umma, exact_umma, ctx->check_word, st));
     if (ev[1]) {  // one interval for the whole expert stage
       EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
       ctx->events_one_launch[ctx->events_used / 3 - 1] = 1;
@@ -477,9 +482,9 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
       EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, nullptr, plan_heavy, xs, nullptr, P, SCATTER_ROWS16, heavy_above,
                                         ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, true, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, exact_umma, false, ctx->check_word, st));
     if (ev[1]) EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
-    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, true, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, exact_umma, false, ctx->check_word, st));
   } else if (use_i8) {
     ksplit = ffn_i8_ksplit(L, T);
     if (one_launch_route)

@@ -105,8 +105,6 @@ cudaError_t launch_ffn_gemv(int phase, const LayerDims& L, const ExpertDev* expe
 bool ffn_mma_supported(const LayerDims& L);
 int ffn_mma_ksplit(const LayerDims& L, int T);
 int ffn_token_tiles(const LayerDims& L, int T);
-bool ffn_many_tokens(const LayerDims& L, int T);
-bool ffn_dense_tokens(const LayerDims& L, int T);
 // plan (nullable): plan_bytes(E) bytes, the work plan for the persistent TMA kernels, filled by block 0.
 // fmt: 0 = bf16, 1 = fp16 tiles (act_tile.cuh, saturating: the TMA-staged kernel's input), 2 = two-limb
 // block-scaled integers (act_q.cuh: the int8 tensor-core kernel's input; xsc receives the block scales).
@@ -178,7 +176,7 @@ bool ffn_umma_supported(const LayerDims& L);
 // zmax: most planes of partial sums the second projection may leave; how many it does is decided on the device and left in
 // the fourth word of the plan's header.
 cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, int* plan, const void* in16, int in_stride,
-                            void* hidden16, int hid_stride, float* o, int n_pairs, int zmax, bool all_experts, int* check_word,
+                            void* hidden16, int hid_stride, float* o, int n_pairs, int zmax, bool exact, bool maybe_empty, int* check_word,
                             cudaStream_t st);
 
 // y[t] = sum_j gates[t][j] * sum_z o_part[z][slot_of_pair[t*k+j]]

@@ -316,11 +316,6 @@ int ffn_token_tiles(const LayerDims& L, int T) {
   return mean <= 12.0 ? 1 : 2;
 }
 
-// Enough tokens per expert (mean of 16 under uniform routing) that the experts with many tokens
-// are a dense contraction: those go to the tcgen05 grouped GEMM.
-bool ffn_many_tokens(const LayerDims& L, int T) { return static_cast<double>(T) * L.top_k / L.E >= 16.0; }
-bool ffn_dense_tokens(const LayerDims& L, int T) { return static_cast<double>(T) * L.top_k / L.E >= 24.0; }
-
 bool ffn_mma_supported(const LayerDims& L) {
   if (!L.act_bf16) return false;
   if (L.d_model % 128 != 0 || L.d_ff % 128 != 0) return false;

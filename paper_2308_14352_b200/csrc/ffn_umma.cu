@@ -24,8 +24,7 @@
 //             lane; later the epilogue: tensor memory -> registers -> activation -> shared memory -> global
 //             memory, where a thread writes 16 bytes of one token (gated: a w1 row and its w3 row lie 16 lanes apart in
 //             one warp and swap halves by shuffles);
-//   warps 11-14 (calls with few tokens per expert) the epilogue of groups up to 160 tokens, two of which have
-//             accumulators at a time, while the others go on with the next unit;
+//   warps 11-14 (EXACT, see the kernel) scales and epilogue, while the others go on with the next unit;
 //   warp 1    one thread issues tcgen05.mma (M128, N = the group's tokens rounded up to 16, in two halves
 //             beyond 256, K16, fp16 x fp16 -> fp32) per 16 inputs and commits each stage back.
 // A step costs two cycles per token in the tensor pipe and some 450 in the dequantisation, so groups of
@@ -61,13 +60,15 @@ constexpr int UM_B_STAGE_BYTES = UM_GROUP_TOK * 128;
 constexpr int UM_OUT_BYTES = 32 * 128 * 2;  // hidden values of a set on their way out: 32 tokens x 128 channels (gated: two turns of 64)
 constexpr int UM_SMEM_BYTES = UM_RAW_STAGES * UM_TILE_BYTES + UM_STAGES * UM_B_STAGE_BYTES + 2 * UM_OUT_BYTES + 1024;  // 224 KB + alignment slack
 constexpr int UM_A_COLS = UM_BK / 2;       // one A stage: 64 fp16 inputs = 32 columns, behind the accumulators
-constexpr int UM_TWO_TOK = UM_GROUP_TOK / 2;  // groups up to this size: accumulators of two units in turn
-constexpr int UM_CAPS = 4;                 // limits of a group that are considered
-__host__ __device__ __forceinline__ constexpr int um_cap(int c) { return c == 0 ? 96 : (c == 1 ? 160 : (c == 2 ? 256 : 320)); }
+constexpr int UM_EXACT_TOK = 64;           // EXACT: tokens of a group, at most
+constexpr int UM_SETS = 4;                 // EXACT: sets of accumulators (two instead: 3 % more time)
+constexpr int UM_CAPS = 4;                 // limits of a group that are considered: 128, 192, 256, 320 tokens
+template <bool EXACT>
+__host__ __device__ __forceinline__ constexpr int um_cap(int c) { return EXACT ? UM_EXACT_TOK : 128 + 64 * c; }
 constexpr int UM_UNPACK_WARPS = 8;         // two sets of four
 constexpr int UM_RAW_WARP = 2 + UM_UNPACK_WARPS;
-constexpr int UM_STORE_WARPS = 4;           // epilogue of small groups
-constexpr int um_threads(bool store_warps) { return (3 + UM_UNPACK_WARPS + (store_warps ? UM_STORE_WARPS : 0)) * 32; }
+constexpr int UM_SCALE_WARPS = 4;           // EXACT: scales and epilogue
+constexpr int um_threads(bool exact) { return (3 + UM_UNPACK_WARPS + (exact ? UM_SCALE_WARPS : 0)) * 32; }
 constexpr int UM_TMEM_COLS = 512;
 
 // a / (1 + exp(-a)) without a branch, so that the 16 columns of a thread overlap (the operator's slow path
@@ -197,6 +198,7 @@ struct UmmaArgs {
   float* o;                  // second projection's output [n_pairs][d_model]
   int zmax;                  // second projection: most slices of the inputs per unit (slice z into plane z of o)
   int n_pairs;
+  bool maybe_empty;          // the plan may well hold nobody
   size_t plane_stride;       // floats between the planes of o
   int* check_word;
 };
@@ -246,10 +248,10 @@ struct TileWalk {
 
 // How a launch is cut (one warp): most tokens of a group, slices of the second projection's inputs.  Larger groups share
 // the dequantisation, smaller ones and slices fill the last round of CTAs.  The estimate, in cycles: a
-// step of 64 inputs takes two per token or the 500 an MMA with A in tensor memory takes at least; storing a unit 30
-// per token with eight warps, behind its last MMA, or 60 with the four that do nothing else, beside the next unit; a further
-// plane of sums costs the combine step its bandwidth (3400 B per cycle).
-__device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, int row_blocks, int kb_total, int lane, bool store_warps) {
+// step of 64 inputs takes two per token or the 450 of the dequantisation (EXACT: 700 for the sums), a unit 1500 + 12
+// per token to start and store; a further plane of sums costs the combine step its bandwidth (3400 B per cycle).
+template <bool EXACT>
+__device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, int row_blocks, int kb_total, int lane) {
   const int n_active = *reinterpret_cast<const volatile int*>(a.plan);
   const PlanRec* recs = reinterpret_cast<const PlanRec*>(reinterpret_cast<const char*>(a.plan) + PLAN_HEADER_BYTES);
   int groups[UM_CAPS] = {}, tokens = 0;
@@ -257,24 +259,24 @@ __device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, int row_blocks, in
     const int cnt = recs[i].cnt;
     tokens += cnt;
 #pragma unroll
-    for (int c = 0; c < UM_CAPS; ++c) groups[c] += (cnt + um_cap(c) - 1) / um_cap(c);
+    for (int c = 0; c < UM_CAPS; ++c) groups[c] += (cnt + um_cap<EXACT>(c) - 1) / um_cap<EXACT>(c);
   }
   tokens = __reduce_add_sync(0xffffffffu, tokens);
-  int2 best = make_int2(um_cap(0), 1);
+  int2 best = make_int2(um_cap<EXACT>(0), 1);
   float best_cost = 3.0e38f;
 #pragma unroll
-  for (int c = 0; c < UM_CAPS; ++c) {
+  for (int c = 0; c < (EXACT ? 1 : UM_CAPS); ++c) {
     const int g = __reduce_add_sync(0xffffffffu, groups[c]);
     const float tok = static_cast<float>(tokens) / static_cast<float>(max(g, 1));
     for (int z = 1; z <= a.zmax; z *= 2) {
       if (z > 1 && (kb_total % z != 0 || kb_total / z % 8 != 0)) break;  // a slice starts on a packed box at every width
       const int rounds = (g * row_blocks * z + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
-      const float steps = static_cast<float>(kb_total / z) * fmaxf(500.0f, 2.0f * tok);
-      const float unit = store_warps && um_cap(c) <= UM_TWO_TOK ? fmaxf(steps + 500.0f, 60.0f * tok) : steps + 3000.0f + 30.0f * tok;
+      const float steps = static_cast<float>(kb_total / z) * fmaxf(EXACT ? 700.0f : 450.0f, 2.0f * tok);
+      const float unit = EXACT ? steps + 1000.0f : steps + 1500.0f + 12.0f * tok;
       const float cost = static_cast<float>(rounds) * unit + static_cast<float>(z - 1) * static_cast<float>(tokens) * static_cast<float>(a.L.d_model) * (8.0f / 3400.0f);
       if (cost < best_cost) {
         best_cost = cost;
-        best = make_int2(um_cap(c), z);
+        best = make_int2(um_cap<EXACT>(c), z);
       }
     }
   }
@@ -285,13 +287,15 @@ __device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, int row_blocks, in
 struct RingPos {
   int raw_it, ab_it;
 };
-// The accumulators of a CTA's n-th unit: where the groups are small enough, two units in turn have columns of their own.
+// The accumulators of a CTA's n-th run of MMAs: a unit, or (EXACT) one scale group of a unit, UM_SETS of which have columns of
+// their own in turn.
+template <bool EXACT>
 struct AccSlot {
   int index, parity, col;
-  __device__ __forceinline__ AccSlot(int n, bool two) {
-    index = two ? n & 1 : 0;
-    parity = two ? (n >> 1) & 1 : n & 1;
-    col = index * UM_TWO_TOK;
+  __device__ __forceinline__ explicit AccSlot(int n) {
+    index = EXACT ? n % UM_SETS : 0;
+    parity = EXACT ? (n / UM_SETS) & 1 : n & 1;
+    col = index * UM_EXACT_TOK;
   }
 };
 struct UmBars {
@@ -300,7 +304,7 @@ struct UmBars {
 
 // One unit's steps by a dequantisation warp of set `part` (steps part, part + 2, ... of every box; boxes hold an even
 // number of steps).  srow: the row's scales from the unit's first step on, spg steps per scale.
-template <int BITS>
+template <int BITS, bool EXACT>
 __device__ __forceinline__ bool dequant_unit(const UmmaArgs& a, const UmBars& b, const unsigned char* raw_ring, uint32_t a_col, const void* sp,
                                              size_t srow, int ngroups, int spg, int kb0, int kb_len, int part, int box, int rin, int lane, RingPos& pos,
                                              volatile int* abort_flag) {
@@ -309,8 +313,11 @@ __device__ __forceinline__ bool dequant_unit(const UmmaArgs& a, const UmBars& b,
   // scales of this set's step, its next one and the one after: a load has two steps to come back from L2; the group
   // index of the step two ahead is kept by counting
   const int first = kb0 + part;
-  float sv = load_scale_ro(sp, sf16, srow + min(first / spg, ngroups - 1)), sv_n1 = load_scale_ro(sp, sf16, srow + min((first + 2) / spg, ngroups - 1)),
-        sv_n2;
+  float sv = 1.0f, sv_n1 = 1.0f, sv_n2 = 1.0f;  // EXACT: the codes alone, whole numbers
+  if (!EXACT) {
+    sv = load_scale_ro(sp, sf16, srow + min(first / spg, ngroups - 1));
+    sv_n1 = load_scale_ro(sp, sf16, srow + min((first + 2) / spg, ngroups - 1));
+  }
   int g2 = (first + 4) / spg, c2 = (first + 4) % spg;
   bool tiny_scale = false;  // q * s below the smallest normal fp16 number would lose bits in the fp16 operand
   for (int kb = 0; kb < kb_len; kb += KBS) {
@@ -321,11 +328,13 @@ __device__ __forceinline__ bool dequant_unit(const UmmaArgs& a, const UmBars& b,
 #pragma unroll 1
     for (int j = part; j < steps; j += 2) {
       const int it = pos.ab_it + j, s = it % UM_STAGES;
-      sv_n2 = load_scale_ro(sp, sf16, srow + min(g2, ngroups - 1));
-      c2 += 2;
-      if (c2 >= spg) {
-        c2 -= spg;
-        ++g2;
+      if (!EXACT) {
+        sv_n2 = load_scale_ro(sp, sf16, srow + min(g2, ngroups - 1));
+        c2 += 2;
+        if (c2 >= spg) {
+          c2 -= spg;
+          ++g2;
+        }
       }
       tiny_scale |= sv != 0.0f && fabsf(sv) < 6.104e-5f;
       const uint32_t s2 = static_cast<uint32_t>(__half_as_ushort(__float2half_rn(sv))) * 0x00010001u;
@@ -350,15 +359,16 @@ __device__ __forceinline__ bool dequant_unit(const UmmaArgs& a, const UmBars& b,
   return true;
 }
 
-// STORE: with the warps that store small groups.  Calls whose experts hold 192 tokens and more on average, and calls that
-// leave only their fullest experts to this kernel, go without: their groups seldom fit two sets of
-// accumulators, and fewer warps may keep more registers (1 to 2 % of the time).  Where they fit, 777 tokens on 32
-// experts of 768 x 3072 take 3 %, 2048 on 128 of 1024 x 4096 6 % less with them.
-template <bool STORE>
-__global__ void __launch_bounds__(um_threads(STORE), 1)
+// EXACT: for calls whose experts the streaming kernel would otherwise serve.  A holds the codes themselves, whole numbers
+// that fp16 holds exactly; four more warps take the sums of each scale group out of tensor memory and add them, times
+// the row's scale, in fp32 registers, as the streaming kernel does.  Groups of up to 64 tokens (their sums
+// fit the registers), four sets of accumulators in turn.  768 x 3072, 32 experts, 2048 tokens: 144 us per layer (streaming
+// 192, rounded 106); the four warps' reads of tensor memory are what bounds it.
+template <bool EXACT>
+__global__ void __launch_bounds__(um_threads(EXACT), 1)
     ffn_umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap tmap_b) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * UM_RAW_STAGES + 2 * UM_STAGES + 4];
+  __shared__ __align__(8) uint64_t bars[2 * UM_RAW_STAGES + 2 * UM_STAGES + 2 * UM_SETS];
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_word;
   __shared__ int2 cut_slot;
@@ -368,13 +378,18 @@ __global__ void __launch_bounds__(um_threads(STORE), 1)
   unsigned char* b_ring = raw_ring + UM_RAW_STAGES * UM_TILE_BYTES;
   const int lane = threadIdx.x & 31, warp = uniform_warp();
 
+  if (a.maybe_empty) {  // nobody is full enough, the common case of an even load: gone before anything is set up
+    pdl_trigger();  // (the kernel behind waits for this one's end, and with it for the one in front)
+    pdl_wait();
+    if (*reinterpret_cast<const volatile int*>(a.plan) == 0) return;
+  }
   UmBars b;
   b.raw_full = smem_u32(bars);
   b.raw_empty = b.raw_full + 8 * UM_RAW_STAGES;
   b.ab_full = b.raw_empty + 8 * UM_RAW_STAGES;
   b.ab_empty = b.ab_full + 8 * UM_STAGES;
   b.acc_full = b.ab_empty + 8 * UM_STAGES;
-  b.acc_empty = b.acc_full + 16;
+  b.acc_empty = b.acc_full + 8 * UM_SETS;
 
   if (threadIdx.x == 0) {
     abort_word = 0;
@@ -406,12 +421,12 @@ __global__ void __launch_bounds__(um_threads(STORE), 1)
 
   TileWalk walk;
   if (warp == 0) {
-    const int2 c = choose_cut(a, row_blocks, kb_total, lane, STORE);
+    const int2 c = choose_cut<EXACT>(a, row_blocks, kb_total, lane);
     if (lane == 0) {
       cut_slot = c;
-      for (int i = 0; i < 2; ++i) {
+      for (int i = 0; i < UM_SETS; ++i) {
         mbar_init(b.acc_full + 8 * i, 1);
-        mbar_init(b.acc_empty + 8 * i, STORE && c.x <= UM_TWO_TOK ? UM_STORE_WARPS : UM_UNPACK_WARPS);
+        mbar_init(b.acc_empty + 8 * i, EXACT ? UM_SCALE_WARPS : UM_UNPACK_WARPS);
       }
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       if (a.phase == 1 && blockIdx.x == 0) a.plan[3] = c.y;  // for the combine step
@@ -419,7 +434,7 @@ __global__ void __launch_bounds__(um_threads(STORE), 1)
   }
   __syncthreads();
   const int2 cut = cut_slot;
-  const bool two = STORE && cut.x <= UM_TWO_TOK;
+  const int spg = (L.group > 0 ? L.group : K) / UM_BK;  // steps per scale: a group is a multiple of 128 inputs, or the whole row
   const int kb_len = kb_total / cut.y;  // steps of a unit
   walk.init(a.plan, row_blocks, cut);
   int tok_first, ntok, rb, z;
@@ -488,18 +503,30 @@ __global__ void __launch_bounds__(um_threads(STORE), 1)
     // rounded up to 16, in two halves where they are more than one MMA takes
     const uint32_t on = elect_one();
     const uint32_t idesc = (1u << 4) | ((UM_ROWS >> 4) << 24);
-    int ab_it = 0, unit_it = 0;
+    int ab_it = 0, run_it = 0;
     bool ok = true;
     while (ok && walk.next(tok_first, ntok, rb, z)) {
       const int cols = (ntok + 15) & ~15;
       const int n1 = cols <= 256 ? cols : ((cols / 2 + 15) & ~15), n2 = cols - n1;
       const uint32_t id1 = idesc | ((n1 >> 3) << 17), id2 = idesc | ((n2 >> 3) << 17);
       const uint32_t on1 = n1 > 0 ? on : 0u, on2 = n2 > 0 ? on : 0u;
-      const AccSlot acc(unit_it, two);
-      const uint32_t d_t = tmem_base + acc.col;
-      if (!mbar_wait_warp(b.acc_empty + 8 * acc.index, acc.parity ^ 1, a.check_word, abort_flag)) break;
-      tc_fence_after();
+      bool fresh = true;  // EXACT: the accumulators start anew
+      uint32_t d_t = tmem_base;
+      if (!EXACT) {
+        if (!mbar_wait_warp(b.acc_empty, (run_it & 1) ^ 1, a.check_word, abort_flag)) break;
+        tc_fence_after();
+      }
+      int run_left = EXACT ? spg - z * kb_len % spg : 0;  // steps to the end of the scale group
       for (int kb = 0; kb < kb_len; ++kb, ++ab_it) {
+        if (EXACT && fresh) {
+          const AccSlot<EXACT> acc(run_it);
+          d_t = tmem_base + acc.col;
+          if (!mbar_wait_warp(b.acc_empty + 8 * acc.index, acc.parity ^ 1, a.check_word, abort_flag)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+        }
         const int s = ab_it % UM_STAGES;
         if (!mbar_wait_warp(b.ab_full + 8 * s, (ab_it / UM_STAGES) & 1, a.check_word, abort_flag)) {
           ok = false;
@@ -511,28 +538,33 @@ __global__ void __launch_bounds__(um_threads(STORE), 1)
         const uint64_t db1 = umma_desc(bs);
 #pragma unroll
         for (int k4 = 0; k4 < UM_BK / 16; ++k4)  // 16 inputs: 8 columns of A, 32 bytes (2 descriptor units) of B
-          umma_f16_ts_if(on1, d_t, a_t + 8 * k4, db1 + 2 * k4, id1, (kb > 0 || k4 > 0) ? 1u : 0u);
-        if (n2 > 0) {
+          umma_f16_ts_if(on1, d_t, a_t + 8 * k4, db1 + 2 * k4, id1, ((EXACT ? !fresh : kb > 0) || k4 > 0) ? 1u : 0u);
+        if (!EXACT && n2 > 0) {
           const uint64_t db2 = umma_desc(bs + n1 * 128);
 #pragma unroll
           for (int k4 = 0; k4 < UM_BK / 16; ++k4)
-            umma_f16_ts_if(on2, d_t + n1, a_t + 8 * k4, db2 + 2 * k4, id2, (kb > 0 || k4 > 0) ? 1u : 0u);
+            umma_f16_ts_if(on2, d_t + n1, a_t + 8 * k4, db2 + 2 * k4, id2, ((EXACT ? !fresh : kb > 0) || k4 > 0) ? 1u : 0u);
         }
         umma_commit_if(on, b.ab_empty + 8 * s);  // the stage may be refilled once these MMAs have read it
+        fresh = EXACT && (kb + 1 == kb_len || --run_left == 0);
+        if (EXACT && fresh) {
+          umma_commit_if(on, b.acc_full + 8 * AccSlot<EXACT>(run_it).index);
+          ++run_it;
+          run_left = spg;
+        }
       }
-      if (ok) umma_commit_if(on, b.acc_full + 8 * acc.index);
-      ++unit_it;
+      if (!EXACT) {
+        if (ok) umma_commit_if(on, b.acc_full);
+        ++run_it;
+      }
     }
   } else {
     // ---------------- dequantise (a thread per weight row) and epilogue ----------------
-    // Groups too large for two sets of accumulators: the dequantising warps store a unit before they go on, eight warps
-    // being faster at it and nothing to overlap it with.  Otherwise the last four warps do, and the others go on.
     const int quarter = warp & 3;          // TMEM lanes this warp may access: 32 * quarter ...
-    const int part = STORE && warp > UM_RAW_WARP ? 2 : (warp - 2) >> 2;  // the set: even or odd steps, or the storing warps
-    const int first_chunk = two ? 0 : 32 * part, chunk_step = two ? 32 : 64;
+    const int part = EXACT && warp > UM_RAW_WARP ? 2 : (warp - 2) >> 2;  // the set: even or odd steps, and 32-token chunks of the epilogue; 2: scales
     const int r = 32 * quarter + lane;     // row of the tile = row of the operand = TMEM lane
     const int G = L.group > 0 ? L.group : K;
-    const int ngroups = K / G, spg = G / UM_BK;  // G is a multiple of 128, or the whole row
+    const int ngroups = K / G;
     const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(32 * quarter) << 16);
     // gated: the upper 16 lanes of a warp hold the w3 rows that belong to the w1 rows of the lower 16
     const bool second = gated && lane >= 16;
@@ -541,7 +573,7 @@ __global__ void __launch_bounds__(um_threads(STORE), 1)
     const int set_tid = 32 * quarter + lane;
     int turn = 0;  // gated: the half of the buffer
     RingPos pos = {0, 0};
-    int unit_it = 0;
+    int run_it = 0;
     while (walk.next(tok_first, ntok, rb, z)) {
       const PlanRec& rec = walk.rec;
       const int bits = rec.bits;
@@ -554,29 +586,57 @@ __global__ void __launch_bounds__(um_threads(STORE), 1)
       bool ok = true;
       if (part < 2) {
         switch (bits) {
-          case 2: ok = dequant_unit<2>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
-          case 4: ok = dequant_unit<4>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
-          default: ok = dequant_unit<8>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
+          case 2: ok = dequant_unit<2, EXACT>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
+          case 4: ok = dequant_unit<4, EXACT>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
+          default: ok = dequant_unit<8, EXACT>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
         }
       }
       if (!ok) break;
-      if (two != (part == 2)) {
-        ++unit_it;
-        continue;
+      if (EXACT && part < 2) continue;
+      // ---- epilogue: this warp's 32 rows x every other 32 token columns (EXACT: all of them) ----
+      uint32_t tot[EXACT ? 2 : 1][32];  // EXACT: the scaled sums
+      int acc_index = 0;
+      if constexpr (EXACT) {
+        float* f = reinterpret_cast<float*>(tot);
+#pragma unroll
+        for (int c = 0; c < 64; ++c) f[c] = 0.0f;
+        const bool sf16 = L.scale_f16 != 0;
+        int gi = kb0 / spg;
+        float sv = load_scale_ro(sp, sf16, srow + min(gi, ngroups - 1));
+        for (int kb = kb0; kb < kb0 + kb_len; kb = (kb / spg + 1) * spg, ++run_it) {
+          const float sv_next = load_scale_ro(sp, sf16, srow + min(++gi, ngroups - 1));
+          const AccSlot<EXACT> acc(run_it);
+          if (!mbar_wait_warp(b.acc_full + 8 * acc.index, acc.parity, a.check_word, abort_flag)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            if (16 * h < ntok) {
+              uint32_t va[16];
+              tmem_ld16(lane_base + acc.col + 16 * h, va);
+              tmem_ld_wait();
+#pragma unroll
+              for (int c = 0; c < 16; ++c) f[16 * h + c] = fmaf(sv, __uint_as_float(va[c]), f[16 * h + c]);
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(b.acc_empty + 8 * acc.index);
+          sv = sv_next;
+        }
+        if (!ok) break;
+      } else {
+        const AccSlot<EXACT> acc(run_it);
+        acc_index = acc.index;
+        if (!mbar_wait_warp(b.acc_full + 8 * acc.index, acc.parity, a.check_word, abort_flag)) break;
+        tc_fence_after();
       }
-      // ---- epilogue: this warp's 32 rows x (every other) 32 token columns ----
-      const AccSlot acc(unit_it, two);
-      if (!mbar_wait_warp(b.acc_full + 8 * acc.index, acc.parity, a.check_word, abort_flag)) break;
-      tc_fence_after();
       const size_t slot0 = static_cast<size_t>(rec.begin) + static_cast<size_t>(tok_first);
       const int u_row0 = rb * (gated ? 64 : UM_ROWS);  // first channel of the unit
       const int hpos = a.phase == 0 ? pair_pos_rt(bits, nrow) : 0;  // (moves a channel inside its 16)
-#pragma unroll 1
-      for (int cc = first_chunk; cc < ntok; cc += chunk_step) {
-        uint32_t va[32];
-        __syncwarp();
-        tmem_ld32(lane_base + acc.col + cc, va);
-        tmem_ld_wait();
+      auto store_chunk = [&](int cc, uint32_t(&va)[32]) {
         const int live = min(32, ntok - cc);  // token columns of this chunk that exist
         // one compact unrolled loop per case (the conditions are uniform)
         if (gated) {
@@ -633,11 +693,26 @@ __global__ void __launch_bounds__(um_threads(STORE), 1)
           }
           asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");  // the buffer has been read
         }
+      };
+      if constexpr (EXACT) {
+        store_chunk(0, tot[0]);
+        if (ntok > 32) store_chunk(32, tot[1]);
+      } else {
+#pragma unroll 1
+        for (int cc = 32 * part; cc < ntok; cc += 64) {
+          uint32_t va[32];
+          __syncwarp();
+          tmem_ld32(lane_base + cc, va);
+          tmem_ld_wait();
+          store_chunk(cc, va);
+        }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(b.acc_empty + 8 * acc.index);
-      ++unit_it;
+      if (!EXACT) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(b.acc_empty + 8 * acc_index);
+        ++run_it;
+      }
     }
   }
 
@@ -660,7 +735,7 @@ bool ffn_umma_supported(const LayerDims& L) {
 }
 
 cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, int* plan, const void* in16, int in_stride,
-                            void* hidden16, int hid_stride, float* o, int n_pairs, int zmax, bool all_experts, int* check_word,
+                            void* hidden16, int hid_stride, float* o, int n_pairs, int zmax, bool exact, bool maybe_empty, int* check_word,
                             cudaStream_t st) {
   const int N = phase == 0 ? L.d_ff : L.d_model;
   const int K = phase == 0 ? L.d_model : L.d_ff;
@@ -684,7 +759,7 @@ cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, in
   const bool gated = phase == 0 && L.act == EMOE_ACT_SWIGLU;
   const long long row_blocks = gated ? N / (UM_ROWS / 2) : (N + UM_ROWS - 1) / UM_ROWS;
   // upper bound of the tile count: every pair alone in a token tile
-  long long tiles = row_blocks * (static_cast<long long>(n_pairs < L.E ? n_pairs : L.E) + n_pairs / um_cap(0)) * (phase == 1 && zmax > 1 ? zmax : 1);
+  long long tiles = row_blocks * (static_cast<long long>(n_pairs < L.E ? n_pairs : L.E) + n_pairs / (exact ? UM_EXACT_TOK : 128)) * (phase == 1 && zmax > 1 ? zmax : 1);
   const int grid = static_cast<int>(tiles < sms_of_device[dev] ? tiles : sms_of_device[dev]);
   UmmaArgs a;
   a.phase = phase;
@@ -696,9 +771,10 @@ cudaError_t launch_ffn_umma(int phase, const LayerDims& L, const void* wmaps, in
   a.o = o;
   a.zmax = phase == 0 || zmax < 1 ? 1 : zmax;
   a.n_pairs = n_pairs;
+  a.maybe_empty = maybe_empty;
   a.plane_stride = static_cast<size_t>(n_pairs) * L.d_model;
   a.check_word = check_word;
-  if (all_experts && n_pairs < 192LL * L.E) return launch_chain(ffn_umma_kernel<true>, dim3(grid), dim3(um_threads(true)), UM_SMEM_BYTES, st, a, tmap_b);
+  if (exact) return launch_chain(ffn_umma_kernel<true>, dim3(grid), dim3(um_threads(true)), UM_SMEM_BYTES, st, a, tmap_b);
   return launch_chain(ffn_umma_kernel<false>, dim3(grid), dim3(um_threads(false)), UM_SMEM_BYTES, st, a, tmap_b);
 }
 
