@@ -233,7 +233,7 @@ int emoe_moe_forward_routed(emoe_ctx* ctx, const emoe_layer_desc* desc, const vo
  * kernel with the TMA-staged weight pipeline (what 0 picks for decode batches), 4 = the tcgen05
  * grouped GEMM (fp16 operands; meant for many tokens per expert), 5 = 3 and 4 in one call: experts
  * with at most 32 tokens take the streaming kernel, the others the grouped GEMM (what 0 picks for
- * large batches), 6 = the weight-streaming kernel on 8-bit integer tcgen05 operands with block-scaled
+ * large batches; where those had the streaming kernel before, the grouped GEMM on exact codes), 6 = the weight-streaming kernel on 8-bit integer tcgen05 operands with block-scaled
  * integer activations (no fp16 range limit; at present slower than 3).
  * 2 to 6 fail with EMOE_ERR_UNSUPPORTED in forward calls whose shape they do not take.  For tests
  * and measurements. */

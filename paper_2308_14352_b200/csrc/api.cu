@@ -382,13 +382,13 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   // more than HYBRID_STREAM_TOKENS tokens, the others stream; from 256 for all (next to nobody would be left to stream).
   const double mean_tokens = static_cast<double>(P) / L.E;
   const bool rounded = mean_tokens >= 16.0 && L.d_model % 512 == 0 && L.d_ff % 512 == 0;
-  // Exact: elsewhere, from 192 (token, expert) pairs.  An uneven load can then fill an expert well beyond the 16 tokens that
+  // Exact: elsewhere, from 256 (token, expert) pairs.  An uneven load can then fill an expert well beyond the 16 tokens that
   // the streaming kernel takes per pass over the weights; an even one pays some 5 us for two launches that find
   // nobody.  From 32 tokens per expert on average for all of them; below, for experts beyond 32 tokens, 48 where even
   // loads reach 32 as well.  us per layer, streaming alone / both, even and skewed (Zipf exponent 1.1) loads:
   // 768 x 3072, 32 experts, 256 tokens 53/58 and 88/78, 512 tokens 77/81 and 138/103; 1024 x 4096, 128 experts, 1024 tokens 220/226
   // and 477/179; 1280 x 4480, 64 experts, 800 tokens 209/218 and 373/197; 2048 tokens on the first, all 192/144 and 510/165.
-  const bool exact_pairs = !rounded && P >= 192;
+  const bool exact_pairs = !rounded && P >= 256;
   const bool one_family = mean_tokens >= (rounded ? 256.0 : 32.0);
   const bool auto_umma = ctx->ffn_path == 0 && (rounded || exact_pairs);
   const bool exact_umma = ctx->ffn_path == 0 && !rounded;

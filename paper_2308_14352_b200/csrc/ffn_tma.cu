@@ -821,6 +821,12 @@ int ffn_tma_ksplit(const LayerDims& L, int T) {
   const int cap = ctas * 4 <= 148 ? steps_max : steps_min;
   if (z > cap) z = cap;
   if (z > 16) z = 16;
+  // ... but not so fine that the items of both projections outnumber the resident CTAs where coarser slices would not: a
+  // second item is a second chain of steps (12 tokens, 8 experts, 512 x 1152: 25 us per layer with nine slices, 21 with
+  // seven; 24 tokens on 512 x 2048 28 and 22)
+  const int rows0 = L.act == EMOE_ACT_SWIGLU ? ST_BOX_ROWS : 2 * ST_BOX_ROWS;
+  const long long room = (ST_CTAS * 148 - active * ((L.d_ff + rows0 - 1) / rows0)) / ctas;
+  if (z > room && room >= 2) z = room;
   if (z < 1) z = 1;
   return static_cast<int>(z);
 }

@@ -486,17 +486,17 @@ def test_forward_tcgen05_path_at_the_edges_of_its_groups(act, group, sdt, d, f, 
 
 
 EXACT_CASES = [
-    # what the default takes on tcgen05 with exact codes: 192 pairs and more, rows that are not multiples of 512 or few
+    # what the default takes on tcgen05 with exact codes: 256 pairs and more, rows that are not multiples of 512 or few
     # tokens on average; router bias exponent (0: none)
-    ("relu", 128, "f16", 640, 768, 3, 1, "softmax", [4, 2, 8], 192, 0.0),              # 64 each, partly filled boxes
-    ("relu", 128, "f16", 640, 512, 1, 1, "softmax", [2], 193, 0.0),                     # groups of 49 tokens
-    ("relu", 0, "f32", 640, 1152, 1, 1, "softmax", [4], 225, 0.0),                      # per-channel scales
-    ("swiglu", 256, "f16", 768, 1280, 4, 2, "softmax_renorm", [4, 8, 2, 4], 161, 0.0),  # four steps per scale
-    ("swiglu", 128, "f32", 640, 1664, 2, 2, "softmax_renorm", [8, 4], 129, 0.0),
-    ("relu", 128, "f16", 512, 6272, 4, 1, "softmax", [4, 2, 8, 4], 210, 0.0),           # several units per CTA
-    ("relu", 128, "f16", 512, 1024, 24, 1, "softmax", [8, 4, 2, 4] * 6, 230, 1.1),      # beside the streaming kernel
-    ("swiglu", 128, "f16", 640, 640, 12, 2, "softmax_renorm", [4, 8, 2, 4] * 3, 120, 1.1),
-    ("relu", 128, "f16", 512, 512, 16, 1, "softmax", [4] * 16, 200, 0.0),               # nobody full enough
+    ("relu", 128, "f16", 640, 768, 3, 1, "softmax", [4, 2, 8], 257, 0.0),              # 64 to 128 each, partly filled boxes
+    ("relu", 128, "f16", 640, 512, 1, 1, "softmax", [2], 257, 0.0),                     # five groups of 52 tokens
+    ("relu", 0, "f32", 640, 1152, 1, 1, "softmax", [4], 256, 0.0),                      # per-channel scales
+    ("swiglu", 256, "f16", 768, 1280, 4, 2, "softmax_renorm", [4, 8, 2, 4], 140, 0.0),  # four steps per scale
+    ("swiglu", 128, "f32", 640, 1664, 2, 2, "softmax_renorm", [8, 4], 128, 0.0),
+    ("relu", 128, "f16", 512, 6272, 4, 1, "softmax", [4, 2, 8, 4], 270, 0.0),           # several units per CTA
+    ("relu", 128, "f16", 512, 1024, 24, 1, "softmax", [8, 4, 2, 4] * 6, 300, 1.1),      # beside the streaming kernel
+    ("swiglu", 128, "f16", 640, 640, 12, 2, "softmax_renorm", [4, 8, 2, 4] * 3, 140, 1.1),
+    ("relu", 128, "f16", 512, 512, 16, 1, "softmax", [4] * 16, 256, 0.0),               # nobody full enough
 ]
 
 
