@@ -117,6 +117,24 @@ def test_forward_tma_pipeline_path(act, group, sdt, d, f, E, k, gate, bits, T):
     assert np.array_equal(y_fused, y_split)
 
 
+TMA_EDGE_CASES = [
+    # slices of the second projection limited by the resident CTAs; tokens of an expert at the limits of a pass (8, 16)
+    ("relu", 0, "f16", 512, 1152, 8, 1, "softmax", [4, 2, 8, 4] * 2, 12),
+    ("relu", 128, "f16", 512, 2048, 8, 1, "softmax", [4, 2, 8, 4] * 2, 24),
+    ("swiglu", 128, "f16", 512, 1536, 8, 2, "softmax_renorm", [4, 8, 2, 4] * 2, 12),
+    ("relu", 128, "f16", 512, 640, 1, 1, "softmax", [4], 8),
+    ("relu", 128, "f16", 512, 640, 1, 1, "softmax", [2], 9),
+    ("swiglu", 128, "f32", 512, 640, 1, 1, "softmax", [8], 16),
+    ("relu", 128, "f16", 512, 640, 1, 1, "softmax", [4], 17),
+]
+
+
+@pytest.mark.parametrize("act,group,sdt,d,f,E,k,gate,bits,T", TMA_EDGE_CASES)
+def test_forward_tma_pipeline_path_at_the_edges_of_its_passes(act, group, sdt, d, f, E, k, gate, bits, T):
+    shape = inputs.LayerShape(d, f, E, k, act, gate, group, sdt, "bf16")
+    _run_case(shape, bits, T, seed=37, path=3)
+
+
 I8_CASES = TMA_CASES + [
     ("relu", 128, "f16", 768, 3072, 32, 1, "softmax", [2, 4, 8, 4] * 8, 64),                # many experts, 2 tokens each
     ("swiglu", 128, "f16", 512, 1024, 8, 2, "softmax_renorm", [8, 8, 4, 4, 2, 2, 4, 8], 4),
