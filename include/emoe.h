@@ -215,6 +215,8 @@ int emoe_permute(emoe_ctx* ctx, const int32_t* ids, int n_pairs, int E, int32_t*
  * GEMM loses bits: both set a flag that emoe_device_status reports as EMOE_ERR_RANGE, and y is then
  * not within the usual bound of the definition.  Kernel family 6 (emoe_set_ffn_path) and the
  * CUDA-core family 1 have no such limit: they follow the full bf16 exponent range.
+ * Order on the GPU: x, router_bias and (given) ids and gates may be written by whatever stands in front
+ * on `stream`, another layer's call among it (layers chain through one stream), as may the weights.
  * Shape limits: d_model and d_ff multiples of 32 with K*bits/8 a multiple of 16 for every
  * matrix; group 0 or a multiple of 32 (INT8), 32 (INT4), 64 (INT2) dividing K.
  * Uses the context workspace (emoe_workspace_bytes). */
@@ -417,7 +419,7 @@ int emoe_cache_release(emoe_ctx* ctx, const int64_t* ids, int n, void* compute_s
  * Expert e of this layer is registered as first_id + e, of the next layer as next_first_id + e.
  * prior: host array as for emoe_rank_experts; ids / gates / y: device buffers as for
  * emoe_moe_forward; pinned_ids: [T][top_k] in pinned host memory, valid when the call returns.
- * Decisions, counters and results are those of the single calls. */
+ * Decisions, counters and results are those of the single calls; order on the GPU as for emoe_moe_forward. */
 int emoe_cached_layer(emoe_ctx* ctx, const emoe_layer_desc* desc, int layer, const void* x, int T, const float* router_W,
                       const float* router_bias, int bias_token_stride, int64_t first_id, const float* prior, int n_prefetch,
                       int64_t next_first_id, int32_t* ids, float* gates, float* y, int32_t* pinned_ids, void* compute_stream,

@@ -440,8 +440,8 @@ int emoe_cached_layer(emoe_ctx* ctx, const emoe_layer_desc* desc, int layer, con
   if (router_bias && bias_token_stride != 0 && bias_token_stride != E) return EMOE_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(compute_stream);
   cudaError_t err = cudaSetDevice(ctx_cache(ctx)->device);
-  // The router kernel forms its product while the layer in front drains, and writes the picks to host memory as well:
-  // they are there some microseconds before a synchronisation would say so.
+  // The router kernel starts while the layer in front drains, and writes the picks to host memory as well: they
+  // are there some microseconds before a synchronisation would say so.
   volatile int32_t* seen_ids = pinned_ids;
   for (int p = 0; p < T * k; ++p) seen_ids[p] = -1;
   g_pdl_enabled = ctx_dependent_launch(ctx);

@@ -46,10 +46,10 @@ struct LayerDims {
 // The kernels of a forward call form a chain on one stream.  When enabled (per host thread,
 // set by the forward call from its context), every launch carries the "programmatic stream
 // serialization" attribute: the next kernel of the chain may start its prologue (barrier set-up,
-// tensor-memory allocation, fetching weights that no kernel of the chain writes) while the
-// current one drains.  Device side, every kernel executes pdl_wait() before it touches anything
-// an earlier kernel of the chain wrote or read, and pdl_trigger() right after, which lets the
-// kernel behind it start.  Without the attribute both are no-ops.
+// tensor-memory allocation, prefetches into L2) while the
+// current one drains.  Device side, every kernel executes pdl_wait() before it reads or writes global memory: the inputs
+// of a call, too, may be what the call in front leaves.  pdl_trigger()
+// lets the kernel behind it start.  Without the attribute both are no-ops.
 extern thread_local bool g_pdl_enabled;
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

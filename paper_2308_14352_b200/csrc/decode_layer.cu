@@ -195,26 +195,32 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
       const int kb = static_cast<int>(static_cast<long long>(d) * r / RS), ke = static_cast<int>(static_cast<long long>(d) * (r + 1) / RS);
       const int e = tid & (EP - 1), part = tid >> a.ep_shift, S = DL_THREADS >> a.ep_shift;
       float acc = 0.0f;
-      if (e < L.E) {
-        constexpr int U = 8;  // independent loads in flight per thread
+      // as in the router kernel, nothing is read before the kernels in front are done
+      prefetch_l2(a.Wr + static_cast<size_t>(kb) * L.E, static_cast<size_t>(ke - kb) * L.E * 4, tid, DL_THREADS);
+      prefetch_l2(static_cast<const char*>(a.x) + (static_cast<size_t>(t) * d + kb) * xsz, (ke - kb) * xsz, tid, DL_THREADS);
+      pdl_wait();
+      const auto product = [&](const auto* xrow) {
+        constexpr int U = 16;  // independent loads in flight per thread: a slice of up to 128 inputs of 32 experts in one round trip
         for (int i = kb + part; i < ke; i += U * S) {
-          float w[U], xv[U];
+          float w[U];
+          std::decay_t<decltype(*xrow)> xv[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int ii = i + u * S;
-            const bool in = ii < ke;
-            w[u] = in ? __ldg(a.Wr + static_cast<size_t>(ii) * L.E + e) : 0.0f;
-            const size_t xi = static_cast<size_t>(t) * d + (in ? ii : kb);
-            xv[u] = bf16 ? __bfloat162float(__ldg(reinterpret_cast<const __nv_bfloat16*>(a.x) + xi))
-                         : __ldg(reinterpret_cast<const float*>(a.x) + xi);
+          for (int u = 0; u < U; ++u) {  // no branch and no conversion between the loads: they are to leave together
+            const int ii = min(i + u * S, ke - 1);
+            w[u] = __ldcg(a.Wr + static_cast<size_t>(ii) * L.E + e);
+            xv[u] = __ldcg(xrow + ii);
           }
 #pragma unroll
-          for (int u = 0; u < U; ++u) acc = fmaf(xv[u], w[u], acc);
+          for (int u = 0; u < U; ++u)
+            if (i + u * S < ke) acc = fmaf(static_cast<float>(xv[u]), w[u], acc);
         }
+      };
+      if (e < L.E) {
+        if (bf16) product(static_cast<const __nv_bfloat16*>(a.x) + static_cast<size_t>(t) * d);
+        else product(static_cast<const float*>(a.x) + static_cast<size_t>(t) * d);
       }
       s_red[part * EP + e] = acc;
       __syncthreads();
-      pdl_wait();  // the kernels in front may still read what is written from here on
       if (tid < EP) {
         float z = 0.0f;
         for (int sidx = 0; sidx < S; ++sidx) z += s_red[sidx * EP + tid];

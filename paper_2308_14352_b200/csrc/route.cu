@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(ROUTER_THREADS)
   // once the whole grid is resident: it cannot take the room of a CTA the wait below needs.
   pdl_trigger();
   const bool one = router_one_supported(E, Wr);  // as the router kernel does it, to the same bits
-  if (one) router_logits_one<ROUTER_THREADS, 4>(smem, x, 1, d, Wr, bias, bias_stride, E, ep_shift, nullptr);  // (both wait on the kernels in front)
+  if (one) router_logits_one<ROUTER_THREADS, 4>(smem, x, 1, d, Wr, bias, bias_stride, E, ep_shift, nullptr);  // (both wait for the kernels in front)
   else router_logits<1>(smem, x, 1, T, d, Wr, bias, bias_stride, E, EP, ep_shift, nullptr);
   // should this CTA's wait run out, the expert kernel behind must find an empty plan, not an old one
   if (t == 0 && tid == 0) plan[0] = 0;

@@ -4,6 +4,8 @@
 #pragma once
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace emoe {
@@ -13,9 +15,21 @@ constexpr int ROUTER_DC = 1024;  // d_model chunk held in shared memory (1 and 8
 // tokens per CTA -> chunk: 32 tokens take chunks of 256 so that their rows still fit shared memory
 __host__ __device__ constexpr int router_dc(int tt) { return tt > 8 ? 256 : ROUTER_DC; }
 
-// Logits of the CTA's TT tokens into zs[TT][EP] (shared memory).  x and the router weights are
-// inputs of the call: the logits are computed while the kernels in front drain; the wait on
-// them comes before the first write to global memory (ids / gates may still be read there).
+// The router comes first in a call, so the kernel in front of it may be the one that writes its inputs (the previous
+// layer, whose last kernel lets this one start before it has stored y): nothing is read before pdl_wait().  Until
+// then the lines are only pulled towards L2, which keeps no stale copy of them, by thread tid of nt.
+__device__ __forceinline__ void prefetch_l2(const void* from, size_t bytes, int tid, int nt) {
+  for (size_t b = 128 * static_cast<size_t>(tid); b < bytes; b += 128 * static_cast<size_t>(nt))
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char*>(from) + b));
+}
+// rows t0 .. t0 + rows - 1 of x, and this CTA's share of the router weights
+__device__ __forceinline__ void router_prefetch(const void* x, int x_bf16, int t0, int rows, int d, const float* Wr, int E, int tid, int nt) {
+  const size_t row_bytes = static_cast<size_t>(d) * (x_bf16 ? 2 : 4), w_bytes = static_cast<size_t>(d) * E * 4;
+  prefetch_l2(static_cast<const char*>(x) + t0 * row_bytes, rows * row_bytes, tid, nt);
+  prefetch_l2(Wr, w_bytes, static_cast<int>(blockIdx.x) * nt + tid, static_cast<int>(gridDim.x) * nt);
+}
+
+// Logits of the CTA's TT tokens into zs[TT][EP] (shared memory).
 template <int TT>
 __device__ __forceinline__ void router_logits(float* smem, const void* __restrict__ x, int x_bf16, int T, int d,
                                               const float* __restrict__ Wr, const float* __restrict__ bias,
@@ -34,6 +48,8 @@ __device__ __forceinline__ void router_logits(float* smem, const void* __restric
 #pragma unroll
   for (int tt = 0; tt < TT; ++tt) acc[tt] = 0.0f;
 
+  router_prefetch(x, x_bf16, t0, min(TT, T - t0), d, Wr, E, tid, ROUTER_THREADS);
+  pdl_wait();
   for (int c0 = 0; c0 < d; c0 += DC) {
     const int dc = min(DC, d - c0);
     __syncthreads();
@@ -59,7 +75,7 @@ __device__ __forceinline__ void router_logits(float* smem, const void* __restric
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int ii = i + u * S;
-          w[u] = ii < dc ? __ldg(Wr + static_cast<size_t>(c0 + ii) * E + e) : 0.0f;
+          w[u] = ii < dc ? __ldcg(Wr + static_cast<size_t>(c0 + ii) * E + e) : 0.0f;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -73,7 +89,6 @@ __device__ __forceinline__ void router_logits(float* smem, const void* __restric
 #pragma unroll
   for (int tt = 0; tt < TT; ++tt) red[(slice * TT + tt) * EP + e] = acc[tt];
   __syncthreads();
-  pdl_wait();
   for (int idx = tid; idx < TT * EP; idx += ROUTER_THREADS) {
     const int tt = idx >> ep_shift, ee = idx & (EP - 1);
     const int t = t0 + tt;
@@ -107,30 +122,36 @@ __device__ __forceinline__ void router_logits_one(float* smem, const void* __res
   float* red = smem + E;   // [rows][E]
   const int tid = threadIdx.x, t = blockIdx.x, sh = ep_shift - 2, quads = 1 << sh;
   const int n = d << sh;   // pieces
-  for (int vt = tid; vt < ROUTER_ONE_THREADS; vt += NT) {
+  router_prefetch(x, x_bf16, t, 1, d, Wr, E, tid, NT);
+  pdl_wait();
+  const auto product = [&](const auto* xrow, int vt) {
     float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     for (int base = vt; base < n; base += FLY * ROUTER_ONE_THREADS) {
       float4 w[FLY];
-      float v[FLY];
+      std::decay_t<decltype(*xrow)> v[FLY];
 #pragma unroll
-      for (int u = 0; u < FLY; ++u) {
+      for (int u = 0; u < FLY; ++u) {  // nothing is converted between the loads: they are to leave together
         const int i = base + u * ROUTER_ONE_THREADS;
-        w[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        v[u] = 0.0f;
         if (i < n) {
-          w[u] = __ldg(reinterpret_cast<const float4*>(Wr) + i);
-          const size_t src = static_cast<size_t>(t) * d + (i >> sh);
-          v[u] = x_bf16 ? __bfloat162float(__ldg(reinterpret_cast<const __nv_bfloat16*>(x) + src)) : __ldg(reinterpret_cast<const float*>(x) + src);
+          w[u] = __ldcg(reinterpret_cast<const float4*>(Wr) + i);
+          v[u] = __ldcg(xrow + (i >> sh));
         }
       }
 #pragma unroll
       for (int u = 0; u < FLY; ++u) {
-        acc.x = fmaf(v[u], w[u].x, acc.x);
-        acc.y = fmaf(v[u], w[u].y, acc.y);
-        acc.z = fmaf(v[u], w[u].z, acc.z);
-        acc.w = fmaf(v[u], w[u].w, acc.w);
+        if (base + u * ROUTER_ONE_THREADS >= n) break;
+        const float xv = static_cast<float>(v[u]);
+        acc.x = fmaf(xv, w[u].x, acc.x);
+        acc.y = fmaf(xv, w[u].y, acc.y);
+        acc.z = fmaf(xv, w[u].z, acc.z);
+        acc.w = fmaf(xv, w[u].w, acc.w);
       }
     }
+    return acc;
+  };
+  for (int vt = tid; vt < ROUTER_ONE_THREADS; vt += NT) {
+    float4 acc = x_bf16 ? product(static_cast<const __nv_bfloat16*>(x) + static_cast<size_t>(t) * d, vt)
+                        : product(static_cast<const float*>(x) + static_cast<size_t>(t) * d, vt);
     for (int o = 16; o >= quads; o >>= 1) {  // lanes with the same experts
       acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
       acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
@@ -141,7 +162,6 @@ __device__ __forceinline__ void router_logits_one(float* smem, const void* __res
       *reinterpret_cast<float4*>(red + static_cast<size_t>(vt / max(32, quads)) * E + 4 * (vt & (quads - 1))) = acc;
   }
   __syncthreads();
-  pdl_wait();
   for (int e = tid; e < E; e += NT) {
     float z = 0.0f;
     for (int row = 0; row < router_one_rows(E); ++row) z += red[row * E + e];
@@ -212,14 +232,16 @@ __device__ __forceinline__ void router_logits_batch(float* smem, const void* __r
       if (in) {
         const size_t at = static_cast<size_t>(tok) * d + k;
         if (x_bf16) {
-          pre[i][0] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(x) + at));
+          pre[i][0] = __ldcg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(x) + at));
         } else {
-          pre[i][0] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(x) + at));
-          pre[i][1] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(x) + at) + 1);
+          pre[i][0] = __ldcg(reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(x) + at));
+          pre[i][1] = __ldcg(reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(x) + at) + 1);
         }
       }
     }
   };
+  router_prefetch(x, x_bf16, t0, min(TT, T - t0), d, Wr, E, tid, ROUTER_BATCH_THREADS);
+  pdl_wait();
   for (int c = 0; c + 1 < stages; ++c) fetch_w(c);
   fetch_x(0);
   for (int c = 0; c < nchunks; ++c) {
@@ -276,7 +298,6 @@ __device__ __forceinline__ void router_logits_batch(float* smem, const void* __r
     *reinterpret_cast<float4*>(to + EP) = make_float4(hi[0], hi[1], hi[2], hi[3]);
   }
   __syncthreads();
-  pdl_wait();
   for (int idx = tid; idx < TT * EP; idx += ROUTER_BATCH_THREADS) {
     const int tt = idx >> ep_shift, ee = idx & (EP - 1);
     const int t = t0 + tt;

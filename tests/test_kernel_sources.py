@@ -1,0 +1,35 @@
+"""Rules that the kernels' sources keep and that no run shows reliably: a read that is too early, or a wait that may
+never end, would be a race or a hang on the GPU."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2308_14352_b200", "csrc")
+
+
+def _source(name):
+    text = open(os.path.join(CSRC, name)).read()
+    text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def _body(text, function):
+    """The text between the braces of the function's definition."""
+    at = text.index("{", text.index(")", re.search(r"\b%s\(" % function, text).end()))
+    depth = 0
+    for i in range(at, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[at:i]
+    raise AssertionError(function)
+
+
+@pytest.mark.parametrize("name,function", [("router.cuh", "router_logits"), ("router.cuh", "router_logits_one"),
+                                           ("router.cuh", "router_logits_batch"), ("decode_layer.cu", "decode_layer_kernel")])
+def test_router_reads_its_inputs_after_the_kernels_in_front_are_done(name, function):
+    """The kernel in front of a call's first one may be the one that writes x: griddepcontrol.wait comes before the first
+    load (prefetches into L2, and the body of a loading lambda, which runs where it is called, aside)."""
+    body = re.sub(r"auto \w+ = \[&\]\(int \w+\) \{.*?\n\s*\};", "", _body(_source(name), function), flags=re.S)
+    reads = [m.start() for m in re.finditer(r"__ldg\(|__ldcg\(|\*>\((a\.)?x\)\[|fetch_[wx]\(|\bx8\(", body)]
+    assert reads and body.index("pdl_wait();") < min(reads)
