@@ -359,6 +359,22 @@ __device__ __forceinline__ bool dequant_unit(const UmmaArgs& a, const UmBars& b,
   return true;
 }
 
+// The four storing warps of a set meet at barriers of their own (the hidden values change hands between them), so they
+// have to leave together: each warp's waits may end differently once another role has given up, and a warp that had
+// left would keep its neighbours at the next barrier for ever.  So they vote once per unit, behind its last wait.
+// (4096 x 14336 gated, 2048 tokens: 1400 us per call with the vote and without; 1450 where the result is not known to be
+// the same in every lane.)
+__device__ __forceinline__ bool set_agrees(int part, bool ok) {
+  uint32_t all;
+  __syncwarp();
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, %2, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(all)
+               : "r"(static_cast<uint32_t>(ok)), "r"(1 + part)
+               : "memory");
+  return __all_sync(0xffffffffu, all != 0);
+}
+__device__ __forceinline__ void set_sync(int part) { asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory"); }
+
 // EXACT: for calls whose experts the streaming kernel would otherwise serve.  A holds the codes themselves, whole numbers
 // that fp16 holds exactly; four more warps take the sums of each scale group out of tensor memory and add them, times
 // the row's scale, in fp32 registers, as the streaming kernel does.  Groups of up to 64 tokens (their sums
@@ -591,8 +607,10 @@ __global__ void __launch_bounds__(um_threads(EXACT), 1)
           default: ok = dequant_unit<8, EXACT>(a, b, raw_ring, a_col, sp, srow, ngroups, spg, kb0, kb_len, part, box, rin, lane, pos, abort_flag); break;
         }
       }
-      if (!ok) break;
-      if (EXACT && part < 2) continue;
+      if (EXACT && part < 2) {
+        if (!ok) break;
+        continue;
+      }
       // ---- epilogue: this warp's 32 rows x every other 32 token columns (EXACT: all of them) ----
       uint32_t tot[EXACT ? 2 : 1][32];  // EXACT: the scaled sums
       int acc_index = 0;
@@ -626,13 +644,13 @@ __global__ void __launch_bounds__(um_threads(EXACT), 1)
           if (lane == 0) mbar_arrive(b.acc_empty + 8 * acc.index);
           sv = sv_next;
         }
-        if (!ok) break;
       } else {
         const AccSlot<EXACT> acc(run_it);
         acc_index = acc.index;
-        if (!mbar_wait_warp(b.acc_full + 8 * acc.index, acc.parity, a.check_word, abort_flag)) break;
+        ok = mbar_wait_warp(b.acc_full + 8 * acc.index, acc.parity, a.check_word, abort_flag) && ok;
         tc_fence_after();
       }
+      if (!set_agrees(part, ok)) break;  // no bounded wait from here to the end of the unit
       const size_t slot0 = static_cast<size_t>(rec.begin) + static_cast<size_t>(tok_first);
       const int u_row0 = rb * (gated ? 64 : UM_ROWS);  // first channel of the unit
       const int hpos = a.phase == 0 ? pair_pos_rt(bits, nrow) : 0;  // (moves a channel inside its 16)
@@ -655,7 +673,7 @@ __global__ void __launch_bounds__(um_threads(EXACT), 1)
             *reinterpret_cast<__half*>(mine + c * 128) = __float2half_rn(fminf(fmaxf(h, -65504.0f), 65504.0f));
           }
           if (beyond) atomicOr(a.check_word, CHECK_F16_RANGE);  // saturated above: reported, not silent
-          asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");
+          set_sync(part);
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
             const int tok = (set_tid >> 3) + 16 * i, piece = set_tid & 7;
@@ -683,7 +701,7 @@ __global__ void __launch_bounds__(um_threads(EXACT), 1)
             *reinterpret_cast<__half*>(mine + c * 256) = __float2half_rn(fminf(h, 65504.0f));
           }
           if (beyond) atomicOr(a.check_word, CHECK_F16_RANGE);
-          asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");
+          set_sync(part);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int tok = (set_tid >> 4) + 8 * i, ch = 8 * (set_tid & 15);
@@ -691,7 +709,7 @@ __global__ void __launch_bounds__(um_threads(EXACT), 1)
               *reinterpret_cast<uint4*>(a.hidden16 + (slot0 + cc + tok) * a.hid_stride + u_row0 + ch) =
                   *reinterpret_cast<const uint4*>(out_stage + tok * 256 + ch * 2);
           }
-          asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");  // the buffer has been read
+          set_sync(part);  // the buffer has been read
         }
       };
       if constexpr (EXACT) {

@@ -33,3 +33,25 @@ def test_router_reads_its_inputs_after_the_kernels_in_front_are_done(name, funct
     body = re.sub(r"auto \w+ = \[&\]\(int \w+\) \{.*?\n\s*\};", "", _body(_source(name), function), flags=re.S)
     reads = [m.start() for m in re.finditer(r"__ldg\(|__ldcg\(|\*>\((a\.)?x\)\[|fetch_[wx]\(|\bx8\(", body)]
     assert reads and body.index("pdl_wait();") < min(reads)
+
+
+BARRIER = r"(?:\b|\\[nt])(?:bar|barrier)(?:\.cta)?\.(?:sync|red|arrive)\b"  # (also right behind an escape in a string)
+
+
+@pytest.mark.parametrize("name", ["ffn_tma.cu", "ffn_i8.cu", "pipe.cuh", "umma.cuh"])
+def test_no_unbounded_barrier_among_the_warps_of_the_pipelined_kernels(name):
+    """A warp whose bounded wait has run out leaves its role; a named barrier that its neighbours stand at would then never
+    open.  (Barriers of the whole CTA stand only where every role passes: at the start and, behind all roles, at the end.)"""
+    assert not re.search(BARRIER, _source(name))
+
+
+def test_the_storing_warps_of_the_grouped_gemm_leave_together():
+    """They have named barriers: each stands behind the set's vote on the unit's waits, and nothing between the vote and
+    the end of the unit waits or leaves."""
+    text = _source("ffn_umma.cu")
+    assert len(re.findall(BARRIER, text)) == 2  # inside set_agrees and set_sync
+    kernel = _body(text, "ffn_umma_kernel")
+    vote = kernel.index("if (!set_agrees(part, ok)) break;")
+    assert kernel.count("set_agrees(") == 1 and kernel.index("set_sync(") > vote
+    unit_end = kernel.index("if (*abort_flag)", vote)
+    assert not re.search(r"mbar_wait|\bbreak;|\breturn\b|\bcontinue;", kernel[vote + len("if (!set_agrees(part, ok)) break;"):unit_end])
