@@ -3,7 +3,7 @@
 // needs and every shared-memory read of it is free of bank conflicts.
 //
 //   tile     [K / 128 segments], at act_tile_offset(first slot of the pass)
-//   segment  [tokens][256 bytes: 128 inputs as fp16]; in passes of at most 8 tokens then 64 bytes: every
+//   segment  [tokens][256 bytes: 128 inputs as fp16]; in passes of at most 8 tokens then 64 bytes: (4 and 2 bits) every
 //            token's share of the code offset, -2^(b-1) * 2^-24 * (sum of its 128 inputs), as fp32,
 //            [2][8]: whole in the first half, or (hidden vectors of a gated layer, whose producers
 //            hold 64 channels each) in two halves to be added up
@@ -84,7 +84,7 @@ __device__ __forceinline__ void act_tile_row(const __nv_bfloat16* __restrict__ s
     const int x = tok & 1;
     *reinterpret_cast<uint4*>(row + ((((2 * b) ^ x) * 4 + t) << 4)) = lo;
     *reinterpret_cast<uint4*>(row + ((((2 * b + 1) ^ x) * 4 + t) << 4)) = hi;
-    if (ntok <= 8) {
+    if (ntok <= 8 && bits != 8) {
       float sum = 0.0f;
       const uint32_t v[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
 #pragma unroll

@@ -27,13 +27,14 @@
 //   * eight consumer warps take one 16-row tile of the stage each (gated projection: eight rows of
 //     w1 and the same eight of w3, so that the activation is formed in one lane).  Sixteen consumer
 //     warps per SM alone, out of shared memory, run at 12 / 7.3 / 3.5 TB/s of 8 / 4 / 2-bit codes;
-//   * up to 8 tokens per pass: a code field is read in place as the mantissa of a SUBNORMAL fp16
+//   * up to 8 tokens per pass, 4 and 2 bits: a code field is read in place as the mantissa of a SUBNORMAL fp16
 //     number ((q + 2^(b-1)) * 2^(p-24) for a field at bit p): one logic instruction per pair of
 //     codes, one shift per word.  Fields at different positions go to accumulators of their own,
 //     which are brought together once per segment; the offset's share 2^(b-1) * sum(x) comes with
-//     the activation tile.  The offset is as small as it can be (8 against codes of magnitude
-//     up to 8), so nothing is lost to cancellation.  9 to 16 tokens per pass: exact codes (one
-//     fp16x2 subtraction more per pair, shared by two token tiles).
+//     the activation tile.  This costs the sums some bits: 0.3 % (4 bits) and 1.7 % (2 bits) of the hidden
+//     values round to the other side of a bf16 tie, with exact codes 0.007 %.  At 8 bits it would be 1 % where
+//     the codes bring 0.007 %, so these are taken exactly, as all are with 9 to 16 tokens per
+//     pass (one fp16x2 subtraction more per pair, there shared by two token tiles).
 // 128 bytes of a row are 128 / 256 / 512 inputs at 8 / 4 / 2 bits, so a stage covers 1 / 2 / 4
 // scale segments.  Every wait is bounded: a wait that runs out sets a bit in the context's
 // check word and the CTA winds down without touching the stage.
@@ -144,6 +145,9 @@ __device__ __forceinline__ uint32_t code_exact(uint32_t w, int pos) {
   const uint32_t c = one | (sign_bits<BITS>() << pos);                         // 2^(10-pos) + 2^(b-1)
   return f16x2_sub(and_xor(w, field_mask<BITS>() << pos, c), c);
 }
+// what passes of up to 8 tokens take
+template <int BITS>
+__device__ __forceinline__ uint32_t code_one(uint32_t w, int pos) { return BITS == 8 ? code_exact<BITS>(w, pos) : code_sub<BITS>(w, pos); }
 
 // Where a lane finds its operands in a stage: its first row of codes (the 16-byte column of segment 0 under the
 // swizzle: the columns of later segments differ by an XOR), the distance to its second row, the even
@@ -176,11 +180,14 @@ __device__ __forceinline__ void consume_segment(const unsigned char* stage, cons
   if constexpr (NT == 1) {
     constexpr int NC = BITS == 2 ? 4 : 2;
     float acc[NC][4];
-    float2 off = *reinterpret_cast<const float2*>(stage + p.init + xoff);
-    if (p.halves) {
-      const float2 o2 = *reinterpret_cast<const float2*>(stage + p.init + xoff + 32);
-      off.x += o2.x;
-      off.y += o2.y;
+    float2 off = make_float2(0.0f, 0.0f);
+    if constexpr (BITS != 8) {
+      off = *reinterpret_cast<const float2*>(stage + p.init + xoff);
+      if (p.halves) {
+        const float2 o2 = *reinterpret_cast<const float2*>(stage + p.init + xoff + 32);
+        off.x += o2.x;
+        off.y += o2.y;
+      }
     }
     acc[0][0] = acc[0][2] = off.x;
     acc[0][1] = acc[0][3] = off.y;
@@ -195,8 +202,8 @@ __device__ __forceinline__ void consume_segment(const unsigned char* stage, cons
       for (int j = 0; j < 2; ++j) {
         const int m = 2 * q + j, pos = field_pos<BITS>(m);
         const uint32_t u0 = w[0][word_of<BITS>(m)], u1 = w[1][word_of<BITS>(m)];
-        mma_f16(acc[code_class<BITS>(m)], code_sub<BITS>(u0, pos), code_sub<BITS>(u1, pos), code_sub<BITS>(u0 >> 8, pos),
-                code_sub<BITS>(u1 >> 8, pos), j ? b.z : b.x, j ? b.w : b.y);
+        mma_f16(acc[code_class<BITS>(m)], code_one<BITS>(u0, pos), code_one<BITS>(u1, pos), code_one<BITS>(u0 >> 8, pos),
+                code_one<BITS>(u1 >> 8, pos), j ? b.z : b.x, j ? b.w : b.y);
       }
     }
 #pragma unroll
@@ -320,7 +327,7 @@ __device__ __forceinline__ void hidden_to_global(const TmaArgs& a, bool gated, i
       const float2 p = __half22float2(*reinterpret_cast<const __half2*>(&v.x)), q = __half22float2(*reinterpret_cast<const __half2*>(&v.y));
       sum = (p.x + p.y) + (q.x + q.y);
     }
-    if (ntok <= 8) {
+    if (ntok <= 8 && bits != 8) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       if (lane == 0) {
@@ -482,7 +489,7 @@ __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, i
   }
   const bool last_pass = p0 + ACT_PASS_MAX >= cnt;
   const int rb = rec.rbz & 0xffff, z = rec.rbz >> 16, ai = rec.ai;
-  if (NT == 1) {  // the subnormal codes weigh 2^-24
+  if (NT == 1 && BITS != 8) {  // the subnormal codes weigh 2^-24
 #pragma unroll
     for (int i = 0; i < 4; ++i) tot[0][i] *= 16777216.0f;
   }

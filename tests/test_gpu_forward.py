@@ -135,6 +135,53 @@ def test_forward_tma_pipeline_path_at_the_edges_of_its_passes(act, group, sdt, d
     _run_case(shape, bits, T, seed=37, path=3)
 
 
+def _one_expert(shape, bits, W, x):
+    """(y, the two dequantised matrices in fp64) of a layer with one expert on the streaming kernel."""
+    T = x.shape[0]
+    with layer.MoELayer(shape, [bits], max_tokens=T) as moe:
+        B.emoe_set_ffn_path(moe.ctx, 3)
+        moe.pack_from_host([W])
+        y, _, _, _ = moe.forward(x, np.zeros((shape.d_model, 1), dtype=np.float32))
+        deq = [oracle.dequantize(moe.packed_host(0, m), moe.scales_host(0, m).astype(np.float32), shape.matrix_shape(m)[1], bits, shape.group)
+               for m in range(2)]
+    return y, [d.astype(np.float64) for d in deq]
+
+
+def _bf16(v):
+    return torch.from_numpy(v.astype(np.float32)).to(torch.bfloat16).double().numpy()
+
+
+@pytest.mark.parametrize("T", [1, 4, 8, 20])
+def test_eight_bit_codes_lose_nothing_in_short_passes(T):
+    """Passes of up to 8 tokens (20: 16 and then 4) over 8-bit experts, with inputs of one sign, where a code offset
+    costs the sums most.  (a) First projection, its 512 hidden values picked out one by one: a segment's eight MMAs
+    each leave at most 2^-23 of the running sum, so a hidden value is off by some 1e-6 of itself, a few times that where
+    the sum nearly vanishes, and falls on the other side of a bf16 tie (half a step: 2^-9 of the value or more) in fewer
+    than 2 of 1000 cases; codes with an offset of 128: 7 to 13.  (b) Second projection, hidden values known exactly
+    (one input each): six segments added with one rounding each, 6 * 2^-24 / sqrt(3) of a sum at most, taken as 2e-7;
+    with the offset 4e-7 and more."""
+    rng = np.random.default_rng(71)
+    flipped = seen = 0
+    for _ in range(max(1, 16 // T)):
+        shape = inputs.LayerShape(1024, 512, 1, 1, "relu", "softmax", 128, "f16", "bf16")
+        pick = np.zeros((1024, 512), dtype=np.float32)
+        pick[np.arange(512), np.arange(512)] = 1.0
+        x = inputs.to_bf16_valued(np.abs(rng.standard_normal((T, 1024))).astype(np.float32))
+        y, (w1, w2) = _one_expert(shape, 8, [(rng.standard_normal((512, 1024)) * 0.02).astype(np.float32), pick], x)
+        h = np.maximum(x.astype(np.float64) @ w1.T, 0.0)
+        want = _bf16(h) @ w2.T
+        on = h > 0
+        flipped += int((np.abs(y - want)[:, :512] > 1e-4 * np.abs(want)[:, :512])[on].sum())
+        seen += int(on.sum())
+    assert flipped < 2e-3 * seen, (flipped, seen)
+    shape = inputs.LayerShape(512, 768, 1, 1, "relu", "softmax", 128, "f16", "bf16")
+    x = np.zeros((T, 512), dtype=np.float32)
+    x[np.arange(T), 7 * np.arange(T)] = 1.0
+    y, (w1, w2) = _one_expert(shape, 8, [(rng.standard_normal(s) * 0.02).astype(np.float32) for s in ((768, 512), (512, 768))], x)
+    want = _bf16(np.maximum(x.astype(np.float64) @ w1.T, 0.0)) @ w2.T
+    assert np.linalg.norm(y - want) < 2e-7 * np.linalg.norm(want), np.linalg.norm(y - want) / np.linalg.norm(want)
+
+
 I8_CASES = TMA_CASES + [
     ("relu", 128, "f16", 768, 3072, 32, 1, "softmax", [2, 4, 8, 4] * 8, 64),                # many experts, 2 tokens each
     ("swiglu", 128, "f16", 512, 1024, 8, 2, "softmax_renorm", [8, 8, 4, 4, 2, 2, 4, 8], 4),
