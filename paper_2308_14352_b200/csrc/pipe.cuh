@@ -6,8 +6,6 @@
 
 namespace emoe {
 
-constexpr unsigned PIPE_WAIT_LIMIT = 1u << 22;  // polls before a polling wait gives up (~0.2 s)
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -40,19 +38,28 @@ __device__ __forceinline__ bool mbar_try_wait_parked(uint32_t bar, uint32_t pari
       : "memory");
   return ok != 0;
 }
-constexpr unsigned long long PIPE_WAIT_NS = 500000000ull;  // a wait gives up after half a second
+constexpr unsigned long long PIPE_WAIT_NS = 500000000ull;  // a wait gives up after half a second of its own
 constexpr uint32_t PIPE_PARK_NS = 20000;                   // how long a waiting thread may be parked at a time
+// The time a wait has had once the clock went from t0 to t1 over one poll: no more than twice what a poll may be parked
+// for, so that a CTA that was switched out meanwhile does not take its absence for a wait that is stuck.
+__host__ __device__ constexpr unsigned long long waited_ns(unsigned long long so_far, unsigned long long t0, unsigned long long t1) {
+  return so_far + (t1 - t0 < 2ull * PIPE_PARK_NS ? t1 - t0 : 2ull * PIPE_PARK_NS);
+}
+static_assert(waited_ns(0, 1000, 21000) == 20000 && waited_ns(70, 5, 5) == 70, "a poll counts what it took");
+static_assert(waited_ns(0, 0, 10 * PIPE_WAIT_NS) < PIPE_WAIT_NS / 1000, "five seconds away are not five seconds of waiting");
 
 // The rest of a wait whose first test failed.  Parked, not polled: the warps that feed a pipeline wait for most
 // of its time, and their polling was a third of the instructions the SM executed.
 static __device__ __noinline__ bool mbar_wait_parked(uint32_t bar, uint32_t parity, int* check_word, volatile int* abort_flag) {
-  unsigned long long t0, t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  unsigned long long before, now, waited = 0;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(before));
   do {
     if (mbar_try_wait_parked(bar, parity, PIPE_PARK_NS)) return true;
     if (*abort_flag) return false;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  } while (t - t0 < PIPE_WAIT_NS);
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+    waited = waited_ns(waited, before, now);
+    before = now;
+  } while (waited < PIPE_WAIT_NS);
   *abort_flag = 1;
   atomicOr(check_word, CHECK_WAIT_TIMEOUT);
   return false;
