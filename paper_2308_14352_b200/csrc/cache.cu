@@ -462,8 +462,9 @@ int emoe_cached_layer(emoe_ctx* ctx, const emoe_layer_desc* desc, int layer, con
   }
   bool seen[EMOE_MAX_EXPERTS] = {};
   for (int p = 0; p < T * k; ++p) {
-    if (pinned_ids[p] < 0 || pinned_ids[p] >= E) return EMOE_ERR_DEVICE_CHECK;
-    seen[pinned_ids[p]] = true;
+    const int32_t e = seen_ids[p];  // (through the volatile pointer: the router kernel wrote them behind the compiler's back)
+    if (e < 0 || e >= E) return EMOE_ERR_DEVICE_CHECK;
+    seen[e] = true;
   }
   int32_t active[EMOE_MAX_EXPERTS];
   int64_t expert_ids[EMOE_MAX_EXPERTS];

@@ -364,3 +364,124 @@ def test_tokens_per_expert_of_the_last_forward_call():
             assert np.array_equal(counts, np.bincount(ids.reshape(-1), minlength=shape.n_experts))
         with pytest.raises(B.EmoeError):
             B.emoe_last_expert_counts(moe.ctx, shape.n_experts + 1)
+
+
+def _stack_on_cache(host, desc, n_slots, max_tokens):
+    ctx = B.emoe_create(0, B.emoe_workspace_bytes(desc, max_tokens))
+    B.emoe_cache_create(ctx, n_slots, host.slot_bytes(), host.n_layers, B.EVICT_FORWARD)
+    host.register_all(ctx, ExpertBufferModel(n_slots, host.n_layers, "forward"))
+    return ctx
+
+
+@pytest.mark.parametrize("T,n_slots,n_prefetch", [(1, 4, 2), (3, 6, 4), (12, 9, 1)])   # one launch per layer, and the chain of launches
+def test_cached_layer_is_the_single_calls(T, n_slots, n_prefetch):
+    """One trace through emoe_cached_layer and, on a context of its own, through the calls it stands for: the same picks,
+    gates and outputs to the bit, the same slots and counters after every layer.  A layer's input is made of the output of
+    the layer in front, on the same stream."""
+    shape = inputs.LayerShape(512, 1024, 4, 2, "relu", "softmax_renorm", 128, "f16", "bf16")
+    n_layers, E, d = 3, 4, 512
+    host = HostExperts(shape, n_layers, lambda l: [[8, 4, 2, 4], [2, 8, 4, 4], [4, 2, 8, 2]][l], seed=43)
+    rng = np.random.default_rng(43)
+    prior = rng.random((E, E)).astype(np.float32)
+    desc = layer.make_desc(shape)
+    dev = torch.device("cuda", 0)
+    Wr = [torch.from_numpy(inputs.router_weight(43, l, d, E, std=0.05)).to(dev) for l in range(n_layers)]
+    bias = torch.from_numpy(rng.normal(0.0, 1.0, size=(T, E)).astype(np.float32)).to(dev)
+    compute, copy = torch.cuda.Stream(device=dev), torch.cuda.Stream(device=dev)
+    cs, cps = compute.cuda_stream, copy.cuda_stream
+    one, many = _stack_on_cache(host, desc, n_slots, T), _stack_on_cache(host, desc, n_slots, T)
+    pinned = torch.full((T, 2), 77, dtype=torch.int32, pin_memory=True)
+    ids = [torch.empty(T, 2, dtype=torch.int32, device=dev) for _ in range(2)]
+    gates = [torch.empty(T, 2, device=dev) for _ in range(2)]
+    try:
+        for step in range(4):
+            x = [torch.from_numpy(inputs.activations(43, 0, T, d, "bf16", batch_tag=step)).to(dev).to(torch.bfloat16) for _ in range(2)]
+            torch.cuda.synchronize()
+            for l in range(n_layers):
+                nxt, b, stride = (l + 1) % n_layers, bias if l else None, E if l else 0
+                y = [torch.full((T, d), float("nan"), device=dev) for _ in range(2)]
+                torch.cuda.synchronize()
+                with torch.cuda.stream(compute):
+                    B.emoe_cached_layer(one, desc, l, x[0].data_ptr(), T, Wr[l].data_ptr(), b.data_ptr() if l else None, stride,
+                                        host.expert_id(l, 0), prior.ctypes.data, n_prefetch, host.expert_id(nxt, 0), ids[0].data_ptr(),
+                                        gates[0].data_ptr(), y[0].data_ptr(), pinned.data_ptr(), cs, cps)
+                    picks = pinned.numpy().copy()   # valid when the call returns
+                    B.emoe_router_topk(many, x[1].data_ptr(), B.DTYPE_BF16, T, d, Wr[l].data_ptr(), b.data_ptr() if l else None, stride, E, 2,
+                                       B.GATE_SOFTMAX_RENORM, ids[1].data_ptr(), gates[1].data_ptr(), None, cs)
+                    compute.synchronize()
+                    want = ids[1].cpu().numpy()
+                    active = sorted(set(want.reshape(-1).tolist()))
+                    order = B.emoe_rank_experts(prior, np.array(active, dtype=np.int32))
+                    B.emoe_prefetch_experts(many, [host.expert_id(nxt, int(e)) for e in order[:n_prefetch]], l, cps)
+                    eids = [host.expert_id(l, e) for e in active]
+                    table = _table_from(B.emoe_cache_acquire(many, eids, l, cs, cps), active, host.bits[l])
+                    B.emoe_moe_forward_routed(many, desc, x[1].data_ptr(), T, ids[1].data_ptr(), gates[1].data_ptr(), table, y[1].data_ptr(), None, cs)
+                    B.emoe_cache_release(many, eids, cs)
+                    for i in range(2):   # a kernel of the caller's writes the next layer's input
+                        x[i].copy_(y[i] * 20.0)
+                compute.synchronize()
+                assert B.emoe_device_status(one, cs) == B.OK and B.emoe_device_status(many, cs) == B.OK
+                assert np.array_equal(picks, want) and torch.equal(ids[0], ids[1])
+                assert torch.equal(gates[0], gates[1]) and torch.equal(y[0], y[1]) and torch.isfinite(y[0]).all()
+                for ll in range(n_layers):
+                    for e in range(E):
+                        assert B.emoe_cache_slot_of(one, host.expert_id(ll, e)) == B.emoe_cache_slot_of(many, host.expert_id(ll, e))
+                assert _bookkeeping(B.emoe_cache_get_stats(one)) == _bookkeeping(B.emoe_cache_get_stats(many))
+        st = B.emoe_cache_get_stats(one)
+        assert st["evictions"] > 0 and st["hits"] > 0 and st["misses"] > 0
+    finally:
+        torch.cuda.synchronize()
+        B.emoe_destroy(one)
+        B.emoe_destroy(many)
+
+
+def test_cached_layer_errors():
+    """Bad arguments are refused before anything runs; a layer that fails after its experts were acquired lets them go."""
+    shape = inputs.LayerShape(512, 1024, 4, 2, "relu", "softmax_renorm", 128, "f16", "bf16")
+    host = HostExperts(shape, 2, lambda l: [8, 4, 2, 4], seed=45)
+    desc = layer.make_desc(shape)
+    dev = torch.device("cuda", 0)
+    x = torch.zeros(8, 512, dtype=torch.bfloat16, device=dev)
+    Wr = torch.from_numpy(inputs.router_weight(45, 0, 512, 4, std=0.05)).to(dev)
+    ids, gates = torch.empty(8, 2, dtype=torch.int32, device=dev), torch.empty(8, 2, device=dev)
+    y, pinned = torch.empty(8, 512, device=dev), torch.empty(8, 2, dtype=torch.int32, pin_memory=True)
+    prior = np.ones((4, 4), dtype=np.float32)
+    torch.cuda.synchronize()
+
+    def call(ctx, **other):
+        a = dict(desc=desc, layer=0, x=x.data_ptr(), T=2, Wr=Wr.data_ptr(), bias=None, stride=0, first=host.expert_id(0, 0), prior=None,
+                 n_prefetch=0, nxt=host.expert_id(1, 0), ids=ids.data_ptr(), gates=gates.data_ptr(), y=y.data_ptr(), pinned=pinned.data_ptr())
+        a.update(other)
+        return B.lib().emoe_cached_layer(ctx, a["desc"], a["layer"], a["x"], a["T"], a["Wr"], a["bias"], a["stride"], a["first"], a["prior"],
+                                         a["n_prefetch"], a["nxt"], a["ids"], a["gates"], a["y"], a["pinned"], None, None)
+
+    bare = B.emoe_create(0, B.emoe_workspace_bytes(desc, 2))
+    ctx, tight = _stack_on_cache(host, desc, 2, 2), _stack_on_cache(host, desc, 1, 2)
+    try:
+        assert call(bare) == B.ERR_INVALID_ARG                          # no cache
+        for name in ("x", "Wr", "ids", "gates", "y", "pinned"):
+            assert call(ctx, **{name: None}) == B.ERR_INVALID_ARG, name
+        assert call(ctx, T=0) == B.ERR_INVALID_ARG
+        assert call(ctx, n_prefetch=-1) == B.ERR_INVALID_ARG
+        assert call(ctx, bias=gates.data_ptr(), stride=3) == B.ERR_INVALID_ARG
+        for field, value, status in (("top_k", 5, B.ERR_INVALID_ARG), ("n_experts", 0, B.ERR_INVALID_ARG), ("d_model", 0, B.ERR_INVALID_ARG),
+                                     ("act_dtype", 9, B.ERR_UNSUPPORTED), ("gate_mode", 9, B.ERR_UNSUPPORTED)):
+            bad = layer.make_desc(shape)
+            setattr(bad, field, value)
+            assert call(ctx, desc=bad) == status, field
+        st = B.emoe_cache_get_stats(ctx)
+        assert st["hits"] == st["misses"] == st["prefetched"] == 0
+        assert call(ctx, first=1000) == B.ERR_INVALID_ARG               # experts nobody registered
+        assert call(ctx, prior=prior.ctypes.data, n_prefetch=1, nxt=1000) == B.ERR_INVALID_ARG
+        assert call(tight) == B.ERR_CACHE_FULL                          # two experts, one slot
+        assert call(ctx, T=8) == B.ERR_WORKSPACE                        # context sized for two tokens
+        for c, eids in ((ctx, [host.expert_id(1, 0), host.expert_id(1, 1)]), (tight, [host.expert_id(1, 0)])):
+            B.emoe_cache_acquire(c, eids, 1, 0, 0)                      # every slot can be had: nothing is held
+            B.emoe_cache_release(c, eids, 0)
+        assert call(ctx) == B.OK
+        torch.cuda.synchronize()
+        assert B.emoe_device_status(ctx) == B.OK
+    finally:
+        torch.cuda.synchronize()
+        for c in (bare, ctx, tight):
+            B.emoe_destroy(c)
