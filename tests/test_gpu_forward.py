@@ -537,7 +537,7 @@ UMMA_EDGE_CASES = [
     ("swiglu", 128, "f16", 512, 512, 1, 1, "softmax", [8], 320),
     ("relu", 128, "f16", 512, 512, 1, 1, "softmax", [4], 321),
     ("relu", 128, "f32", 512, 2048, 1, 1, "softmax", [2], 129),       # second projection in slices of its inputs
-    # several units per CTA: accumulators in turn, stored by warps of their own (small groups) or not (large ones)
+    # several units per CTA: the accumulators are free again only when the unit in front has been stored
     ("relu", 128, "f16", 512, 8192, 4, 1, "softmax", [4, 2, 8, 4], 150),
     ("swiglu", 128, "f16", 512, 6144, 3, 2, "softmax_renorm", [8, 4, 2], 200),
     ("swiglu", 128, "f16", 512, 6144, 2, 2, "softmax_renorm", [4, 2], 210),
@@ -548,6 +548,35 @@ UMMA_EDGE_CASES = [
 def test_forward_tcgen05_path_at_the_edges_of_its_groups(act, group, sdt, d, f, E, k, gate, bits, T):
     shape = inputs.LayerShape(d, f, E, k, act, gate, group, sdt, "bf16")
     _run_case(shape, bits, T, seed=33, path=4)
+
+
+def test_gated_activation_of_the_tcgen05_path():
+    """silu(a) * b over both signs of a, from small values past the point where exp(-a) overflows, with a and b exact in
+    either path (one input, one 2-bit code per row).  Against 64 bits: the bf16 rounding of the hidden value (2^-8) and
+    the smallest steps of fp16.  Against the streaming path, which divides: the same fp32 value but for a few
+    units in the last place, so at most a step of bf16 where that lies at a tie (about one in 4000).  Sixteen tokens, a
+    pass that takes the codes exactly there: with 8 and fewer a small hidden value beside large ones carries the rounding
+    of their sum times the code offset, 2^-24 of it or so (values of 2e-3 beside a sum of 1e3: 6e-5 off)."""
+    a = np.concatenate([np.geomspace(1e-3, 80.0, 180), np.linspace(80.0, 110.0, 60), np.geomspace(110.0, 1000.0, 16)])
+    a = np.concatenate([a, -a]).astype(np.float16).astype(np.float32)
+    w1, w3 = np.zeros((512, 512), dtype=np.float32), np.zeros((512, 512), dtype=np.float32)
+    w1[:, 0], w3[:, 0] = a, 0.25
+    T = 16
+    x = np.zeros((T, 512), dtype=np.float32)
+    x[:, 0] = 2.0 ** (np.arange(T) % 5 - 2)
+    shape = inputs.LayerShape(512, 512, 1, 1, "swiglu", "softmax", 128, "f16", "bf16")
+    y = {}
+    for path in (3, 4):
+        with layer.MoELayer(shape, [2], max_tokens=T) as moe:
+            B.emoe_set_ffn_path(moe.ctx, path)
+            moe.pack_from_host([[w1, w3, np.eye(512, dtype=np.float32)]])
+            y[path] = moe.forward(x, np.zeros((512, 1), dtype=np.float32))[0].astype(np.float64)
+    av = x[:, :1].astype(np.float64) * a
+    with np.errstate(over="ignore"):
+        want = av / (1.0 + np.exp(-av)) * (0.25 * x[:, :1])
+    assert np.all(np.abs(y[4] - want) <= 2.0 ** -8 * np.abs(want) + 2.0 ** -24)
+    assert np.all(np.abs(y[4] - y[3]) <= 2.0 ** -7 * np.abs(want) + 2.0 ** -24)
+    assert np.count_nonzero(y[4] != y[3]) <= 16
 
 
 EXACT_CASES = [
