@@ -9,6 +9,10 @@
 
 namespace emoe {
 
+// Multiprocessors of the GPU this library is built for, for the rules that also size a workspace (where no device is at
+// hand); grids that must be resident at once go by the device's own number.
+constexpr int GPU_SMS = 148;
+
 // Device copy of one layer's expert table (one entry per expert).
 struct ExpertDev {
   int32_t bits;

@@ -453,8 +453,6 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
   }
 }
 
-size_t decode_layer_smem() { return 0; }
-
 }  // namespace
 
 bool decode_layer_supported(const LayerDims& L, int T) {
@@ -465,7 +463,7 @@ bool decode_layer_supported(const LayerDims& L, int T) {
 
 int decode_layer_resident_ctas(int device) {
   int per_sm = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_layer_kernel<DL_R_MAX>, DL_THREADS, decode_layer_smem()) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_layer_kernel<DL_R_MAX>, DL_THREADS, 0) != cudaSuccess)
     return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
   return per_sm * sms;
@@ -526,7 +524,7 @@ cudaError_t launch_decode_layer(const LayerDims& L, const ExpertDev* experts, co
   while (a.wpr > 1 && static_cast<long long>(T) * (L.d_model / DL_R_MAX) > static_cast<long long>(grid) * (DL_WARPS / a.wpr)) a.wpr >>= 1;
   while (a.rsplit > 1 && T * a.rsplit > grid) a.rsplit >>= 1;  // a small device: fewer slices than CTAs
   if (per_sm < 1 || grid < T) return cudaErrorInvalidConfiguration;
-  return launch_chain(decode_layer_kernel<DL_R_MAX>, dim3(grid), dim3(DL_THREADS), decode_layer_smem(), st, a);
+  return launch_chain(decode_layer_kernel<DL_R_MAX>, dim3(grid), dim3(DL_THREADS), 0, st, a);
 }
 
 }  // namespace emoe

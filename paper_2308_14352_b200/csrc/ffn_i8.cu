@@ -1085,10 +1085,10 @@ int ffn_i8_ksplit(const LayerDims& L, int T) {
   const long long units = row_blocks * active;
   // enough slices that the second projection's items outnumber the CTAs (one per SM) about three
   // times: short items at the end of the launch keep its tail short
-  long long z = (3 * 148 + units - 1) / units;
+  long long z = (3 * GPU_SMS + units - 1) / units;
   const int steps_min = (L.d_ff + 511) / 512;  // stages at the widest span (2 bits)
   const int steps_max = (L.d_ff + 127) / 128;
-  const int cap = units * 2 <= 148 ? steps_max : steps_min;
+  const int cap = units * 2 <= GPU_SMS ? steps_max : steps_min;
   if (z > cap) z = cap;
   if (z > 16) z = 16;
   if (z < 1) z = 1;

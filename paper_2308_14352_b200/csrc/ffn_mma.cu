@@ -328,7 +328,7 @@ int ffn_mma_ksplit(const LayerDims& L, int T) {
   const long long active = T * static_cast<long long>(L.top_k) < L.E ? T * static_cast<long long>(L.top_k) : L.E;
   const long long ctas = row_blocks * active;
   const int chunks = (L.d_ff + MMA_KCH - 1) / MMA_KCH;
-  long long z = (4 * 148 + ctas - 1) / ctas;
+  long long z = (4 * GPU_SMS + ctas - 1) / ctas;
   if (z > chunks) z = chunks;
   if (z > 16) z = 16;
   if (z < 1) z = 1;

@@ -59,10 +59,7 @@ constexpr int ST_CTAS = 2;                       // per SM
 constexpr int ST_BOX_ROWS = 64;
 constexpr int ST_BOX_BYTES = ST_BOX_ROWS * 128;  // 8 KB
 constexpr int ST_X_OFFSET = 2 * ST_BOX_BYTES + 2 * ST_BOX_ROWS * 16;  // a stage: two boxes, 16 bytes of scales per row, the activation slice
-#ifndef EMOE_ST_RING_KB
-#define EMOE_ST_RING_KB 96
-#endif
-constexpr int ST_RING = EMOE_ST_RING_KB * 1024;
+constexpr int ST_RING = 96 * 1024;
 constexpr int ST_SLOTS = 8;                      // stages in flight at most (barriers, records)
 constexpr int ST_HID_BYTES = ACT_PASS_MAX * 256;  // one segment of hidden values on their way out
 constexpr int ST_SMEM = ST_RING + 2 * ST_HID_BYTES + 1024;  // + slack to align the base to 1024
@@ -357,7 +354,6 @@ __device__ __forceinline__ void store_output(const TmaArgs& a, int rb, int z, in
 // Item k of the CTA's list, decoded by one thread.  Every CTA takes every gridDim.x-th item: the items of the
 // first projection, then those of the second, most expensive bitwidth first, so that the shares are even to
 // about one of the cheapest items; the list is known without asking, 32 items are decoded at a time.
-template <bool SF16>
 __device__ __forceinline__ void decode_item(const TmaArgs& a, const PlanRec* s_plan, const PlanRec* recs, int n_active, int k, ItemRec* out) {
   const int n_items0 = a.phase_begin == 0 ? n_active * a.row_blocks[0] : 0;
   const int n_items1 = a.phase_end == 2 ? n_active * a.row_blocks[1] * a.ksplit : 0;
@@ -570,7 +566,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
     int it = 0, oldest = 0, head = 0, phys = 0;
     int more = 1;
     for (int k0 = 0; more; k0 += 32) {
-      decode_item<SF16>(a, s_plan, recs, s_active, k0 + lane, &queue[(k0 + lane) % ST_QUEUE]);
+      decode_item(a, s_plan, recs, s_active, k0 + lane, &queue[(k0 + lane) % ST_QUEUE]);
       __syncwarp();
       if (lane == 0) {
         for (int k = k0; k < k0 + 32 && more; ++k) {
@@ -819,20 +815,20 @@ int ffn_tma_ksplit(const LayerDims& L, int T) {
   const int steps_min = (L.d_ff + 511) / 512;  // stages at the widest span (2 bits)
   // enough slices that the second projection's items outnumber the resident CTAs (2 per SM)
   // several times: short items at the end of the launch keep its tail short
-  long long z = (12 * 148 + ctas - 1) / ctas;
+  long long z = (12 * GPU_SMS + ctas - 1) / ctas;
   // A handful of tokens leaves most SMs without an item: the slices are then cut as fine as the
   // 8-bit stages allow (narrower experts get empty slices, which only store zeros), so that the
   // second projection of the one or two activated experts is a short step on many SMs instead
   // of a chain of stages on a few.
   const int steps_max = (L.d_ff + 127) / 128;
-  const int cap = ctas * 4 <= 148 ? steps_max : steps_min;
+  const int cap = ctas * 4 <= GPU_SMS ? steps_max : steps_min;
   if (z > cap) z = cap;
   if (z > 16) z = 16;
   // ... but not so fine that the items of both projections outnumber the resident CTAs where coarser slices would not: a
   // second item is a second chain of steps (12 tokens, 8 experts, 512 x 1152: 25 us per layer with nine slices, 21 with
   // seven; 24 tokens on 512 x 2048 28 and 22)
   const int rows0 = L.act == EMOE_ACT_SWIGLU ? ST_BOX_ROWS : 2 * ST_BOX_ROWS;
-  const long long room = (ST_CTAS * 148 - active * ((L.d_ff + rows0 - 1) / rows0)) / ctas;
+  const long long room = (ST_CTAS * GPU_SMS - active * ((L.d_ff + rows0 - 1) / rows0)) / ctas;
   if (z > room && room >= 2) z = room;
   if (z < 1) z = 1;
   return static_cast<int>(z);

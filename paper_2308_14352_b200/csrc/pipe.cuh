@@ -102,21 +102,11 @@ __device__ __forceinline__ void mbar_expect_tx_if(uint32_t on, uint32_t bar, uin
                "r"(bytes), "r"(on)
                : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_if(uint32_t on, uint32_t bar) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"(on) : "memory");
-}
 __device__ __forceinline__ void tma_load_2d_if(uint32_t on, uint32_t dst, const void* tmap, int c0, int c1, uint32_t bar) {
   asm volatile(
       "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
       "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}" ::"r"(dst),
       "l"(tmap), "r"(c0), "r"(c1), "r"(bar), "r"(on)
-      : "memory");
-}
-__device__ __forceinline__ void bulk_load_if(uint32_t on, uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
-      "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar), "r"(on)
       : "memory");
 }
 

@@ -285,14 +285,14 @@ cudaError_t launch_router_topk(const void* x, int x_bf16, int T, int d, const fl
     if (router_batch_chunk(EP) == 128) return launch(router_topk_kernel<16, 128>, 16, smem);
     return launch(router_topk_kernel<16, 64>, 16, smem);
   }
-  if (tiled && T >= 148) {
+  if (tiled && T >= GPU_SMS) {
     const size_t smem = router_batch_smem(8, EP);
     if (router_batch_chunk(EP) == 512) return launch(router_topk_kernel<8, 512>, 8, smem);
     if (router_batch_chunk(EP) == 256) return launch(router_topk_kernel<8, 256>, 8, smem);
     if (router_batch_chunk(EP) == 128) return launch(router_topk_kernel<8, 128>, 8, smem);
     return launch(router_topk_kernel<8, 64>, 8, smem);
   }
-  if (T < 148 && router_one_supported(E, Wr))
+  if (T < GPU_SMS && router_one_supported(E, Wr))
     return launch(router_topk_kernel<1, -1>, 1, router_one_smem(E), ROUTER_ONE_THREADS);
   if (T >= 8 * 64) return launch(router_topk_kernel<8, 0>, 8, sizeof(float) * (8 * ROUTER_DC + ROUTER_THREADS * 8 + 8 * EP), ROUTER_THREADS);  // <= 48 KB
   return launch(router_topk_kernel<1, 0>, 1, sizeof(float) * (ROUTER_DC + ROUTER_THREADS + EP), ROUTER_THREADS);

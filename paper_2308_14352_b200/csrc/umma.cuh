@@ -15,24 +15,6 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr) {
          (1ull << 46) | (2ull << 61);
 }
 
-// fp16 x fp16 -> fp32, both operands from shared memory
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      :
-      : "r"(d_tmem), "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// ... or A from tensor memory (row i of A in lane i, two fp16 inputs per 32-bit column)
-__device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t db, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      :
-      : "r"(d_tmem), "r"(a_tmem), "l"(db), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
 // 8-bit integers -> int32: A from shared memory ...
 __device__ __forceinline__ void umma_i8_ss(uint32_t d_tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -56,7 +38,8 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// ... by one elected lane of a convergent warp (see pipe.cuh)
+// fp16 x fp16 -> fp32, A from tensor memory (row i of A in lane i, two fp16 inputs per 32-bit column), and the commit, by one
+// elected lane of a convergent warp (see pipe.cuh)
 __device__ __forceinline__ void umma_f16_ts_if(uint32_t on, uint32_t d_tmem, uint32_t a_tmem, uint64_t db, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
