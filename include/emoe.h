@@ -241,13 +241,14 @@ int emoe_moe_forward_routed(emoe_ctx* ctx, const emoe_layer_desc* desc, const vo
  * and measurements. */
 int emoe_set_ffn_path(emoe_ctx* ctx, int path);
 
-/* Every wait inside the weight-streaming kernel (on a pipeline stage, on tensor memory, on the
- * completion of an expert's hidden vectors) is bounded: after `polls` unsuccessful polls the
+/* Every wait inside a kernel (on a pipeline stage, on tensor memory, on the completion of an
+ * expert's hidden vectors, on the other CTAs of a grid) is bounded: when it runs out the
  * kernel records the failure, lets its copies in flight land, releases what it holds and
  * returns; emoe_device_status then reports EMOE_ERR_TIMEOUT and the context stays usable.  This
  * is the library's form of failure detection (the paper's only failure path is a mispredicted
- * preload, Section 3.3, which is corrected by loading the right expert).  polls = 0 restores the
- * default (about 0.2 s).  Applies to the forward calls that follow. */
+ * preload, Section 3.3, which is corrected by loading the right expert).  `polls` sets the limit of
+ * kernel family 6, of the one-launch layer and of the one-launch routing, in unsuccessful polls, for the forward calls
+ * that follow (0: the default, about 0.2 s); the other kernels give up after a tenth of a second to half a second. */
 int emoe_set_wait_limit(emoe_ctx* ctx, unsigned polls);
 
 /* Test hook for the above: the second projection of every expert waits for `extra` more
@@ -294,8 +295,8 @@ int emoe_set_fused_routing(emoe_ctx* ctx, int enabled);
  * within the accumulation-order difference (fp32 sums of the same products).  A wait that runs out reports EMOE_ERR_TIMEOUT through
  * emoe_device_status (limit: emoe_set_wait_limit).
  * mode 0: never; 1: every call inside the limits; 2 (the default): calls of up to eight pairs,
- * where it was measured faster than the chain of launches (1.8 x for one pair, 1.5 x for two to
- * four on a Switch-base-sized layer, 1.25 x for eight; for sixteen the chain wins).  Other values:
+ * where it was measured faster than the chain of launches on a Switch-base-sized layer (1.75 x for one
+ * pair, 1.35 x for two, 1.2 x for four, 1.05 x for eight; for sixteen the chain wins).  Other values:
  * EMOE_ERR_INVALID_ARG. */
 int emoe_set_fused_layer(emoe_ctx* ctx, int mode);
 

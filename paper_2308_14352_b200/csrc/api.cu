@@ -337,8 +337,9 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
 
   // a handful of tokens on a small layer: router, both projections and the gate-weighted sum in one launch
   bool one_launch_layer = false;
-  // as measured on a Switch-base-sized layer: 1.8 x faster than the chain of launches for one pair, 1.5 x for two to four, 1.25 x
-  // for eight, slower for sixteen (the projections then take several passes of dependent loads per warp)
+  // us per 12 layers of 768 x 3072, 32 experts, chain of launches / one launch: one token 280/160, two 285/210, four 292/242,
+  // eight 350/331, twelve 416/476, sixteen 422/533 (the projections then take several passes of dependent loads per warp);
+  // gated layers of 768 x 2048 with two picks lose earlier (us per four layers: one token 107/82, two 100/99, four 100/136)
   const bool layer_wanted = ctx->fuse_layer == 1 || (ctx->fuse_layer == 2 && T * L.top_k <= 8);
   if (layer_wanted && ctx->ffn_path == 0 && decode_layer_supported(L, T)) {
     if (ctx->resident_layer_ctas < 0) {
@@ -386,8 +387,9 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   // the streaming kernel takes per pass over the weights; an even one pays some 5 us for two launches that find
   // nobody.  From 32 tokens per expert on average for all of them; below, for experts beyond 32 tokens, 48 where even
   // loads reach 32 as well.  us per layer, streaming alone / both, even and skewed (Zipf exponent 1.1) loads:
-  // 768 x 3072, 32 experts, 256 tokens 53/58 and 88/78, 512 tokens 77/81 and 138/103; 1024 x 4096, 128 experts, 1024 tokens 220/226
-  // and 477/179; 1280 x 4480, 64 experts, 800 tokens 209/218 and 373/197; 2048 tokens on the first, all 192/144 and 510/165.
+  // 768 x 3072, 32 experts, 256 tokens 58/62 and 88/85, 512 tokens 79/85 and 141/103; 1024 x 4096, 128 experts, 256 tokens 180/183 and
+  // 200/132, 1024 tokens 233/238 and 583/183; 1280 x 4480, 64 experts, 800 tokens 217/225 and 497/206; 2048 tokens on the
+  // first, all 193/146 and 505/166.
   const bool exact_pairs = !rounded && P >= 256;
   const bool one_family = mean_tokens >= (rounded ? 256.0 : 32.0);
   const bool auto_umma = ctx->ffn_path == 0 && (rounded || exact_pairs);

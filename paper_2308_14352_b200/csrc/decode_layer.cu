@@ -512,7 +512,8 @@ cudaError_t launch_decode_layer(const LayerDims& L, const ExpertDev* experts, co
   // Every CTA must be resident at once.  As few CTAs as give every block of four rows of the
   // first projection a warp of its own (one, two or three per SM): each further CTA makes the two
   // grid-wide waits longer (as measured, one token: 0.139 ms per 12-layer step with one CTA per
-  // SM, 0.154 with two, 0.173 with three; four tokens: 0.307 / 0.259 / 0.224).
+  // SM, 0.154 with two, 0.173 with three; four tokens: 0.307 / 0.259 / 0.224; since then the router product, which used to run
+  // ahead of the kernels in front, has added some 10 us to each).
   const long long blocks = static_cast<long long>(T) * L.top_k * L.d_ff / DL_R_MAX;
   const int max_per_sm = resident_ctas / sms < 3 ? resident_ctas / sms : 3;
   int per_sm = 1;

@@ -13,7 +13,7 @@
 //     128-bit loads (16 / 32 / 64 weights each), the next loads on their way while one set is used;
 //   * the fields of a 32-bit word are masked into bytes together, a byte becomes a float by one byte
 //     permute into the mantissa of 2^23 and one (exact) subtraction, shared by the tokens.
-// Measured: Switch-base-like layers with 8 experts and 16 fp32 tokens, forward call of eight layers 878 -> 333 us
+// Measured: Switch-base-like layers with 8 experts and 16 fp32 tokens, forward call of eight layers 878 -> 340 us
 // (one row per warp, all inputs in turn, activations from global memory before); what is left is the
 // latency of five launches and of the first loads of each.
 #include "common.cuh"

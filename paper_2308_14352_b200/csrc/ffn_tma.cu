@@ -26,7 +26,7 @@
 //     and whatever it does per stage shows;
 //   * eight consumer warps take one 16-row tile of the stage each (gated projection: eight rows of
 //     w1 and the same eight of w3, so that the activation is formed in one lane).  Sixteen consumer
-//     warps per SM alone, out of shared memory, run at 12 / 7.3 / 3.5 TB/s of 8 / 4 / 2-bit codes;
+//     warps per SM alone, out of shared memory, run at 12 / 7.3 / 3.5 TB/s of 8 / 4 / 2-bit codes (all read in place);
 //   * up to 8 tokens per pass, 4 and 2 bits: a code field is read in place as the mantissa of a SUBNORMAL fp16
 //     number ((q + 2^(b-1)) * 2^(p-24) for a field at bit p): one logic instruction per pair of
 //     codes, one shift per word.  Fields at different positions go to accumulators of their own,
@@ -40,8 +40,9 @@
 // check word and the CTA winds down without touching the stage.
 //
 // Measured (expert launch alone, start of comparison: one feeding and four computing warps per CTA, three CTAs,
-// 16 / 8-token tiles by the launch's mean): Mixtral-like layer (d 4096, f 14336), 23 tokens 245 -> 218 us
-// (3.7 TB/s of packed bytes), 4 tokens of 4-bit experts 2.8 -> 3.6 TB/s, 8 bits 4.7 -> 4.9, 2 bits 1.8 -> 2.2.
+// 16 / 8-token tiles by the launch's mean): Mixtral-like layer (d 4096, f 14336), 23 tokens 245 -> 217 us
+// (3.8 TB/s of packed bytes), 4 tokens of 4-bit experts 2.8 -> 3.6 TB/s, 8 bits 4.7 -> 4.85 (5.0 with the codes read
+// in place, which is not exact), 2 bits 1.8 -> 2.15.
 #include <cuda.h>
 
 #include "act_tile.cuh"

@@ -378,8 +378,8 @@ __device__ __forceinline__ void set_sync(int part) { asm volatile("bar.sync %0, 
 // EXACT: for calls whose experts the streaming kernel would otherwise serve.  A holds the codes themselves, whole numbers
 // that fp16 holds exactly; four more warps take the sums of each scale group out of tensor memory and add them, times
 // the row's scale, in fp32 registers, as the streaming kernel does.  Groups of up to 64 tokens (their sums
-// fit the registers), four sets of accumulators in turn.  768 x 3072, 32 experts, 2048 tokens: 144 us per layer (streaming
-// 192, rounded 106); the four warps' reads of tensor memory are what bounds it.
+// fit the registers), four sets of accumulators in turn.  768 x 3072, 32 experts, 2048 tokens: 146 us per layer (streaming
+// 193, rounded 106); the four warps' reads of tensor memory are what bounds it.
 template <bool EXACT>
 __global__ void __launch_bounds__(um_threads(EXACT), 1)
     ffn_umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap tmap_b) {

@@ -106,7 +106,7 @@ __device__ __forceinline__ void router_logits(float* smem, const void* __restric
 // Logits of one token into zs[EP]: bound by the round trips to memory, so everything a thread reads is requested at
 // once, with nothing staged in front: ROUTER_ONE_FLY pieces of four experts' weights per thread and the activation that
 // belongs to each (up to 32 K products per round trip).  E a power of two, at least four: a thread keeps to four
-// experts.  4 tokens x 4096 x 8 experts, back to back: 12.3 us with chunks staged in shared memory, 8.2 so.
+// experts.  4 tokens x 4096 x 8 experts, back to back: 12.3 us with chunks staged in shared memory, 8.0 so.
 constexpr int ROUTER_ONE_THREADS = 512, ROUTER_ONE_FLY = 16;
 __host__ __device__ constexpr int router_one_rows(int E) { return ROUTER_ONE_THREADS * 4 / (E > 128 ? E : 128); }  // partial sums per expert
 __host__ __device__ constexpr int router_one_smem(int E) { return (router_one_rows(E) + 1) * E * 4; }
