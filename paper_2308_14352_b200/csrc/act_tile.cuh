@@ -5,8 +5,9 @@
 //   tile     [K / 128 segments], at act_tile_offset(first slot of the pass)
 //   segment  [tokens][256 bytes: 128 inputs as fp16]; in passes of at most 8 tokens then 64 bytes: (4 and 2 bits) every
 //            token's share of the code offset, -2^(b-1) * 2^-24 * (sum of its 128 inputs), as fp32,
-//            [2][8]: whole in the first half, or (hidden vectors of a gated layer, whose producers
-//            hold 64 channels each) in two halves to be added up
+//            [8][2]: two halves to be added up, which one 16-byte read brings for a lane's two tokens (hidden vectors of
+//            a gated layer, whose producers hold 64 channels each, fill one half at a time; others the first, the
+//            second being zero)
 //   row      sixteen 16-byte chunks; chunk (q ^ (token & 1)) * 4 + t holds what lane t of an MMA quad
 //            needs for the two MMAs 2q and 2q+1 of the segment (its inputs 32t .. 32t+31), so the
 //            eight lanes of one shared-memory phase (two tokens x four t) cover all 32 banks.
@@ -29,9 +30,12 @@ __host__ __device__ __forceinline__ constexpr int act_seg_bytes(int ntok) { retu
 __host__ __device__ __forceinline__ constexpr size_t act_slot_bytes(int K) { return static_cast<size_t>(K) * 2 + static_cast<size_t>(K / 128) * 64; }
 __host__ __device__ __forceinline__ size_t act_tile_offset(int slot0, int K) { return static_cast<size_t>(slot0) * act_slot_bytes(K); }
 
-// the share of the code offset of token `tok` from the sum of (half of) its inputs; `at`: behind the segment's rows
+// the share of the code offset of token `tok` from the sum of its inputs (half 0 or 1: of those 64; -1: of all); `at`:
+// behind the segment's rows
 __device__ __forceinline__ void act_tile_offset_share(unsigned char* at, int tok, int half, float sum, int bits) {
-  reinterpret_cast<float*>(at)[8 * half + tok] = -static_cast<float>(1 << (bits - 1)) * 5.9604644775390625e-8f * sum;
+  const float share = -static_cast<float>(1 << (bits - 1)) * 5.9604644775390625e-8f * sum;
+  if (half < 0) reinterpret_cast<float2*>(at)[tok] = make_float2(share, 0.0f);
+  else reinterpret_cast<float*>(at)[2 * tok + half] = share;
 }
 
 // byte offset of input n (inside its segment) in the row of token `tok`
@@ -95,7 +99,7 @@ __device__ __forceinline__ void act_tile_row(const __nv_bfloat16* __restrict__ s
       const unsigned group = 0xffu << (threadIdx.x & 24);
 #pragma unroll
       for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(group, sum, o);
-      if ((u & 7) == 0) act_tile_offset_share(tile + static_cast<size_t>(seg) * seg_bytes + ntok * 256, tok, 0, sum, bits);
+      if ((u & 7) == 0) act_tile_offset_share(tile + static_cast<size_t>(seg) * seg_bytes + ntok * 256, tok, -1, sum, bits);
     }
   }
   // a value the fp16 operand cannot hold was saturated: the result is no longer the definition's

@@ -24,9 +24,11 @@
 //     schedulers favour old warps.  Items are decoded 32 at a time by the lanes of the first; a
 //     feeding thread between eight computing warps needs about twenty cycles per instruction,
 //     and whatever it does per stage shows;
-//   * eight consumer warps take one 16-row tile of the stage each (gated projection: eight rows of
-//     w1 and the same eight of w3, so that the activation is formed in one lane).  Sixteen consumer
-//     warps per SM alone, out of shared memory, run at 12 / 7.3 / 3.5 TB/s of 8 / 4 / 2-bit codes (all read in place);
+//   * eight consumer warps take one 16-row tile of the stage each: eight rows of either box (gated projection: of
+//     w1 and the same eight of w3, so that the activation is formed in one lane).  The two rows of a lane then always lie
+//     one box apart, and with the lane's places worked out once per pass and the scales of a stage read as whole words a
+//     segment costs few instructions beside its unpacking (4 bits, 4 tokens of the Mixtral-like layer: 156 -> 149 per
+//     16 rows x 128 inputs, expert launch 129 -> 121 us; 768 x 3072, 32 experts, 64 tokens 37 -> 35 us);
 //   * up to 8 tokens per pass, 4 and 2 bits: a code field is read in place as the mantissa of a SUBNORMAL fp16
 //     number ((q + 2^(b-1)) * 2^(p-24) for a field at bit p): one logic instruction per pair of
 //     codes, one shift per word.  Fields at different positions go to accumulators of their own,
@@ -86,7 +88,6 @@ struct TmaArgs {
   int ksplit;         // split-K slices of the second projection
   int row_blocks[2];  // row blocks of an expert per projection
   int ngroups[2];     // scale groups per row, per projection
-  bool scale_pairs[2];  // one fp16 scale per segment, an even number of them per row, per projection
   unsigned gmul;      // scale group of segment s: (s * gmul) >> 20 (2^20 / segments per group, rounded up; 0: one group per row)
   int n_pairs;
   int* check_word;
@@ -147,30 +148,34 @@ __device__ __forceinline__ uint32_t code_exact(uint32_t w, int pos) {
 template <int BITS>
 __device__ __forceinline__ uint32_t code_one(uint32_t w, int pos) { return BITS == 8 ? code_exact<BITS>(w, pos) : code_sub<BITS>(w, pos); }
 
-// Where a lane finds its operands in a stage: its first row of codes (the 16-byte column of segment 0 under the
-// swizzle: the columns of later segments differ by an XOR), the distance to its second row, the even
-// chunks of the activation tile (the odd ones: XOR 64), the code offset's shares, and its rows' scales.
+// Where a lane finds its operands in a stage, from the stage's start.  Everything that does not change from stage to stage
+// is worked out once per pass: a segment's reads then are a register and a constant each.
 struct StageLane {
-  int row, drow, xe, init, sc, dsc;
-  bool halves;  // the offset's share comes in two halves
+  int row;      // its first row of codes, at the 16-byte column of segment 0 under the swizzle (the second: ROW2 behind it)
+  int d1, d2;   // to the columns of the next segment and of the one after that (the swizzle makes them differ from lane to lane)
+  int xe, xo;   // the even and the odd chunks of the activation tile
+  int init;     // the code offset's shares
+  int sc;       // the scales of its first row (the second's: SCALE2 behind it)
 };
+constexpr int ROW2 = ST_BOX_BYTES, SCALE2 = ST_BOX_ROWS * 16;  // a warp takes eight rows of each of the stage's two boxes
 
-// One segment (128 inputs) of the warp's 16 rows; SG: its index in the stage.
+// One segment (128 inputs) of the warp's 16 rows: codes at wp (8 bits: and wp + d1), activations at x0 / x1 (even and odd
+// chunks), the offset's shares at init.
 template <int BITS, int NT>
-__device__ __forceinline__ void consume_segment(const unsigned char* stage, const StageLane& p, int sg, int xoff, float s0, float s1,
-                                                float (&tot)[NT][4]) {
+__device__ __forceinline__ void consume_segment(const unsigned char* wp, int d1, const unsigned char* x0, const unsigned char* x1,
+                                                const unsigned char* init, float s0, float s1, float (&tot)[NT][4]) {
   constexpr int NW = BITS;  // 32-bit words of the lane's 32 codes of a row
   uint32_t w[2][NW];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     if constexpr (BITS == 2) {
-      const uint2 v = *reinterpret_cast<const uint2*>(stage + (p.row ^ (sg << 5)) + i * p.drow);
+      const uint2 v = *reinterpret_cast<const uint2*>(wp + i * ROW2);
       w[i][0] = v.x, w[i][1] = v.y;
     } else {
-      const uint4 v = *reinterpret_cast<const uint4*>(stage + (p.row ^ (BITS == 4 ? sg << 6 : 0)) + i * p.drow);
+      const uint4 v = *reinterpret_cast<const uint4*>(wp + i * ROW2);
       w[i][0] = v.x, w[i][1] = v.y, w[i][2] = v.z, w[i][3] = v.w;
       if constexpr (BITS == 8) {
-        const uint4 u = *reinterpret_cast<const uint4*>(stage + (p.row ^ 16) + i * p.drow);
+        const uint4 u = *reinterpret_cast<const uint4*>(wp + d1 + i * ROW2);
         w[i][4] = u.x, w[i][5] = u.y, w[i][6] = u.z, w[i][7] = u.w;
       }
     }
@@ -180,12 +185,8 @@ __device__ __forceinline__ void consume_segment(const unsigned char* stage, cons
     float acc[NC][4];
     float2 off = make_float2(0.0f, 0.0f);
     if constexpr (BITS != 8) {
-      off = *reinterpret_cast<const float2*>(stage + p.init + xoff);
-      if (p.halves) {
-        const float2 o2 = *reinterpret_cast<const float2*>(stage + p.init + xoff + 32);
-        off.x += o2.x;
-        off.y += o2.y;
-      }
+      const float4 o = *reinterpret_cast<const float4*>(init);
+      off = make_float2(o.x + o.y, o.z + o.w);
     }
     acc[0][0] = acc[0][2] = off.x;
     acc[0][1] = acc[0][3] = off.y;
@@ -195,7 +196,7 @@ __device__ __forceinline__ void consume_segment(const unsigned char* stage, cons
       for (int i = 0; i < 4; ++i) acc[c][i] = 0.0f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const uint4 b = *reinterpret_cast<const uint4*>(stage + (p.xe ^ ((q & 1) << 6)) + xoff + 128 * (q >> 1));
+      const uint4 b = *reinterpret_cast<const uint4*>((q & 1 ? x1 : x0) + 128 * (q >> 1));
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int m = 2 * q + j, pos = field_pos<BITS>(m);
@@ -232,7 +233,7 @@ __device__ __forceinline__ void consume_segment(const unsigned char* stage, cons
         }
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
-        const uint4 b = *reinterpret_cast<const uint4*>(stage + (p.xe ^ ((q & 1) << 6)) + xoff + 128 * (q >> 1) + nt * 2048);
+        const uint4 b = *reinterpret_cast<const uint4*>((q & 1 ? x1 : x0) + 128 * (q >> 1) + nt * 2048);
         mma_f16(acc[nt], c[0][0], c[1][0], c[0][1], c[1][1], b.x, b.y);
         mma_f16(acc[nt], c[0][2], c[1][2], c[0][3], c[1][3], b.z, b.w);
       }
@@ -261,7 +262,7 @@ __device__ __forceinline__ void count_item_done(PlanRec* recs, int ai, int lane)
 __device__ __forceinline__ __half hidden_half(float h) { return f32_to_f16_sat(__bfloat162float(__float2bfloat16_rn(h))); }
 __device__ __forceinline__ bool half_saturated(__half v) { return (__half_as_ushort(v) & 0x7fffu) == 0x7bffu; }
 
-// Hidden values of a first-projection item: the lane's results (rows gp, gp+8 x tokens 2t, 2t+1 of
+// Hidden values of a first-projection item: the lane's results (row gp of either box x tokens 2t, 2t+1 of
 // every 8-token tile) into the warp-shared tile segment in shared memory, in the order the second
 // projection reads them.
 template <int BITS, int NT>
@@ -301,7 +302,7 @@ __device__ __forceinline__ void hidden_to_smem(bool gated, int rb, int ntok, int
       for (int i = 0; i < 4; ++i) {
         const int tok = nt * 8 + 2 * t + (i & 1);
         if (tok < ntok) {
-          *reinterpret_cast<__half*>(hid + tok * 256 + act_tile_pos<BITS>(16 * warp + gp + 8 * (i >> 1), tok)) = hv[i];
+          *reinterpret_cast<__half*>(hid + tok * 256 + act_tile_pos<BITS>(8 * warp + gp + 64 * (i >> 1), tok)) = hv[i];
           beyond |= half_saturated(hv[i]);
         }
       }
@@ -329,7 +330,7 @@ __device__ __forceinline__ void hidden_to_global(const TmaArgs& a, bool gated, i
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       if (lane == 0) {
-        act_tile_offset_share(tile + ntok * 256, tok, half, sum, bits);
+        act_tile_offset_share(tile + ntok * 256, tok, gated ? half : -1, sum, bits);
       }
     }
   }
@@ -340,14 +341,14 @@ __device__ __forceinline__ void store_output(const TmaArgs& a, int rb, int z, in
                                              const float (&tot)[NT][4]) {
   const int g = lane >> 2, t = lane & 3;
   const int N = a.L.d_model;
-  float* dst = a.o_part + (static_cast<size_t>(z) * a.n_pairs + slot0) * N + rb * 128 + 16 * warp + box_row_of<BITS>(g);
+  float* dst = a.o_part + (static_cast<size_t>(z) * a.n_pairs + slot0) * N + rb * 128 + 8 * warp + box_row_of<BITS>(g);
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) {
     if (nt * 8 >= ntok) break;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int tok = nt * 8 + 2 * t + (i & 1);
-      if (tok < ntok) dst[static_cast<size_t>(tok) * N + 8 * (i >> 1)] = tot[nt][i];
+      if (tok < ntok) dst[static_cast<size_t>(tok) * N + ST_BOX_ROWS * (i >> 1)] = tot[nt][i];
     }
   }
 }
@@ -399,17 +400,20 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 
-template <bool SF16>
+// How a row's scales lie: one fp16 number per segment and an even number of them, so that a stage's are whole aligned
+// 4-byte words; fp16 or fp32 in any other number.
+constexpr int SC_PAIRS = 0, SC_F16 = 1, SC_F32 = 2;
+template <int SC>
 __device__ __forceinline__ float scale_at(const unsigned char* p) {
-  if constexpr (SF16) return __half2float(*reinterpret_cast<const __half*>(p));
+  if constexpr (SC != SC_F32) return __half2float(*reinterpret_cast<const __half*>(p));
   else return *reinterpret_cast<const float*>(p);
 }
+__device__ __forceinline__ float2 scale_pair(uint32_t w) { return __half22float2(*reinterpret_cast<const __half2*>(&w)); }
 
 // what the consumer warps share
 struct Pipe {
   const unsigned char* ring;
   unsigned char* hid_stage;
-  const int* offset;  // of the stage in a slot
   const ItemRec* queue;
   uint32_t bar_full, bar_empty, bar_issued, bar_hid;
   PlanRec* recs;
@@ -419,12 +423,16 @@ struct Pipe {
 // where a consumer warp stands
 struct Cursor {
   int it;          // next stage
+  int phys;        // ... and the first place in the ring for it
   int n_hidden;    // first-projection items stored so far
   int pending_ai;  // expert whose finished item is still to be counted (-1: none)
 };
 
+// bytes of a stage in the ring
+__device__ __forceinline__ int stage_bytes(int nseg, int xseg) { return nseg > 0 ? ST_X_OFFSET + ((nseg * xseg + 1023) & ~1023) : 0; }
+
 // One pass of an item by a consumer warp, its first stage having arrived: all its stages, then the results.
-template <int BITS, bool SF16, int NT>
+template <int BITS, int SC, int NT>
 __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, int k, int p0, int warp, int lane, Cursor& cur) {
   constexpr int SEGS = 8 / BITS;
   const ItemRec& rec = pp.queue[k % ST_QUEUE];
@@ -432,48 +440,69 @@ __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, i
   const int ntok = min(ACT_PASS_MAX, cnt - p0);
   const int phase = rec.flags & ITEM_SECOND ? 1 : 0;
   const bool gated = phase == 0 && a.L.act == EMOE_ACT_SWIGLU;
-  constexpr int ssz = SF16 ? 2 : 4;
+  constexpr int ssz = SC == SC_F32 ? 4 : 2;
   const int g = lane >> 2, t = lane & 3;
-  const int gp = box_row_of<BITS>(g);
+  const int gp = box_row_of<BITS>(g), row = 8 * warp + gp;  // in its box
   StageLane p;
-  // rows of a warp: 16 of one matrix, or eight of w1 (first box) and the same eight of w3 (second).  8 bits:
+  // eight rows of either box: of w1 and the same of w3, or of one matrix and those 64 further down.  8 bits:
   // columns 2t and 2t+1; 4 bits: column t of the segment's four; 2 bits: half of column t/2 of its two
-  p.row = ((gated ? 8 : 16) * warp + gp) * 128 + (((BITS == 8 ? 2 * t : (BITS == 4 ? t : t >> 1)) ^ gp) << 4) + (BITS == 2 ? (t & 1) << 3 : 0);
-  p.drow = gated ? ST_BOX_BYTES : 8 * 128;
+  p.row = row * 128 + (((BITS == 8 ? 2 * t : (BITS == 4 ? t : t >> 1)) ^ gp) << 4) + (BITS == 2 ? (t & 1) << 3 : 0);
+  p.d1 = (p.row ^ (BITS == 8 ? 16 : (BITS == 4 ? 64 : 32))) - p.row;
+  p.d2 = (p.row ^ 64) - p.row;  // (2 bits)
   p.xe = ST_X_OFFSET + g * 256 + t * 16 + ((g & 1) << 6);
-  p.init = ST_X_OFFSET + ntok * 256 + t * 8;
-  p.halves = phase == 1 && a.L.act == EMOE_ACT_SWIGLU;
+  p.xo = p.xe ^ 64;
+  p.init = ST_X_OFFSET + ntok * 256 + t * 16;
   const int xstride = act_seg_bytes(ntok);
+  const int need_full = stage_bytes(SEGS, xstride), need_last = stage_bytes(last, xstride);
   float tot[NT][4];
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
     for (int i = 0; i < 4; ++i) tot[nt][i] = 0.0f;
   // scales: 16 bytes per row of the stage, from the 4-byte boundary at or below the first one
-  p.sc = 2 * ST_BOX_BYTES + ((gated ? 8 : 16) * warp + gp) * 16;
-  p.dsc = gated ? ST_BOX_ROWS * 16 : 8 * 16;
-  const int row_bytes = a.ngroups[phase] * ssz, row_off = (rec.row0 + (gated ? 8 : 16) * warp + gp) * row_bytes;
+  p.sc = 2 * ST_BOX_BYTES + row * 16;
+  const int row_off = (rec.row0 + row) * a.ngroups[phase] * ssz;
 #pragma unroll 1
   for (int s = 0; s < nst; ++s) {
-    const int slot = cur.it % ST_SLOTS;
+    const int slot = cur.it % ST_SLOTS, need = s == nst - 1 ? need_last : need_full;
+    if (cur.phys + need > ST_RING) cur.phys = 0;  // as the weight warp places it
+    const unsigned char* stage = pp.ring + cur.phys;
+    cur.phys += need;
     if (s > 0 && !__all_sync(0xffffffffu, mbar_wait(pp.bar_full + 8 * slot, (cur.it / ST_SLOTS) & 1, a.check_word, pp.abort_flag)))
       return false;
-    const unsigned char* stage = pp.ring + pp.offset[slot];
-    const int seg = seg0 + s * SEGS, g0 = group_of_seg(a, seg);
-    const unsigned char* sc = stage + p.sc + ((row_off + g0 * ssz) & 3);
-    const int nseg = s == nst - 1 ? last : SEGS;
-    if (nseg == SEGS) {
+    const int seg = seg0 + s * SEGS, nseg = s == nst - 1 ? last : SEGS;
+    const unsigned char *wp = stage + p.row, *x0 = stage + p.xe, *x1 = stage + p.xo, *init = stage + p.init, *sc = stage + p.sc;
+    uint32_t sw[2][2];
+    int g0 = 0;
+    if constexpr (SC == SC_PAIRS) {
 #pragma unroll
-      for (int sg = 0; sg < SEGS; ++sg) {
-        const int d = sg == 0 ? 0 : (group_of_seg(a, seg + sg) - g0) * ssz;
-        consume_segment<BITS, NT>(stage, p, sg, sg * xstride, scale_at<SF16>(sc + d), scale_at<SF16>(sc + d + p.dsc), tot);
+      for (int i = 0; i < 2; ++i) {
+        if constexpr (BITS == 8) {
+          sw[i][0] = *reinterpret_cast<const unsigned short*>(sc + i * SCALE2 + 2 * (seg & 1));
+        } else if constexpr (BITS == 4) {
+          sw[i][0] = *reinterpret_cast<const uint32_t*>(sc + i * SCALE2);
+        } else {
+          const uint2 v = *reinterpret_cast<const uint2*>(sc + i * SCALE2);
+          sw[i][0] = v.x, sw[i][1] = v.y;
+        }
       }
     } else {
-#pragma unroll 1
-      for (int sg = 0; sg < nseg; ++sg) {
-        const int d = (group_of_seg(a, seg + sg) - g0) * ssz;
-        consume_segment<BITS, NT>(stage, p, sg, sg * xstride, scale_at<SF16>(sc + d), scale_at<SF16>(sc + d + p.dsc), tot);
+      g0 = group_of_seg(a, seg);
+      sc += (row_off + g0 * ssz) & 3;
+    }
+#pragma unroll
+    for (int sg = 0; sg < SEGS; ++sg) {
+      if (sg >= nseg) break;
+      float s0, s1;
+      if constexpr (SC == SC_PAIRS) {
+        const float2 u0 = scale_pair(sw[0][sg >> 1]), u1 = scale_pair(sw[1][sg >> 1]);
+        s0 = sg & 1 ? u0.y : u0.x, s1 = sg & 1 ? u1.y : u1.x;
+      } else {
+        const int d = sg == 0 ? 0 : (group_of_seg(a, seg + sg) - g0) * ssz;
+        s0 = scale_at<SC>(sc + d), s1 = scale_at<SC>(sc + d + SCALE2);
       }
+      const unsigned char* w = BITS == 2 ? wp + (sg & 1 ? p.d1 : 0) + (sg & 2 ? p.d2 : 0) : wp + (BITS == 4 && sg ? p.d1 : 0);
+      consume_segment<BITS, NT>(w, p.d1, x0 + sg * xstride, x1 + sg * xstride, init + sg * xstride, s0, s1, tot);
     }
     // shared memory of the stage is no longer needed
     __syncwarp();
@@ -506,7 +535,7 @@ __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, i
   return true;
 }
 
-template <bool SF16>
+template <int SC>
 __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __grid_constant__ TmaArgs a) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bars[3 * ST_SLOTS + 1];  // full, empty, issued (weight warp -> activation warp), hidden segment staged
@@ -590,8 +619,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
           const int c_first = rec.seg0 * 16 * bits;  // byte column: 128 inputs = 16 * bits bytes
           for (int p0 = 0; p0 < cnt && more; p0 += ACT_PASS_MAX) {
             const int xseg = act_seg_bytes(min(ACT_PASS_MAX, cnt - p0));
-            const int need_full = ST_X_OFFSET + (((8 / bits) * xseg + 1023) & ~1023);
-            const int need_last = last > 0 ? ST_X_OFFSET + ((last * xseg + 1023) & ~1023) : 0;
+            const int need_full = stage_bytes(8 / bits, xseg), need_last = stage_bytes(last, xseg);
             for (int s = 0, c0 = c_first; s < nst; ++s, ++it, c0 += 128) {
               const int need = s == nst - 1 ? need_last : need_full;
               if (phys + need > ST_RING) {  // does not fit in front of the end of the ring
@@ -644,7 +672,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
       }
       const int phase = flags & ITEM_SECOND ? 1 : 0, bits = flags >> 8, nst = rec.nst, last = rec.last, cnt = rec.cnt, seg0 = rec.seg0;
       const bool gated = phase == 0 && L.act == EMOE_ACT_SWIGLU;
-      constexpr int ssz = SF16 ? 2 : 4;
+      constexpr int ssz = SC == SC_F32 ? 4 : 2;
       // the lane's rows of the stage: lane, lane + 32, ...
       const int row_bytes = a.ngroups[phase] * ssz;
       const char* sc_a = rec.scales[0];
@@ -653,7 +681,6 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         sc_row[i] = (gated && i >= 2 ? sc_b : sc_a) + static_cast<size_t>(rec.row0 + (gated ? (lane + 32 * i) & 63 : lane + 32 * i)) * row_bytes;
-      const bool pairs = a.scale_pairs[phase];
       {  // pull the item's scales towards L2, where the copies below find them
         for (int b = lane * 128; b < (gated ? ST_BOX_ROWS : 2 * ST_BOX_ROWS) * row_bytes && (phase == 0 || a.ksplit == 1); b += 32 * 128) {
           asm volatile("prefetch.global.L2 [%0];" ::"l"(sc_a + static_cast<size_t>(rec.row0) * row_bytes + b));
@@ -706,7 +733,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
             src += nseg * xseg;
             const int seg = seg0 + s * (8 / bits);
             const uint32_t dst = st + 2 * ST_BOX_BYTES + lane * 16;
-            if (pairs) {  // one scale per segment, rows of whole 4-byte words: one word, or two at 2 bits
+            if constexpr (SC == SC_PAIRS) {  // one word, or two at 2 bits
               const int b0 = (seg * 2) & ~3;
 #pragma unroll
               for (int i = 0; i < 4; ++i) cp_async4(dst + 512 * i, sc_row[i] + b0);
@@ -733,11 +760,11 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
     }
   } else {
     // ---------------- consumer warps ----------------
-    const Pipe pp = {ring, hid_stage, s_offset, queue, bar_full, bar_empty, bar_issued, bar_hid, recs, fused, abort_flag};
+    const Pipe pp = {ring, hid_stage, queue, bar_full, bar_empty, bar_issued, bar_hid, recs, fused, abort_flag};
     // A finished first-projection item is counted one stage late: by then its stores have long
     // been acknowledged and the fence in front of the count costs nothing.  It is never held back
     // across a wait, because the stage waited for may be the one that waits for this count.
-    Cursor cur = {0, 0, -1};
+    Cursor cur = {0, 0, 0, -1};
     bool ok = true;
     for (int k = 0, p0 = 0; ok;) {
       const int slot = cur.it % ST_SLOTS;
@@ -752,15 +779,15 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
       if (flags & ITEM_STOP) break;
       if (cnt - p0 <= 8) {
         switch (flags >> 8) {
-          case 2: ok = consume_pass<2, SF16, 1>(a, pp, k, p0, warp, lane, cur); break;
-          case 4: ok = consume_pass<4, SF16, 1>(a, pp, k, p0, warp, lane, cur); break;
-          default: ok = consume_pass<8, SF16, 1>(a, pp, k, p0, warp, lane, cur); break;
+          case 2: ok = consume_pass<2, SC, 1>(a, pp, k, p0, warp, lane, cur); break;
+          case 4: ok = consume_pass<4, SC, 1>(a, pp, k, p0, warp, lane, cur); break;
+          default: ok = consume_pass<8, SC, 1>(a, pp, k, p0, warp, lane, cur); break;
         }
       } else {
         switch (flags >> 8) {
-          case 2: ok = consume_pass<2, SF16, 2>(a, pp, k, p0, warp, lane, cur); break;
-          case 4: ok = consume_pass<4, SF16, 2>(a, pp, k, p0, warp, lane, cur); break;
-          default: ok = consume_pass<8, SF16, 2>(a, pp, k, p0, warp, lane, cur); break;
+          case 2: ok = consume_pass<2, SC, 2>(a, pp, k, p0, warp, lane, cur); break;
+          case 4: ok = consume_pass<4, SC, 2>(a, pp, k, p0, warp, lane, cur); break;
+          default: ok = consume_pass<8, SC, 2>(a, pp, k, p0, warp, lane, cur); break;
         }
       }
       p0 += ACT_PASS_MAX;
@@ -779,25 +806,25 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
   }
 }
 
-template <bool SF16>
-cudaError_t launch_sf(const TmaArgs& a, long long items, cudaStream_t st) {
+template <int SC>
+cudaError_t launch_sc(const TmaArgs& a, long long items, cudaStream_t st) {
   static int ctas_per_device[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!ctas_per_device[dev]) {
-    e = cudaFuncSetAttribute(ffn_tma_kernel<SF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM);
+    e = cudaFuncSetAttribute(ffn_tma_kernel<SC>, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM);
     if (e != cudaSuccess) return e;
     int per_sm = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ffn_tma_kernel<SF16>, ST_THREADS, ST_SMEM);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ffn_tma_kernel<SC>, ST_THREADS, ST_SMEM);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     ctas_per_device[dev] = (per_sm > 0 ? per_sm : 1) * sms;
   }
   const int grid = items < ctas_per_device[dev] ? static_cast<int>(items) : ctas_per_device[dev];
-  return launch_chain(ffn_tma_kernel<SF16>, dim3(grid), dim3(ST_THREADS), ST_SMEM, st, a);
+  return launch_chain(ffn_tma_kernel<SC>, dim3(grid), dim3(ST_THREADS), ST_SMEM, st, a);
 }
 
 }  // namespace
@@ -854,7 +881,6 @@ cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, c
   a.ngroups[0] = L.group > 0 ? L.d_model / L.group : 1;
   a.ngroups[1] = L.group > 0 ? L.d_ff / L.group : 1;
   a.gmul = L.group > 0 ? ((1u << 20) + static_cast<unsigned>(L.group / 128) - 1) / static_cast<unsigned>(L.group / 128) : 0u;
-  for (int p = 0; p < 2; ++p) a.scale_pairs[p] = L.scale_f16 && L.group == 128 && a.ngroups[p] % 2 == 0;
   a.n_pairs = n_pairs;
   a.check_word = check_word;
   for (int p = 0; p < 2; ++p) {
@@ -868,7 +894,9 @@ cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, c
   if (phase_begin == 0) per_expert += a.row_blocks[0];
   if (phase_end == 2) per_expert += static_cast<long long>(a.row_blocks[1]) * ksplit;
   const long long items = active_max * per_expert;
-  return L.scale_f16 ? launch_sf<true>(a, items, st) : launch_sf<false>(a, items, st);
+  if (!L.scale_f16) return launch_sc<SC_F32>(a, items, st);
+  const bool pairs = L.group == 128 && a.ngroups[0] % 2 == 0 && a.ngroups[1] % 2 == 0;
+  return pairs ? launch_sc<SC_PAIRS>(a, items, st) : launch_sc<SC_F16>(a, items, st);
 }
 
 // Host-side tensor-map encoder (driver entry point looked up once; no link against libcuda).
