@@ -47,6 +47,8 @@
 // in place, which is not exact), 2 bits 1.8 -> 2.15.
 #include <cuda.h>
 
+#include <climits>
+
 #include "act_tile.cuh"
 #include "common.cuh"
 #include "ffn_tile.cuh"
@@ -353,19 +355,8 @@ __device__ __forceinline__ void store_output(const TmaArgs& a, int rb, int z, in
   }
 }
 
-// Item k of the CTA's list, decoded by one thread.  Every CTA takes every gridDim.x-th item: the items of the
-// first projection, then those of the second, most expensive bitwidth first, so that the shares are even to
-// about one of the cheapest items; the list is known without asking, 32 items are decoded at a time.
-__device__ __forceinline__ void decode_item(const TmaArgs& a, const PlanRec* s_plan, const PlanRec* recs, int n_active, int k, ItemRec* out) {
-  const int n_items0 = a.phase_begin == 0 ? n_active * a.row_blocks[0] : 0;
-  const int n_items1 = a.phase_end == 2 ? n_active * a.row_blocks[1] * a.ksplit : 0;
-  const int item = static_cast<int>(blockIdx.x) + k * static_cast<int>(gridDim.x);
-  if (item >= n_items0 + n_items1) {
-    out->flags = ITEM_STOP;
-    return;
-  }
-  const int phase = item < n_items0 ? 0 : 1;
-  const int li = item - (phase == 0 ? 0 : n_items0);
+// Item li of a projection, decoded by one thread.  The items are listed by expert, most expensive bitwidth first.
+__device__ __forceinline__ void decode_item(const TmaArgs& a, const PlanRec* s_plan, const PlanRec* recs, int phase, int li, ItemRec* out) {
   const bool gated = phase == 0 && a.L.act == EMOE_ACT_SWIGLU;
   const int row_blocks = a.row_blocks[phase], ksplit = phase == 0 ? 1 : a.ksplit;
   const int mat_first = phase == 0 ? 0 : (a.L.act == EMOE_ACT_SWIGLU ? 2 : 1);
@@ -593,13 +584,27 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
     // beginning again.  head and vstart are positions on an endless tape; a stage may be written
     // once nothing live lies within a ring's length behind its end.  This thread feeds eight
     // computing warps: whatever it does per stage is kept to a few instructions.
+    // Every CTA takes every n-th item of the first projection and, going on so, one of the second; these are known without
+    // asking and decoded 32 at a time.  From then on whoever is free claims the next one (one claim ahead, so that nobody
+    // waits for the answer).
+    const int n = static_cast<int>(gridDim.x), me = static_cast<int>(blockIdx.x);
+    const int n_items0 = a.phase_begin == 0 ? s_active * a.row_blocks[0] : 0, n_items1 = a.phase_end == 2 ? s_active * a.row_blocks[1] * a.ksplit : 0;
+    const int n_fixed = n_items0 + min(n, n_items1);
     int it = 0, oldest = 0, head = 0, phys = 0;
-    int more = 1;
+    int more = 1, claim = n_items1;
     for (int k0 = 0; more; k0 += 32) {
-      decode_item(a, s_plan, recs, s_active, k0 + lane, &queue[(k0 + lane) % ST_QUEUE]);
+      const int item = me + (k0 + lane) * n;
+      ItemRec* out = &queue[(k0 + lane) % ST_QUEUE];
+      if (item < n_fixed) decode_item(a, s_plan, recs, item < n_items0 ? 0 : 1, item < n_items0 ? item : item - n_items0, out);
+      else out->flags = ITEM_STOP;
       __syncwarp();
       if (lane == 0) {
         for (int k = k0; k < k0 + 32 && more; ++k) {
+          if (n_items1 > n && me + (k + 1) * n >= n_fixed) {  // this item is the last known one, or a claimed one
+            const int now = claim;
+            claim = n + atomicAdd(a.plan + 1, 1);
+            if (me + k * n >= n_fixed && now < n_items1) decode_item(a, s_plan, recs, 1, now, &queue[k % ST_QUEUE]);
+          }
           const ItemRec& rec = queue[k % ST_QUEUE];
           const int flags = rec.flags;
           if (flags & ITEM_STOP) {  // tell the others that nothing else comes
