@@ -7,9 +7,10 @@
 // products accumulate in fp32 per 128-input segment, then total += scale * segment.  The work is
 // bound by streaming packed weights from HBM and, at 4 and 2 bits, by the logic pipe (one
 // instruction per pair of codes, at half the issue rate), so both are kept lean:
-//   * the kernel is persistent and runs BOTH projections of a layer.  Every CTA takes every n-th item of
-//     a list: the first projection's (activated expert, block of output rows), then the second's
-//     (.., split-K slice), most expensive bitwidth first.  The stream runs ahead across items, so
+//   * the kernel is persistent and runs BOTH projections of a layer.  The items are the first projection's (activated
+//     expert, block of output rows), then the second's (.., split-K slice), most expensive bitwidth first.  A CTA takes every
+//     n-th of the first and whichever is next of the second (fixed shares let the slowest CTA end a tenth of the launch
+//     behind the others; Mixtral-like layer, 4 tokens 133 -> 125 us).  The stream runs ahead across items, so
 //     it never drains between tiles; an item of the second projection waits until the expert's
 //     hidden vectors are complete (release / acquire on a counter in the expert's plan record);
 //   * a stage holds two 64-row x 128-byte boxes of packed codes (two TMA tensor copies, 128-byte
@@ -24,7 +25,7 @@
 //     schedulers favour old warps.  Items are decoded 32 at a time by the lanes of the first; a
 //     feeding thread between eight computing warps needs about twenty cycles per instruction,
 //     and whatever it does per stage shows;
-//   * eight consumer warps take one 16-row tile of the stage each: eight rows of either box (gated projection: of
+//   * eight consumer warps take one 16-row tile of the stage each, or four warps two (see the launch): eight rows of either box (gated projection: of
 //     w1 and the same eight of w3, so that the activation is formed in one lane).  The two rows of a lane then always lie
 //     one box apart, and with the lane's places worked out once per pass and the scales of a stage read as whole words a
 //     segment costs few instructions beside its unpacking (4 bits, 4 tokens of the Mixtral-like layer: 156 -> 149 per
@@ -41,10 +42,10 @@
 // scale segments.  Every wait is bounded: a wait that runs out sets a bit in the context's
 // check word and the CTA winds down without touching the stage.
 //
-// Measured (expert launch alone, start of comparison: one feeding and four computing warps per CTA, three CTAs,
-// 16 / 8-token tiles by the launch's mean): Mixtral-like layer (d 4096, f 14336), 23 tokens 245 -> 217 us
-// (3.8 TB/s of packed bytes), 4 tokens of 4-bit experts 2.8 -> 3.6 TB/s, 8 bits 4.7 -> 4.85 (5.0 with the codes read
-// in place, which is not exact), 2 bits 1.8 -> 2.15.
+// Measured (expert launch alone; one feeding and four computing warps per CTA, three CTAs -> eight computing warps, fixed items
+// -> now): Mixtral-like layer (d 4096, f 14336), 23 tokens 245 -> 223 -> 200 us (4.1 TB/s of packed bytes), 4 tokens 143 -> 121
+// (4.3); of 8-bit experts 4.7 -> 4.7 -> 5.35 TB/s, 4 bits 2.8 -> 3.5 -> 4.1, 2 bits 1.8 -> 2.1 -> 2.5; 768 x 3072, 32 experts, 64 tokens
+// 37 -> 35.5 us.  With the consumers idle the same launch takes 103 us at 4 tokens, with nothing loaded 113.
 #include <cuda.h>
 
 #include <climits>
@@ -57,11 +58,13 @@
 namespace emoe {
 namespace {
 
-constexpr int ST_WARPS = 8;                      // consumer warps of a CTA
-constexpr int ST_THREADS = (ST_WARPS + 2) * 32;  // + the weight warp and the activation warp
+// A CTA has W consumer warps, eight or four, which take one or two 16-row tiles of every stage, and the weight and the
+// activation warp.
+__host__ __device__ constexpr int st_threads(int w) { return (w + 2) * 32; }
 constexpr int ST_PLAN_CACHE = 64;                // plan records a CTA keeps in shared memory
 constexpr int ST_CTAS = 2;                       // per SM
 constexpr int ST_BOX_ROWS = 64;
+__host__ __device__ constexpr int st_tiles(int w) { return ST_BOX_ROWS / (8 * w); }  // 16-row tiles of a warp: eight rows of each box per tile
 constexpr int ST_BOX_BYTES = ST_BOX_ROWS * 128;  // 8 KB
 constexpr int ST_X_OFFSET = 2 * ST_BOX_BYTES + 2 * ST_BOX_ROWS * 16;  // a stage: two boxes, 16 bytes of scales per row, the activation slice
 constexpr int ST_RING = 96 * 1024;
@@ -161,89 +164,108 @@ struct StageLane {
 };
 constexpr int ROW2 = ST_BOX_BYTES, SCALE2 = ST_BOX_ROWS * 16;  // a warp takes eight rows of each of the stage's two boxes
 
-// One segment (128 inputs) of the warp's 16 rows: codes at wp (8 bits: and wp + d1), activations at x0 / x1 (even and odd
-// chunks), the offset's shares at init.
-template <int BITS, int NT>
+// One segment (128 inputs) of the warp's tiles: codes at wp (8 bits: and wp + d1), activations at x0 / x1 (even and odd
+// chunks), the offset's shares at init; sc: the rows' scales.
+template <int BITS, int NT, int TILES>
 __device__ __forceinline__ void consume_segment(const unsigned char* wp, int d1, const unsigned char* x0, const unsigned char* x1,
-                                                const unsigned char* init, float s0, float s1, float (&tot)[NT][4]) {
+                                                const unsigned char* init, const float (&sc)[TILES][2], float (&tot)[TILES][NT][4]) {
   constexpr int NW = BITS;  // 32-bit words of the lane's 32 codes of a row
-  uint32_t w[2][NW];
+  uint32_t w[TILES][2][NW];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    if constexpr (BITS == 2) {
-      const uint2 v = *reinterpret_cast<const uint2*>(wp + i * ROW2);
-      w[i][0] = v.x, w[i][1] = v.y;
-    } else {
-      const uint4 v = *reinterpret_cast<const uint4*>(wp + i * ROW2);
-      w[i][0] = v.x, w[i][1] = v.y, w[i][2] = v.z, w[i][3] = v.w;
-      if constexpr (BITS == 8) {
-        const uint4 u = *reinterpret_cast<const uint4*>(wp + d1 + i * ROW2);
-        w[i][4] = u.x, w[i][5] = u.y, w[i][6] = u.z, w[i][7] = u.w;
+  for (int j = 0; j < TILES; ++j)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const unsigned char* at = wp + i * ROW2 + j * 1024;
+      if constexpr (BITS == 2) {
+        const uint2 v = *reinterpret_cast<const uint2*>(at);
+        w[j][i][0] = v.x, w[j][i][1] = v.y;
+      } else {
+        const uint4 v = *reinterpret_cast<const uint4*>(at);
+        w[j][i][0] = v.x, w[j][i][1] = v.y, w[j][i][2] = v.z, w[j][i][3] = v.w;
+        if constexpr (BITS == 8) {
+          const uint4 u = *reinterpret_cast<const uint4*>(at + d1);
+          w[j][i][4] = u.x, w[j][i][5] = u.y, w[j][i][6] = u.z, w[j][i][7] = u.w;
+        }
       }
     }
-  }
   if constexpr (NT == 1) {
     constexpr int NC = BITS == 2 ? 4 : 2;
-    float acc[NC][4];
+    float acc[TILES][NC][4];
     float2 off = make_float2(0.0f, 0.0f);
     if constexpr (BITS != 8) {
       const float4 o = *reinterpret_cast<const float4*>(init);
       off = make_float2(o.x + o.y, o.z + o.w);
     }
-    acc[0][0] = acc[0][2] = off.x;
-    acc[0][1] = acc[0][3] = off.y;
 #pragma unroll
-    for (int c = 1; c < NC; ++c)
+    for (int j = 0; j < TILES; ++j) {
+      acc[j][0][0] = acc[j][0][2] = off.x;
+      acc[j][0][1] = acc[j][0][3] = off.y;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) acc[c][i] = 0.0f;
+      for (int c = 1; c < NC; ++c)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[j][c][i] = 0.0f;
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const uint4 b = *reinterpret_cast<const uint4*>((q & 1 ? x1 : x0) + 128 * (q >> 1));
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int m = 2 * q + j, pos = field_pos<BITS>(m);
-        const uint32_t u0 = w[0][word_of<BITS>(m)], u1 = w[1][word_of<BITS>(m)];
-        mma_f16(acc[code_class<BITS>(m)], code_one<BITS>(u0, pos), code_one<BITS>(u1, pos), code_one<BITS>(u0 >> 8, pos),
-                code_one<BITS>(u1 >> 8, pos), j ? b.z : b.x, j ? b.w : b.y);
+      for (int h = 0; h < 2; ++h) {
+        const int m = 2 * q + h, pos = field_pos<BITS>(m);
+#pragma unroll
+        for (int j = 0; j < TILES; ++j) {
+          const uint32_t u0 = w[j][0][word_of<BITS>(m)], u1 = w[j][1][word_of<BITS>(m)];
+          mma_f16(acc[j][code_class<BITS>(m)], code_one<BITS>(u0, pos), code_one<BITS>(u1, pos), code_one<BITS>(u0 >> 8, pos),
+                  code_one<BITS>(u1 >> 8, pos), h ? b.z : b.x, h ? b.w : b.y);
+        }
       }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float v;
-      if constexpr (BITS == 8) v = acc[0][i] + acc[1][i];
-      else if constexpr (BITS == 4) v = fmaf(acc[1][i], 0.0625f, acc[0][i]);
-      else v = fmaf(fmaf(acc[3][i], 0.25f, acc[2][i]), 0.0625f, fmaf(acc[1][i], 0.25f, acc[0][i]));
-      tot[0][i] = fmaf(i < 2 ? s0 : s1, v, tot[0][i]);
-    }
+    for (int j = 0; j < TILES; ++j)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float v;
+        if constexpr (BITS == 8) v = acc[j][0][i] + acc[j][1][i];
+        else if constexpr (BITS == 4) v = fmaf(acc[j][1][i], 0.0625f, acc[j][0][i]);
+        else v = fmaf(fmaf(acc[j][3][i], 0.25f, acc[j][2][i]), 0.0625f, fmaf(acc[j][1][i], 0.25f, acc[j][0][i]));
+        tot[j][0][i] = fmaf(sc[j][i >> 1], v, tot[j][0][i]);
+      }
   } else {
-    float acc[NT][4];
+    float acc[TILES][NT][4];
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
+    for (int j = 0; j < TILES; ++j)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) acc[nt][i] = 0.0f;
+      for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[j][nt][i] = 0.0f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      uint32_t c[2][4];
+      uint32_t c[TILES][2][4];
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
+      for (int j = 0; j < TILES; ++j)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int m = 2 * q + j, pos = field_pos<BITS>(m);
-          const uint32_t u = w[i][word_of<BITS>(m)];
-          c[i][2 * j] = code_exact<BITS>(u, pos);
-          c[i][2 * j + 1] = code_exact<BITS>(u >> 8, pos);
-        }
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int m = 2 * q + h, pos = field_pos<BITS>(m);
+            const uint32_t u = w[j][i][word_of<BITS>(m)];
+            c[j][i][2 * h] = code_exact<BITS>(u, pos);
+            c[j][i][2 * h + 1] = code_exact<BITS>(u >> 8, pos);
+          }
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
         const uint4 b = *reinterpret_cast<const uint4*>((q & 1 ? x1 : x0) + 128 * (q >> 1) + nt * 2048);
-        mma_f16(acc[nt], c[0][0], c[1][0], c[0][1], c[1][1], b.x, b.y);
-        mma_f16(acc[nt], c[0][2], c[1][2], c[0][3], c[1][3], b.z, b.w);
+#pragma unroll
+        for (int j = 0; j < TILES; ++j) mma_f16(acc[j][nt], c[j][0][0], c[j][1][0], c[j][0][1], c[j][1][1], b.x, b.y);
+#pragma unroll
+        for (int j = 0; j < TILES; ++j) mma_f16(acc[j][nt], c[j][0][2], c[j][1][2], c[j][0][3], c[j][1][3], b.z, b.w);
       }
     }
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
+    for (int j = 0; j < TILES; ++j)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) tot[nt][i] = fmaf(i < 2 ? s0 : s1, acc[nt][i], tot[nt][i]);
+      for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tot[j][nt][i] = fmaf(sc[j][i >> 1], acc[j][nt][i], tot[j][nt][i]);
   }
 }
 
@@ -268,13 +290,12 @@ __device__ __forceinline__ bool half_saturated(__half v) { return (__half_as_ush
 // every 8-token tile) into the warp-shared tile segment in shared memory, in the order the second
 // projection reads them.
 template <int BITS, int NT>
-__device__ __forceinline__ void hidden_to_smem(bool gated, int rb, int ntok, int warp, int lane, const float (&tot)[NT][4],
+__device__ __forceinline__ void hidden_to_smem(bool gated, int rb, int ntok, int row, int lane, const float (&tot)[NT][4],
                                                unsigned char* hid, int* check_word) {
-  const int g = lane >> 2, t = lane & 3;
-  const int gp = box_row_of<BITS>(g);
+  const int t = lane & 3;
   bool beyond = false;
   if (gated) {
-    const int n = (rb & 1) * 64 + 8 * warp + gp;  // channel inside its 128-input segment
+    const int n = (rb & 1) * 64 + row;  // channel inside its 128-input segment
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
       if (nt * 8 >= ntok) break;
@@ -304,7 +325,7 @@ __device__ __forceinline__ void hidden_to_smem(bool gated, int rb, int ntok, int
       for (int i = 0; i < 4; ++i) {
         const int tok = nt * 8 + 2 * t + (i & 1);
         if (tok < ntok) {
-          *reinterpret_cast<__half*>(hid + tok * 256 + act_tile_pos<BITS>(8 * warp + gp + 64 * (i >> 1), tok)) = hv[i];
+          *reinterpret_cast<__half*>(hid + tok * 256 + act_tile_pos<BITS>(row + 64 * (i >> 1), tok)) = hv[i];
           beyond |= half_saturated(hv[i]);
         }
       }
@@ -316,11 +337,11 @@ __device__ __forceinline__ void hidden_to_smem(bool gated, int rb, int ntok, int
 // The staged segment to global memory, a warp per token: 8 bytes per lane, and the sum of the
 // token's values for the offset codes of the second projection.
 __device__ __forceinline__ void hidden_to_global(const TmaArgs& a, bool gated, int rb, int slot0, int ntok, int bits, int warp,
-                                                 int lane, const unsigned char* hid) {
+                                                 int warps, int lane, const unsigned char* hid) {
   const int seg = gated ? rb >> 1 : rb, half = gated ? rb & 1 : 0;
   unsigned char* tile = a.hidden + act_tile_offset(slot0, a.L.d_ff) + static_cast<size_t>(seg) * act_seg_bytes(ntok);
   const bool mine = !gated || ((lane >> 2) & 1) == half;  // a gated item fills half of the segment: inputs of lanes t = 2*half, 2*half+1
-  for (int tok = warp; tok < ntok; tok += ST_WARPS) {
+  for (int tok = warp; tok < ntok; tok += warps) {
     float sum = 0.0f;
     if (mine) {
       const uint2 v = *reinterpret_cast<const uint2*>(hid + tok * 256 + lane * 8);
@@ -339,11 +360,11 @@ __device__ __forceinline__ void hidden_to_global(const TmaArgs& a, bool gated, i
 }
 
 template <int BITS, int NT>
-__device__ __forceinline__ void store_output(const TmaArgs& a, int rb, int z, int slot0, int ntok, int warp, int lane,
+__device__ __forceinline__ void store_output(const TmaArgs& a, int rb, int z, int slot0, int ntok, int row, int lane,
                                              const float (&tot)[NT][4]) {
-  const int g = lane >> 2, t = lane & 3;
+  const int t = lane & 3;
   const int N = a.L.d_model;
-  float* dst = a.o_part + (static_cast<size_t>(z) * a.n_pairs + slot0) * N + rb * 128 + 8 * warp + box_row_of<BITS>(g);
+  float* dst = a.o_part + (static_cast<size_t>(z) * a.n_pairs + slot0) * N + rb * 128 + row;
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) {
     if (nt * 8 >= ntok) break;
@@ -423,9 +444,9 @@ struct Cursor {
 __device__ __forceinline__ int stage_bytes(int nseg, int xseg) { return nseg > 0 ? ST_X_OFFSET + ((nseg * xseg + 1023) & ~1023) : 0; }
 
 // One pass of an item by a consumer warp, its first stage having arrived: all its stages, then the results.
-template <int BITS, int SC, int NT>
+template <int BITS, int SC, int NT, int W>
 __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, int k, int p0, int warp, int lane, Cursor& cur) {
-  constexpr int SEGS = 8 / BITS;
+  constexpr int SEGS = 8 / BITS, TILES = st_tiles(W);
   const ItemRec& rec = pp.queue[k % ST_QUEUE];
   const int nst = rec.nst, seg0 = rec.seg0, last = rec.last, cnt = rec.cnt, tok0 = rec.begin + p0;
   const int ntok = min(ACT_PASS_MAX, cnt - p0);
@@ -433,9 +454,9 @@ __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, i
   const bool gated = phase == 0 && a.L.act == EMOE_ACT_SWIGLU;
   constexpr int ssz = SC == SC_F32 ? 4 : 2;
   const int g = lane >> 2, t = lane & 3;
-  const int gp = box_row_of<BITS>(g), row = 8 * warp + gp;  // in its box
+  const int gp = box_row_of<BITS>(g), row = 8 * TILES * warp + gp;  // in its box; of the warp's next tile: eight further down
   StageLane p;
-  // eight rows of either box: of w1 and the same of w3, or of one matrix and those 64 further down.  8 bits:
+  // a tile has eight rows of either box: of w1 and the same of w3, or of one matrix and those 64 further down.  8 bits:
   // columns 2t and 2t+1; 4 bits: column t of the segment's four; 2 bits: half of column t/2 of its two
   p.row = row * 128 + (((BITS == 8 ? 2 * t : (BITS == 4 ? t : t >> 1)) ^ gp) << 4) + (BITS == 2 ? (t & 1) << 3 : 0);
   p.d1 = (p.row ^ (BITS == 8 ? 16 : (BITS == 4 ? 64 : 32))) - p.row;
@@ -445,11 +466,13 @@ __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, i
   p.init = ST_X_OFFSET + ntok * 256 + t * 16;
   const int xstride = act_seg_bytes(ntok);
   const int need_full = stage_bytes(SEGS, xstride), need_last = stage_bytes(last, xstride);
-  float tot[NT][4];
+  float tot[TILES][NT][4];
 #pragma unroll
-  for (int nt = 0; nt < NT; ++nt)
+  for (int j = 0; j < TILES; ++j)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) tot[nt][i] = 0.0f;
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) tot[j][nt][i] = 0.0f;
   // scales: 16 bytes per row of the stage, from the 4-byte boundary at or below the first one
   p.sc = 2 * ST_BOX_BYTES + row * 16;
   const int row_off = (rec.row0 + row) * a.ngroups[phase] * ssz;
@@ -463,20 +486,23 @@ __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, i
       return false;
     const int seg = seg0 + s * SEGS, nseg = s == nst - 1 ? last : SEGS;
     const unsigned char *wp = stage + p.row, *x0 = stage + p.xe, *x1 = stage + p.xo, *init = stage + p.init, *sc = stage + p.sc;
-    uint32_t sw[2][2];
+    uint32_t sw[TILES][2][2];
     int g0 = 0;
     if constexpr (SC == SC_PAIRS) {
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        if constexpr (BITS == 8) {
-          sw[i][0] = *reinterpret_cast<const unsigned short*>(sc + i * SCALE2 + 2 * (seg & 1));
-        } else if constexpr (BITS == 4) {
-          sw[i][0] = *reinterpret_cast<const uint32_t*>(sc + i * SCALE2);
-        } else {
-          const uint2 v = *reinterpret_cast<const uint2*>(sc + i * SCALE2);
-          sw[i][0] = v.x, sw[i][1] = v.y;
+      for (int j = 0; j < TILES; ++j)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const unsigned char* at = sc + i * SCALE2 + j * 128;
+          if constexpr (BITS == 8) {
+            sw[j][i][0] = *reinterpret_cast<const unsigned short*>(at + 2 * (seg & 1));
+          } else if constexpr (BITS == 4) {
+            sw[j][i][0] = *reinterpret_cast<const uint32_t*>(at);
+          } else {
+            const uint2 v = *reinterpret_cast<const uint2*>(at);
+            sw[j][i][0] = v.x, sw[j][i][1] = v.y;
+          }
         }
-      }
     } else {
       g0 = group_of_seg(a, seg);
       sc += (row_off + g0 * ssz) & 3;
@@ -484,16 +510,21 @@ __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, i
 #pragma unroll
     for (int sg = 0; sg < SEGS; ++sg) {
       if (sg >= nseg) break;
-      float s0, s1;
-      if constexpr (SC == SC_PAIRS) {
-        const float2 u0 = scale_pair(sw[0][sg >> 1]), u1 = scale_pair(sw[1][sg >> 1]);
-        s0 = sg & 1 ? u0.y : u0.x, s1 = sg & 1 ? u1.y : u1.x;
-      } else {
-        const int d = sg == 0 ? 0 : (group_of_seg(a, seg + sg) - g0) * ssz;
-        s0 = scale_at<SC>(sc + d), s1 = scale_at<SC>(sc + d + SCALE2);
-      }
+      float f[TILES][2];
+      const int d = SC == SC_PAIRS || sg == 0 ? 0 : (group_of_seg(a, seg + sg) - g0) * ssz;
+#pragma unroll
+      for (int j = 0; j < TILES; ++j)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if constexpr (SC == SC_PAIRS) {
+            const float2 u = scale_pair(sw[j][i][sg >> 1]);
+            f[j][i] = sg & 1 ? u.y : u.x;
+          } else {
+            f[j][i] = scale_at<SC>(sc + d + i * SCALE2 + j * 128);
+          }
+        }
       const unsigned char* w = BITS == 2 ? wp + (sg & 1 ? p.d1 : 0) + (sg & 2 ? p.d2 : 0) : wp + (BITS == 4 && sg ? p.d1 : 0);
-      consume_segment<BITS, NT>(w, p.d1, x0 + sg * xstride, x1 + sg * xstride, init + sg * xstride, s0, s1, tot);
+      consume_segment<BITS, NT, TILES>(w, p.d1, x0 + sg * xstride, x1 + sg * xstride, init + sg * xstride, f, tot);
     }
     // shared memory of the stage is no longer needed
     __syncwarp();
@@ -508,26 +539,30 @@ __device__ __forceinline__ bool consume_pass(const TmaArgs& a, const Pipe& pp, i
   const int rb = rec.rbz & 0xffff, z = rec.rbz >> 16, ai = rec.ai;
   if (NT == 1 && BITS != 8) {  // the subnormal codes weigh 2^-24
 #pragma unroll
-    for (int i = 0; i < 4; ++i) tot[0][i] *= 16777216.0f;
+    for (int j = 0; j < TILES; ++j)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) tot[j][0][i] *= 16777216.0f;
   }
   if (phase == 0) {
     // two staging buffers in turn: a warp can be one item ahead of the slowest, not two
     unsigned char* hid = pp.hid_stage + (cur.n_hidden & 1) * ST_HID_BYTES;
-    hidden_to_smem<BITS, NT>(gated, rb, ntok, warp, lane, tot, hid, a.check_word);
+#pragma unroll
+    for (int j = 0; j < TILES; ++j) hidden_to_smem<BITS, NT>(gated, rb, ntok, row + 8 * j, lane, tot[j], hid, a.check_word);
     __syncwarp();
     if (lane == 0) mbar_arrive(pp.bar_hid);
     if (!__all_sync(0xffffffffu, mbar_wait(pp.bar_hid, cur.n_hidden & 1, a.check_word, pp.abort_flag))) return false;
     ++cur.n_hidden;
-    hidden_to_global(a, gated, rb, tok0, ntok, BITS, warp, lane, hid);
+    hidden_to_global(a, gated, rb, tok0, ntok, BITS, warp, W, lane, hid);
     if (pp.fused && last_pass) cur.pending_ai = ai;
   } else {
-    store_output<BITS, NT>(a, rb, z, tok0, ntok, warp, lane, tot);
+#pragma unroll
+    for (int j = 0; j < TILES; ++j) store_output<BITS, NT>(a, rb, z, tok0, ntok, row + 8 * j, lane, tot[j]);
   }
   return true;
 }
 
-template <int SC>
-__global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __grid_constant__ TmaArgs a) {
+template <int SC, int W>
+__global__ void __launch_bounds__(st_threads(W), ST_CTAS) ffn_tma_kernel(const __grid_constant__ TmaArgs a) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bars[3 * ST_SLOTS + 1];  // full, empty, issued (weight warp -> activation warp), hidden segment staged
   __shared__ ItemRec queue[ST_QUEUE];
@@ -540,7 +575,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
   unsigned char* hid_stage = ring + ST_RING;
   // The feeding warps come first: the schedulers favour the oldest warp, and a feeding warp that has to wait for
   // eight computing ones to stall leaves them without work soon after.
-  const int lane = threadIdx.x & 31, warp_id = threadIdx.x >> 5, warp = warp_id < 2 ? ST_WARPS + warp_id : warp_id - 2;
+  const int lane = threadIdx.x & 31, warp_id = threadIdx.x >> 5, warp = warp_id < 2 ? W + warp_id : warp_id - 2;
   const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + ST_SLOTS), bar_issued = smem_u32(bars + 2 * ST_SLOTS), bar_hid = smem_u32(bars + 3 * ST_SLOTS);
 
   if (threadIdx.x == 0) {
@@ -548,14 +583,14 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
     for (int s = 0; s < ST_SLOTS; ++s) {
       mbar_init(bar_full + 8 * s, 34);          // weight warp and activation warp (+ the bytes of their copies), every lane's scale copies
       mbar_init(bar_issued + 8 * s, 1);
-      mbar_init(bar_empty + 8 * s, ST_WARPS);   // one arrival per consumer warp
+      mbar_init(bar_empty + 8 * s, W);   // one arrival per consumer warp
     }
-    mbar_init(bar_hid, ST_WARPS);
+    mbar_init(bar_hid, W);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   // Everything above overlaps the tail of the kernel in front.
-  if (warp == ST_WARPS) {
+  if (warp == W) {
     // The tensor maps are older than every kernel of the chain: pull them towards L2 now, so that
     // the first copy of an expert's matrix does not wait for its descriptor to come from HBM.
     const int n_maps = 3 * a.L.E;
@@ -567,7 +602,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
   {  // the plan into shared memory: header and records in one round trip
     const int4* src = reinterpret_cast<const int4*>(reinterpret_cast<const char*>(a.plan) + PLAN_HEADER_BYTES);
     const int n = min(a.L.E, ST_PLAN_CACHE) * static_cast<int>(sizeof(PlanRec) / 16);
-    for (int i = threadIdx.x; i < n; i += ST_THREADS) reinterpret_cast<int4*>(s_plan)[i] = __ldcg(src + i);
+    for (int i = threadIdx.x; i < n; i += st_threads(W)) reinterpret_cast<int4*>(s_plan)[i] = __ldcg(src + i);
     if (threadIdx.x == 0) s_active = __ldcg(a.plan);
     __syncthreads();
   }
@@ -578,7 +613,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
   // hidden vectors are complete (PlanRec::done, raised by the consumers of the first projection)
   const bool fused = a.phase_begin == 0 && a.phase_end == 2;
 
-  if (warp == ST_WARPS) {
+  if (warp == W) {
     // ---------------- weight warp: items, ring, packed codes ----------------
     // The ring: stages lie one behind the other, a stage that would run over the end starts at the
     // beginning again.  head and vstart are positions on an endless tape; a stage may be written
@@ -660,7 +695,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
       }
       more = __shfl_sync(0xffffffffu, more, 0);
     }
-  } else if (warp == ST_WARPS + 1) {
+  } else if (warp == W + 1) {
     // ---------------- activation warp: the activation slice and the scales of every stage ----------------
     // On its own so that a wait for hidden vectors does not keep the weight stream from running ahead.
     int ready_ai = -1;  // the expert whose hidden vectors are known to be complete
@@ -695,7 +730,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
       if (fused && phase == 1 && rec.ai != ready_ai && last > 0) {
         // The codes of the stage are on their way; the hidden vectors may still be in the making on other
         // SMs.  (Every lane acquires the counter itself.)
-        const int expect = a.row_blocks[0] * ST_WARPS;  // every consumer warp counts once per item
+        const int expect = a.row_blocks[0] * W;  // every consumer warp counts once per item
         const int* done = &recs[rec.ai].done;
         bool ready = false;
         for (unsigned i = 0; i < DEP_WAIT_LIMIT; ++i) {
@@ -784,15 +819,15 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
       if (flags & ITEM_STOP) break;
       if (cnt - p0 <= 8) {
         switch (flags >> 8) {
-          case 2: ok = consume_pass<2, SC, 1>(a, pp, k, p0, warp, lane, cur); break;
-          case 4: ok = consume_pass<4, SC, 1>(a, pp, k, p0, warp, lane, cur); break;
-          default: ok = consume_pass<8, SC, 1>(a, pp, k, p0, warp, lane, cur); break;
+          case 2: ok = consume_pass<2, SC, 1, W>(a, pp, k, p0, warp, lane, cur); break;
+          case 4: ok = consume_pass<4, SC, 1, W>(a, pp, k, p0, warp, lane, cur); break;
+          default: ok = consume_pass<8, SC, 1, W>(a, pp, k, p0, warp, lane, cur); break;
         }
       } else {
         switch (flags >> 8) {
-          case 2: ok = consume_pass<2, SC, 2>(a, pp, k, p0, warp, lane, cur); break;
-          case 4: ok = consume_pass<4, SC, 2>(a, pp, k, p0, warp, lane, cur); break;
-          default: ok = consume_pass<8, SC, 2>(a, pp, k, p0, warp, lane, cur); break;
+          case 2: ok = consume_pass<2, SC, 2, W>(a, pp, k, p0, warp, lane, cur); break;
+          case 4: ok = consume_pass<4, SC, 2, W>(a, pp, k, p0, warp, lane, cur); break;
+          default: ok = consume_pass<8, SC, 2, W>(a, pp, k, p0, warp, lane, cur); break;
         }
       }
       p0 += ACT_PASS_MAX;
@@ -811,7 +846,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) ffn_tma_kernel(const __gr
   }
 }
 
-template <int SC>
+template <int SC, int W>
 cudaError_t launch_sc(const TmaArgs& a, long long items, cudaStream_t st) {
   static int ctas_per_device[64] = {};
   int dev = 0;
@@ -819,17 +854,17 @@ cudaError_t launch_sc(const TmaArgs& a, long long items, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!ctas_per_device[dev]) {
-    e = cudaFuncSetAttribute(ffn_tma_kernel<SC>, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM);
+    e = cudaFuncSetAttribute(ffn_tma_kernel<SC, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM);
     if (e != cudaSuccess) return e;
     int per_sm = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ffn_tma_kernel<SC>, ST_THREADS, ST_SMEM);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ffn_tma_kernel<SC, W>, st_threads(W), ST_SMEM);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     ctas_per_device[dev] = (per_sm > 0 ? per_sm : 1) * sms;
   }
   const int grid = items < ctas_per_device[dev] ? static_cast<int>(items) : ctas_per_device[dev];
-  return launch_chain(ffn_tma_kernel<SC>, dim3(grid), dim3(ST_THREADS), ST_SMEM, st, a);
+  return launch_chain(ffn_tma_kernel<SC, W>, dim3(grid), dim3(st_threads(W)), ST_SMEM, st, a);
 }
 
 }  // namespace
@@ -899,9 +934,15 @@ cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, c
   if (phase_begin == 0) per_expert += a.row_blocks[0];
   if (phase_end == 2) per_expert += static_cast<long long>(a.row_blocks[1]) * ksplit;
   const long long items = active_max * per_expert;
-  if (!L.scale_f16) return launch_sc<SC_F32>(a, items, st);
+  // Few tokens per activated expert and long rows: four warps with two tiles each, which read the activations once for both
+  // and meet a stage half as often (Mixtral-like layer, expert launch with eight / four warps: 1 token 77.8 / 73.7 us, 4
+  // tokens 125 / 121, 23 tokens 203 / 200; 768 x 3072, 32 experts, 64 tokens 35.5 / 36.0, 256 tokens 51 / 57, 777 tokens 79 / 86:
+  // wider passes, and items of a few stages, need the eight warps to hide their latencies).
+  const bool few = n_pairs <= 6 * active_max && L.d_model >= 1536;
+  if (!L.scale_f16) return few ? launch_sc<SC_F32, 4>(a, items, st) : launch_sc<SC_F32, 8>(a, items, st);
   const bool pairs = L.group == 128 && a.ngroups[0] % 2 == 0 && a.ngroups[1] % 2 == 0;
-  return pairs ? launch_sc<SC_PAIRS>(a, items, st) : launch_sc<SC_F16>(a, items, st);
+  if (pairs) return few ? launch_sc<SC_PAIRS, 4>(a, items, st) : launch_sc<SC_PAIRS, 8>(a, items, st);
+  return few ? launch_sc<SC_F16, 4>(a, items, st) : launch_sc<SC_F16, 8>(a, items, st);
 }
 
 // Host-side tensor-map encoder (driver entry point looked up once; no link against libcuda).
