@@ -420,7 +420,8 @@ int emoe_cache_release(emoe_ctx* ctx, const int64_t* ids, int n, void* compute_s
  * Expert e of this layer is registered as first_id + e, of the next layer as next_first_id + e.
  * prior: host array as for emoe_rank_experts; ids / gates / y: device buffers as for
  * emoe_moe_forward; pinned_ids: [T][top_k] in pinned host memory, valid when the call returns.
- * Decisions, counters and results are those of the single calls; order on the GPU as for emoe_moe_forward. */
+ * Decisions, counters and results are those of the single calls; order on the GPU as for emoe_moe_forward.  The copies
+ * of preloads are enqueued behind those of the experts this layer waits for. */
 int emoe_cached_layer(emoe_ctx* ctx, const emoe_layer_desc* desc, int layer, const void* x, int T, const float* router_W,
                       const float* router_bias, int bias_token_stride, int64_t first_id, const float* prior, int n_prefetch,
                       int64_t next_first_id, int32_t* ids, float* gates, float* y, int32_t* pinned_ids, void* compute_stream,

@@ -282,6 +282,32 @@ void expert_pointers(const ExpertCache* c, const CacheExpert& e, emoe_expert* ou
   }
 }
 
+// Preloads that are decided (the experts have their slots) and whose copies are still to be enqueued.
+struct Preloads {
+  int experts[EMOE_MAX_EXPERTS];
+  int n = 0;
+  bool take(int ei) {  // is it among them?  then not any more
+    const int at = static_cast<int>(std::find(experts, experts + n, ei) - experts);
+    if (at == n) return false;
+    std::copy(experts + at + 1, experts + n, experts + at);
+    --n;
+    return true;
+  }
+};
+
+// the decisions of a prefetch of at most EMOE_MAX_EXPERTS experts
+int decide_prefetch(ExpertCache* c, const int64_t* ids, int n, int current_layer, Preloads* later) {
+  for (int i = 0; i < n; ++i) {
+    const int ei = c->policy.find(ids[i]);
+    if (ei < 0) return EMOE_ERR_INVALID_ARG;
+    int evicted;
+    if (c->policy.prefetch(ei, current_layer, &evicted) < 0) continue;  // resident already, or every slot is in use: a prefetch never waits
+    if (evicted >= 0) later->take(evicted);
+    later->experts[later->n++] = ei;
+  }
+  return EMOE_OK;
+}
+
 }  // namespace
 
 // ---- accessors into the context (api.cu) ----------------------------------------------------
@@ -289,6 +315,21 @@ ExpertCache*& ctx_cache(emoe_ctx* ctx);
 int ctx_device(const emoe_ctx* ctx);
 bool ctx_dependent_launch(const emoe_ctx* ctx);
 int ctx_cuda_fail(emoe_ctx* ctx, cudaError_t e);
+
+namespace {
+int enqueue_preloads(emoe_ctx* ctx, Preloads* later, void* copy_stream) {
+  ExpertCache* c = ctx_cache(ctx);
+  cudaError_t err = cudaSetDevice(c->device);
+  for (int i = 0; i < later->n && err == cudaSuccess; ++i) {
+    const CacheExpert& e = c->policy.expert(later->experts[i]);
+    err = load_into_slot(c, e, e.slot, static_cast<cudaStream_t>(copy_stream));
+  }
+  later->n = 0;
+  return err == cudaSuccess ? EMOE_OK : ctx_cuda_fail(ctx, err);
+}
+int acquire(emoe_ctx* ctx, const int64_t* ids, int n, int current_layer, void* compute_stream, void* copy_stream, emoe_expert* out_experts,
+            Preloads* later);
+}  // namespace
 
 }  // namespace emoe
 
@@ -355,6 +396,17 @@ int emoe_prefetch_experts(emoe_ctx* ctx, const int64_t* ids, int n, int current_
 
 int emoe_cache_acquire(emoe_ctx* ctx, const int64_t* ids, int n, int current_layer, void* compute_stream, void* copy_stream,
                        emoe_expert* out_experts) {
+  Preloads none;
+  return acquire(ctx, ids, n, current_layer, compute_stream, copy_stream, out_experts, &none);
+}
+
+}  // extern "C"
+
+namespace emoe {
+namespace {
+
+int acquire(emoe_ctx* ctx, const int64_t* ids, int n, int current_layer, void* compute_stream, void* copy_stream, emoe_expert* out_experts,
+            Preloads* later) {
   if (!ctx || !ctx_cache(ctx) || n <= 0 || !ids || !out_experts) return EMOE_ERR_INVALID_ARG;
   ExpertCache* c = ctx_cache(ctx);
   cudaError_t err = cudaSetDevice(c->device);
@@ -383,6 +435,8 @@ int emoe_cache_acquire(emoe_ctx* ctx, const int64_t* ids, int n, int current_lay
       rc = EMOE_ERR_CACHE_FULL;
       break;
     }
+    if (later->take(ei)) load = 1;             // decided as a preload a moment ago, and needed now
+    if (evicted >= 0) later->take(evicted);  // a preload that leaves before its copy was made
     if (load) {
       err = load_into_slot(c, c->policy.expert(ei), s, static_cast<cudaStream_t>(copy_stream));
       if (err != cudaSuccess) rc = ctx_cuda_fail(ctx, err);
@@ -405,6 +459,11 @@ int emoe_cache_acquire(emoe_ctx* ctx, const int64_t* ids, int n, int current_lay
   }
   return rc;
 }
+
+}  // namespace
+}  // namespace emoe
+
+extern "C" {
 
 int emoe_cache_release(emoe_ctx* ctx, const int64_t* ids, int n, void* compute_stream) {
   if (!ctx || !ctx_cache(ctx) || n <= 0 || !ids) return EMOE_ERR_INVALID_ARG;
@@ -471,18 +530,27 @@ int emoe_cached_layer(emoe_ctx* ctx, const emoe_layer_desc* desc, int layer, con
   int n = 0;
   for (int e = 0; e < E; ++e)
     if (seen[e]) active[n++] = e;
+  // What the next layer will probably need is decided first, as the single calls would, but its copies go behind those
+  // that this layer waits for: the host link is the bottleneck, and a load on demand behind a preload stands in a queue
+  // of one expert (6 layers 768 x 3072, 32 experts, a quarter of them resident, 16 steps of one token: 5.0 -> 4.7 ms).
+  Preloads later;
+  int rc = EMOE_OK;
   if (prior && n_prefetch > 0) {
     int32_t order[EMOE_MAX_EXPERTS];
-    int rc = emoe_rank_experts(prior, E, active, n, order);
+    rc = emoe_rank_experts(prior, E, active, n, order);
     const int m = n_prefetch < E ? n_prefetch : E;
     for (int i = 0; i < m; ++i) expert_ids[i] = next_first_id + order[i];
-    if (rc == EMOE_OK) rc = emoe_prefetch_experts(ctx, expert_ids, m, layer, copy_stream);
-    if (rc != EMOE_OK) return rc;
+    if (rc == EMOE_OK) rc = decide_prefetch(ctx_cache(ctx), expert_ids, m, layer, &later);
   }
   for (int i = 0; i < n; ++i) expert_ids[i] = first_id + active[i];
   emoe_expert got[EMOE_MAX_EXPERTS], table[EMOE_MAX_EXPERTS];
-  int rc = emoe_cache_acquire(ctx, expert_ids, n, layer, compute_stream, copy_stream, got);
+  if (rc == EMOE_OK) rc = acquire(ctx, expert_ids, n, layer, compute_stream, copy_stream, got, &later);
+  const int rc_later = enqueue_preloads(ctx, &later, copy_stream);  // whatever else happened: their slots are taken
   if (rc != EMOE_OK) return rc;
+  if (rc_later != EMOE_OK) {
+    emoe_cache_release(ctx, expert_ids, n, compute_stream);
+    return rc_later;
+  }
   // entries of experts nobody picked are never read; they borrow an acquired expert whole (pointers AND
   // width, so that whatever is derived from an entry stays inside that expert's slot)
   for (int e = 0, i = 0; e < E; ++e) table[e] = seen[e] ? got[i++] : got[0];

@@ -435,6 +435,43 @@ def test_cached_layer_is_the_single_calls(T, n_slots, n_prefetch):
         B.emoe_destroy(many)
 
 
+@pytest.mark.parametrize("n_slots,n_prefetch", [(3, 4), (4, 2), (4, 4)])
+def test_cached_layer_preloads_that_are_needed_at_once_or_leave_again(n_slots, n_prefetch):
+    """A stack of one layer preloads its own experts: some are needed by the very call that decided so, some lose their slot
+    to a load on demand before their copy was made.  Every slot has to hold the expert the books say it holds."""
+    shape = inputs.LayerShape(512, 1024, 4, 2, "relu", "softmax_renorm", 128, "f16", "bf16")
+    host = HostExperts(shape, 1, lambda l: [8, 4, 2, 4], seed=47)
+    rng = np.random.default_rng(47)
+    prior, desc = rng.random((4, 4)).astype(np.float32), layer.make_desc(shape)
+    dev = torch.device("cuda", 0)
+    Wr = torch.from_numpy(inputs.router_weight(47, 0, 512, 4, std=0.05)).to(dev)
+    stream = torch.cuda.Stream(device=dev)
+    ctx = _stack_on_cache(host, desc, n_slots, 1)
+    ids, gates, y = torch.empty(1, 2, dtype=torch.int32, device=dev), torch.empty(1, 2, device=dev), torch.empty(1, 512, device=dev)
+    pinned = torch.empty(1, 2, dtype=torch.int32, pin_memory=True)
+    dense = layer.MoELayer(shape, host.bits[0], max_tokens=1)
+    try:
+        for e in range(4):
+            for m in range(2):
+                dense.packed[e][m].copy_(host.pin[0][e][0][m].reshape(-1))
+                dense.scales[e][m].copy_(host.pin[0][e][1][m].reshape(-1))
+        for step in range(12):
+            x = torch.from_numpy(inputs.activations(47, 0, 1, 512, "bf16", batch_tag=step)).to(dev).to(torch.bfloat16)
+            torch.cuda.synchronize()
+            B.emoe_cached_layer(ctx, desc, 0, x.data_ptr(), 1, Wr.data_ptr(), None, 0, host.expert_id(0, 0), prior.ctypes.data, n_prefetch,
+                                host.expert_id(0, 0), ids.data_ptr(), gates.data_ptr(), y.data_ptr(), pinned.data_ptr(), 0, stream.cuda_stream)
+            want = torch.empty_like(y)
+            B.emoe_moe_forward_routed(dense.ctx, desc, x.data_ptr(), 1, ids.data_ptr(), gates.data_ptr(), dense.table, want.data_ptr(), None, 0)
+            torch.cuda.synchronize()
+            assert torch.equal(y, want), step
+        st = B.emoe_cache_get_stats(ctx)
+        assert st["prefetched"] > 0 and st["hits"] > 0
+    finally:
+        torch.cuda.synchronize()
+        dense.close()
+        B.emoe_destroy(ctx)
+
+
 def test_cached_layer_errors():
     """Bad arguments are refused before anything runs; a layer that fails after its experts were acquired lets them go."""
     shape = inputs.LayerShape(512, 1024, 4, 2, "relu", "softmax_renorm", 128, "f16", "bf16")
