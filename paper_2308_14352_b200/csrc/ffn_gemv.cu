@@ -4,20 +4,25 @@
 //
 // The path for fp32 activations (fp32 products and sums throughout) and the fallback for shapes the
 // tensor-core paths do not take.  At these sizes a layer is a few microseconds of arithmetic, so
-// the time is latency: the work is cut fine enough that all of it is on the SMs at once.
-//   * a CTA takes a few rows of one expert, a slice of at most 1024 inputs (second projection: one
-//     slice per CTA, summed by the combine step; first projection: all slices in turn) and up to
-//     four tokens, whose activations it stages in shared memory as fp32 (read from there by every
-//     warp; from global memory each step of the loop below waited for the L1 or L2);
-//   * a warp is cut into groups of lanes; a group owns two rows and its lanes stream them with
-//     128-bit loads (16 / 32 / 64 weights each), the next loads on their way while one set is used;
+// the time is latency: the second projection's weights are fetched while the first still runs, and all of the work is
+// on the SMs at once.
+//   * a CTA takes some blocks of 32 rows of one expert and a slice of at most 1024 inputs (second projection: one
+//     slice per CTA, summed by the combine step; first projection: all slices in turn).  Their codes come into shared
+//     memory by bulk copies, all of them asked for at once; the number of blocks is such that every CTA is resident
+//     at once;
+//   * up to four tokens at a time have their activations in shared memory as fp32 (from global memory each
+//     step of the loop below waited for the L1 or L2);
+//   * a warp is cut into groups of lanes; a group owns four rows of a block and its lanes take 128-bit words of them (16 / 32 / 64
+//     weights each), so that an activation read serves four rows (two: the reads of shared memory bound passes of four tokens);
 //   * the fields of a 32-bit word are masked into bytes together, a byte becomes a float by one byte
-//     permute into the mantissa of 2^23 and one (exact) subtraction, shared by the tokens.
-// Measured: Switch-base-like layers with 8 experts and 16 fp32 tokens, forward call of eight layers 878 -> 340 us
-// (one row per warp, all inputs in turn, activations from global memory before); what is left is the
-// latency of five launches and of the first loads of each.
+//     permute into the mantissa of 2^23 and one (exact) subtraction for two of them, shared by the tokens; products and sums go
+//     by twos as well.
+// Measured (forward call per layer; two rows per group, codes through registers, a variant of the loop per width and number
+// of tokens -> now): 768 x 3072, 8 experts, 16 fp32 tokens 41.8 -> 33.3 us; 640 x 2560, 16 experts, 64 tokens 78 -> 59; 1024 x 4096,
+// 4 experts, two picks, 64 tokens 211 -> 142; 512 x 1536, 16 experts, 9 tokens 21.3 -> 21.5 (five launches).
 #include "common.cuh"
 #include "ffn_tile.cuh"
+#include "pipe.cuh"
 
 namespace emoe {
 namespace {
@@ -26,27 +31,50 @@ constexpr int GEMV_WARPS = 4;
 constexpr int GEMV_THREADS = GEMV_WARPS * 32;
 constexpr int GEMV_TOK = 4;       // tokens of a pass
 constexpr int GEMV_SLICE = 1024;  // inputs staged at a time
-constexpr int GEMV_R = 2;         // rows of a group of lanes
+constexpr int GEMV_R = 4;         // rows of a group of lanes
 constexpr int GEMV_LANES = 16;    // lanes of a group: a slice is one to four words per lane at 2 bits to 8, and a lane's share about 64 weights per row
-constexpr int GEMV_ROWS = GEMV_WARPS * (32 / GEMV_LANES) * GEMV_R;  // rows of a CTA
+constexpr int GEMV_ROWS = GEMV_WARPS * (32 / GEMV_LANES) * GEMV_R;  // rows of a block, which a CTA takes at a time
+constexpr int GEMV_CTAS = 4;      // per SM (registers)
+constexpr int GEMV_BLOCKS = 4;    // of a CTA, at most
+constexpr int GEMV_SMEM = 226 * 1024;  // of an SM, with what the system keeps per CTA taken off below
 
-// The codes of a 32-bit word (two's-complement fields, low bits first) as bytes q + 2^(b-1): code i is byte i / S of
-// out[i % S], S = 8 / BITS fields to a byte.
-template <int BITS>
-__device__ __forceinline__ void code_bytes(uint32_t word, uint32_t (&out)[8 / BITS]) {
-  constexpr uint32_t mask = ((1u << BITS) - 1) * 0x01010101u, flip = (1u << (BITS - 1)) * 0x01010101u;
-#pragma unroll
-  for (int i = 0; i < 8 / BITS; ++i) out[i] = and_xor(word >> (BITS * i), mask, flip);
+// two fp32 numbers in a register pair: sums and products of both by one instruction
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pair_of(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
 }
-// code i of the word as fp32: its byte in the mantissa of 2^23 by one byte permute, the constant subtracted (exact)
-template <int BITS>
-__device__ __forceinline__ float code_f32(const uint32_t (&bytes)[8 / BITS], int i) {
-  constexpr int S = 8 / BITS;
-  return __uint_as_float(prmt(bytes[i % S], 0x4B000000u, 0x7540u + i / S)) - (8388608.0f + static_cast<float>(1 << (BITS - 1)));
+__device__ __forceinline__ float pair_sum(f32x2 v) {
+  float lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+  return lo + hi;
 }
 
-__device__ __forceinline__ float load_scale(const void* scales, bool f16, size_t idx) {
-  return f16 ? __half2float(__ldg(reinterpret_cast<const __half*>(scales) + idx)) : __ldg(reinterpret_cast<const float*>(scales) + idx);
+// How codes of b bits are taken: field f of a 32-bit word's four bytes at a time (one, two or four fields to a byte), as bytes
+// q + 2^(b-1).  The width is data here, not a variant of the code: with a variant per width and number of tokens the CTAs of an
+// SM ran nine loops, and a third of all cycles went into waiting for instructions.
+struct Width {
+  int bits, fields;     // 8 / bits
+  uint32_t mask, flip;  // of a field, and its sign bit, in every byte
+  f32x2 minus;          // -(2^23 + 2^(b-1)), twice
+};
+__device__ __forceinline__ Width width_of(int bits) {
+  Width w;
+  w.bits = bits;
+  w.fields = 8 / bits;
+  w.mask = ((1u << bits) - 1) * 0x01010101u;
+  w.flip = (1u << (bits - 1)) * 0x01010101u;
+  const float m = -(8388608.0f + static_cast<float>(1 << (bits - 1)));
+  w.minus = pair_of(m, m);
+  return w;
+}
+// bytes 2h and 2h + 1 as fp32: each in the mantissa of 2^23 by a byte permute, the constant subtracted from both (exact)
+template <int H>
+__device__ __forceinline__ f32x2 code_pair(uint32_t bytes, f32x2 minus) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pair_of(__uint_as_float(prmt(bytes, 0x4B000000u, 0x7540u + 2 * H)), __uint_as_float(prmt(bytes, 0x4B000000u, 0x7541u + 2 * H)))), "l"(minus));
+  return r;
 }
 
 struct GemvArgs {
@@ -60,175 +88,335 @@ struct GemvArgs {
   float* o;      // [ksplit][n_pairs][d_model]
   int slice;     // inputs of a slice
   int nslices, ksplit, n_pairs;
+  int blocks;    // blocks of rows per CTA (one where there are several slices in turn)
+  int G, ngroups;  // inputs per scale, scales of a row
+  int groups;    // scales of a row that a slice touches, at most
+  int* check_word;
 };
+
+// shared memory: [matrices][rows][slice] codes, [matrices][rows][groups] scales, [GEMV_TOK][slice] activations
+struct Staged {
+  unsigned char* codes;
+  float* scales;
+  float* xs;
+};
+
+// a slice of the inputs of an expert's rows
+struct Slice {
+  int k0, len, bytes;  // its first input, inputs, bytes of a row
+  int g0, ng;          // first scale, scales
+  int wpg, gshift;     // 128-bit words per scale, its logarithm (negative: not a power of two)
+};
+__device__ __forceinline__ Slice slice_of(const GemvArgs& a, int sl, int bits) {
+  const int K = a.phase == 0 ? a.L.d_model : a.L.d_ff;
+  Slice s;
+  s.k0 = sl * a.slice;
+  s.len = min(a.slice, K - s.k0);
+  s.bytes = s.len * bits / 8;
+  s.g0 = a.nslices == 1 ? 0 : s.k0 / a.G;
+  s.ng = a.nslices == 1 ? a.ngroups : (s.k0 + s.len - 1) / a.G - s.g0 + 1;
+  s.wpg = a.G * bits / 128;
+  s.gshift = (s.wpg & (s.wpg - 1)) == 0 ? 31 - __clz(s.wpg) : -1;
+  return s;
+}
 
 // where one matrix's rows of a lane group lie
 struct Rows {
-  const uint4* w;      // first row, first word of the row
-  const void* scales;
-  size_t srow;         // index of the first row's first scale
+  const unsigned char* w;  // first row
+  const float* s;          // its scales
+  int row_bytes, srow;     // distance to the second row
 };
 
-// acc[r][m] += sum_k q[r][k] * s[r][k/G] * x_m[k] over the words l, l + L, ... of the slice [j0, j0 + nv) of two rows.
-// xs: [MT][chunk of 4 inputs][word] in shared memory, tokens GEMV_SLICE floats apart.
-template <int BITS, int MT>
-__device__ __forceinline__ void rows_dot(const Rows& m, int nvec, bool scale_f16, int ngroups, int gshift, int wpg, int j0, int nv, const float* xs,
-                                         int l, float (&acc)[GEMV_R][MT]) {
-  constexpr int PER = 32 / BITS;
-  uint4 nw[GEMV_R];
-  if (l < nv)
-#pragma unroll
-    for (int r = 0; r < GEMV_R; ++r) nw[r] = __ldg(m.w + static_cast<size_t>(r) * nvec + j0 + l);
+// acc[r][m] += sum_k q[r][k] * s[r][k/G] * x_m[k] over the words l, l + L, ... of a slice of the group's rows.
+// xs: [MT][32-bit word of a 128-bit one][field][128-bit word][byte], tokens xstride floats apart.
+template <int MT>
+__device__ __forceinline__ void rows_dot(const Rows& m, const Width& wd, const Slice& sc, const float* xs, int xstride, int l, float (&acc)[GEMV_R][MT]) {
+  const int nv = sc.bytes >> 4, j0 = sc.k0 * wd.bits / 128;
 #pragma unroll 1
   for (int j = l; j < nv; j += GEMV_LANES) {
     uint32_t w[GEMV_R][4];
-    float s[GEMV_R], part[GEMV_R][MT];
-    const int g = gshift >= 0 ? (j0 + j) >> gshift : (j0 + j) / wpg;  // words per scale group
+    float s[GEMV_R];
+    f32x2 part[GEMV_R][MT];  // the sums over even and over odd bytes
+    const int g = sc.ng == 1 ? 0 : (sc.gshift >= 0 ? (j0 + j) >> sc.gshift : (j0 + j) / sc.wpg) - sc.g0;
 #pragma unroll
     for (int r = 0; r < GEMV_R; ++r) {
-      w[r][0] = nw[r].x, w[r][1] = nw[r].y, w[r][2] = nw[r].z, w[r][3] = nw[r].w;
-      s[r] = load_scale(m.scales, scale_f16, m.srow + static_cast<size_t>(r) * ngroups + g);
+      const uint4 v = *reinterpret_cast<const uint4*>(m.w + r * m.row_bytes + 16 * j);
+      w[r][0] = v.x, w[r][1] = v.y, w[r][2] = v.z, w[r][3] = v.w;
+      s[r] = m.s[r * m.srow + g];
 #pragma unroll
-      for (int t = 0; t < MT; ++t) part[r][t] = 0.0f;
+      for (int t = 0; t < MT; ++t) part[r][t] = 0ull;
     }
-    if (j + GEMV_LANES < nv)
-#pragma unroll
-      for (int r = 0; r < GEMV_R; ++r) nw[r] = __ldg(m.w + static_cast<size_t>(r) * nvec + j0 + j + GEMV_LANES);
     const float* xp = xs + j * 4;
-    constexpr int AT_ONCE = BITS / 2;  // 32-bit words: 16 weights (the kernel holds nine variants of this loop: unrolled further, it waits for its instructions)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
 #pragma unroll 1
-    for (int i0 = 0; i0 < 4; i0 += AT_ONCE) {
+      for (int f = 0; f < 8; f += wd.bits) {
+        ulonglong2 xv[MT];
 #pragma unroll
-      for (int i = 0; i < AT_ONCE; ++i) {
-        uint32_t by[GEMV_R][8 / BITS];
+        for (int t = 0; t < MT; ++t) xv[t] = *reinterpret_cast<const ulonglong2*>(xp + t * xstride);
+        xp += nv * 4;
 #pragma unroll
-        for (int r = 0; r < GEMV_R; ++r) code_bytes<BITS>(w[r][i], by[r]);
+        for (int r = 0; r < GEMV_R; ++r) {
+          const uint32_t by = and_xor(w[r][i] >> f, wd.mask, wd.flip);
+          const f32x2 q0 = code_pair<0>(by, wd.minus), q1 = code_pair<1>(by, wd.minus);
 #pragma unroll
-        for (int c = 0; c < PER / 4; ++c) {
-          float4 xv[MT];
-#pragma unroll
-          for (int t = 0; t < MT; ++t) xv[t] = *reinterpret_cast<const float4*>(xp + t * GEMV_SLICE);
-          xp += nv * 4;
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int r = 0; r < GEMV_R; ++r) {
-              const float q = code_f32<BITS>(by[r], 4 * c + k);
-#pragma unroll
-              for (int t = 0; t < MT; ++t) part[r][t] = fmaf(q, k == 0 ? xv[t].x : (k == 1 ? xv[t].y : (k == 2 ? xv[t].z : xv[t].w)), part[r][t]);
-            }
+          for (int t = 0; t < MT; ++t) {
+            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(part[r][t]) : "l"(q0), "l"(xv[t].x));
+            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(part[r][t]) : "l"(q1), "l"(xv[t].y));
+          }
         }
       }
-#pragma unroll
-      for (int r = 0; r < GEMV_R; ++r)
-#pragma unroll
-        for (int i = 0; i + AT_ONCE < 4; ++i) w[r][i] = w[r][i + AT_ONCE];
     }
 #pragma unroll
     for (int r = 0; r < GEMV_R; ++r)
 #pragma unroll
-      for (int t = 0; t < MT; ++t) acc[r][t] = fmaf(s[r], part[r][t], acc[r][t]);
+      for (int t = 0; t < MT; ++t) acc[r][t] = fmaf(s[r], pair_sum(part[r][t]), acc[r][t]);
   }
 }
 
-// the rows' sums over the slices [sl0, sl1) for MT tokens in slots slot0 ..
-template <int BITS, bool GATED, int MT>
-__device__ __forceinline__ void expert_pass(const GemvArgs& a, const ExpertDev& ex, int slot0, int ntok, int sl0, int sl1, int n0, float* xs) {
+// The activations of `tokens` tokens (the last of ntok repeated) in the slice of `len` inputs from k0 on, in the order rows_dot
+// takes them.
+__device__ __forceinline__ void stage_inputs(const GemvArgs& a, const Width& wd, int slot0, int ntok, int tokens, int k0, int len, float* xs) {
   const LayerDims& L = a.L;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int N = a.phase == 0 ? L.d_ff : L.d_model, K = a.phase == 0 ? L.d_model : L.d_ff;
-  const int nvec = K * BITS / 128;
-  const int n = n0 + (warp * (32 / GEMV_LANES) + lane / GEMV_LANES) * GEMV_R, l = lane & (GEMV_LANES - 1);
-  const int G = L.group > 0 ? L.group : K, ngroups = K / G;
-  const int wpg = G * BITS / 128;
-  const int gshift = (wpg & (wpg - 1)) == 0 ? 31 - __clz(wpg) : -1;
-  const int mat = a.phase == 0 ? 0 : (L.act == EMOE_ACT_RELU ? 1 : 2);
-  const Rows m0 = {reinterpret_cast<const uint4*>(ex.packed[mat]) + static_cast<size_t>(n) * nvec, ex.scales[mat], static_cast<size_t>(n) * ngroups};
-  const Rows m1 = {reinterpret_cast<const uint4*>(ex.packed[1]) + static_cast<size_t>(n) * nvec, ex.scales[1], static_cast<size_t>(n) * ngroups};
-  float v[GEMV_R][MT], u[GEMV_R][MT];
-#pragma unroll
-  for (int r = 0; r < GEMV_R; ++r)
-#pragma unroll
-    for (int t = 0; t < MT; ++t) v[r][t] = u[r][t] = 0.0f;
-  for (int sl = sl0; sl < sl1; ++sl) {
-    const int k0 = sl * a.slice, len = min(a.slice, K - k0), nv = len * BITS / 128;
-    __syncthreads();  // the slice in front is used up
-    for (int i = threadIdx.x; i < MT * (len / 4); i += GEMV_THREADS) {
-      const int t = i / (len / 4), c4 = i - t * (len / 4);  // token, chunk of four inputs
-      const int slot = slot0 + min(t, ntok - 1);
-      const size_t row = a.phase == 0 ? static_cast<size_t>(L.top_k == 1 ? a.perm[slot] : a.perm[slot] / L.top_k) : static_cast<size_t>(slot);
-      const size_t at = row * K + k0 + 4 * c4;
-      const void* src = a.phase == 0 ? a.x : a.hidden;
-      float4 f;
+  const int K = a.phase == 0 ? L.d_model : L.d_ff, nv = len * wd.bits / 128;
+  const int sh = wd.bits == 8 ? 0 : (wd.bits == 4 ? 1 : 2);  // log2 of the fields
+  for (int t = 0; t < tokens; ++t) {
+    const int slot = slot0 + min(t, ntok - 1);
+    const size_t row = a.phase == 0 ? static_cast<size_t>(L.top_k == 1 ? a.perm[slot] : a.perm[slot] / L.top_k) : static_cast<size_t>(slot);
+    const void* src = a.phase == 0 ? a.x : a.hidden;
+    float* to = xs + t * a.slice;
+    for (int k = 4 * threadIdx.x; k < len; k += 4 * GEMV_THREADS) {
+      const size_t at = row * K + k0 + k;
+      float4 v;
       if (L.act_bf16) {
         const uint2 b = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(src) + at);
-        f = make_float4(__uint_as_float(b.x << 16), __uint_as_float(b.x & 0xffff0000u), __uint_as_float(b.y << 16), __uint_as_float(b.y & 0xffff0000u));
+        v = make_float4(__uint_as_float(b.x << 16), __uint_as_float(b.x & 0xffff0000u), __uint_as_float(b.y << 16), __uint_as_float(b.y & 0xffff0000u));
       } else {
-        f = *reinterpret_cast<const float4*>(static_cast<const float*>(src) + at);
+        v = *reinterpret_cast<const float4*>(static_cast<const float*>(src) + at);
       }
-      constexpr int CH = 32 / BITS;  // chunks of a 128-bit word; chunk-major, so that neighbouring words' readers read neighbouring 16 bytes
-      *reinterpret_cast<float4*>(xs + t * GEMV_SLICE + ((c4 % CH) * nv + c4 / CH) * 4) = f;
+      // input k of the slice: 128-bit word k / (16 << sh), and in it 32-bit word, byte and field
+      const int word = k >> (4 + sh), i = (k >> (2 + sh)) & 3, o = k & ((4 << sh) - 1);
+      if (sh == 0) {
+        *reinterpret_cast<float4*>(to + (i * nv + word) * 4) = v;
+      } else if (sh == 1) {  // two fields, two bytes
+        float* p = to + (i * 2 * nv + word) * 4 + (o >> 1);
+        *reinterpret_cast<float2*>(p) = make_float2(v.x, v.z);
+        *reinterpret_cast<float2*>(p + nv * 4) = make_float2(v.y, v.w);
+      } else {  // four fields, one byte
+        float* p = to + (i * 4 * nv + word) * 4 + (o >> 2);
+        p[0] = v.x;
+        p[nv * 4] = v.y;
+        p[nv * 8] = v.z;
+        p[nv * 12] = v.w;
+      }
     }
-    __syncthreads();
-    rows_dot<BITS, MT>(m0, nvec, L.scale_f16, ngroups, gshift, wpg, k0 * BITS / 128, nv, xs, l, v);
-    if (GATED) rows_dot<BITS, MT>(m1, nvec, L.scale_f16, ngroups, gshift, wpg, k0 * BITS / 128, nv, xs, l, u);
   }
+}
+
+// asks for the codes of a slice of the CTA's rows (one arrival at `bar`, with the bytes)
+template <bool GATED>
+__device__ __forceinline__ void fetch_codes(const GemvArgs& a, const ExpertDev& ex, const Slice& sc, int n0, int rows, const Staged& sm, uint32_t bar) {
+  const int K = a.phase == 0 ? a.L.d_model : a.L.d_ff, mat = a.phase == 0 ? 0 : (a.L.act == EMOE_ACT_RELU ? 1 : 2);
+  const size_t row_bytes = static_cast<size_t>(K) * ex.bits / 8;
+  if (threadIdx.x >= 32) return;
 #pragma unroll
-  for (int o = GEMV_LANES >> 1; o > 0; o >>= 1)
+  for (int i = 0; i < (GATED ? 2 : 1); ++i) {
+    const int m = GATED ? i : mat;
+    const uint8_t* from = (m == 0 ? ex.packed[0] : (m == 1 ? ex.packed[1] : ex.packed[2])) + n0 * row_bytes + static_cast<size_t>(sc.k0) * ex.bits / 8;
+    const uint32_t to = smem_u32(sm.codes + i * a.blocks * GEMV_ROWS * a.slice);
+    if (threadIdx.x == 0 && i == 0) mbar_expect_tx(bar, (GATED ? 2 : 1) * rows * sc.bytes);
+    if (sc.len == K) {  // whole rows follow each other
+      if (threadIdx.x == 0) bulk_load(to, from, rows * sc.bytes, bar);
+    } else {
+      __syncwarp();  // (behind the announcement of the bytes)
+      for (int r = threadIdx.x; r < rows; r += 32) bulk_load(to + r * sc.bytes, from + r * row_bytes, sc.bytes, bar);
+    }
+  }
+}
+// ... and their scales; `staging` runs between the first loads and the first store
+template <bool GATED, typename F>
+__device__ __forceinline__ void fetch_scales(const GemvArgs& a, const ExpertDev& ex, const Slice& sc, int n0, int rows, const Staged& sm, F staging) {
+  const int mat = a.phase == 0 ? 0 : (a.L.act == EMOE_ACT_RELU ? 1 : 2);
+  const auto scale = [&](int m, int u) {
+    const int r = sc.ng == 1 ? u : u / sc.ng;
+    const void* scales = m == 0 ? ex.scales[0] : (m == 1 ? ex.scales[1] : ex.scales[2]);
+    return load_scale_ro(scales, a.L.scale_f16, static_cast<size_t>(n0 + r) * a.ngroups + sc.g0 + u - r * sc.ng);
+  };
+  const int n = rows * sc.ng, tid = threadIdx.x;
+  float first[GATED ? 2 : 1];
+#pragma unroll
+  for (int i = 0; i < (GATED ? 2 : 1); ++i) first[i] = tid < n ? scale(GATED ? i : mat, tid) : 0.0f;
+  staging();
+#pragma unroll
+  for (int i = 0; i < (GATED ? 2 : 1); ++i) {
+    float* to = sm.scales + i * a.blocks * GEMV_ROWS * a.groups;
+    if (tid < n) to[tid] = first[i];
+    for (int u = tid + GEMV_THREADS; u < n; u += GEMV_THREADS) to[u] = scale(GATED ? i : mat, u);
+  }
+}
+
+// the sums of a block's rows in the staged slice, for MT tokens
+template <bool GATED, int MT>
+__device__ __forceinline__ void block_dot(const GemvArgs& a, const Width& wd, int b, const Slice& sc, const Staged& sm, float (&v)[GEMV_R][MT], float (&u)[GEMV_R][MT]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l = lane & (GEMV_LANES - 1);
+  const int r = b * GEMV_ROWS + (warp * (32 / GEMV_LANES) + lane / GEMV_LANES) * GEMV_R;
+  const Rows m0 = {sm.codes + r * sc.bytes, sm.scales + r * sc.ng, sc.bytes, sc.ng};
+  rows_dot<MT>(m0, wd, sc, sm.xs, a.slice, l, v);
+  if (GATED) {
+    const Rows m1 = {m0.w + a.blocks * GEMV_ROWS * a.slice, m0.s + a.blocks * GEMV_ROWS * a.groups, sc.bytes, sc.ng};
+    rows_dot<MT>(m1, wd, sc, sm.xs, a.slice, l, u);
+  }
+}
+
+// Adds up the V values of every lane over its group of lanes; lane i keeps value i % V.  Half of the values go to
+// the partner in each of the first steps.
+template <int V>
+__device__ __forceinline__ float sum_lanes(const float (&v)[V], int l) {
+  static_assert(V == 1 || V == 2 || V == 4 || V == 8 || V == 16, "");
+  float x[V];
+#pragma unroll
+  for (int i = 0; i < V; ++i) x[i] = v[i];
+  int o = 1;
+#pragma unroll
+  for (int n = V; n > 1; n >>= 1, o <<= 1) {  // value 2i stays in the lanes without bit o, 2i + 1 in those with it
+    const bool odd = l & o;
+#pragma unroll
+    for (int i = 0; i < n / 2; ++i) {
+      const float keep = odd ? x[2 * i + 1] : x[2 * i], give = odd ? x[2 * i] : x[2 * i + 1];
+      x[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  for (; o < GEMV_LANES; o <<= 1) x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+  return x[0];
+}
+
+// adds the lanes up and stores a block's results
+template <bool GATED, int MT>
+__device__ __forceinline__ void store_block(const GemvArgs& a, int z, int n0, int slot0, int ntok, float (&v)[GEMV_R][MT], float (&u)[GEMV_R][MT]) {
+  const LayerDims& L = a.L;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l = lane & (GEMV_LANES - 1);
+  const int N = a.phase == 0 ? L.d_ff : L.d_model;
+  float f[GEMV_R * MT], h[GEMV_R * MT];
+#pragma unroll
+  for (int i = 0; i < GEMV_R * MT; ++i) f[i] = v[i / MT][i % MT], h[i] = u[i / MT][i % MT];
+  const float x = sum_lanes(f, l), y = GATED ? sum_lanes(h, l) : 0.0f;
+  const int i = l % (GEMV_R * MT), t = i % MT;
+  const int n = n0 + (warp * (32 / GEMV_LANES) + lane / GEMV_LANES) * GEMV_R + i / MT;
+  if (l >= GEMV_R * MT || t >= ntok) return;
+  const size_t slot = static_cast<size_t>(slot0 + t);
+  if (a.phase == 0) {
+    const float r = GATED ? x / (1.0f + expf(-x)) * y : fmaxf(x, 0.0f);
+    if (L.act_bf16) static_cast<__nv_bfloat16*>(a.hidden)[slot * N + n] = __float2bfloat16_rn(r);
+    else static_cast<float*>(a.hidden)[slot * N + n] = r;
+  } else {
+    a.o[(static_cast<size_t>(z) * a.n_pairs + slot) * N + n] = x;
+  }
+}
+
+// What a CTA does; the codes of its first slice are on their way.
+struct Work {
+  int begin, cnt;      // the expert's slots
+  int n0, rows;        // its rows
+  int sl0, sl1, z;     // slices and plane
+};
+
+template <bool GATED, int MT>
+__device__ __forceinline__ bool token_pass(const GemvArgs& a, const ExpertDev& ex, const Width& wd, const Work& w, int c0, int ntok, const Staged& sm, uint32_t bar,
+                                           Slice& sc, uint32_t& parity, bool& first, volatile int* abort_flag) {
+  const int slot0 = w.begin + c0;
+  const bool one = w.sl1 - w.sl0 == 1;
+  float v[GEMV_R][MT], u[GEMV_R][MT];
+  for (int b = 0; b < w.rows / GEMV_ROWS; ++b) {
 #pragma unroll
     for (int r = 0; r < GEMV_R; ++r)
 #pragma unroll
-      for (int t = 0; t < MT; ++t) {
-        v[r][t] += __shfl_xor_sync(0xffffffffu, v[r][t], o);
-        if (GATED) u[r][t] += __shfl_xor_sync(0xffffffffu, u[r][t], o);
+      for (int t = 0; t < MT; ++t) v[r][t] = u[r][t] = 0.0f;
+    for (int sl = w.sl0; sl < w.sl1; ++sl) {
+      if (b == 0) {  // (with several slices there is one block)
+        __syncthreads();  // what is staged has been used
+        if (!one && !first) {
+          sc = slice_of(a, sl, wd.bits);
+          fetch_codes<GATED>(a, ex, sc, w.n0, w.rows, sm, bar);
+        }
+        const auto staging = [&] { stage_inputs(a, wd, slot0, ntok, MT, sc.k0, sc.len, sm.xs); };
+        if (first || !one) fetch_scales<GATED>(a, ex, sc, w.n0, w.rows, sm, staging);
+        else staging();
+        if (first || !one) {
+          const bool ok = mbar_wait(bar, parity, a.check_word, abort_flag);
+          parity ^= 1;
+          if (!__syncthreads_and(ok)) return false;
+        } else {
+          __syncthreads();
+        }
+        first = false;
       }
-  // every lane of the group holds all sums: lane i stores the i-th
-#pragma unroll
-  for (int r = 0; r < GEMV_R; ++r)
-#pragma unroll
-    for (int t = 0; t < MT; ++t) {
-      if (((r * MT + t) & (GEMV_LANES - 1)) != l || t >= ntok) continue;
-      const size_t slot = static_cast<size_t>(slot0 + t);
-      if (a.phase == 0) {
-        const float h = GATED ? v[r][t] / (1.0f + expf(-v[r][t])) * u[r][t] : fmaxf(v[r][t], 0.0f);
-        if (L.act_bf16) static_cast<__nv_bfloat16*>(a.hidden)[slot * N + n + r] = __float2bfloat16_rn(h);
-        else static_cast<float*>(a.hidden)[slot * N + n + r] = h;
-      } else {
-        a.o[(static_cast<size_t>(blockIdx.y % a.ksplit) * a.n_pairs + slot) * N + n + r] = v[r][t];
-      }
+      block_dot<GATED, MT>(a, wd, b, sc, sm, v, u);
     }
+    store_block<GATED, MT>(a, w.z, w.n0 + b * GEMV_ROWS, slot0, ntok, v, u);
+  }
+  return true;
 }
 
-template <int BITS, bool GATED>
-__device__ __forceinline__ void expert_rows(const GemvArgs& a, const ExpertDev& ex, int begin, int cnt, float* xs) {
-  const int n0 = static_cast<int>(blockIdx.x) * GEMV_ROWS;
-  // second projection: slices z, z + 1, ... of this plane
-  const int z = a.phase == 0 ? 0 : blockIdx.y % a.ksplit, per = a.phase == 0 ? a.nslices : (a.nslices + a.ksplit - 1) / a.ksplit;
-  const int sl0 = z * per, sl1 = min(a.nslices, sl0 + per);
-  for (int c0 = blockIdx.z * GEMV_TOK; c0 < cnt; c0 += gridDim.z * GEMV_TOK) {
-    const int ntok = min(GEMV_TOK, cnt - c0);
-    if (ntok > 2) expert_pass<BITS, GATED, 4>(a, ex, begin + c0, ntok, sl0, sl1, n0, xs);
-    else if (ntok == 2) expert_pass<BITS, GATED, 2>(a, ex, begin + c0, ntok, sl0, sl1, n0, xs);
-    else expert_pass<BITS, GATED, 1>(a, ex, begin + c0, ntok, sl0, sl1, n0, xs);
+template <bool GATED>
+__device__ __forceinline__ void expert_rows(const GemvArgs& a, const ExpertDev& ex, const Work& w, Slice sc, const Staged& sm, uint32_t bar, volatile int* abort_flag) {
+  const Width wd = width_of(ex.bits);
+  uint32_t parity = 0;
+  bool first = true, ok = true;
+  for (int c0 = blockIdx.z * GEMV_TOK; c0 < w.cnt && ok; c0 += gridDim.z * GEMV_TOK) {
+    const int ntok = min(GEMV_TOK, w.cnt - c0);
+    if (ntok > 2) ok = token_pass<GATED, 4>(a, ex, wd, w, c0, ntok, sm, bar, sc, parity, first, abort_flag);
+    else ok = token_pass<GATED, 2>(a, ex, wd, w, c0, ntok, sm, bar, sc, parity, first, abort_flag);
   }
+  if (!ok)
+    for (int i = 0; i < 2000; ++i) __nanosleep(100);  // let copies in flight land
 }
 
 template <bool GATED>  // first projection of a gated layer: two matrices
-__global__ void __launch_bounds__(GEMV_THREADS, GATED ? 4 : 5) ffn_gemv_kernel(const __grid_constant__ GemvArgs a) {
-  __shared__ __align__(16) float xs[GEMV_TOK * GEMV_SLICE];
-  pdl_wait();
-  pdl_trigger();
-  const int e = a.phase == 0 ? blockIdx.y : blockIdx.y / a.ksplit;
-  const int begin = a.off[e];
-  const int cnt = a.off[e + 1] - begin;
-  if (cnt <= 0) return;  // only activated experts are touched
-  const ExpertDev ex = a.experts[e];
-  switch (ex.bits) {
-    case 2: expert_rows<2, GATED>(a, ex, begin, cnt, xs); break;
-    case 4: expert_rows<4, GATED>(a, ex, begin, cnt, xs); break;
-    case 8: expert_rows<8, GATED>(a, ex, begin, cnt, xs); break;
-    default: break;
+__global__ void __launch_bounds__(GEMV_THREADS, GEMV_CTAS) ffn_gemv_kernel(const __grid_constant__ GemvArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(8) uint64_t bar_word;
+  __shared__ int abort_word;
+  const int rows_max = (GATED ? 2 : 1) * a.blocks * GEMV_ROWS;
+  Staged sm;
+  sm.codes = smem;
+  sm.xs = reinterpret_cast<float*>(smem + rows_max * a.slice);
+  sm.scales = sm.xs + GEMV_TOK * a.slice;
+  const uint32_t bar = smem_u32(&bar_word);
+  if (threadIdx.x == 0) {
+    abort_word = 0;
+    mbar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  const int N = a.phase == 0 ? a.L.d_ff : a.L.d_model;
+  const int e = a.phase == 0 ? blockIdx.y : blockIdx.y / a.ksplit;
+  Work w;
+  w.n0 = static_cast<int>(blockIdx.x) * a.blocks * GEMV_ROWS;
+  w.rows = min(a.blocks * GEMV_ROWS, N - w.n0);
+  // second projection: slices z, z + 1, ... of this plane
+  w.z = a.phase == 0 ? 0 : blockIdx.y % a.ksplit;
+  const int per = a.phase == 0 ? a.nslices : (a.nslices + a.ksplit - 1) / a.ksplit;
+  w.sl0 = w.z * per;
+  w.sl1 = min(a.nslices, w.sl0 + per);
+  // The table of experts is older than the kernel in front, and for the second projection so are the offsets: the first
+  // projection had waited for them when it let this kernel start.  What does not depend on the kernel in front is fetched
+  // beside it; only activated experts are touched.
+  const ExpertDev ex = a.experts[e];
+  if (a.phase == 0) {
+    pdl_wait();
+    pdl_trigger();
+  }
+  w.begin = __ldcg(a.off + e);
+  w.cnt = __ldcg(a.off + e + 1) - w.begin;
+  const bool idle = w.cnt <= static_cast<int>(blockIdx.z) * GEMV_TOK;
+  const Slice sc = slice_of(a, w.sl0, ex.bits);
+  if (!idle && w.sl0 < w.sl1) fetch_codes<GATED>(a, ex, sc, w.n0, w.rows, sm, bar);  // (the last planes may be without a slice)
+  if (a.phase == 1) {
+    pdl_wait();
+    pdl_trigger();
+  }
+  if (idle) return;
+  __syncthreads();
+  expert_rows<GATED>(a, ex, w, sc, sm, bar, &abort_word);
 }
 
 // slices of a projection over K inputs: as long as shared memory holds, of equal length, whole 128-bit words at every width
@@ -243,17 +431,45 @@ int ffn_gemv_ksplit(const LayerDims& L) {
 }
 
 cudaError_t launch_ffn_gemv(int phase, const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* perm, const int32_t* off,
-                            void* hidden, float* o, int ksplit, int n_pairs, cudaStream_t st) {
+                            void* hidden, float* o, int ksplit, int n_pairs, int* check_word, cudaStream_t st) {
   const int N = phase == 0 ? L.d_ff : L.d_model, K = phase == 0 ? L.d_model : L.d_ff;
-  GemvArgs a{phase, L, experts, x, perm, off, hidden, o, 0, 0, ksplit, n_pairs};
+  const bool gated = phase == 0 && L.act == EMOE_ACT_SWIGLU;
+  const int G = L.group > 0 ? L.group : K;
+  GemvArgs a{phase, L, experts, x, perm, off, hidden, o, 0, 0, ksplit, n_pairs, 1, G, K / G, 0, check_word};
   const int want = gemv_slices(K);
   a.slice = ((K + want - 1) / want + 63) / 64 * 64;
   a.nslices = (K + a.slice - 1) / a.slice;
-  // passes of four tokens side by side: what even routing would fill (empty CTAs cost more than a second turn of a full one)
+  a.groups = a.nslices == 1 ? K / G : (a.slice + G - 1) / G + 1;
+  const int turns = phase == 0 ? a.nslices : (a.nslices + ksplit - 1) / ksplit;  // slices a CTA takes one after another
+  const int gy = phase == 0 ? L.E : L.E * ksplit, row_blocks = N / GEMV_ROWS;
+  const size_t per_block = static_cast<size_t>(gated ? 2 : 1) * GEMV_ROWS * (a.slice + 4 * a.groups), fixed = sizeof(float) * GEMV_TOK * a.slice;
+  // Blocks of rows per CTA: a CTA's start (offsets, activations, first codes) costs about a block's time, and so does every
+  // wave of CTAs.  At least three CTAs of an SM have to be resident.
+  const auto resident = [&](int blocks) {
+    const long long by_smem = GEMV_SMEM / static_cast<long long>(fixed + blocks * per_block + 1280);
+    return by_smem < GEMV_CTAS ? by_smem : GEMV_CTAS;
+  };
+  const long long active = static_cast<long long>(n_pairs < L.E ? n_pairs : L.E) * (gy / L.E);
+  const auto waves = [&](int blocks) {
+    const long long at_once = resident(blocks) * GPU_SMS;
+    return (active * ((row_blocks + blocks - 1) / blocks) + at_once - 1) / at_once;
+  };
+  for (int b = 2; b <= GEMV_BLOCKS && turns == 1 && resident(b) >= 3; ++b)
+    if (waves(b) * (b + 1) <= waves(a.blocks) * (a.blocks + 1)) a.blocks = b;
+  const int gx = (row_blocks + a.blocks - 1) / a.blocks;
+  // passes of four tokens side by side while there is room for their CTAs
   const int passes = (n_pairs / L.E + GEMV_TOK - 1) / GEMV_TOK + (n_pairs < L.E ? 1 : 0);
-  const dim3 grid(N / GEMV_ROWS, phase == 0 ? L.E : L.E * ksplit, passes < 16 ? passes : 16);
-  if (phase == 0 && L.act == EMOE_ACT_SWIGLU) return launch_chain(ffn_gemv_kernel<true>, grid, dim3(GEMV_THREADS), 0, st, a);
-  return launch_chain(ffn_gemv_kernel<false>, grid, dim3(GEMV_THREADS), 0, st, a);
+  const long long room = resident(a.blocks) * GPU_SMS / (gx * active);
+  const int gz = room < 1 ? 1 : static_cast<int>(room < passes ? room : passes);
+  const size_t smem = fixed + a.blocks * per_block;
+  const auto launch = [&](auto kernel) -> cudaError_t {
+    if (smem > 48 * 1024) {
+      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+      if (e != cudaSuccess) return e;
+    }
+    return launch_chain(kernel, dim3(gx, gy, gz < 16 ? gz : 16), dim3(GEMV_THREADS), smem, st, a);
+  };
+  return gated ? launch(ffn_gemv_kernel<true>) : launch(ffn_gemv_kernel<false>);
 }
 
 }  // namespace emoe
