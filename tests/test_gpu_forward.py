@@ -77,6 +77,19 @@ def test_forward_cuda_core_path_at_the_edges_of_its_slices(act, adt, group, sdt,
     _run_case(shape, bits, T, seed=23, path=1)
 
 
+GEMV_BLOCK_CASES = [
+    # CTAs with several blocks of rows, the last of them with fewer; several passes of tokens over staged or refetched codes
+    ("relu", "f32", 0, "f32", 64, 4128, 8, 1, "softmax", [8, 4, 8, 4, 8, 4, 4, 8], 40),
+    ("swiglu", "f32", 64, "f16", 128, 4160, 8, 2, "softmax_renorm", [8, 4, 2, 4, 2, 8, 4, 4], 12),
+    ("relu", "f32", 0, "f16", 4128, 64, 8, 1, "softmax", [8, 4, 4, 8, 8, 4, 8, 4], 37),
+]
+
+
+@pytest.mark.parametrize("act,adt,group,sdt,d,f,E,k,gate,bits,T", GEMV_BLOCK_CASES)
+def test_forward_cuda_core_path_with_several_blocks_per_cta(act, adt, group, sdt, d, f, E, k, gate, bits, T):
+    _run_case(inputs.LayerShape(d, f, E, k, act, gate, group, sdt, adt), bits, T, seed=25, path=1)
+
+
 MMA_CASES = [
     ("relu", 128, "f16", 256, 512, 4, 1, "softmax", [2, 4, 8, 4], 10),
     ("relu", 128, "f16", 768, 3072, 8, 1, "softmax", [8, 4, 2, 4, 8, 2, 4, 8], 64),
