@@ -29,6 +29,7 @@ namespace {
 constexpr int DL_THREADS = ROUTER_THREADS;
 constexpr int DL_WARPS = DL_THREADS / 32;
 constexpr int DL_MAX_PAIRS = 16;
+constexpr int DL_TABLE = 64;                 // records of experts a CTA has at hand
 constexpr int DL_WPR_MAX = 4;                // most warps that share a row block of the second projection (a.wpr: 1, 2 or 4)
 constexpr int DL_R_MAX = 4;                  // consecutive rows of a matrix one warp takes at once
 constexpr long long DL_MAX_WEIGHTS = 8LL << 20;  // per matrix: beyond this a layer is bandwidth-bound and streams better
@@ -174,6 +175,7 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
   __shared__ float s_part[DL_WARPS][DL_R_MAX];  // [row block of the CTA][warp of the block][row]
   __shared__ float s_red[DL_THREADS];            // router product: [parts][EP]
   __shared__ float s_z[DL_WARPS][EMOE_MAX_EXPERTS];  // logits of the token a warp picks for
+  __shared__ __align__(16) ExpertDev s_table[DL_TABLE];
   __shared__ int s_flag;
   const LayerDims& L = a.L;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -184,6 +186,10 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
   // The next kernel of the chain is scheduled once every CTA of this grid has executed this, i.e.
   // once the whole grid is resident: it cannot take the room of a CTA the waits below need.
   pdl_trigger();
+  // the table of experts is older than every kernel in front (an upload is not overtaken)
+  for (int i = tid; i < min(L.E, DL_TABLE) * static_cast<int>(sizeof(ExpertDev) / 8); i += DL_THREADS)
+    reinterpret_cast<uint2*>(s_table)[i] = __ldg(reinterpret_cast<const uint2*>(a.experts) + i);
+  const auto expert = [&](int e) -> const ExpertDev& { return e < DL_TABLE ? s_table[e] : a.experts[e]; };
 
   // ---- 1. routing ----
   if (a.Wr) {
@@ -287,7 +293,7 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
       for (int j = 0; j < L.top_k; ++j) {
         const int e = s_ids[t * L.top_k + j];
         if (e < 0) continue;
-        const ExpertDev ex = a.experts[e];
+        const ExpertDev ex = expert(e);
         const int nvec = K * ex.bits / 128;
         const size_t b0 = static_cast<size_t>(static_cast<long long>(nvec) * sub / wpr) * 16;
         const size_t b1 = static_cast<size_t>(static_cast<long long>(nvec) * (sub + 1) / wpr) * 16;
@@ -335,7 +341,7 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
       const int n = static_cast<int>(u - static_cast<long long>(p) * NB) * DL_R;
       const int e = s_ids[p];
       if (e < 0) continue;
-      const ExpertDev ex = a.experts[e];
+      const ExpertDev ex = expert(e);
       const size_t bytes = static_cast<size_t>(K) * ex.bits / 8 * DL_R;  // the unit's rows follow each other
       const int n_mat = L.act == EMOE_ACT_RELU ? 1 : 2;
       for (int m = 0; m < n_mat; ++m) {
@@ -352,7 +358,7 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
 #pragma unroll
       for (int r = 0; r < DL_R; ++r) h[r] = 0.0f;
       if (e >= 0) {
-        const ExpertDev ex = a.experts[e];
+        const ExpertDev ex = expert(e);
         const int nvec = K * ex.bits / 128;
         const size_t row_bytes = static_cast<size_t>(K) * ex.bits / 8;
         const void* xrow = static_cast<const char*>(a.x) + static_cast<size_t>(p / L.top_k) * K * xsz;
@@ -415,7 +421,7 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
           const int p = t * L.top_k + j;
           const int e = s_ids[p];
           if (e < 0) continue;
-          const ExpertDev ex = a.experts[e];
+          const ExpertDev ex = expert(e);
           const int nvec = K * ex.bits / 128;
           const int j0 = static_cast<int>(static_cast<long long>(nvec) * sub / wpr);
           const int j1 = static_cast<int>(static_cast<long long>(nvec) * (sub + 1) / wpr);

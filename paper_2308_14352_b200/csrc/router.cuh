@@ -314,9 +314,10 @@ __device__ __forceinline__ void router_logits_batch(float* smem, const void* __r
 
 // Softmax and Top-K of one token by one warp from its row of logits zrow[EP] (shared memory):
 // K rounds of arg-max, ties to the lower expert index.  Lane r < top_k returns the r-th pick.
-__device__ __forceinline__ void router_pick(const float* zrow, int E, int top_k, int renorm, int lane, int& out_id,
-                                            float& out_gate) {
-  constexpr int MAXJ = EMOE_MAX_EXPERTS / 32;
+// MAXJ: values per lane (one suffices up to 32 experts).
+template <int MAXJ>
+__device__ __forceinline__ void router_pick_of(const float* zrow, int E, int top_k, int renorm, int lane, int& out_id,
+                                               float& out_gate) {
   float zv[MAXJ], pe[MAXJ];
   float m = -CUDART_INF_F;
 #pragma unroll
@@ -376,6 +377,11 @@ __device__ __forceinline__ void router_pick(const float* zrow, int E, int top_k,
   }
   out_id = my_id;
   out_gate = renorm ? my_p / psel : my_p;
+}
+
+__device__ __forceinline__ void router_pick(const float* zrow, int E, int top_k, int renorm, int lane, int& out_id, float& out_gate) {
+  if (E <= 32) router_pick_of<1>(zrow, E, top_k, renorm, lane, out_id, out_gate);
+  else router_pick_of<EMOE_MAX_EXPERTS / 32>(zrow, E, top_k, renorm, lane, out_id, out_gate);
 }
 
 }  // namespace emoe
