@@ -934,11 +934,11 @@ cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, c
   if (phase_begin == 0) per_expert += a.row_blocks[0];
   if (phase_end == 2) per_expert += static_cast<long long>(a.row_blocks[1]) * ksplit;
   const long long items = active_max * per_expert;
-  // Few tokens per activated expert and long rows: four warps with two tiles each, which read the activations once for both
-  // and meet a stage half as often (Mixtral-like layer, expert launch with eight / four warps: 1 token 77.8 / 73.7 us, 4
-  // tokens 125 / 121, 23 tokens 203 / 200; 768 x 3072, 32 experts, 64 tokens 35.5 / 36.0, 256 tokens 51 / 57, 777 tokens 79 / 86:
-  // wider passes, and items of a few stages, need the eight warps to hide their latencies).
-  const bool few = n_pairs <= 6 * active_max && L.d_model >= 1536;
+  // Few tokens per activated expert: four warps with two tiles each, which read the activations once for both and meet a stage
+  // half as often (Mixtral-like layer, expert launch with eight / four warps: 1 token 77.8 / 73.7 us, 4 tokens 125 / 121, 23
+  // tokens 203 / 200; twelve layers of 768 x 3072, 32 experts, 64 tokens 507 / 499 us, where the launch alone takes 35.5 / 36.0;
+  // per launch with 256 tokens 51 / 57, 777 tokens 79 / 86: wider passes need the eight warps to hide their latencies).
+  const bool few = n_pairs <= 6 * active_max;
   if (!L.scale_f16) return few ? launch_sc<SC_F32, 4>(a, items, st) : launch_sc<SC_F32, 8>(a, items, st);
   const bool pairs = L.group == 128 && a.ngroups[0] % 2 == 0 && a.ngroups[1] % 2 == 0;
   if (pairs) return few ? launch_sc<SC_PAIRS, 4>(a, items, st) : launch_sc<SC_PAIRS, 8>(a, items, st);
