@@ -83,7 +83,9 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 // ... by a whole warp: a branch on one lane's answer may leave the lanes apart for as long as the compiler likes, and
 // instructions that need the warp together (tcgen05.ld, tcgen05.st) may follow the wait
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* check_word, volatile int* abort_flag) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, check_word, abort_flag));
+  const bool done = mbar_try_wait(bar, parity);
+  if (__all_sync(0xffffffffu, done)) return true;
+  return __all_sync(0xffffffffu, done || mbar_wait_parked(bar, parity, check_word, abort_flag));
 }
 
 // ---- the same operations for a whole warp that runs convergent, one elected lane of which acts ----
@@ -91,11 +93,17 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, in
 // enters, every operand is moved there anew and each instruction of the loop costs its full latency
 // (a loop of four MMAs, two waits and a commit took 850 cycles); a warp that stays together, with a
 // warp index the compiler knows to be uniform, has them there already.
+__device__ __forceinline__ int warp_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 __device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x) >> 5, 0); }
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t on;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(on));
   return on;
+}
+__device__ __forceinline__ void mbar_arrive_if(uint32_t on, uint32_t bar, int count = 1) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q mbarrier.arrive.shared::cta.b64 _, [%0], %2;\n\t}" ::"r"(bar), "r"(on),
+               "r"(count)
+               : "memory");
 }
 __device__ __forceinline__ void mbar_expect_tx_if(uint32_t on, uint32_t bar, uint32_t bytes) {
   asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar),
