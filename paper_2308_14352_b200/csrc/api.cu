@@ -379,19 +379,22 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   const bool can_umma = ffn_umma_supported(L) && tmaps != nullptr;
   // The tcgen05 grouped GEMM comes in two forms (ffn_umma.cu): one rounds code x scale to fp16 and shares the dequantised
   // weights among up to 320 tokens; the other keeps the codes exact and takes 64 tokens at a time.
-  // Rounded: from 16 tokens per expert on average, on rows of whole packed boxes at every width, for the experts with
-  // more than HYBRID_STREAM_TOKENS tokens, the others stream; from 256 for all (next to nobody would be left to stream).
+  // Rounded: on rows of whole packed boxes at every width, from 48 tokens per expert on average, with more than 32 experts from 16, for
+  // the experts with more than HYBRID_STREAM_TOKENS tokens, the others stream; from 256 for all (next to nobody would be
+  // left to stream).  us per layer, rounded and streaming / exact for all, even and skewed (Zipf exponent 1.1) loads: 512 x 2048, 16
+  // experts, 500 tokens 61/39 and 60/43, 2000 tokens 57/62; 1536 x 5632, 32 experts, 800 tokens 243/154 and 167/170; 1024 x 4096, 128
+  // experts, 2048 tokens 313/268 and 183/198.
   const double mean_tokens = static_cast<double>(P) / L.E;
-  const bool rounded = mean_tokens >= 16.0 && L.d_model % 512 == 0 && L.d_ff % 512 == 0;
-  // Exact: elsewhere, from 256 (token, expert) pairs.  An uneven load can then fill an expert well beyond the 16 tokens that
-  // the streaming kernel takes per pass over the weights; an even one pays some 5 us for two launches that find
-  // nobody.  From 32 tokens per expert on average for all of them; below, for experts beyond 32 tokens, 48 where even
-  // loads reach 32 as well.  us per layer, streaming alone / both, even and skewed (Zipf exponent 1.1) loads:
-  // 768 x 3072, 32 experts, 256 tokens 58/62 and 88/85, 512 tokens 79/85 and 141/103; 1024 x 4096, 128 experts, 256 tokens 180/183 and
-  // 200/132, 1024 tokens 233/238 and 583/183; 1280 x 4480, 64 experts, 800 tokens 217/225 and 497/206; 2048 tokens on the
-  // first, all 193/146 and 505/166.
-  const bool exact_pairs = !rounded && P >= 256;
-  const bool one_family = mean_tokens >= (rounded ? 256.0 : 32.0);
+  const bool rounded = mean_tokens >= (L.E > 32 ? 16.0 : 48.0) && L.d_model % 512 == 0 && L.d_ff % 512 == 0;
+  // Exact, for all experts: elsewhere, from 14 tokens per expert on average, where about half of them need a second pass over
+  // their weights in the streaming kernel.  us, streaming / exact: 768 x 3072, 32 experts, 777 tokens 88/73; 8 experts, 128 tokens 43.5/36.3,
+  // 64 tokens (8 on average) 37/35; 512 x 2048, 8 experts, 96 tokens 27.2/28.7, 128 tokens 30.5/29.5; Mixtral-like layer, 40 tokens 229/241,
+  // 56 tokens 245/247, 64 tokens 326/248.
+  // Below that, from 256 (token, expert) pairs, for the experts beyond HYBRID_STREAM_TOKENS: an uneven load can fill an expert well beyond the
+  // 16 tokens that the streaming kernel takes per pass; an even one pays some 5 us for two launches that find nobody.  Streaming alone / both,
+  // even and skewed: 768 x 3072, 32 experts, 256 tokens 53/58 and 83/73; 1024 x 4096, 128 experts, 1024 tokens 210/215 and 483/154.
+  const bool exact_pairs = !rounded && (mean_tokens >= 14.0 || P >= 256);
+  const bool one_family = mean_tokens >= (rounded ? 256.0 : 14.0);
   const bool auto_umma = ctx->ffn_path == 0 && (rounded || exact_pairs);
   const bool exact_umma = ctx->ffn_path == 0 && !rounded;
   const bool use_hybrid = can_umma && can_tma && (ctx->ffn_path == 5 || (auto_umma && !one_family));
@@ -452,7 +455,7 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   // families can share the buffers
   const int xs_stride = static_cast<int>(act_slot_bytes(L.d_model) / 2), hid_stride = static_cast<int>(act_slot_bytes(L.d_ff) / 2);
   int* plan_heavy = reinterpret_cast<int*>(reinterpret_cast<char*>(plan) + align_up(plan_bytes(L.E)));
-  const int heavy_above = use_umma ? 0 : HYBRID_STREAM_TOKENS + (exact_umma && mean_tokens >= 16.0 ? 16 : 0);  // experts with more tokens than this are the tcgen05 kernel's
+  const int heavy_above = use_umma ? 0 : HYBRID_STREAM_TOKENS;  // experts with more tokens than this are the tcgen05 kernel's
   const int zmax = w.ksplit < 4 ? w.ksplit : 4;  // planes of partial sums its second projection may use
   if (use_hybrid) {
     // Each family has its own plan and writes only its own slots of xs / hidden / o_part.

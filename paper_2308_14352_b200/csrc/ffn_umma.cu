@@ -60,7 +60,7 @@ __host__ __device__ __forceinline__ constexpr int um_cap(int c) { return EXACT ?
 constexpr int UM_SCALE_SETS = 2;            // EXACT: sets of four warps for scales and epilogue: every other unit, or (SCALE_TOK
 constexpr int UM_SCALE_TOK = 32;            // tokens, whose sums a thread holds, and more) half of the tokens each
 constexpr int UM_SCALE_WARPS = 4 * UM_SCALE_SETS;
-constexpr int UM_SCALE_AHEAD = 4;           // EXACT: scales of a row on their way
+constexpr int UM_SCALE_AHEAD = 2;           // EXACT: scales of a row on their way
 constexpr int UM_TMEM_COLS = 512;
 // What the two forms of the kernel (see there) are made of
 template <bool EXACT>
@@ -237,10 +237,11 @@ struct TileWalk {
   const PlanRec* recs;
   int mat0, mat1;        // matrices of the projection (mat1: w3 of a gated one)
   const void *my_sp0, *my_sp1;
-  int n_active, row_blocks, cap, zs, lane;
+  int n_active, row_blocks, cap, z_log, lane;  // 2^z_log slices
   int lin;               // the next unit, from the chunk's first on
   int chunk;             // first of the 32 experts at hand
   int my_end, my_units;  // lane's expert: units up to and including it, its own
+  int my_tok;            // tokens of its groups but the last: at most cap, which is a multiple of 16
   int my_e, my_begin, my_cnt, my_bits, owner;
   int e, begin, cnt, bits;  // of the unit at hand
   __device__ __forceinline__ void load_chunk(int limit) {
@@ -265,7 +266,9 @@ struct TileWalk {
     if (lane >= n_active) my_cnt = 0;  // what an earlier call left behind
   }
   __device__ __forceinline__ void sum_units() {
-    my_units = (my_cnt + cap - 1) / cap * row_blocks * zs;
+    const int groups = (my_cnt + cap - 1) / cap;
+    my_tok = groups > 0 ? ((my_cnt + groups - 1) / groups + 15) & ~15 : 0;
+    my_units = groups * row_blocks << z_log;
     my_end = my_units;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -275,7 +278,7 @@ struct TileWalk {
   }
   __device__ __forceinline__ void start(int rb, int2 choice) {
     cap = choice.x;
-    zs = choice.y;
+    z_log = 31 - __clz(choice.y);
     row_blocks = rb;
     lin = blockIdx.x;
     sum_units();
@@ -293,17 +296,16 @@ struct TileWalk {
       sum_units();
     }
     owner = __ffs(__ballot_sync(0xffffffffu, my_end > lin)) - 1;
-    const int local = lin - __shfl_sync(0xffffffffu, my_end - my_units, owner);
+    int local = lin - __shfl_sync(0xffffffffu, my_end - my_units, owner);
     e = __shfl_sync(0xffffffffu, my_e, owner);
     begin = __shfl_sync(0xffffffffu, my_begin, owner);
     cnt = __shfl_sync(0xffffffffu, my_cnt, owner);
     bits = __shfl_sync(0xffffffffu, my_bits, owner);
-    const int groups = (cnt + cap - 1) / cap;
-    const int tok_group = ((cnt + groups - 1) / groups + 15) & ~15;  // at most cap, which is a multiple of 16
-    const int tt = local / (row_blocks * zs);
-    const int rz = local - tt * row_blocks * zs;  // the slices of a row block lie next to each other
-    rb = rz / zs;
-    z = rz - rb * zs;
+    const int tok_group = __shfl_sync(0xffffffffu, my_tok, owner);
+    int tt = 0;  // an expert has few groups: no division
+    for (; local >= row_blocks << z_log; local -= row_blocks << z_log) ++tt;
+    rb = local >> z_log;  // the slices of a row block lie next to each other
+    z = local & ((1 << z_log) - 1);
     tok0 = tt * tok_group;
     ntok = max(0, min(tok_group, cnt - tok0));  // (rounding to 16 may leave the last of many groups without tokens)
     lin += gridDim.x;
@@ -341,7 +343,7 @@ __device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, const TileWalk<!EX
     for (int z = 1; z <= a.zmax; z *= 2) {
       if (z > 1 && (kb_total % z != 0 || kb_total / z % (512 / Um<EXACT>::BK) != 0)) break;  // a slice starts on a packed box at every width
       const int rounds = (g * row_blocks * z + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
-      const float steps = static_cast<float>(kb_total / z) * fmaxf(EXACT ? 1400.0f : 450.0f, 2.0f * tok);
+      const float steps = static_cast<float>(kb_total / z) * fmaxf(EXACT ? 500.0f : 330.0f, 2.0f * tok);
       const float unit = EXACT ? steps + 1000.0f : steps + 1500.0f + 12.0f * tok;
       const float cost = static_cast<float>(rounds) * unit + static_cast<float>(z - 1) * static_cast<float>(tokens) * static_cast<float>(a.L.d_model) * (8.0f / 3400.0f);
       if (cost < best_cost) {
@@ -779,6 +781,7 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
           bool beyond = false;
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
+            if (c % 4 == 0 && c >= live) break;
             const uint32_t other = __shfl_xor_sync(0xffffffffu, second ? va[c] : va[16 + c], 16);
             const float av = __uint_as_float(second ? other : va[c]), bv = __uint_as_float(second ? va[16 + c] : other);
             // the hidden vector is a bf16 tensor
@@ -801,20 +804,26 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
           if (nrow < N) {
 #pragma unroll
             for (int c = 0; c < 32; ++c) {
+              if (c % 8 == 0 && c >= live) break;
               if (c < live) *dst = __uint_as_float(va[c]);
               dst += N;
             }
           }
         } else {
           unsigned char* mine = out_stage + (hpos - u_row0) * 2;  // [32 tokens][128 channels]
-          bool beyond = false;
+          float most = 0.0f;
 #pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            const float h = __bfloat162float(__float2bfloat16_rn(fmaxf(__uint_as_float(va[c]), 0.0f)));
-            beyond |= c < live && nrow < N && beyond_f16(h);
-            *reinterpret_cast<__half*>(mine + c * 256) = __float2half_rn(fminf(h, 65504.0f));
+          for (int c = 0; c < 32; c += 2) {
+            if (c % 8 == 0 && c >= live) break;
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(fmaxf(__uint_as_float(va[c]), 0.0f), fmaxf(__uint_as_float(va[c + 1]), 0.0f));
+            const float h0 = __low2float(h2), h1 = __high2float(h2);
+            if (c < live) most = fmaxf(most, h0);
+            if (c + 1 < live) most = fmaxf(most, h1);
+            const __half2 f2 = __floats2half2_rn(fminf(h0, 65504.0f), fminf(h1, 65504.0f));
+            *reinterpret_cast<__half*>(mine + c * 256) = __low2half(f2);
+            *reinterpret_cast<__half*>(mine + (c + 1) * 256) = __high2half(f2);
           }
-          if (beyond) atomicOr(a.check_word, CHECK_F16_RANGE);
+          if (nrow < N && beyond_f16(most)) atomicOr(a.check_word, CHECK_F16_RANGE);
           set_sync(part);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
