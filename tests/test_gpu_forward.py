@@ -615,6 +615,29 @@ def test_forward_default_with_exact_codes_on_tcgen05(act, group, sdt, d, f, E, k
     _run_case(shape, bits, T, seed=36, path=0, bias=bias)
 
 
+# One expert's tokens per group, at the edges of what an exact tcgen05 unit takes: boxes of 16 tokens, 32 sums per scaling thread (beyond,
+# both sets of scaling warps share a unit), groups of 64; steps per scale: one (two issuers), two and three (one issuer), a whole row;
+# an odd number of units and of steps, so that the sets of accumulators, stages and scaling warps meet every parity.
+EXACT_EDGE_CASES = [
+    # act, group, scale_dtype, d, f, bits, tokens of the expert
+    *[("relu", 128, "f16", 640, 768, 4, n) for n in (14, 16, 17, 31, 32, 33, 48, 64, 65, 129)],
+    ("relu", 256, "f16", 768, 1280, 2, 33),
+    ("relu", 384, "f32", 1152, 768, 8, 40),
+    ("relu", 0, "f32", 640, 1920, 8, 70),
+    ("swiglu", 128, "f16", 640, 1408, 2, 15),
+    ("swiglu", 128, "f32", 896, 640, 8, 63),
+    ("swiglu", 0, "f16", 640, 1152, 4, 97),
+]
+
+
+@pytest.mark.parametrize("act,group,sdt,d,f,bits,n", EXACT_EDGE_CASES)
+def test_forward_exact_codes_on_tcgen05_at_the_edges_of_its_units(act, group, sdt, d, f, bits, n):
+    """Two experts, the picks of every token both: n tokens each, above the mean from which the exact form takes all experts.  Sums in
+    another order move hidden values by one bf16 unit now and then: the path's tolerance, as in the other cases."""
+    shape = inputs.LayerShape(d, f, 2, 2, act, "softmax_renorm", group, sdt, "bf16")
+    assert _run_case(shape, [bits, {2: 8, 4: 2, 8: 4}[bits]], n, 700 + n, 0) <= 2e-3
+
+
 PERMUTE_EDGE_CASES = [
     # pairs of a call around the limits of the one-launch permutation (1024 pairs: one per CTA; 4096: four)
     (3, 1024, 1), (3, 1025, 1), (3, 2047, 2), (3, 2048, 2), (3, 2049, 2), (4, 1366, 3), (5, 1367, 3),
