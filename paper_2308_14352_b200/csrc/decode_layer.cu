@@ -186,9 +186,15 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
   // The next kernel of the chain is scheduled once every CTA of this grid has executed this, i.e.
   // once the whole grid is resident: it cannot take the room of a CTA the waits below need.
   pdl_trigger();
-  // the table of experts is older than every kernel in front (an upload is not overtaken)
-  for (int i = tid; i < min(L.E, DL_TABLE) * static_cast<int>(sizeof(ExpertDev) / 8); i += DL_THREADS)
-    reinterpret_cast<uint2*>(s_table)[i] = __ldg(reinterpret_cast<const uint2*>(a.experts) + i);
+  // the records of the experts come into shared memory while the routing runs, behind the wait for the kernels in front like
+  // every other read
+  const auto fetch_table = [&]() {
+    for (int i = tid; i < min(L.E, DL_TABLE) * static_cast<int>(sizeof(ExpertDev) / 8); i += DL_THREADS)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(reinterpret_cast<uint2*>(s_table) + i))),
+                   "l"(reinterpret_cast<const uint2*>(a.experts) + i)
+                   : "memory");
+  };
+  const auto table_here = []() { asm volatile("cp.async.wait_all;" ::: "memory"); };
   const auto expert = [&](int e) -> const ExpertDev& { return e < DL_TABLE ? s_table[e] : a.experts[e]; };
 
   // ---- 1. routing ----
@@ -205,6 +211,7 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
       prefetch_l2(a.Wr + static_cast<size_t>(kb) * L.E, static_cast<size_t>(ke - kb) * L.E * 4, tid, DL_THREADS);
       prefetch_l2(static_cast<const char*>(a.x) + (static_cast<size_t>(t) * d + kb) * xsz, (ke - kb) * xsz, tid, DL_THREADS);
       pdl_wait();
+      fetch_table();
       const auto product = [&](const auto* xrow) {
         constexpr int U = 16;  // independent loads in flight per thread: a slice of up to 128 inputs of 32 experts in one round trip
         for (int i = kb + part; i < ke; i += U * S) {
@@ -234,10 +241,12 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
       }
     } else {
       pdl_wait();
+      fetch_table();
     }
-    if (!grid_arrive_wait(a.sync, static_cast<unsigned>(n_route + a.extra_arrivals), static_cast<int>(blockIdx.x) < n_route,
-                          a.wait_limit, a.check_word, &s_flag))
-      return;
+    const bool routed = grid_arrive_wait(a.sync, static_cast<unsigned>(n_route + a.extra_arrivals), static_cast<int>(blockIdx.x) < n_route,
+                                         a.wait_limit, a.check_word, &s_flag);
+    table_here();
+    if (!routed) return;
     // every CTA makes the picks of every token from the same numbers in the same order
     for (int t = warp; t < a.T; t += DL_WARPS) {
       float* zrow = s_z[warp];
@@ -265,6 +274,7 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
     }
   } else {
     pdl_wait();
+    fetch_table();
     if (tid < P) {
       int id = __ldcg(a.ids_in + tid);
       if (id < 0 || id >= L.E) {  // only a caller's picks can be out of range
@@ -274,6 +284,7 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
       s_ids[tid] = id;
       s_gates[tid] = __ldcg(a.gates_in + tid);
     }
+    table_here();
   }
   __syncthreads();
 
