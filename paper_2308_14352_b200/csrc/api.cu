@@ -382,19 +382,19 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   // Rounded: on rows of whole packed boxes at every width, from 48 tokens per expert on average, with more than 32 experts from 16, for
   // the experts with more than HYBRID_STREAM_TOKENS tokens, the others stream; from 256 for all (next to nobody would be
   // left to stream).  us per layer, rounded and streaming / exact for all, even and skewed (Zipf exponent 1.1) loads: 512 x 2048, 16
-  // experts, 500 tokens 61/39 and 60/43, 2000 tokens 57/62; 1536 x 5632, 32 experts, 800 tokens 243/154 and 167/170; 1024 x 4096, 128
-  // experts, 2048 tokens 313/268 and 183/198.
+  // experts, 500 tokens 61/35 and 60/39, 2000 tokens 57/62 (even); 1536 x 5632, 32 experts, 800 tokens 243/145 and 167/156; 64 experts, 2048
+  // tokens 388/276 and 249/274; 1024 x 4096, 128 experts, 2048 tokens 313/250 and 177/184.
   const double mean_tokens = static_cast<double>(P) / L.E;
   const bool rounded = mean_tokens >= (L.E > 32 ? 16.0 : 48.0) && L.d_model % 512 == 0 && L.d_ff % 512 == 0;
-  // Exact, for all experts: elsewhere, from 14 tokens per expert on average, where about half of them need a second pass over
-  // their weights in the streaming kernel.  us, streaming / exact: 768 x 3072, 32 experts, 777 tokens 88/73; 8 experts, 128 tokens 43.5/36.3,
-  // 64 tokens (8 on average) 37/35; 512 x 2048, 8 experts, 96 tokens 27.2/28.7, 128 tokens 30.5/29.5; Mixtral-like layer, 40 tokens 229/241,
-  // 56 tokens 245/247, 64 tokens 326/248.
-  // Below that, from 256 (token, expert) pairs, for the experts beyond HYBRID_STREAM_TOKENS: an uneven load can fill an expert well beyond the
-  // 16 tokens that the streaming kernel takes per pass; an even one pays some 5 us for two launches that find nobody.  Streaming alone / both,
-  // even and skewed: 768 x 3072, 32 experts, 256 tokens 53/58 and 83/73; 1024 x 4096, 128 experts, 1024 tokens 210/215 and 483/154.
-  const bool exact_pairs = !rounded && (mean_tokens >= 14.0 || P >= 256);
-  const bool one_family = mean_tokens >= (rounded ? 256.0 : 14.0);
+  // Exact, for all experts: elsewhere, from 10 tokens per expert on average, from 8 with 256 (token, expert) pairs, which an uneven load
+  // may give to a few experts; the streaming kernel takes 16 tokens per pass over the weights.  us, streaming / exact: 768 x 3072, 32 experts,
+  // 777 tokens 88/65, 256 tokens 52/53 (skewed 82/49); 8 experts, 64 tokens 36.8/30.5; 512 x 2048, 8 experts, 64 tokens 25.6/26.4, 96
+  // tokens 27.5/26.9; Mixtral-like layer, 32 tokens 217/230, 40 tokens 228/231, 64 tokens 326/240; 1024 x 4096, 128 experts,
+  // 1024 tokens 209/208 (skewed 474/132), 200 tokens 146/200.
+  // Below that, from 256 pairs, for the experts beyond HYBRID_STREAM_TOKENS; an even load pays some 5 us for two launches that find nobody.
+  // Streaming alone / both, even and skewed: 1024 x 4096, 128 experts, 256 tokens 180/183 and 200/132.
+  const bool exact_pairs = !rounded && (mean_tokens >= 10.0 || P >= 256);
+  const bool one_family = mean_tokens >= (rounded ? 256.0 : P >= 256 ? 8.0 : 10.0);
   const bool auto_umma = ctx->ffn_path == 0 && (rounded || exact_pairs);
   const bool exact_umma = ctx->ffn_path == 0 && !rounded;
   const bool use_hybrid = can_umma && can_tma && (ctx->ffn_path == 5 || (auto_umma && !one_family));

@@ -52,7 +52,7 @@ struct LayerDims {
 // serialization" attribute: the next kernel of the chain may start its prologue (barrier set-up,
 // tensor-memory allocation, prefetches into L2) while the
 // current one drains.  Device side, every kernel executes pdl_wait() before it reads or writes global memory: the inputs
-// of a call, too, may be what the call in front leaves.  pdl_trigger()
+// of a call, too, may be what the call in front leaves.  (One exception, which says why: ffn_umma.cu's second projection.)  pdl_trigger()
 // lets the kernel behind it start.  Without the attribute both are no-ops.
 extern thread_local bool g_pdl_enabled;
 

@@ -511,7 +511,11 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
-  pdl_wait();  // barrier set-up and the tensor-memory allocation overlap the kernel in front
+  // Barrier set-up and the tensor-memory allocation overlap the kernel in front.  The second projection needs nothing of the first
+  // but its hidden values: the plan was complete before the first started (it waits itself before it lets this one in), so only
+  // the producer of the activations waits, and codes, scales and dequantisation are under way where the first has left an SM
+  // (768 x 3072, 32 experts, 777 tokens: 72.8 -> 64.9 us per layer; Mixtral-like layer, 64 tokens 257 -> 241).
+  if (a.phase == 0) pdl_wait();
   pdl_trigger();
 
   const LayerDims& L = a.L;
@@ -533,6 +537,7 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
 
   if (warp == 0) {
     // ---------------- producer of the activations ----------------
+    if (a.phase != 0) pdl_wait();
     const uint32_t on = elect_one();
     int it = 0;
     bool ok = true;
@@ -780,14 +785,18 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
           unsigned char* mine = stage + c0 * 128 + (((hpos - u_row0) * 2) ^ (second ? 64 : 0));
           bool beyond = false;
 #pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            if (c % 4 == 0 && c >= live) break;
-            const uint32_t other = __shfl_xor_sync(0xffffffffu, second ? va[c] : va[16 + c], 16);
-            const float av = __uint_as_float(second ? other : va[c]), bv = __uint_as_float(second ? va[16 + c] : other);
-            // the hidden vector is a bf16 tensor
-            const float h = __bfloat162float(__float2bfloat16_rn(silu_branchless(av) * bv));
-            beyond |= c0 + c < live && beyond_f16(h);  // columns past the last token read whatever lies behind it
-            *reinterpret_cast<__half*>(mine + c * 128) = __float2half_rn(fminf(fmaxf(h, -65504.0f), 65504.0f));
+          for (int b4 = 0; b4 < 16; b4 += 4) {
+            if (b4 < live) {
+#pragma unroll
+              for (int c = b4; c < b4 + 4; ++c) {
+                const uint32_t other = __shfl_xor_sync(0xffffffffu, second ? va[c] : va[16 + c], 16);
+                const float av = __uint_as_float(second ? other : va[c]), bv = __uint_as_float(second ? va[16 + c] : other);
+                // the hidden vector is a bf16 tensor
+                const float h = __bfloat162float(__float2bfloat16_rn(silu_branchless(av) * bv));
+                beyond |= c0 + c < live && beyond_f16(h);  // columns past the last token read whatever lies behind it
+                *reinterpret_cast<__half*>(mine + c * 128) = __float2half_rn(fminf(fmaxf(h, -65504.0f), 65504.0f));
+              }
+            }
           }
           if (beyond) atomicOr(a.check_word, CHECK_F16_RANGE);  // saturated above: reported, not silent
           set_sync(part);
@@ -803,25 +812,33 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
           float* dst = a.o + z * a.plane_stride + (slot0 + cc) * N + nrow;
           if (nrow < N) {
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              if (c % 8 == 0 && c >= live) break;
-              if (c < live) *dst = __uint_as_float(va[c]);
-              dst += N;
+            for (int b8 = 0; b8 < 32; b8 += 8) {
+              if (b8 < live) {
+#pragma unroll
+                for (int c = b8; c < b8 + 8; ++c) {
+                  if (c < live) *dst = __uint_as_float(va[c]);
+                  dst += N;
+                }
+              }
             }
           }
         } else {
           unsigned char* mine = out_stage + (hpos - u_row0) * 2;  // [32 tokens][128 channels]
           float most = 0.0f;
 #pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            if (c % 8 == 0 && c >= live) break;
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(fmaxf(__uint_as_float(va[c]), 0.0f), fmaxf(__uint_as_float(va[c + 1]), 0.0f));
-            const float h0 = __low2float(h2), h1 = __high2float(h2);
-            if (c < live) most = fmaxf(most, h0);
-            if (c + 1 < live) most = fmaxf(most, h1);
-            const __half2 f2 = __floats2half2_rn(fminf(h0, 65504.0f), fminf(h1, 65504.0f));
-            *reinterpret_cast<__half*>(mine + c * 256) = __low2half(f2);
-            *reinterpret_cast<__half*>(mine + (c + 1) * 256) = __high2half(f2);
+          for (int b8 = 0; b8 < 32; b8 += 8) {
+            if (b8 < live) {
+#pragma unroll
+              for (int c = b8; c < b8 + 8; c += 2) {
+                const __nv_bfloat162 h2 = __floats2bfloat162_rn(fmaxf(__uint_as_float(va[c]), 0.0f), fmaxf(__uint_as_float(va[c + 1]), 0.0f));
+                const float h0 = __low2float(h2), h1 = __high2float(h2);
+                if (c < live) most = fmaxf(most, h0);
+                if (c + 1 < live) most = fmaxf(most, h1);
+                const __half2 f2 = __floats2half2_rn(fminf(h0, 65504.0f), fminf(h1, 65504.0f));
+                *reinterpret_cast<__half*>(mine + c * 256) = __low2half(f2);
+                *reinterpret_cast<__half*>(mine + (c + 1) * 256) = __high2half(f2);
+              }
+            }
           }
           if (nrow < N && beyond_f16(most)) atomicOr(a.check_word, CHECK_F16_RANGE);
           set_sync(part);
