@@ -27,7 +27,7 @@
 //   warps 11-18 (EXACT, see the kernel) scales and epilogue, two sets of four, while the others go on with the next unit;
 //   warp 1    one thread issues tcgen05.mma (M128, N = the group's tokens rounded up to 16, in two halves
 //             beyond 256, K16, fp16 x fp16 -> fp32) per 16 inputs and commits each stage back (EXACT: warp 19 every other one).
-// A step costs two cycles per token in the tensor pipe and some 450 in the dequantisation, so groups of
+// A step costs two cycles per token in the tensor pipe and some 330 to 450 in the dequantisation, so groups of
 // about 256 tokens and more are tensor-bound; an expert's tokens are split evenly (choose_cut, TileWalk).
 // Measured (4096 x 14336 gated, 8 experts, 2048 tokens, 4 bits, both launches): 2040 us with one issuing lane in a branch
 // and groups of whole 128-token tiles, 1053 us now: 1.37 PFLOP/s, 0.85 of the measured dense rate.  Few tokens are bound by
@@ -322,7 +322,7 @@ struct TileWalk {
 
 // How a launch is cut (every warp works it out for itself): most tokens of a group, slices of the second projection's inputs.  Larger groups share
 // the dequantisation, smaller ones and slices fill the last round of CTAs.  The estimate, in cycles: a
-// step of 64 inputs takes two per token or the 450 of the dequantisation (EXACT: 700 for the sums), a unit 1500 + 12
+// step of 64 inputs takes two per token or the 330 of the dequantisation (EXACT: 500 for one of 128), a unit 1500 + 12
 // per token to start and store; a further plane of sums costs the combine step its bandwidth (3400 B per cycle).
 template <bool EXACT>
 __device__ __forceinline__ int2 choose_cut(const UmmaArgs& a, const TileWalk<!EXACT>& walk, int row_blocks, int kb_total) {
@@ -458,11 +458,11 @@ __device__ __forceinline__ void set_sync(int part) { asm volatile("bar.sync %0, 
 // group out of tensor memory and add them, times the row's scale, in fp32 registers, as the streaming kernel does.
 // Groups of up to 64 tokens, four sets of accumulators in turn, steps of 128 inputs (the usual scale group).  What bounds it is the
 // hand-over between the roles, hence: two issuing warps; every other unit to the other set of scaling warps, whose
-// epilogue then hides behind the next unit; two runs read at a time; scales asked for four groups ahead; activations in boxes of 16
+// epilogue then hides behind the next unit; two runs read at a time; scales asked for two groups ahead; activations in boxes of 16
 // tokens (boxes of 64 were four times the L2 traffic at few tokens).  One set of scaling warps of 64 tokens each: 10 us more at 4096 x
 // 14336 and at 768 x 3072 alike; three sets of dequantising warps: nothing.
-// us per layer, before -> after: 768 x 3072, 32 experts, 512 tokens 84.7 -> 65.9, 777 tokens 90.7 -> 74.5, 2048 tokens 121 -> 99;
-// Mixtral-like layer, 23 tokens 440 -> 242, 2048 tokens (for comparison) 3214 -> 2290.
+// us per layer, before -> after: 768 x 3072, 32 experts, 512 tokens 84.7 -> 65.9, 777 tokens 90.7 -> 74.5, 2048 tokens 121 -> 99
+// (and 64.9 and 90 with the early start of the second projection); Mixtral-like layer, 23 tokens 440 -> 242 (231).
 template <bool EXACT>
 __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
     ffn_umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap tmap_b) {

@@ -615,6 +615,14 @@ def test_forward_default_with_exact_codes_on_tcgen05(act, group, sdt, d, f, E, k
     _run_case(shape, bits, T, seed=36, path=0, bias=bias)
 
 
+@pytest.mark.parametrize("act,d,f,E,k,bits,T", [("relu", 512, 512, 40, 1, [8, 4, 2, 4] * 10, 300),
+                                                ("swiglu", 640, 640, 48, 2, [4, 8, 2, 4] * 12, 160)])
+def test_forward_default_with_some_experts_on_tcgen05_beside_the_streaming_kernel(act, d, f, E, k, bits, T):
+    """Fewer than 8 tokens per expert on average, uneven loads: the experts beyond 32 tokens take the exact form, the others stream."""
+    shape = inputs.LayerShape(d, f, E, k, act, "softmax" if k == 1 else "softmax_renorm", 128, "f16", "bf16")
+    _run_case(shape, bits, T, seed=41, path=0, bias=(-2.2 * np.log(np.arange(1, E + 1))).astype(np.float32))
+
+
 # One expert's tokens per group, at the edges of what an exact tcgen05 unit takes: boxes of 16 tokens, 32 sums per scaling thread (beyond,
 # both sets of scaling warps share a unit), groups of 64; steps per scale: one (two issuers), two and three (one issuer), a whole row;
 # an odd number of units and of steps, so that the sets of accumulators, stages and scaling warps meet every parity.
