@@ -463,10 +463,9 @@ cudaError_t launch_ffn_gemv(int phase, const LayerDims& L, const ExpertDev* expe
   const int gz = room < 1 ? 1 : static_cast<int>(room < passes ? room : passes);
   const size_t smem = fixed + a.blocks * per_block;
   const auto launch = [&](auto kernel) -> cudaError_t {
-    if (smem > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-      if (e != cudaSuccess) return e;
-    }
+    // whatever the size: the 48 KB that need no asking hold the kernel's static words too
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
     return launch_chain(kernel, dim3(gx, gy, gz < 16 ? gz : 16), dim3(GEMV_THREADS), smem, st, a);
   };
   return gated ? launch(ffn_gemv_kernel<true>) : launch(ffn_gemv_kernel<false>);

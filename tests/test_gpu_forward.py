@@ -4,6 +4,10 @@ Bars: permutation bit-exact; ids exact outside the 1e-4 logit margin; outputs wi
 max|y - y_ref| / max|y_ref| <= 2e-3 (bf16 activations) or 1e-5 (fp32 activations).  The
 reference is always evaluated with the ids the GPU picked, so a legal tie-break difference
 does not leak into the output comparison."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -88,6 +92,16 @@ GEMV_BLOCK_CASES = [
 @pytest.mark.parametrize("act,adt,group,sdt,d,f,E,k,gate,bits,T", GEMV_BLOCK_CASES)
 def test_forward_cuda_core_path_with_several_blocks_per_cta(act, adt, group, sdt, d, f, E, k, gate, bits, T):
     _run_case(inputs.LayerShape(d, f, E, k, act, gate, group, sdt, adt), bits, T, seed=25, path=1)
+
+
+@pytest.mark.parametrize("d,f,group", [(512, 64, 16), (576, 96, 48)])
+def test_forward_cuda_core_path_with_exactly_48_kb(d, f, group):
+    """A first projection of one block of rows whose codes, scales and activations are 49152 bytes of shared memory: what a kernel may
+    take without asking, less its static words.  In a process of its own, where no other launch has raised the limit."""
+    assert 2 * 32 * (d + 4 * (d // group)) + 4 * 4 * d == 48 * 1024
+    code = ("from tests.test_gpu_forward import _run_case, inputs\n"
+            f"_run_case(inputs.LayerShape({d}, {f}, 2, 1, 'swiglu', 'softmax', {group}, 'f32', 'f32'), [8, 8], 3, seed=24, path=0)")
+    subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))), check=True, timeout=300)
 
 
 MMA_CASES = [
