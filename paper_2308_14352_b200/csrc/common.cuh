@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/emoe.h"
 
 namespace emoe {
@@ -75,6 +77,23 @@ inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block,
     cfg.numAttrs = 1;
   }
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Lets every launch of a kernel have up to `most` bytes of dynamic shared memory, the most that any of them asks for.  The limit
+// belongs to the kernel on a device, not to a launch, and contexts of other host threads launch the same kernel: it is raised
+// once per device and never written again (a thread that set its own launch's size could lower it under
+// another thread's, whose launch was then refused).
+template <auto KERNEL>
+inline cudaError_t allow_smem(int most) {
+  static std::atomic<bool> raised[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (raised[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, most);  // (two threads may: to the same value)
+  if (e == cudaSuccess) raised[dev].store(true, std::memory_order_release);
+  return e;
 }
 
 // expert cache of a context (cache.cu)

@@ -37,6 +37,10 @@ constexpr int GEMV_ROWS = GEMV_WARPS * (32 / GEMV_LANES) * GEMV_R;  // rows of a
 constexpr int GEMV_CTAS = 4;      // per SM (registers)
 constexpr int GEMV_BLOCKS = 4;    // of a CTA, at most
 constexpr int GEMV_SMEM = 226 * 1024;  // of an SM, with what the system keeps per CTA taken off below
+constexpr int GEMV_GROUP = 16;    // inputs per scale, at least: a 128-bit word of 8-bit codes
+// codes, scales and activations of one block of a gated first projection: the most a CTA takes (several blocks: a third of an SM)
+constexpr int GEMV_CTA_SMEM = 2 * GEMV_ROWS * (GEMV_SLICE + 4 * (GEMV_SLICE / GEMV_GROUP + 1)) + 4 * GEMV_TOK * GEMV_SLICE;
+static_assert(GEMV_SMEM / 3 <= GEMV_CTA_SMEM && GEMV_CTA_SMEM <= GEMV_SMEM, "shared memory");
 
 // two fp32 numbers in a register pair: sums and products of both by one instruction
 typedef unsigned long long f32x2;
@@ -462,13 +466,11 @@ cudaError_t launch_ffn_gemv(int phase, const LayerDims& L, const ExpertDev* expe
   const long long room = resident(a.blocks) * GPU_SMS / (gx * active);
   const int gz = room < 1 ? 1 : static_cast<int>(room < passes ? room : passes);
   const size_t smem = fixed + a.blocks * per_block;
-  const auto launch = [&](auto kernel) -> cudaError_t {
-    // whatever the size: the 48 KB that need no asking hold the kernel's static words too
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    return launch_chain(kernel, dim3(gx, gy, gz < 16 ? gz : 16), dim3(GEMV_THREADS), smem, st, a);
-  };
-  return gated ? launch(ffn_gemv_kernel<true>) : launch(ffn_gemv_kernel<false>);
+  if (smem > GEMV_CTA_SMEM) return cudaErrorInvalidValue;
+  const dim3 grid(gx, gy, gz < 16 ? gz : 16), block(GEMV_THREADS);
+  const cudaError_t e = gated ? allow_smem<ffn_gemv_kernel<true>>(GEMV_CTA_SMEM) : allow_smem<ffn_gemv_kernel<false>>(GEMV_CTA_SMEM);
+  if (e != cudaSuccess) return e;
+  return gated ? launch_chain(ffn_gemv_kernel<true>, grid, block, smem, st, a) : launch_chain(ffn_gemv_kernel<false>, grid, block, smem, st, a);
 }
 
 }  // namespace emoe

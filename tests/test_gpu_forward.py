@@ -7,6 +7,7 @@ does not leak into the output comparison."""
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -102,6 +103,62 @@ def test_forward_cuda_core_path_with_exactly_48_kb(d, f, group):
     code = ("from tests.test_gpu_forward import _run_case, inputs\n"
             f"_run_case(inputs.LayerShape({d}, {f}, 2, 1, 'swiglu', 'softmax', {group}, 'f32', 'f32'), [8, 8], 3, seed=24, path=0)")
     subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))), check=True, timeout=300)
+
+
+def _side_by_side(jobs, rounds):
+    """Runs every job (a function of the stream) `rounds` times in a host thread and on a stream of its own; raises what one of them raised."""
+    errors, start = [], threading.Barrier(len(jobs))
+
+    def work(job):
+        try:
+            stream = torch.cuda.Stream()
+            start.wait()
+            for i in range(rounds):
+                job(stream.cuda_stream)
+                if i % 16 == 15:  # threads that wait for a place in a full queue do not meet
+                    stream.synchronize()
+            stream.synchronize()
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(j,)) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    if errors:
+        raise errors[0]
+
+
+def test_forward_cuda_core_path_in_several_host_threads():
+    """A context per thread, layers whose launches of the same kernel need 50 and 80 KB of shared memory: the one's launches must not
+    take away what the other's need, and each must get what it gets alone."""
+    moes, jobs, ys, want = [], [], [], []
+    try:
+        for i, d in enumerate((1024, 640, 1024, 640)):
+            shape = inputs.LayerShape(d, 64, 1, 1, "swiglu", "softmax", 0, "f32", "f32")
+            moe = layer.MoELayer(shape, [8], max_tokens=1)
+            moes.append(moe)
+            moe.pack_from_host(inputs.expert_set(51 + i, 0, shape, 0.02))
+            x = torch.from_numpy(inputs.activations(51 + i, 0, 1, d, "f32")).cuda()
+            Wr = torch.from_numpy(inputs.router_weight(51 + i, 0, d, 1, std=0.05)).cuda()
+            y = torch.empty(1, d, device="cuda")
+            B.emoe_set_ffn_path(moe.ctx, 1)
+            B.emoe_set_fused_layer(moe.ctx, 0)
+            moe.forward_device(x, Wr, None, y)
+            torch.cuda.synchronize()
+            want.append(y.clone())
+            y.fill_(float("nan"))
+            ys.append(y)
+            jobs.append(lambda st, a=(moe, x, Wr, y): a[0].forward_device(a[1], a[2], None, a[3], stream=st))
+        torch.cuda.synchronize()
+        _side_by_side(jobs, 10000)
+        for y, w in zip(ys, want):
+            assert torch.equal(y, w)
+    finally:
+        torch.cuda.synchronize()
+        for moe in moes:
+            moe.close()
 
 
 MMA_CASES = [
