@@ -12,6 +12,8 @@
 // per-warp count table, so no order-dependent atomics decide a position.
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "router.cuh"
 #include "scatter.cuh"
@@ -270,31 +272,32 @@ cudaError_t launch_router_topk(const void* x, int x_bf16, int T, int d, const fl
   // CTA (every CTA reads the whole router matrix from L2).  Experts in groups of four, rows in
   // 16-byte pieces: the register-tiled product.
   const bool tiled = E >= 4 && E % 4 == 0 && d % 8 == 0 && reinterpret_cast<uintptr_t>(Wr) % 16 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
-  const auto launch = [&](auto kernel, int tt, size_t smem, int threads = ROUTER_BATCH_THREADS) -> cudaError_t {
-    if (smem > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-      if (e != cudaSuccess) return e;
-    }
+  const auto launch = [&](auto kernel, int tt, size_t smem, int threads) -> cudaError_t {
     return launch_chain(kernel, dim3((T + tt - 1) / tt), dim3(threads), smem, st, x, x_bf16, T, d, Wr, bias, bias_stride, E, EP, sh,
                         top_k, renorm, ids, ids_copy, gates, logits);
   };
-  if (tiled && T >= 96 * 16) {
-    const size_t smem = router_batch_smem(16, EP);
-    if (router_batch_chunk(EP) == 512) return launch(router_topk_kernel<16, 512>, 16, smem);
-    if (router_batch_chunk(EP) == 256) return launch(router_topk_kernel<16, 256>, 16, smem);
-    if (router_batch_chunk(EP) == 128) return launch(router_topk_kernel<16, 128>, 16, smem);
-    return launch(router_topk_kernel<16, 64>, 16, smem);
-  }
-  if (tiled && T >= GPU_SMS) {
-    const size_t smem = router_batch_smem(8, EP);
-    if (router_batch_chunk(EP) == 512) return launch(router_topk_kernel<8, 512>, 8, smem);
-    if (router_batch_chunk(EP) == 256) return launch(router_topk_kernel<8, 256>, 8, smem);
-    if (router_batch_chunk(EP) == 128) return launch(router_topk_kernel<8, 128>, 8, smem);
-    return launch(router_topk_kernel<8, 64>, 8, smem);
-  }
-  if (T < GPU_SMS && router_one_supported(E, Wr))
+  // the register-tiled product of TT tokens per CTA in chunks of BC inputs
+  const auto batch = [&](auto tt, auto bc) -> cudaError_t {
+    constexpr int TT = decltype(tt)::value, BC = decltype(bc)::value;
+    const cudaError_t e = allow_smem<router_topk_kernel<TT, BC>>(router_batch_most(TT, BC));
+    return e != cudaSuccess ? e : launch(router_topk_kernel<TT, BC>, TT, router_batch_smem(TT, EP), ROUTER_BATCH_THREADS);
+  };
+  const auto batch_of = [&](auto tt) -> cudaError_t {
+    switch (router_batch_chunk(EP)) {
+      case 512: return batch(tt, std::integral_constant<int, 512>());
+      case 256: return batch(tt, std::integral_constant<int, 256>());
+      case 128: return batch(tt, std::integral_constant<int, 128>());
+      default: return batch(tt, std::integral_constant<int, 64>());
+    }
+  };
+  if (tiled && T >= 96 * 16) return batch_of(std::integral_constant<int, 16>());
+  if (tiled && T >= GPU_SMS) return batch_of(std::integral_constant<int, 8>());
+  if (T < GPU_SMS && router_one_supported(E, Wr)) {
+    static_assert(router_one_smem(EMOE_MAX_EXPERTS) <= 48 * 1024, "no larger limit is asked for");
     return launch(router_topk_kernel<1, -1>, 1, router_one_smem(E), ROUTER_ONE_THREADS);
-  if (T >= 8 * 64) return launch(router_topk_kernel<8, 0>, 8, sizeof(float) * (8 * ROUTER_DC + ROUTER_THREADS * 8 + 8 * EP), ROUTER_THREADS);  // <= 48 KB
+  }
+  static_assert(sizeof(float) * (8 * ROUTER_DC + ROUTER_THREADS * 8 + 8 * EMOE_MAX_EXPERTS) <= 48 * 1024, "no larger limit is asked for");
+  if (T >= 8 * 64) return launch(router_topk_kernel<8, 0>, 8, sizeof(float) * (8 * ROUTER_DC + ROUTER_THREADS * 8 + 8 * EP), ROUTER_THREADS);
   return launch(router_topk_kernel<1, 0>, 1, sizeof(float) * (ROUTER_DC + ROUTER_THREADS + EP), ROUTER_THREADS);
 }
 

@@ -189,6 +189,13 @@ __host__ __device__ constexpr int router_batch_floats_w(int tt, int EP) {
 __host__ __device__ constexpr int router_batch_smem(int tt, int EP) {
   return (router_batch_floats_w(tt, EP) + tt * router_batch_chunk(EP) + tt * EP) * 4;
 }
+// the most that any number of experts with chunks of bc inputs takes
+constexpr int router_batch_most(int tt, int bc) {
+  int most = 0;
+  for (int EP = 4; EP <= EMOE_MAX_EXPERTS; EP *= 2)
+    if (router_batch_chunk(EP) == bc && router_batch_smem(tt, EP) > most) most = router_batch_smem(tt, EP);
+  return most;
+}
 
 template <int TT, int BC>
 __device__ __forceinline__ void router_logits_batch(float* smem, const void* __restrict__ x, int x_bf16, int T, int d,

@@ -1,5 +1,8 @@
 """Shared helpers of the GPU parity tests: oracle-side packing of a layer and the metrics."""
+import threading
+
 import numpy as np
+import torch
 
 import oracle
 from paper_2308_14352_b200 import inputs
@@ -43,3 +46,28 @@ def check_ids(ids_gpu, logits_ref, k, margin=1e-4):
                 assert abs(z[ids_gpu[t, j]] - srt[j]) <= margin
             assert len(set(ids_gpu[t].tolist())) == k
     return strict
+
+
+def side_by_side(jobs, rounds):
+    """Runs every job (a function of the stream) `rounds` times in a host thread and on a stream of its own; raises what one of them raised."""
+    errors, start = [], threading.Barrier(len(jobs))
+
+    def work(job):
+        try:
+            stream = torch.cuda.Stream()
+            start.wait()
+            for i in range(rounds):
+                job(stream.cuda_stream)
+                if i % 16 == 15:  # threads that wait for a place in a full queue do not meet
+                    stream.synchronize()
+            stream.synchronize()
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(j,)) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    if errors:
+        raise errors[0]

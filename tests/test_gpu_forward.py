@@ -7,7 +7,6 @@ does not leak into the output comparison."""
 import os
 import subprocess
 import sys
-import threading
 
 import numpy as np
 import pytest
@@ -15,7 +14,7 @@ import torch
 
 import oracle
 from paper_2308_14352_b200 import binding as B, inputs, layer
-from tests.helpers import check_ids, oracle_pack_layer, output_tolerance, rel_to_max
+from tests.helpers import check_ids, oracle_pack_layer, output_tolerance, rel_to_max, side_by_side
 
 pytestmark = pytest.mark.gpu
 
@@ -105,31 +104,6 @@ def test_forward_cuda_core_path_with_exactly_48_kb(d, f, group):
     subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))), check=True, timeout=300)
 
 
-def _side_by_side(jobs, rounds):
-    """Runs every job (a function of the stream) `rounds` times in a host thread and on a stream of its own; raises what one of them raised."""
-    errors, start = [], threading.Barrier(len(jobs))
-
-    def work(job):
-        try:
-            stream = torch.cuda.Stream()
-            start.wait()
-            for i in range(rounds):
-                job(stream.cuda_stream)
-                if i % 16 == 15:  # threads that wait for a place in a full queue do not meet
-                    stream.synchronize()
-            stream.synchronize()
-        except Exception as e:  # noqa: BLE001
-            errors.append(e)
-
-    threads = [threading.Thread(target=work, args=(j,)) for j in jobs]
-    for t in threads:
-        t.start()
-    for t in threads:
-        t.join()
-    if errors:
-        raise errors[0]
-
-
 def test_forward_cuda_core_path_in_several_host_threads():
     """A context per thread, layers whose launches of the same kernel need 50 and 80 KB of shared memory: the one's launches must not
     take away what the other's need, and each must get what it gets alone."""
@@ -152,7 +126,7 @@ def test_forward_cuda_core_path_in_several_host_threads():
             ys.append(y)
             jobs.append(lambda st, a=(moe, x, Wr, y): a[0].forward_device(a[1], a[2], None, a[3], stream=st))
         torch.cuda.synchronize()
-        _side_by_side(jobs, 10000)
+        side_by_side(jobs, 10000)
         for y, w in zip(ys, want):
             assert torch.equal(y, w)
     finally:

@@ -57,7 +57,7 @@ def test_the_storing_warps_of_the_grouped_gemm_leave_together():
     assert not re.search(r"mbar_wait|\bbreak;|\breturn\b|\bcontinue;", kernel[vote + len("if (!set_agrees(part, ok)) break;"):unit_end])
 
 
-@pytest.mark.parametrize("name", ["common.cuh", "ffn_gemv.cu", "ffn_i8.cu", "ffn_tma.cu", "ffn_umma.cu"])
+@pytest.mark.parametrize("name", ["common.cuh", "ffn_gemv.cu", "ffn_i8.cu", "ffn_tma.cu", "ffn_umma.cu", "route.cu"])
 def test_limits_of_dynamic_shared_memory_are_set_once(name):
     """The limit belongs to a kernel on a device and is shared by the contexts of all host threads: a launch that sets its own
     size may lower it between another thread's setting and its launch, which is then refused."""
