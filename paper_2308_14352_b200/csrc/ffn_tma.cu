@@ -9,8 +9,8 @@
 // instruction per pair of codes, at half the issue rate), so both are kept lean:
 //   * the kernel is persistent and runs BOTH projections of a layer.  The items are the first projection's (activated
 //     expert, block of output rows), then the second's (.., split-K slice), most expensive bitwidth first.  A CTA takes every
-//     n-th of the first and whichever is next of the second (fixed shares let the slowest CTA end a tenth of the launch
-//     behind the others; Mixtral-like layer, 4 tokens 133 -> 125 us).  The stream runs ahead across items, so
+//     n-th of the first and, where the second has more than three items per CTA, whichever is next of those (fixed shares let the
+//     slowest CTA end a tenth of the launch behind the others; Mixtral-like layer, 4 tokens 133 -> 125 us).  The stream runs ahead across items, so
 //     it never drains between tiles; an item of the second projection waits until the expert's
 //     hidden vectors are complete (release / acquire on a counter in the expert's plan record);
 //   * a stage holds two 64-row x 128-byte boxes of packed codes (two TMA tensor copies, 128-byte
@@ -621,10 +621,15 @@ __global__ void __launch_bounds__(st_threads(W), ST_CTAS) ffn_tma_kernel(const _
     // computing warps: whatever it does per stage is kept to a few instructions.
     // Every CTA takes every n-th item of the first projection and, going on so, one of the second; these are known without
     // asking and decoded 32 at a time.  From then on whoever is free claims the next one (one claim ahead, so that nobody
-    // waits for the answer).
+    // waits for the answer).  Up to three items of the second projection per CTA the fixed shares go on to the end: a claimed
+    // item is decoded alone, in front of its first copy, and the shares are as even as claims could make them (us per layer, fixed /
+    // claimed, at 1.7 to 2 items per CTA: 1024 x 4096, 8 experts, 64 tokens 36.4/39.4; 768 x 3072, 16 experts, 96 tokens 37.1/39.7;
+    // 512 x 2048, 32 experts, 192 tokens 35.0/36.9; at 3.5 to 4: 2048 x 8192, 4 experts, 16 tokens 48.1/46.9, 768 x 3072, 32 experts, 192
+    // tokens 53.0/49.9, Mixtral-like layer, 8 tokens 188/179).
     const int n = static_cast<int>(gridDim.x), me = static_cast<int>(blockIdx.x);
     const int n_items0 = a.phase_begin == 0 ? s_active * a.row_blocks[0] : 0, n_items1 = a.phase_end == 2 ? s_active * a.row_blocks[1] * a.ksplit : 0;
-    const int n_fixed = n_items0 + min(n, n_items1);
+    const bool claims = n_items1 > 3 * n;
+    const int n_fixed = n_items0 + (claims ? n : n_items1);
     int it = 0, oldest = 0, head = 0, phys = 0;
     int more = 1, claim = n_items1;
     for (int k0 = 0; more; k0 += 32) {
@@ -635,7 +640,7 @@ __global__ void __launch_bounds__(st_threads(W), ST_CTAS) ffn_tma_kernel(const _
       __syncwarp();
       if (lane == 0) {
         for (int k = k0; k < k0 + 32 && more; ++k) {
-          if (n_items1 > n && me + (k + 1) * n >= n_fixed) {  // this item is the last known one, or a claimed one
+          if (claims && me + (k + 1) * n >= n_fixed) {  // this item is the last known one, or a claimed one
             const int now = claim;
             claim = n + atomicAdd(a.plan + 1, 1);
             if (me + k * n >= n_fixed && now < n_items1) decode_item(a, s_plan, recs, 1, now, &queue[k % ST_QUEUE]);

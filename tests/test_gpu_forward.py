@@ -569,6 +569,14 @@ def test_fp16_operand_kernels_report_values_outside_their_range(path):
             moe.forward(x_ok, inputs.router_weight(28, 0, shape.d_model, shape.n_experts, std=0.05))
 
 
+@pytest.mark.parametrize("f,T", [(6656, 1), (7168, 1), (7168, 9)])
+def test_forward_streaming_kernel_about_three_items_per_cta(f, T):
+    """All picks of four experts: 4 x 16 row blocks x a slice per 512 inputs, 832 items of the second projection in fixed shares (at most
+    three per CTA, two CTAs on each of 148 SMs) and 896 that are claimed."""
+    assert (4 * 16 * (f // 512) > 3 * 2 * 148) == (f == 7168)
+    _run_case(inputs.LayerShape(2048, f, 4, 4, "relu", "softmax_renorm", 128, "f16", "bf16"), [8, 4, 2, 4], T, seed=29, path=3)
+
+
 UMMA_CASES = [
     ("relu", 128, "f16", 512, 1024, 4, 1, "softmax", [8, 4, 2, 4], 200),              # ~50 tokens per expert
     ("relu", 128, "f16", 512, 1024, 2, 1, "softmax", [4, 2], 300),                    # two token tiles per expert
