@@ -554,9 +554,9 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
   } else {
     ksplit = ffn_gemv_ksplit(L) < w.ksplit ? ffn_gemv_ksplit(L) : w.ksplit;
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
-    EMOE_LAUNCH(ctx, launch_ffn_gemv(0, L, table, x, perm, off, hidden, o_part, ksplit, P, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_gemv(0, L, table, x, perm, off, hidden, o_part, ksplit, P, st));
     if (ev[1]) EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
-    EMOE_LAUNCH(ctx, launch_ffn_gemv(1, L, table, x, perm, off, hidden, o_part, ksplit, P, ctx->check_word, st));
+    EMOE_LAUNCH(ctx, launch_ffn_gemv(1, L, table, x, perm, off, hidden, o_part, ksplit, P, st));
   }
   if (ev[2]) EMOE_CUDA(ctx, cudaEventRecord(ev[2], st));
   EMOE_LAUNCH(ctx, launch_combine(o_part, ksplit, static_cast<size_t>(P), gates_use, slot_of_pair, T, L.top_k, L.d_model, y, ids_use, counts,

@@ -120,7 +120,7 @@ cudaError_t launch_permute(const int32_t* ids, int n_pairs, int E, int32_t* coun
 // The second projection leaves ksplit partial sums, o: [ksplit][n_pairs][d_model].
 int ffn_gemv_ksplit(const LayerDims& L);
 cudaError_t launch_ffn_gemv(int phase, const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* perm, const int32_t* off,
-                            void* hidden, float* o, int ksplit, int n_pairs, int* check_word, cudaStream_t st);
+                            void* hidden, float* o, int ksplit, int n_pairs, cudaStream_t st);
 
 // Tensor-core (mma.sync bf16) grouped kernel for bf16 activations.
 // xs: x rows scattered into expert order with the per-bitwidth k-interleave, [n_pairs][d_model] bf16.

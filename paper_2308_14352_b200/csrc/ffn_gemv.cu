@@ -8,21 +8,21 @@
 // on the SMs at once.
 //   * a CTA takes some blocks of 32 rows of one expert and a slice of at most 1024 inputs (second projection: one
 //     slice per CTA, summed by the combine step; first projection: all slices in turn).  Their codes come into shared
-//     memory by bulk copies, all of them asked for at once; the number of blocks is such that every CTA is resident
-//     at once;
+//     memory by asynchronous 16-byte copies of all threads, all of them asked for at once (a bulk copy takes longer to its first
+//     byte); the number of blocks is such that every CTA is resident at once;
 //   * up to four tokens at a time have their activations in shared memory as fp32 (from global memory each
-//     step of the loop below waited for the L1 or L2);
+//     step of the loop below waited for the L1 or L2); the loads of a pass are in flight together;
 //   * a warp is cut into groups of lanes; a group owns four rows of a block and its lanes take 128-bit words of them (16 / 32 / 64
 //     weights each), so that an activation read serves four rows (two: the reads of shared memory bound passes of four tokens);
 //   * the fields of a 32-bit word are masked into bytes together, a byte becomes a float by one byte
 //     permute into the mantissa of 2^23 and one (exact) subtraction for two of them, shared by the tokens; products and sums go
 //     by twos as well.
-// Measured (forward call per layer; two rows per group, codes through registers, a variant of the loop per width and number
-// of tokens -> now): 768 x 3072, 8 experts, 16 fp32 tokens 41.8 -> 33.3 us; 640 x 2560, 16 experts, 64 tokens 78 -> 59; 1024 x 4096,
-// 4 experts, two picks, 64 tokens 211 -> 142; 512 x 1536, 16 experts, 9 tokens 21.3 -> 21.5 (five launches).
+// Measured (us per layer of a forward call; two rows per group, codes through registers, a variant of the loop per width and number
+// of tokens -> bulk copies, tokens staged one after the other, one token as two -> now): 768 x 3072, 8 experts, fp32, 16 tokens 41.8 ->
+// 34.5 -> 30.5; 1024 x 4096, 4 experts, two picks, 64 tokens 211 -> 148 -> 136; 4096 x 14336 gated, 8 experts, two picks, one token
+// 204 -> 228 -> 194, 4 tokens 405 -> 436 -> 368, 64 tokens 3690 -> 3240 -> 2630; 64 x 128, 4 experts, two picks, 64 tokens (bf16) 23.8 -> 26.9 -> 23.6.
 #include "common.cuh"
 #include "ffn_tile.cuh"
-#include "pipe.cuh"
 
 namespace emoe {
 namespace {
@@ -95,7 +95,6 @@ struct GemvArgs {
   int blocks;    // blocks of rows per CTA (one where there are several slices in turn)
   int G, ngroups;  // inputs per scale, scales of a row
   int groups;    // scales of a row that a slice touches, at most
-  int* check_word;
 };
 
 // shared memory: [matrices][rows][slice] codes, [matrices][rows][groups] scales, [GEMV_TOK][slice] activations
@@ -178,62 +177,79 @@ __device__ __forceinline__ void rows_dot(const Rows& m, const Width& wd, const S
   }
 }
 
-// The activations of `tokens` tokens (the last of ntok repeated) in the slice of `len` inputs from k0 on, in the order rows_dot
-// takes them.
-__device__ __forceinline__ void stage_inputs(const GemvArgs& a, const Width& wd, int slot0, int ntok, int tokens, int k0, int len, float* xs) {
+// The activations of MT tokens (the last of ntok repeated) in the slice of `len` inputs from k0 on, in the order rows_dot takes
+// them.  The loads of all tokens are in flight together.
+template <int MT>
+__device__ __forceinline__ void stage_inputs(const GemvArgs& a, const Width& wd, int slot0, int ntok, int k0, int len, float* xs) {
   const LayerDims& L = a.L;
   const int K = a.phase == 0 ? L.d_model : L.d_ff, nv = len * wd.bits / 128;
   const int sh = wd.bits == 8 ? 0 : (wd.bits == 4 ? 1 : 2);  // log2 of the fields
-  for (int t = 0; t < tokens; ++t) {
+  const void* src = a.phase == 0 ? a.x : a.hidden;
+  size_t at[MT];
+#pragma unroll
+  for (int t = 0; t < MT; ++t) {
     const int slot = slot0 + min(t, ntok - 1);
-    const size_t row = a.phase == 0 ? static_cast<size_t>(L.top_k == 1 ? a.perm[slot] : a.perm[slot] / L.top_k) : static_cast<size_t>(slot);
-    const void* src = a.phase == 0 ? a.x : a.hidden;
-    float* to = xs + t * a.slice;
-    for (int k = 4 * threadIdx.x; k < len; k += 4 * GEMV_THREADS) {
-      const size_t at = row * K + k0 + k;
-      float4 v;
-      if (L.act_bf16) {
-        const uint2 b = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(src) + at);
-        v = make_float4(__uint_as_float(b.x << 16), __uint_as_float(b.x & 0xffff0000u), __uint_as_float(b.y << 16), __uint_as_float(b.y & 0xffff0000u));
-      } else {
-        v = *reinterpret_cast<const float4*>(static_cast<const float*>(src) + at);
-      }
-      // input k of the slice: 128-bit word k / (16 << sh), and in it 32-bit word, byte and field
-      const int word = k >> (4 + sh), i = (k >> (2 + sh)) & 3, o = k & ((4 << sh) - 1);
+    at[t] = static_cast<size_t>(a.phase == 0 ? a.perm[slot] : slot);
+  }
+#pragma unroll
+  for (int t = 0; t < MT; ++t) at[t] = (a.phase == 0 && L.top_k != 1 ? static_cast<int>(at[t]) / L.top_k : at[t]) * K + k0;
+  for (int k = 4 * threadIdx.x; k < len; k += 4 * GEMV_THREADS) {
+    float4 v[MT];
+    if (L.act_bf16) {
+      uint2 b[MT];
+#pragma unroll
+      for (int t = 0; t < MT; ++t) b[t] = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(src) + at[t] + k);
+#pragma unroll
+      for (int t = 0; t < MT; ++t)
+        v[t] = make_float4(__uint_as_float(b[t].x << 16), __uint_as_float(b[t].x & 0xffff0000u), __uint_as_float(b[t].y << 16), __uint_as_float(b[t].y & 0xffff0000u));
+    } else {
+#pragma unroll
+      for (int t = 0; t < MT; ++t) v[t] = *reinterpret_cast<const float4*>(static_cast<const float*>(src) + at[t] + k);
+    }
+    // input k of the slice: 128-bit word k / (16 << sh), and in it 32-bit word, byte and field
+    const int word = k >> (4 + sh), i = (k >> (2 + sh)) & 3, o = k & ((4 << sh) - 1);
+#pragma unroll
+    for (int t = 0; t < MT; ++t) {
+      float* to = xs + t * a.slice;
       if (sh == 0) {
-        *reinterpret_cast<float4*>(to + (i * nv + word) * 4) = v;
+        *reinterpret_cast<float4*>(to + (i * nv + word) * 4) = v[t];
       } else if (sh == 1) {  // two fields, two bytes
         float* p = to + (i * 2 * nv + word) * 4 + (o >> 1);
-        *reinterpret_cast<float2*>(p) = make_float2(v.x, v.z);
-        *reinterpret_cast<float2*>(p + nv * 4) = make_float2(v.y, v.w);
+        *reinterpret_cast<float2*>(p) = make_float2(v[t].x, v[t].z);
+        *reinterpret_cast<float2*>(p + nv * 4) = make_float2(v[t].y, v[t].w);
       } else {  // four fields, one byte
         float* p = to + (i * 4 * nv + word) * 4 + (o >> 2);
-        p[0] = v.x;
-        p[nv * 4] = v.y;
-        p[nv * 8] = v.z;
-        p[nv * 12] = v.w;
+        p[0] = v[t].x;
+        p[nv * 4] = v[t].y;
+        p[nv * 8] = v[t].z;
+        p[nv * 12] = v[t].w;
       }
     }
   }
 }
 
-// asks for the codes of a slice of the CTA's rows (one arrival at `bar`, with the bytes)
+__device__ __forceinline__ void cp_async16(void* to, const void* from) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(to))), "l"(from) : "memory");
+}
+
+// asks for the codes of a slice of the CTA's rows
 template <bool GATED>
-__device__ __forceinline__ void fetch_codes(const GemvArgs& a, const ExpertDev& ex, const Slice& sc, int n0, int rows, const Staged& sm, uint32_t bar) {
+__device__ __forceinline__ void fetch_codes(const GemvArgs& a, const ExpertDev& ex, const Slice& sc, int n0, int rows, const Staged& sm) {
   const int K = a.phase == 0 ? a.L.d_model : a.L.d_ff, mat = a.phase == 0 ? 0 : (a.L.act == EMOE_ACT_RELU ? 1 : 2);
   const size_t row_bytes = static_cast<size_t>(K) * ex.bits / 8;
-  if (threadIdx.x >= 32) return;
 #pragma unroll
   for (int i = 0; i < (GATED ? 2 : 1); ++i) {
     const int m = GATED ? i : mat;
     const uint8_t* from = (m == 0 ? ex.packed[0] : (m == 1 ? ex.packed[1] : ex.packed[2])) + n0 * row_bytes + static_cast<size_t>(sc.k0) * ex.bits / 8;
-    const uint32_t to = smem_u32(sm.codes + i * a.blocks * GEMV_ROWS * a.slice);
-    if (threadIdx.x == 0 && i == 0) mbar_expect_tx(bar, (GATED ? 2 : 1) * rows * sc.bytes);
+    unsigned char* to = sm.codes + i * a.blocks * GEMV_ROWS * a.slice;
     if (sc.len == K) {  // whole rows follow each other
-      if (threadIdx.x == 0) bulk_load(to, from, rows * sc.bytes, bar);
+      for (int u = 16 * threadIdx.x; u < rows * sc.bytes; u += 16 * GEMV_THREADS) cp_async16(to + u, from + u);
     } else {
-      __syncwarp();  // (behind the announcement of the bytes)
-      for (int r = threadIdx.x; r < rows; r += 32) bulk_load(to + r * sc.bytes, from + r * row_bytes, sc.bytes, bar);
+      const int words = sc.bytes >> 4;
+      for (int u = threadIdx.x; u < rows * words; u += GEMV_THREADS) {
+        const int r = u / words, c = 16 * (u - r * words);
+        cp_async16(to + r * sc.bytes + c, from + r * row_bytes + c);
+      }
     }
   }
 }
@@ -325,8 +341,8 @@ struct Work {
 };
 
 template <bool GATED, int MT>
-__device__ __forceinline__ bool token_pass(const GemvArgs& a, const ExpertDev& ex, const Width& wd, const Work& w, int c0, int ntok, const Staged& sm, uint32_t bar,
-                                           Slice& sc, uint32_t& parity, bool& first, volatile int* abort_flag) {
+__device__ __forceinline__ void token_pass(const GemvArgs& a, const ExpertDev& ex, const Width& wd, const Work& w, int c0, int ntok, const Staged& sm, Slice& sc,
+                                           bool& first) {
   const int slot0 = w.begin + c0;
   const bool one = w.sl1 - w.sl0 == 1;
   float v[GEMV_R][MT], u[GEMV_R][MT];
@@ -340,57 +356,41 @@ __device__ __forceinline__ bool token_pass(const GemvArgs& a, const ExpertDev& e
         __syncthreads();  // what is staged has been used
         if (!one && !first) {
           sc = slice_of(a, sl, wd.bits);
-          fetch_codes<GATED>(a, ex, sc, w.n0, w.rows, sm, bar);
+          fetch_codes<GATED>(a, ex, sc, w.n0, w.rows, sm);
         }
-        const auto staging = [&] { stage_inputs(a, wd, slot0, ntok, MT, sc.k0, sc.len, sm.xs); };
+        const auto staging = [&] { stage_inputs<MT>(a, wd, slot0, ntok, sc.k0, sc.len, sm.xs); };
         if (first || !one) fetch_scales<GATED>(a, ex, sc, w.n0, w.rows, sm, staging);
         else staging();
-        if (first || !one) {
-          const bool ok = mbar_wait(bar, parity, a.check_word, abort_flag);
-          parity ^= 1;
-          if (!__syncthreads_and(ok)) return false;
-        } else {
-          __syncthreads();
-        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
         first = false;
       }
       block_dot<GATED, MT>(a, wd, b, sc, sm, v, u);
     }
     store_block<GATED, MT>(a, w.z, w.n0 + b * GEMV_ROWS, slot0, ntok, v, u);
   }
-  return true;
 }
 
 template <bool GATED>
-__device__ __forceinline__ void expert_rows(const GemvArgs& a, const ExpertDev& ex, const Work& w, Slice sc, const Staged& sm, uint32_t bar, volatile int* abort_flag) {
+__device__ __forceinline__ void expert_rows(const GemvArgs& a, const ExpertDev& ex, const Work& w, Slice sc, const Staged& sm) {
   const Width wd = width_of(ex.bits);
-  uint32_t parity = 0;
-  bool first = true, ok = true;
-  for (int c0 = blockIdx.z * GEMV_TOK; c0 < w.cnt && ok; c0 += gridDim.z * GEMV_TOK) {
+  bool first = true;
+  for (int c0 = blockIdx.z * GEMV_TOK; c0 < w.cnt; c0 += gridDim.z * GEMV_TOK) {
     const int ntok = min(GEMV_TOK, w.cnt - c0);
-    if (ntok > 2) ok = token_pass<GATED, 4>(a, ex, wd, w, c0, ntok, sm, bar, sc, parity, first, abort_flag);
-    else ok = token_pass<GATED, 2>(a, ex, wd, w, c0, ntok, sm, bar, sc, parity, first, abort_flag);
+    if (ntok > 2) token_pass<GATED, 4>(a, ex, wd, w, c0, ntok, sm, sc, first);
+    else if (ntok == 2) token_pass<GATED, 2>(a, ex, wd, w, c0, ntok, sm, sc, first);
+    else token_pass<GATED, 1>(a, ex, wd, w, c0, ntok, sm, sc, first);
   }
-  if (!ok)
-    for (int i = 0; i < 2000; ++i) __nanosleep(100);  // let copies in flight land
 }
 
 template <bool GATED>  // first projection of a gated layer: two matrices
 __global__ void __launch_bounds__(GEMV_THREADS, GEMV_CTAS) ffn_gemv_kernel(const __grid_constant__ GemvArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ __align__(8) uint64_t bar_word;
-  __shared__ int abort_word;
   const int rows_max = (GATED ? 2 : 1) * a.blocks * GEMV_ROWS;
   Staged sm;
   sm.codes = smem;
   sm.xs = reinterpret_cast<float*>(smem + rows_max * a.slice);
   sm.scales = sm.xs + GEMV_TOK * a.slice;
-  const uint32_t bar = smem_u32(&bar_word);
-  if (threadIdx.x == 0) {
-    abort_word = 0;
-    mbar_init(bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
   const int N = a.phase == 0 ? a.L.d_ff : a.L.d_model;
   const int e = a.phase == 0 ? blockIdx.y : blockIdx.y / a.ksplit;
   Work w;
@@ -413,14 +413,13 @@ __global__ void __launch_bounds__(GEMV_THREADS, GEMV_CTAS) ffn_gemv_kernel(const
   w.cnt = __ldcg(a.off + e + 1) - w.begin;
   const bool idle = w.cnt <= static_cast<int>(blockIdx.z) * GEMV_TOK;
   const Slice sc = slice_of(a, w.sl0, ex.bits);
-  if (!idle && w.sl0 < w.sl1) fetch_codes<GATED>(a, ex, sc, w.n0, w.rows, sm, bar);  // (the last planes may be without a slice)
+  if (!idle && w.sl0 < w.sl1) fetch_codes<GATED>(a, ex, sc, w.n0, w.rows, sm);  // (the last planes may be without a slice)
   if (a.phase == 1) {
     pdl_wait();
     pdl_trigger();
   }
   if (idle) return;
-  __syncthreads();
-  expert_rows<GATED>(a, ex, w, sc, sm, bar, &abort_word);
+  expert_rows<GATED>(a, ex, w, sc, sm);
 }
 
 // slices of a projection over K inputs: as long as shared memory holds, of equal length, whole 128-bit words at every width
@@ -435,11 +434,11 @@ int ffn_gemv_ksplit(const LayerDims& L) {
 }
 
 cudaError_t launch_ffn_gemv(int phase, const LayerDims& L, const ExpertDev* experts, const void* x, const int32_t* perm, const int32_t* off,
-                            void* hidden, float* o, int ksplit, int n_pairs, int* check_word, cudaStream_t st) {
+                            void* hidden, float* o, int ksplit, int n_pairs, cudaStream_t st) {
   const int N = phase == 0 ? L.d_ff : L.d_model, K = phase == 0 ? L.d_model : L.d_ff;
   const bool gated = phase == 0 && L.act == EMOE_ACT_SWIGLU;
   const int G = L.group > 0 ? L.group : K;
-  GemvArgs a{phase, L, experts, x, perm, off, hidden, o, 0, 0, ksplit, n_pairs, 1, G, K / G, 0, check_word};
+  GemvArgs a{phase, L, experts, x, perm, off, hidden, o, 0, 0, ksplit, n_pairs, 1, G, K / G, 0};
   const int want = gemv_slices(K);
   a.slice = ((K + want - 1) / want + 63) / 64 * 64;
   a.nslices = (K + a.slice - 1) / a.slice;

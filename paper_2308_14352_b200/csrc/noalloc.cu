@@ -170,8 +170,8 @@ extern "C" int emoe_moe_forward_routed_static(int device, const emoe_layer_desc*
                             reinterpret_cast<__nv_bfloat16*>(hidden), o_part, w.ksplit, P, T, st));
     EMOE_TRY(launch_combine(o_part, w.ksplit, static_cast<size_t>(P), gates, slot_of_pair, T, L.top_k, L.d_model, y, nullptr, nullptr, 0, nullptr, st));
   } else {
-    EMOE_TRY(launch_ffn_gemv(0, L, table, x, perm, off, hidden, o_part, w.ksplit, P, check, st));
-    EMOE_TRY(launch_ffn_gemv(1, L, table, x, perm, off, hidden, o_part, w.ksplit, P, check, st));
+    EMOE_TRY(launch_ffn_gemv(0, L, table, x, perm, off, hidden, o_part, w.ksplit, P, st));
+    EMOE_TRY(launch_ffn_gemv(1, L, table, x, perm, off, hidden, o_part, w.ksplit, P, st));
     EMOE_TRY(launch_combine(o_part, w.ksplit, static_cast<size_t>(P), gates, slot_of_pair, T, L.top_k, L.d_model, y, nullptr, nullptr, 0, nullptr, st));
   }
 #undef EMOE_TRY
