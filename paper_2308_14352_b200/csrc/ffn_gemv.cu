@@ -20,7 +20,7 @@
 // Measured (us per layer of a forward call; two rows per group, codes through registers, a variant of the loop per width and number
 // of tokens -> bulk copies, tokens staged one after the other, one token as two -> now): 768 x 3072, 8 experts, fp32, 16 tokens 41.8 ->
 // 34.5 -> 30.5; 1024 x 4096, 4 experts, two picks, 64 tokens 211 -> 148 -> 136; 4096 x 14336 gated, 8 experts, two picks, one token
-// 204 -> 228 -> 194, 4 tokens 405 -> 436 -> 368, 64 tokens 3690 -> 3240 -> 2630; 64 x 128, 4 experts, two picks, 64 tokens (bf16) 23.8 -> 26.9 -> 23.6.
+// 204 -> 228 -> 194, 4 tokens 405 -> 436 -> 368, 64 tokens 3690 -> 3240 -> 2630; 64 x 128, 4 experts, two picks, 64 tokens (bf16) 23.8 -> 26.9 -> 22.2.
 #include "common.cuh"
 #include "ffn_tile.cuh"
 
