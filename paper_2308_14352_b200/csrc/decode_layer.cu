@@ -29,7 +29,7 @@ namespace {
 constexpr int DL_THREADS = ROUTER_THREADS;
 constexpr int DL_WARPS = DL_THREADS / 32;
 constexpr int DL_MAX_PAIRS = 16;
-constexpr int DL_TABLE = 64;                 // records of experts a CTA has at hand
+constexpr int DL_MAXJ = EMOE_MAX_EXPERTS / 32;
 constexpr int DL_WPR_MAX = 4;                // most warps that share a row block of the second projection (a.wpr: 1, 2 or 4)
 constexpr int DL_R_MAX = 4;                  // consecutive rows of a matrix one warp takes at once
 constexpr long long DL_MAX_WEIGHTS = 8LL << 20;  // per matrix: beyond this a layer is bandwidth-bound and streams better
@@ -168,14 +168,19 @@ __device__ __forceinline__ bool grid_arrive_wait(unsigned* counter, unsigned tar
   return *s_flag != 0;
 }
 
-template <int DL_R>
+// MAXJ: logits per lane of a warp that makes the picks.  One (up to 32 experts): the records of the experts come into shared memory
+// while the routing runs.  Both forms in one kernel, chosen by the number of experts at run time, made calls of 2 to 8 tokens on
+// small layers slower than neither (us per layer, without / both at run time / as variants: 256 x 512, 16 experts, 8 tokens 15.0/16.0/15.0;
+// 256 x 896, 8 experts, 4 tokens 14.7/15.8/14.7; 768 x 3072, 32 experts, one token 14.3/14.2/14.1, 4 tokens 20.0/19.7/19.5).
+template <int DL_R, int MAXJ>
 __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const DecodeLayerArgs a) {
   __shared__ int s_ids[DL_MAX_PAIRS];
   __shared__ float s_gates[DL_MAX_PAIRS];
   __shared__ float s_part[DL_WARPS][DL_R_MAX];  // [row block of the CTA][warp of the block][row]
   __shared__ float s_red[DL_THREADS];            // router product: [parts][EP]
   __shared__ float s_z[DL_WARPS][EMOE_MAX_EXPERTS];  // logits of the token a warp picks for
-  __shared__ __align__(16) ExpertDev s_table[DL_TABLE];
+  constexpr bool TABLE = MAXJ == 1;
+  __shared__ __align__(16) ExpertDev s_table[TABLE ? 32 : 1];
   __shared__ int s_flag;
   const LayerDims& L = a.L;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -189,13 +194,19 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
   // the records of the experts come into shared memory while the routing runs, behind the wait for the kernels in front like
   // every other read
   const auto fetch_table = [&]() {
-    for (int i = tid; i < min(L.E, DL_TABLE) * static_cast<int>(sizeof(ExpertDev) / 8); i += DL_THREADS)
+    if constexpr (!TABLE) return;
+    for (int i = tid; i < min(L.E, 32) * static_cast<int>(sizeof(ExpertDev) / 8); i += DL_THREADS)
       asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(reinterpret_cast<uint2*>(s_table) + i))),
                    "l"(reinterpret_cast<const uint2*>(a.experts) + i)
                    : "memory");
   };
-  const auto table_here = []() { asm volatile("cp.async.wait_all;" ::: "memory"); };
-  const auto expert = [&](int e) -> const ExpertDev& { return e < DL_TABLE ? s_table[e] : a.experts[e]; };
+  const auto table_here = []() {
+    if constexpr (TABLE) asm volatile("cp.async.wait_all;" ::: "memory");
+  };
+  const auto expert = [&](int e) -> const ExpertDev& {
+    if constexpr (TABLE) return s_table[e];
+    else return a.experts[e];
+  };
 
   // ---- 1. routing ----
   if (a.Wr) {
@@ -261,7 +272,7 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
       __syncwarp();
       int my_id;
       float my_gate;
-      router_pick(zrow, L.E, L.top_k, a.renorm, lane, my_id, my_gate);
+      router_pick_of<MAXJ>(zrow, L.E, L.top_k, a.renorm, lane, my_id, my_gate);
       if (lane < L.top_k) {
         s_ids[t * L.top_k + lane] = my_id;
         s_gates[t * L.top_k + lane] = my_gate;
@@ -479,9 +490,11 @@ bool decode_layer_supported(const LayerDims& L, int T) {
 }
 
 int decode_layer_resident_ctas(int device) {
-  int per_sm = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_layer_kernel<DL_R_MAX>, DL_THREADS, 0) != cudaSuccess)
+  int per_sm = 0, sms = 0, other = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_layer_kernel<DL_R_MAX, 1>, DL_THREADS, 0) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&other, decode_layer_kernel<DL_R_MAX, DL_MAXJ>, DL_THREADS, 0) != cudaSuccess)
     return 0;
+  per_sm = per_sm < other ? per_sm : other;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
   return per_sm * sms;
 }
@@ -542,7 +555,8 @@ cudaError_t launch_decode_layer(const LayerDims& L, const ExpertDev* experts, co
   while (a.wpr > 1 && static_cast<long long>(T) * (L.d_model / DL_R_MAX) > static_cast<long long>(grid) * (DL_WARPS / a.wpr)) a.wpr >>= 1;
   while (a.rsplit > 1 && T * a.rsplit > grid) a.rsplit >>= 1;  // a small device: fewer slices than CTAs
   if (per_sm < 1 || grid < T) return cudaErrorInvalidConfiguration;
-  return launch_chain(decode_layer_kernel<DL_R_MAX>, dim3(grid), dim3(DL_THREADS), 0, st, a);
+  if (L.E <= 32) return launch_chain(decode_layer_kernel<DL_R_MAX, 1>, dim3(grid), dim3(DL_THREADS), 0, st, a);
+  return launch_chain(decode_layer_kernel<DL_R_MAX, DL_MAXJ>, dim3(grid), dim3(DL_THREADS), 0, st, a);
 }
 
 }  // namespace emoe

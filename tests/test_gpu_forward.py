@@ -351,6 +351,9 @@ LAYER_CASES = [
     ("relu", "f32", 0, "f32", 128, 256, 4, 1, "softmax", [5, 1]),
     ("swiglu", "f32", 64, "f16", 192, 320, 3, 2, "softmax_renorm", [7, 2]),
     ("relu", "bf16", 64, "f16", 512, 512, 128, 1, "softmax", [3, 16]),
+    # the last number of experts whose records are at hand, and the next
+    ("relu", "f32", 64, "f16", 128, 128, 32, 2, "softmax_renorm", [8, 1]),
+    ("relu", "f32", 64, "f16", 128, 128, 33, 2, "softmax_renorm", [8, 1]),
 ]
 
 
