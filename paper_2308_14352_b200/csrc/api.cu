@@ -155,6 +155,7 @@ namespace {
 
 int cuda_fail(emoe_ctx* ctx, cudaError_t e) {
   if (ctx) ctx->last_cuda = static_cast<int>(e);
+  cudaGetLastError();  // told to the caller: no later call that asks for launch errors reports it once more
   return EMOE_ERR_CUDA;
 }
 

@@ -167,6 +167,15 @@ class CachePolicy {
     --slots_[static_cast<size_t>(s)].pins;
     return s;
   }
+  // the expert was placed but its copy could not be enqueued: the slot holds nothing
+  void forget(int ei) {
+    CacheExpert& e = experts_[static_cast<size_t>(ei)];
+    if (e.slot < 0) return;
+    slots_[static_cast<size_t>(e.slot)].expert = -1;
+    e.slot = -1;
+    e.by_prefetch = false;
+    for (int m = 0; m < 6; ++m) stats_.bytes_copied -= static_cast<int64_t>(e.bytes[m]);
+  }
 
  private:
   int n_layers_, policy_;
@@ -317,12 +326,14 @@ bool ctx_dependent_launch(const emoe_ctx* ctx);
 int ctx_cuda_fail(emoe_ctx* ctx, cudaError_t e);
 
 namespace {
+// Whatever could not be enqueued has no slot any more: nobody takes it for loaded.
 int enqueue_preloads(emoe_ctx* ctx, Preloads* later, void* copy_stream) {
   ExpertCache* c = ctx_cache(ctx);
   cudaError_t err = cudaSetDevice(c->device);
-  for (int i = 0; i < later->n && err == cudaSuccess; ++i) {
+  for (int i = 0; i < later->n; ++i) {
     const CacheExpert& e = c->policy.expert(later->experts[i]);
-    err = load_into_slot(c, e, e.slot, static_cast<cudaStream_t>(copy_stream));
+    if (err == cudaSuccess) err = load_into_slot(c, e, e.slot, static_cast<cudaStream_t>(copy_stream));
+    if (err != cudaSuccess) c->policy.forget(later->experts[i]);
   }
   later->n = 0;
   return err == cudaSuccess ? EMOE_OK : ctx_cuda_fail(ctx, err);
@@ -389,7 +400,10 @@ int emoe_prefetch_experts(emoe_ctx* ctx, const int64_t* ids, int n, int current_
     const int s = c->policy.prefetch(ei, current_layer, &evicted);
     if (s < 0) continue;  // resident already, or every slot is in use: a prefetch never waits
     err = load_into_slot(c, c->policy.expert(ei), s, static_cast<cudaStream_t>(copy_stream));
-    if (err != cudaSuccess) return ctx_cuda_fail(ctx, err);
+    if (err != cudaSuccess) {
+      c->policy.forget(ei);
+      return ctx_cuda_fail(ctx, err);
+    }
   }
   return EMOE_OK;
 }
@@ -413,7 +427,7 @@ int acquire(emoe_ctx* ctx, const int64_t* ids, int n, int current_layer, void* c
   if (err != cudaSuccess) return ctx_cuda_fail(ctx, err);
   for (int i = 0; i < n; ++i)  // nothing is touched unless every id is known
     if (c->policy.find(ids[i]) < 0) return EMOE_ERR_INVALID_ARG;
-  int rc = EMOE_OK, done = 0;
+  int rc = EMOE_OK, done = 0, not_loaded = -1;
   cudaEvent_t t_after = nullptr;
   if (c->timing) {
     while (c->timed.size() < c->timed_used + 2) {
@@ -439,7 +453,10 @@ int acquire(emoe_ctx* ctx, const int64_t* ids, int n, int current_layer, void* c
     if (evicted >= 0) later->take(evicted);  // a preload that leaves before its copy was made
     if (load) {
       err = load_into_slot(c, c->policy.expert(ei), s, static_cast<cudaStream_t>(copy_stream));
-      if (err != cudaSuccess) rc = ctx_cuda_fail(ctx, err);
+      if (err != cudaSuccess) {
+        rc = ctx_cuda_fail(ctx, err);
+        not_loaded = ei;
+      }
     }
     // the compute stream goes on when the slot's contents are complete (no host wait)
     if (rc == EMOE_OK) {
@@ -456,6 +473,7 @@ int acquire(emoe_ctx* ctx, const int64_t* ids, int n, int current_layer, void* c
     // all or nothing: the experts acquired so far by this call are let go again, so that a failed
     // call leaves no slot protected (their activation counts keep the increment)
     for (int i = 0; i < done; ++i) c->policy.release(c->policy.find(ids[i]));
+    if (not_loaded >= 0) c->policy.forget(not_loaded);
   }
   return rc;
 }

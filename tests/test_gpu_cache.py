@@ -3,6 +3,8 @@ copy stream, used by the routed forward on a compute stream.  Checks (i) data: t
 cached experts matches the CPU checker within the output bar, and bit-for-bit the forward on the
 same experts resident in ordinary device memory; (ii) bookkeeping: slots, evictions and counters
 equal the plain model's, operation by operation (integer work: exact)."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -469,6 +471,66 @@ def test_cached_layer_preloads_that_are_needed_at_once_or_leave_again(n_slots, n
     finally:
         torch.cuda.synchronize()
         dense.close()
+        B.emoe_destroy(ctx)
+
+
+@pytest.mark.parametrize("call", ["prefetch", "acquire", "layer"])
+def test_an_expert_whose_copy_cannot_be_enqueued_holds_no_slot(call):
+    """The copy stream is being captured, and a slot's last reader lies outside the capture: the runtime refuses the copy.  Nobody
+    may then find the expert resident; the next use loads it."""
+    shape = inputs.LayerShape(512, 1024, 4, 2, "relu", "softmax_renorm", 128, "f16", "bf16")
+    host = HostExperts(shape, 2, lambda l: [8, 4, 2, 4], seed=53)
+    desc, dev = layer.make_desc(shape), torch.device("cuda", 0)
+    cudart = ctypes.CDLL("libcudart.so.12")
+    Wr = torch.from_numpy(inputs.router_weight(53, 0, 512, 4, std=0.05)).to(dev)
+    x = torch.from_numpy(inputs.activations(53, 0, 1, 512, "bf16")).to(dev).to(torch.bfloat16)
+    ids, gates, y = torch.empty(1, 2, dtype=torch.int32, device=dev), torch.empty(1, 2, device=dev), torch.empty(1, 512, device=dev)
+    pinned = torch.empty(1, 2, dtype=torch.int32, pin_memory=True)
+    prior = np.zeros((4, 4), dtype=np.float32)
+    prior[:, 2:] = 1.0  # the last two of the next layer
+    stream, compute = torch.cuda.Stream(device=dev), torch.cuda.Stream(device=dev)
+    copy, ctx = ctypes.c_void_p(stream.cuda_stream), _stack_on_cache(host, desc, 6, 1)
+    wanted = [host.expert_id(1, 2), host.expert_id(1, 3)]
+
+    def layer_call():
+        B.emoe_cached_layer(ctx, desc, 0, x.data_ptr(), 1, Wr.data_ptr(), None, 0, host.expert_id(0, 0), prior.ctypes.data, 2, host.expert_id(1, 0),
+                            ids.data_ptr(), gates.data_ptr(), y.data_ptr(), pinned.data_ptr(), compute.cuda_stream, stream.cuda_stream)
+
+    try:
+        # all of layer 0 and the other two of layer 1, each with a reader behind it
+        first = [host.expert_id(0, e) for e in range(4)] + [host.expert_id(1, e) for e in range(2)]
+        B.emoe_cache_acquire(ctx, first, 0, compute.cuda_stream, stream.cuda_stream)
+        B.emoe_cache_release(ctx, first, compute.cuda_stream)
+        torch.cuda.synchronize()
+        copied = B.emoe_cache_get_stats(ctx)["bytes_copied"]
+        assert cudart.cudaStreamBeginCapture(copy, 2) == 0  # (2: of this stream alone)
+        try:
+            with pytest.raises(B.EmoeError) as ei:
+                if call == "prefetch":
+                    B.emoe_prefetch_experts(ctx, wanted, 0, stream.cuda_stream)
+                elif call == "acquire":
+                    B.emoe_cache_acquire(ctx, wanted, 0, compute.cuda_stream, stream.cuda_stream)
+                else:
+                    layer_call()
+        finally:
+            graph = ctypes.c_void_p()
+            cudart.cudaStreamEndCapture(copy, ctypes.byref(graph))  # the refused copy has invalidated it
+            cudart.cudaGetLastError()                                # ... which this runtime remembers
+        assert ei.value.status == B.ERR_CUDA
+        assert [B.emoe_cache_slot_of(ctx, e) for e in wanted] == [-1, -1]
+        before = B.emoe_cache_get_stats(ctx)
+        if call != "layer":  # (there the second takes the slot of the first, which counts as copied)
+            assert before["bytes_copied"] == copied
+        B.emoe_cache_acquire(ctx, wanted, 1, compute.cuda_stream, stream.cuda_stream)
+        B.emoe_cache_release(ctx, wanted, compute.cuda_stream)
+        assert B.emoe_cache_get_stats(ctx)["misses"] == before["misses"] + 2
+        layer_call()
+        with layer.MoELayer(shape, host.bits[0]) as moe:  # launches that are asked for their errors
+            moe.pack_matrix(0, 0, torch.zeros(1024, 512, device=dev))
+        torch.cuda.synchronize()
+        assert B.emoe_device_status(ctx) == B.OK
+    finally:
+        torch.cuda.synchronize()
         B.emoe_destroy(ctx)
 
 
