@@ -568,8 +568,8 @@ __global__ void __launch_bounds__(st_threads(W), ST_CTAS) ffn_tma_kernel(const _
   __shared__ ItemRec queue[ST_QUEUE];
   __shared__ __align__(16) PlanRec s_plan[ST_PLAN_CACHE];
   __shared__ int s_active, s_vstart[ST_SLOTS], s_offset[ST_SLOTS];
-  __shared__ int abort_word;
-  volatile int* abort_flag = &abort_word;
+  __shared__ int wait_words[PIPE_WORDS];
+  volatile int* abort_flag = wait_words + PIPE_ABORT;
   // an offset from the array, not a rounded address: the compiler then knows that every access is to shared memory
   unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* hid_stage = ring + ST_RING;
@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(st_threads(W), ST_CTAS) ffn_tma_kernel(const _
   const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + ST_SLOTS), bar_issued = smem_u32(bars + 2 * ST_SLOTS), bar_hid = smem_u32(bars + 3 * ST_SLOTS);
 
   if (threadIdx.x == 0) {
-    abort_word = 0;
+    wait_words[PIPE_ABORT] = wait_words[PIPE_FRONT] = 0;
     for (int s = 0; s < ST_SLOTS; ++s) {
       mbar_init(bar_full + 8 * s, 34);          // weight warp and activation warp (+ the bytes of their copies), every lane's scale copies
       mbar_init(bar_issued + 8 * s, 1);

@@ -470,8 +470,8 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bars[2 * U::RAW_STAGES + 2 * U::STAGES + (1 + UM_SCALE_SETS) * UM_SETS];
   __shared__ uint32_t tmem_base_slot;
-  __shared__ int abort_word;
-  volatile int* abort_flag = &abort_word;
+  __shared__ int wait_words[PIPE_WORDS];
+  volatile int* abort_flag = wait_words + PIPE_ABORT;
   // an offset from the array, not a rounded address: the compiler then knows that every access is to shared memory
   unsigned char* raw_ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* b_ring = raw_ring + U::RAW_STAGES * UM_TILE_BYTES;
@@ -491,7 +491,8 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
   b.acc_empty = b.acc_full + 8 * UM_SCALE_SETS * UM_SETS;
 
   if (threadIdx.x == 0) {
-    abort_word = 0;
+    wait_words[PIPE_ABORT] = 0;
+    wait_words[PIPE_FRONT] = a.phase != 0;
     for (int s = 0; s < U::RAW_STAGES; ++s) {
       mbar_init(b.raw_full + 8 * s, 1);
       mbar_init(b.raw_empty + 8 * s, U::UNPACK_WARPS);
@@ -538,7 +539,10 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
 
   if (warp == 0) {
     // ---------------- producer of the activations ----------------
-    if (a.phase != 0) pdl_wait();
+    if (a.phase != 0) {
+      pdl_wait();
+      if (lane == 0) abort_flag[PIPE_FRONT] = 0;
+    }
     const uint32_t on = elect_one();
     int it = 0;
     bool ok = true;

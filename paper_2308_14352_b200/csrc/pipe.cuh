@@ -1,6 +1,7 @@
 // mbarrier / TMA / bulk-copy wrappers shared by the pipelined expert kernels.  Every wait is
 // bounded: a wait that runs out sets CHECK_WAIT_TIMEOUT in the context's check word, raises the
-// CTA's abort flag and returns false, and the caller winds down without touching the stage.
+// CTA's abort flag and returns false, and the caller winds down without touching the stage.  The word behind the flag
+// says whether the CTA still waits for the kernel in front (whose own waits are bounded): then waits go on but count no time.
 #pragma once
 #include "common.cuh"
 
@@ -40,13 +41,16 @@ __device__ __forceinline__ bool mbar_try_wait_parked(uint32_t bar, uint32_t pari
 }
 constexpr unsigned long long PIPE_WAIT_NS = 500000000ull;  // a wait gives up after half a second of its own
 constexpr uint32_t PIPE_PARK_NS = 20000;                   // how long a waiting thread may be parked at a time
+// The words of a CTA's waits, in shared memory: the first is the abort flag.
+enum : int { PIPE_ABORT = 0, PIPE_FRONT = 1, PIPE_WORDS = 2 };
 // The time a wait has had once the clock went from t0 to t1 over one poll: no more than twice what a poll may be parked
 // for, so that a CTA that was switched out meanwhile does not take its absence for a wait that is stuck.
-__host__ __device__ constexpr unsigned long long waited_ns(unsigned long long so_far, unsigned long long t0, unsigned long long t1) {
-  return so_far + (t1 - t0 < 2ull * PIPE_PARK_NS ? t1 - t0 : 2ull * PIPE_PARK_NS);
+__host__ __device__ constexpr unsigned long long waited_ns(unsigned long long so_far, unsigned long long t0, unsigned long long t1, bool front) {
+  return front ? 0 : so_far + (t1 - t0 < 2ull * PIPE_PARK_NS ? t1 - t0 : 2ull * PIPE_PARK_NS);
 }
-static_assert(waited_ns(0, 1000, 21000) == 20000 && waited_ns(70, 5, 5) == 70, "a poll counts what it took");
-static_assert(waited_ns(0, 0, 10 * PIPE_WAIT_NS) < PIPE_WAIT_NS / 1000, "five seconds away are not five seconds of waiting");
+static_assert(waited_ns(0, 1000, 21000, false) == 20000 && waited_ns(70, 5, 5, false) == 70, "a poll counts what it took");
+static_assert(waited_ns(0, 0, 10 * PIPE_WAIT_NS, false) < PIPE_WAIT_NS / 1000, "five seconds away are not five seconds of waiting");
+static_assert(waited_ns(PIPE_WAIT_NS - 1, 1000, 21000, true) == 0, "the time of the kernel in front is not this one's");
 
 // The rest of a wait whose first test failed.  Parked, not polled: the warps that feed a pipeline wait for most
 // of its time, and their polling was a third of the instructions the SM executed.
@@ -56,8 +60,9 @@ static __device__ __noinline__ bool mbar_wait_parked(uint32_t bar, uint32_t pari
   do {
     if (mbar_try_wait_parked(bar, parity, PIPE_PARK_NS)) return true;
     if (*abort_flag) return false;
+    const bool front = abort_flag[PIPE_FRONT] != 0;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-    waited = waited_ns(waited, before, now);
+    waited = waited_ns(waited, before, now, front);
     before = now;
   } while (waited < PIPE_WAIT_NS);
   *abort_flag = 1;

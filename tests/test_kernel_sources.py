@@ -64,3 +64,18 @@ def test_limits_of_dynamic_shared_memory_are_set_once(name):
     text = _source(name)
     for m in re.finditer(r"cudaFuncSetAttribute\(", text):
         assert re.search(r"raised\[dev\]\.load|if \(!(ctas_per_device|sms_of_device)\[dev\]\) \{", text[:m.start()][-400:])
+
+
+def test_waits_beside_the_kernel_in_front_count_no_time():
+    """The second projection of the grouped GEMM starts while the first is running, which may take longer than a wait is bounded
+    by: until its producer of the activations is past its own wait for the first, the CTA says so beside its abort flag and
+    no wait counts (pipe.cuh checks the count itself when it is compiled).  Every kernel with such waits sets both words."""
+    kernel = _body(_source("ffn_umma.cu"), "ffn_umma_kernel")
+    assert "wait_words[PIPE_FRONT] = a.phase != 0;" in kernel
+    released = [m.start() for m in re.finditer(r"abort_flag\[PIPE_FRONT\] = 0;", kernel)]
+    assert len(released) == 1 and kernel.rindex("pdl_wait();") < released[0] < kernel.index("walk.next(")
+    assert "waited_ns(waited, before, now, front)" in _body(_source("pipe.cuh"), "mbar_wait_parked")
+    for name in sorted(n for n in os.listdir(CSRC) if n.endswith(".cu")):
+        text = _source(name)
+        if re.search(r"mbar_wait(_warp|_parked)?\(", text):
+            assert "__shared__ int wait_words[PIPE_WORDS];" in text and re.search(r"wait_words\[PIPE_FRONT\] = ", text), name
