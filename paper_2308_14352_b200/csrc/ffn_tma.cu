@@ -940,13 +940,15 @@ cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, c
   if (phase_end == 2) per_expert += static_cast<long long>(a.row_blocks[1]) * ksplit;
   const long long items = active_max * per_expert;
   // Few tokens per activated expert: four warps with two tiles each, which read the activations once for both and meet a stage
-  // half as often.  Wider passes need the eight warps to hide their latencies, the sooner the shorter the rows: four warps for one token
-  // per 256 inputs on average, six at most (us per layer, eight / four warps at 2, 3, 4, 5, 6, 8 tokens per expert: 512 x 2048, 16 experts
-  // 27.0/26.8, 28.4/28.3, 29.1/29.4, 30.1/31.0, 30.4/32.4, 31.6/32.4; 768 x 3072, 32 experts 42.4/41.4, 44.4/43.7, 47.1/48.9, 48.4/51.5,
-  // 49.9/55.8; 1024 x 4096, 16 experts 42.1/40.5, 42.9/42.0, 43.4/42.4, 44.9/48.6, 45.5/50.0, 46.9/51.6; 2048 x 8192, 16 experts 80.5/76.9,
-  // 92.4/89.2, 97.3/93.6, 99.9/97.9, 102/101, 110/113; Mixtral-like layer, 8 experts 179/170, 198/189, 199/189, 204/196, 209/205).
-  const int few_mean = L.d_model / 256 < 6 ? L.d_model / 256 : 6;
-  const bool few = n_pairs <= few_mean * active_max;
+  // half as often.  Passes of more than 8 tokens need the eight warps to hide their latencies, the sooner the shorter the rows, and an uneven
+  // load has such passes at any mean.  So on rows below 1024 four warps only up to 16 pairs; beyond, for one token per 256
+  // inputs less one on average, six at most.  us per layer, eight / four warps, even and skewed (Zipf exponent 1.1) loads: 512 x 2048, 16 experts,
+  // 32 tokens 29.5/28.9 and 24.3/26.6; 768 x 3072, 32 experts, 12 tokens 36.0/34.8 and 30.5/29.8, 64 tokens 42.6/41.8 and 41.9/43.8;
+  // 1024 x 4096, 64 experts, 128 tokens 90.1/86.0 and 72.5/74.5, 256 tokens 114/116 and 96.5/100; 1536 x 5632, 32 experts, 64 tokens
+  // 89.1/86.1 and 68.1/69.9, 192 tokens 110/110 and 121/122; 2048 x 6144, 16 experts, 32 tokens 71.6/68.6 and 56.5/55.6, 80 tokens 79.5/78.6
+  // and 76.2/76.2; 3072 x 8192 gated, 8 experts, two picks, 20 tokens 109/106 and 104/102.
+  const int few_mean = L.d_model / 256 - 1 < 6 ? L.d_model / 256 - 1 : 6;
+  const bool few = n_pairs <= (L.d_model < 1024 ? 16 : few_mean * active_max);
   if (!L.scale_f16) return few ? launch_sc<SC_F32, 4>(a, items, st) : launch_sc<SC_F32, 8>(a, items, st);
   const bool pairs = L.group == 128 && a.ngroups[0] % 2 == 0 && a.ngroups[1] % 2 == 0;
   if (pairs) return few ? launch_sc<SC_PAIRS, 4>(a, items, st) : launch_sc<SC_PAIRS, 8>(a, items, st);

@@ -580,6 +580,16 @@ def test_forward_streaming_kernel_about_three_items_per_cta(f, T):
     _run_case(inputs.LayerShape(2048, f, 4, 4, "relu", "softmax_renorm", 128, "f16", "bf16"), [8, 4, 2, 4], T, seed=29, path=3)
 
 
+@pytest.mark.parametrize("act,d,k,E,T", [("relu", 768, 1, 16, 16), ("relu", 768, 1, 16, 17), ("swiglu", 512, 2, 6, 9),
+                                         ("relu", 1024, 1, 4, 12), ("relu", 1024, 1, 4, 13), ("swiglu", 1024, 2, 3, 5)])
+@pytest.mark.parametrize("skew", [0.0, 2.2])
+def test_forward_streaming_kernel_at_the_limits_of_its_four_warps(act, d, k, E, T, skew):
+    """16 pairs and the next call beyond them on short rows, a mean of three tokens per expert and beyond on rows of 1024; evenly
+    loaded and with an expert whose passes are wide."""
+    shape = inputs.LayerShape(d, 1024, E, k, act, "softmax" if k == 1 else "softmax_renorm", 128, "f16", "bf16")
+    _run_case(shape, ([8, 4, 2, 4] * E)[:E], T, seed=44, path=3, bias=(-skew * np.log(np.arange(1, E + 1))).astype(np.float32) if skew else None)
+
+
 UMMA_CASES = [
     ("relu", 128, "f16", 512, 1024, 4, 1, "softmax", [8, 4, 2, 4], 200),              # ~50 tokens per expert
     ("relu", 128, "f16", 512, 1024, 2, 1, "softmax", [4, 2], 300),                    # two token tiles per expert
