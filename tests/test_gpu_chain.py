@@ -21,6 +21,9 @@ CASES = [
     ("bf16", 40, 8, False),
     ("bf16", 40, 8, True),
     ("bf16", 200, 8, False),
+    ("bf16", 300, 48, False),   # the streaming kernel in front of two tcgen05 launches that find nobody
+    ("bf16", 300, 4, False),    # ... of the rounded tcgen05 form for most experts, whose second projection starts early
+    ("bf16", 600, 2, False),    # the rounded form alone
 ]
 
 

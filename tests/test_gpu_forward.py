@@ -660,17 +660,17 @@ def test_gated_activation_of_the_tcgen05_path():
 
 
 EXACT_CASES = [
-    # what the default takes on tcgen05 with exact codes: 256 pairs and more, rows that are not multiples of 512 or few
-    # tokens on average; router bias exponent (0: none)
+    # what the default takes on tcgen05 with exact codes for all experts: 8 tokens each on average and more from 256 pairs, rows
+    # that are not multiples of 512 or fewer than 48 tokens on average; router bias exponent (0: none)
     ("relu", 128, "f16", 640, 768, 3, 1, "softmax", [4, 2, 8], 257, 0.0),              # 64 to 128 each, partly filled boxes
     ("relu", 128, "f16", 640, 512, 1, 1, "softmax", [2], 257, 0.0),                     # five groups of 52 tokens
     ("relu", 0, "f32", 640, 1152, 1, 1, "softmax", [4], 256, 0.0),                      # per-channel scales
     ("swiglu", 256, "f16", 768, 1280, 4, 2, "softmax_renorm", [4, 8, 2, 4], 140, 0.0),  # four steps per scale
     ("swiglu", 128, "f32", 640, 1664, 2, 2, "softmax_renorm", [8, 4], 128, 0.0),
     ("relu", 128, "f16", 512, 6272, 4, 1, "softmax", [4, 2, 8, 4], 270, 0.0),           # several units per CTA
-    ("relu", 128, "f16", 512, 1024, 24, 1, "softmax", [8, 4, 2, 4] * 6, 300, 1.1),      # beside the streaming kernel
+    ("relu", 128, "f16", 512, 1024, 24, 1, "softmax", [8, 4, 2, 4] * 6, 300, 1.1),      # uneven loads, some experts without tokens
     ("swiglu", 128, "f16", 640, 640, 12, 2, "softmax_renorm", [4, 8, 2, 4] * 3, 140, 1.1),
-    ("relu", 128, "f16", 512, 512, 16, 1, "softmax", [4] * 16, 256, 0.0),               # nobody full enough
+    ("relu", 128, "f16", 512, 512, 16, 1, "softmax", [4] * 16, 256, 0.0),               # some 16 tokens each
 ]
 
 
@@ -687,6 +687,26 @@ def test_forward_default_with_some_experts_on_tcgen05_beside_the_streaming_kerne
     """Fewer than 8 tokens per expert on average, uneven loads: the experts beyond 32 tokens take the exact form, the others stream."""
     shape = inputs.LayerShape(d, f, E, k, act, "softmax" if k == 1 else "softmax_renorm", 128, "f16", "bf16")
     _run_case(shape, bits, T, seed=41, path=0, bias=(-2.2 * np.log(np.arange(1, E + 1))).astype(np.float32))
+
+
+@pytest.mark.parametrize("act,d,f,E,k,bits,T", [("relu", 512, 2048, 48, 1, [8, 4, 2, 4] * 12, 300),
+                                                ("swiglu", 640, 1024, 40, 2, [4, 8, 2, 4] * 10, 150),
+                                                ("relu", 512, 512, 128, 1, [4, 2, 8, 4] * 32, 1000)])
+def test_forward_default_with_nobody_full_enough_for_tcgen05(act, d, f, E, k, bits, T):
+    """256 pairs and more, fewer than 8 tokens per expert on average, even loads: both tcgen05 launches find nobody and leave, and what an uneven
+    call in front left in their plan is not read.  To the bit what the streaming kernel alone computes."""
+    shape = inputs.LayerShape(d, f, E, k, act, "softmax" if k == 1 else "softmax_renorm", 128, "f16", "bf16")
+    W, x = inputs.expert_set(43, 0, shape), inputs.activations(43, 0, T, d, "bf16")
+    Wr = inputs.router_weight(43, 0, d, E, std=0.05)
+    with layer.MoELayer(shape, bits, max_tokens=T) as moe:
+        moe.pack_from_host(W)
+        moe.forward(x, Wr, (-2.2 * np.log(np.arange(1, E + 1))).astype(np.float32))
+        assert B.emoe_last_expert_counts(moe.ctx, E).max() > 32
+        y, ids, gates, _ = moe.forward(x, Wr)
+        assert B.emoe_last_expert_counts(moe.ctx, E).max() <= 32
+        B.emoe_set_ffn_path(moe.ctx, 3)
+        y_stream, ids_stream, gates_stream, _ = moe.forward(x, Wr)
+    assert np.array_equal(ids, ids_stream) and np.array_equal(gates, gates_stream) and np.array_equal(y, y_stream)
 
 
 # One expert's tokens per group, at the edges of what an exact tcgen05 unit takes: boxes of 16 tokens, 32 sums per scaling thread (beyond,
