@@ -31,8 +31,8 @@ enum : int {
 };
 
 // Work plan of the persistent expert kernels, built on the device after the permutation:
-// a 16-byte header {activated experts, item counter of the first projection, of the second, 0}
-// followed by one record per activated expert, widest codes first.  `done` counts the finished
+// a 16-byte header followed by one record per activated expert, widest codes first.  The header: activated experts, two counters of
+// claimed items (ffn_tma.cu: of the second projection, in the first; ffn_i8.cu: one per projection), planes of the tcgen05 kernel's second projection.  `done` counts the finished
 // pieces of the expert's first projection (zeroed with the plan): the fused expert kernel starts
 // an expert's second projection once the count is complete.
 struct PlanRec {
@@ -54,8 +54,11 @@ struct LayerDims {
 // serialization" attribute: the next kernel of the chain may start its prologue (barrier set-up,
 // tensor-memory allocation, prefetches into L2) while the
 // current one drains.  Device side, every kernel executes pdl_wait() before it reads or writes global memory: the inputs
-// of a call, too, may be what the call in front leaves.  (One exception, which says why: ffn_umma.cu's second projection.)  pdl_trigger()
-// lets the kernel behind it start.  Without the attribute both are no-ops.
+// of a call, too, may be what the call in front leaves.  pdl_trigger() lets the kernel behind it start.  Without the attribute both are no-ops.
+// Two kernels read some of their inputs earlier: ffn_umma.cu's second projection the plan, codes and scales; ffn_gemv.cu the table of
+// experts, its second projection offsets, codes and scales too.  That is sound only because the kernel DIRECTLY in front (the first
+// projection; the permutation in front of ffn_gemv.cu's first) has executed its own pdl_wait() before its trigger: what is older than that
+// kernel is then complete.  No launch may come between, and no trigger of theirs may move in front of the wait.
 extern thread_local bool g_pdl_enabled;
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -194,11 +194,12 @@ __global__ void __launch_bounds__(DL_THREADS, 3) decode_layer_kernel(const Decod
   // the records of the experts come into shared memory while the routing runs, behind the wait for the kernels in front like
   // every other read
   const auto fetch_table = [&]() {
-    if constexpr (!TABLE) return;
-    for (int i = tid; i < min(L.E, 32) * static_cast<int>(sizeof(ExpertDev) / 8); i += DL_THREADS)
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(reinterpret_cast<uint2*>(s_table) + i))),
-                   "l"(reinterpret_cast<const uint2*>(a.experts) + i)
-                   : "memory");
+    if constexpr (TABLE) {
+      for (int i = tid; i < min(L.E, 32) * static_cast<int>(sizeof(ExpertDev) / 8); i += DL_THREADS)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(reinterpret_cast<uint2*>(s_table) + i))),
+                     "l"(reinterpret_cast<const uint2*>(a.experts) + i)
+                     : "memory");
+    }
   };
   const auto table_here = []() {
     if constexpr (TABLE) asm volatile("cp.async.wait_all;" ::: "memory");

@@ -59,14 +59,13 @@ __device__ __forceinline__ float pair_sum(f32x2 v) {
 // q + 2^(b-1).  The width is data here, not a variant of the code: with a variant per width and number of tokens the CTAs of an
 // SM ran nine loops, and a third of all cycles went into waiting for instructions.
 struct Width {
-  int bits, fields;     // 8 / bits
+  int bits;
   uint32_t mask, flip;  // of a field, and its sign bit, in every byte
   f32x2 minus;          // -(2^23 + 2^(b-1)), twice
 };
 __device__ __forceinline__ Width width_of(int bits) {
   Width w;
   w.bits = bits;
-  w.fields = 8 / bits;
   w.mask = ((1u << bits) - 1) * 0x01010101u;
   w.flip = (1u << (bits - 1)) * 0x01010101u;
   const float m = -(8388608.0f + static_cast<float>(1 << (bits - 1)));
@@ -407,7 +406,7 @@ __global__ void __launch_bounds__(GEMV_THREADS, GEMV_CTAS) ffn_gemv_kernel(const
   const ExpertDev ex = a.experts[e];
   if (a.phase == 0) {
     pdl_wait();
-    pdl_trigger();
+    pdl_trigger();  // behind the wait: the second projection relies on what it lets through being complete (common.cuh)
   }
   w.begin = __ldcg(a.off + e);
   w.cnt = __ldcg(a.off + e + 1) - w.begin;

@@ -427,7 +427,7 @@ struct Pipe {
   const unsigned char* ring;
   unsigned char* hid_stage;
   const ItemRec* queue;
-  uint32_t bar_full, bar_empty, bar_issued, bar_hid;
+  uint32_t bar_full, bar_empty, bar_hid;
   PlanRec* recs;
   bool fused;
   volatile int* abort_flag;
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(st_threads(W), ST_CTAS) ffn_tma_kernel(const _
     }
   } else {
     // ---------------- consumer warps ----------------
-    const Pipe pp = {ring, hid_stage, queue, bar_full, bar_empty, bar_issued, bar_hid, recs, fused, abort_flag};
+    const Pipe pp = {ring, hid_stage, queue, bar_full, bar_empty, bar_hid, recs, fused, abort_flag};
     // A finished first-projection item is counted one stage late: by then its stores have long
     // been acknowledged and the fence in front of the count costs nothing.  It is never held back
     // across a wait, because the stage waited for may be the one that waits for this count.

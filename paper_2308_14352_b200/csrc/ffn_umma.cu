@@ -459,7 +459,8 @@ __device__ __forceinline__ void set_sync(int part) { asm volatile("bar.sync %0, 
 // Groups of up to 64 tokens, four sets of accumulators in turn, steps of 128 inputs (the usual scale group).  What bounds it is the
 // hand-over between the roles, hence: two issuing warps; every other unit to the other set of scaling warps, whose
 // epilogue then hides behind the next unit; two runs read at a time; scales asked for two groups ahead; activations in boxes of 16
-// tokens (boxes of 64 were four times the L2 traffic at few tokens).  One set of scaling warps of 64 tokens each: 10 us more at 4096 x
+// tokens (boxes of 64 were four times the L2 traffic at few tokens).  Its 20 warps leave 96 registers a thread, of which 40 bytes
+// spill (none in the rounded form's 142).  One set of scaling warps of 64 tokens each: 10 us more at 4096 x
 // 14336 and at 768 x 3072 alike; three sets of dequantising warps: nothing.
 // us per layer, before -> after: 768 x 3072, 32 experts, 512 tokens 84.7 -> 65.9, 777 tokens 90.7 -> 74.5, 2048 tokens 121 -> 99
 // (and 64.9 and 90 with the early start of the second projection); Mixtral-like layer, 23 tokens 440 -> 242 (231).
@@ -516,6 +517,7 @@ __global__ void __launch_bounds__(Um<EXACT>::THREADS, 1)
   // but its hidden values: the plan was complete before the first started (it waits itself before it lets this one in), so only
   // the producer of the activations waits, and codes, scales and dequantisation are under way where the first has left an SM
   // (768 x 3072, 32 experts, 777 tokens: 72.8 -> 64.9 us per layer; Mixtral-like layer, 64 tokens 257 -> 241).
+  // (where the plan may be empty, everybody has waited above, in both launches)
   if (a.phase == 0) pdl_wait();
   else __threadfence();  // nothing that an earlier kernel left in this SM's L1 is taken for the plan
   pdl_trigger();

@@ -79,3 +79,26 @@ def test_waits_beside_the_kernel_in_front_count_no_time():
         text = _source(name)
         if re.search(r"mbar_wait(_warp|_parked)?\(", text):
             assert "__shared__ int wait_words[PIPE_WORDS];" in text and re.search(r"wait_words\[PIPE_FRONT\] = ", text), name
+
+
+def test_reads_in_front_of_the_wait_rest_on_a_kernel_that_waited_before_its_trigger():
+    """The CUDA-core kernel and the second tcgen05 projection read inputs before griddepcontrol.wait: those are older than the kernel
+    directly in front, which has to have waited before it lets this one start, and nothing is launched between."""
+    permute = _body(_source("route.cu"), "permute_kernel")
+    assert permute.index("pdl_wait();") < permute.index("pdl_trigger();")
+    gemv = _body(_source("ffn_gemv.cu"), "ffn_gemv_kernel")
+    first = gemv.index("if (a.phase == 0)")
+    assert re.findall(r"pdl_\w+", gemv) == ["pdl_wait", "pdl_trigger"] * 2 and gemv.index("pdl_wait") > first
+    assert re.findall(r"a\.(?:experts|off|x|perm|hidden|o)\b", gemv[:first]) == ["a.experts"]
+    umma = _body(_source("ffn_umma.cu"), "ffn_umma_kernel")
+    empty, rest = umma[:umma.index("UmBars b;")], umma[umma.index("UmBars b;"):]
+    assert empty.index("pdl_wait();") < empty.index("a.plan") < empty.index("return;")  # with this wait the others are no-ops
+    assert rest.index("if (a.phase == 0) pdl_wait();") < rest.index("pdl_trigger();") < rest.index("walk.open(a.plan")
+    for name in ("api.cu", "noalloc.cu"):
+        launches = re.findall(r"launch_(\w+)\((\d?)", _source(name))
+        for i, launch in enumerate(launches):
+            if launch == ("ffn_gemv", "0"):
+                assert launches[i + 1] == ("ffn_gemv", "1")
+            if launch == ("ffn_umma", "0"):
+                assert launches[i + 1] == ("ffn_umma", "1")
+        assert ("ffn_gemv", "0") in launches
