@@ -374,7 +374,8 @@ typedef struct emoe_cache_stats {
   int64_t prefetch_redundant; /* prefetch requests for experts already in a slot */
   int64_t prefetch_refused;   /* prefetch requests dropped because every slot was in use */
   int64_t evictions;
-  int64_t bytes_copied;       /* host -> device bytes of all loads started */
+  int64_t bytes_copied;       /* host -> device bytes of all loads started (emoe_cached_layer counts as the single calls do, also
+                                 a preload whose slot goes to a load on demand before its copy is enqueued) */
   int64_t exposed_copy_ns;    /* device time the compute stream stood still inside emoe_cache_acquire, waiting for
                                  slot contents (loading not hidden under compute: Section 3.3, the pipeline's
                                  failed-prediction case); counted only while emoe_cache_set_timing is on */
