@@ -468,10 +468,10 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
       EMOE_LAUNCH(ctx, launch_scatter_x(L, table, x, ids_use, perm, off, plan, plan_heavy, xs, nullptr, P, 1, heavy_above, ctx->check_word, st));
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
     if (ctx->fuse_projections) {
-      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, true, ctx->check_word, st));
     } else {
-      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
-      EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, tmaps, xs, plan, hidden, o_part, ksplit, P, true, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, true, ctx->check_word, st));
     }
     EMOE_LAUNCH(ctx, launch_ffn_umma(0, L, tmaps, plan_heavy, xs, xs_stride, hidden, hid_stride, o_part, P, 1, exact_umma, exact_umma, ctx->check_word, st));
     EMOE_LAUNCH(ctx, launch_ffn_umma(1, L, tmaps, plan_heavy, hidden, hid_stride, hidden, hid_stride, o_part, P, zmax, exact_umma, exact_umma, ctx->check_word, st));
@@ -533,16 +533,16 @@ int forward_impl(emoe_ctx* ctx, const emoe_layer_desc* desc, const void* x, int 
     if (ev[0]) EMOE_CUDA(ctx, cudaEventRecord(ev[0], st));
     if (ctx->fuse_projections) {
       // one launch: an expert's second projection starts when its hidden vectors are complete
-      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, false, ctx->check_word, st));
       if (ev[1]) {  // one interval only: the end event of the triple stays unused
         EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
         ctx->events_one_launch[ctx->events_used / 3 - 1] = 1;
         ev[2] = nullptr;
       }
     } else {
-      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(0, 1, L, tmaps, xs, plan, hidden, o_part, ksplit, P, false, ctx->check_word, st));
       if (ev[1]) EMOE_CUDA(ctx, cudaEventRecord(ev[1], st));
-      EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, ctx->check_word, st));
+      EMOE_LAUNCH(ctx, launch_ffn_tma(1, 2, L, tmaps, xs, plan, hidden, o_part, ksplit, P, false, ctx->check_word, st));
     }
   } else if (use_mma) {
     ksplit = ffn_mma_ksplit(L, T);

@@ -172,9 +172,9 @@ int ffn_tma_ksplit(const LayerDims& L, int T);
 int encode_weight_tmap(void* out_map, const void* packed, int N, int K, int bits);
 // Phases [phase_begin, phase_end) of the FFN in one launch: (0,1) first projection, (1,2) second,
 // (0,2) both, the second projection of an expert starting as soon as its hidden vectors are complete.
-// xs / hidden: activation tiles (act_tile.cuh).
+// xs / hidden: activation tiles (act_tile.cuh).  uneven: the experts' numbers of tokens differ much (how the work is handed out).
 cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, const void* tmaps, const void* xs, int* plan,
-                           void* hidden, float* o_part, int ksplit, int n_pairs, int* check_word, cudaStream_t st);
+                           void* hidden, float* o_part, int ksplit, int n_pairs, bool uneven, int* check_word, cudaStream_t st);
 
 // The weight-streaming kernel on 8-bit integer tensor-core operands (tcgen05 kind::i8, accumulators
 // and unpacked codes in tensor memory).  xq / hq: activations as two-limb block-scaled integers

@@ -95,6 +95,7 @@ struct TmaArgs {
   int ngroups[2];     // scale groups per row, per projection
   unsigned gmul;      // scale group of segment s: (s * gmul) >> 20 (2^20 / segments per group, rounded up; 0: one group per row)
   int n_pairs;
+  int claim_above;    // items of the second projection per CTA beyond which they are claimed
   int* check_word;
   // floor(2^32 / d) + 1 for the divisors of the item index, per projection: n / d = umulhi(n, magic) for the
   // small n and d met here (n * d < 2^32), instead of an integer division in front of every item's first copy
@@ -621,14 +622,17 @@ __global__ void __launch_bounds__(st_threads(W), ST_CTAS) ffn_tma_kernel(const _
     // computing warps: whatever it does per stage is kept to a few instructions.
     // Every CTA takes every n-th item of the first projection and, going on so, one of the second; these are known without
     // asking and decoded 32 at a time.  From then on whoever is free claims the next one (one claim ahead, so that nobody
-    // waits for the answer).  Up to three items of the second projection per CTA the fixed shares go on to the end: a claimed
+    // waits for the answer).  Up to three items of the second projection per CTA (one beside the tcgen05 kernel, where few experts are left
+    // to stream and have 1 to 32 tokens each) the fixed shares go on to the end: a claimed
     // item is decoded alone, in front of its first copy, and the shares are as even as claims could make them (us per layer, fixed /
     // claimed, at 1.7 to 2 items per CTA: 1024 x 4096, 8 experts, 64 tokens 36.4/39.4; 768 x 3072, 16 experts, 96 tokens 37.1/39.7;
     // 512 x 2048, 32 experts, 192 tokens 35.0/36.9; at 3.5 to 4: 2048 x 8192, 4 experts, 16 tokens 48.1/46.9, 768 x 3072, 32 experts, 192
-    // tokens 53.0/49.9, Mixtral-like layer, 8 tokens 188/179).
+    // tokens 53.0/49.9, Mixtral-like layer, 8 tokens 188/179; beside the tcgen05 kernel, Zipf exponent 1.1: 1024 x 4096, 64 experts, 300 tokens
+    // 101/98, 500 tokens 109/110, 128 experts, 1000 tokens 144/140, 1280 x 4480, 128 experts, 1000 tokens 210/200; even loads there leave
+    // more than three).
     const int n = static_cast<int>(gridDim.x), me = static_cast<int>(blockIdx.x);
     const int n_items0 = a.phase_begin == 0 ? s_active * a.row_blocks[0] : 0, n_items1 = a.phase_end == 2 ? s_active * a.row_blocks[1] * a.ksplit : 0;
-    const bool claims = n_items1 > 3 * n;
+    const bool claims = n_items1 > a.claim_above * n;
     const int n_fixed = n_items0 + (claims ? n : n_items1);
     int it = 0, oldest = 0, head = 0, phys = 0;
     int more = 1, claim = n_items1;
@@ -908,7 +912,7 @@ int ffn_tma_ksplit(const LayerDims& L, int T) {
 }
 
 cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, const void* tmaps, const void* xs, int* plan,
-                           void* hidden, float* o_part, int ksplit, int n_pairs, int* check_word, cudaStream_t st) {
+                           void* hidden, float* o_part, int ksplit, int n_pairs, bool uneven, int* check_word, cudaStream_t st) {
   if (phase_begin < 0 || phase_end > 2 || phase_begin >= phase_end) return cudaErrorInvalidValue;
   const int rows_first = L.act == EMOE_ACT_SWIGLU ? ST_BOX_ROWS : 2 * ST_BOX_ROWS;
   TmaArgs a;
@@ -927,6 +931,7 @@ cudaError_t launch_ffn_tma(int phase_begin, int phase_end, const LayerDims& L, c
   a.ngroups[1] = L.group > 0 ? L.d_ff / L.group : 1;
   a.gmul = L.group > 0 ? ((1u << 20) + static_cast<unsigned>(L.group / 128) - 1) / static_cast<unsigned>(L.group / 128) : 0u;
   a.n_pairs = n_pairs;
+  a.claim_above = uneven ? 1 : 3;
   a.check_word = check_word;
   for (int p = 0; p < 2; ++p) {
     const int ks = p == 0 ? 1 : ksplit;

@@ -709,6 +709,30 @@ def test_forward_default_with_nobody_full_enough_for_tcgen05(act, d, f, E, k, bi
     assert np.array_equal(ids, ids_stream) and np.array_equal(gates, gates_stream) and np.array_equal(y, y_stream)
 
 
+def test_forward_claims_items_early_beside_tcgen05():
+    """Beside the tcgen05 kernel the second projection's items are claimed from one per CTA on: with up to three of them, a token whose expert
+    streams has to the bit what the streaming kernel alone gives it, whose CTAs take fixed shares."""
+    d, f, E, T = 1024, 2048, 64, 300
+    shape = inputs.LayerShape(d, f, E, 1, "relu", "softmax", 128, "f16", "bf16")
+    x, Wr = inputs.activations(45, 0, T, d, "bf16"), inputs.router_weight(45, 0, d, E, std=0.05)
+    bias = (-1.6 * np.log(np.arange(1, E + 1))).astype(np.float32)
+    with layer.MoELayer(shape, [8, 4, 2, 4] * 16, max_tokens=T) as moe:
+        gen = torch.Generator(device="cuda").manual_seed(45)
+        for e in range(E):
+            for m in range(2):
+                moe.pack_matrix(e, m, torch.randn(*shape.matrix_shape(m), generator=gen, device="cuda") * 0.02)
+        y, ids, _, _ = moe.forward(x, Wr, bias)
+        counts = B.emoe_last_expert_counts(moe.ctx, E)
+        B.emoe_set_ffn_path(moe.ctx, 3)
+        y_stream, ids_stream, _, _ = moe.forward(x, Wr, bias)
+    streams = (counts > 0) & (counts <= 32)
+    assert 2 * 148 < streams.sum() * (d // 128) * (f // 512) <= 3 * 2 * 148 and counts.max() > 32
+    assert np.array_equal(ids, ids_stream)
+    light = streams[ids[:, 0]]
+    assert np.array_equal(y[light], y_stream[light])
+    assert rel_to_max(y, y_stream) <= 2 * output_tolerance("bf16")  # either is within the bar of the definition
+
+
 # One expert's tokens per group, at the edges of what an exact tcgen05 unit takes: boxes of 16 tokens, 32 sums per scaling thread (beyond,
 # both sets of scaling warps share a unit), groups of 64; steps per scale: one (two issuers), two and three (one issuer), a whole row;
 # an odd number of units and of steps, so that the sets of accumulators, stages and scaling warps meet every parity.
